@@ -137,14 +137,17 @@ class Clocks:
 # slices of 256 x 64, keyed "kernel@batch"; coarse: one slice of 128 x 32; the
 # stage-kernel traffic summary in profiles/), valid only while the kernel
 # sources are those that were captured.
-NCU_TRAFFIC_SOURCES = ("paper_2001_01609_gb300/csrc/rbc_kernels.cu", "paper_2001_01609_gb300/csrc/rbc_internal.h")
-NCU_TRAFFIC_SHA256 = "bccf5326cefa87d23c30c873735b605116d20294072d2c0e5a25ffdcbd076c31"
+NCU_TRAFFIC_SOURCES = (
+    "paper_2001_01609_gb300/csrc/rbc_kernels.cu",
+    "paper_2001_01609_gb300/csrc/rbc_rows_fx.cu",
+    "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
+    "paper_2001_01609_gb300/csrc/rbc_internal.h",
+)
+NCU_TRAFFIC_SHA256 = "14b5cb7099fd2f3c67d58d101e9c8d4854ffc574521d322c5bde380c822e2e24"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 130202, "coarse:k_rows": 483123, "coarse:k_zfwd": 116864, "coarse:k_solve": 826752,
-    "fine:k_zinv@32": 8907264, "fine:k_rows@32": 56720845, "fine:k_zfwd@32": 12620800, "fine:k_solve@32": 23538240,
-    # batch of 2 with the heuristic shapes (the clustered row kernel; the tuned one-block-per-row
-    # kernel reads and writes the same rows)
-    "fine:k_zinv@2": 661350, "fine:k_rows@2": 3586304, "fine:k_zfwd@2": 821824, "fine:k_solve@2": 2441088,
+    "coarse:k_zinv": 127437, "coarse:k_rows": 400026, "coarse:k_zfwd": 118144, "coarse:k_solve": 827264,
+    "fine:k_zinv@32": 8581376, "fine:k_rows@32": 37900288, "fine:k_zfwd@32": 12622080, "fine:k_solve@32": 23538880,
+    "fine:k_zinv@2": 662118, "fine:k_rows@2": 2501325, "fine:k_zfwd@2": 821376, "fine:k_solve@2": 2441728,
 }
 
 

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -111,6 +112,61 @@ Mat lobatto_interp(int N, const std::vector<double>& theta) {
       W[(size_t)n * N + j] = 2.0 / (N - 1) * std::cos(n * theta[j]) / (cn * cj);
     }
   return W;
+}
+
+// ---------------------------------------------------------------------------
+// Fixed-point tables (62 fractional bits), in double-double arithmetic: the
+// same integers on every host.
+// ---------------------------------------------------------------------------
+struct DD {
+  double h, l;
+};
+DD dd_fast(double a, double b) {
+  const double s = a + b;
+  return {s, b - (s - a)};
+}
+DD dd_add(DD a, DD b) {
+  const double s = a.h + b.h, t = s - a.h;
+  const double e = (a.h - (s - t)) + (b.h - t);
+  return dd_fast(s, e + (a.l + b.l));
+}
+DD dd_mul(DD a, DD b) {
+  const double p = a.h * b.h, e = std::fma(a.h, b.h, -p);
+  return dd_fast(p, e + (a.h * b.l + a.l * b.h));
+}
+DD dd_div(DD a, double b) {
+  const double q = a.h / b;
+  const double r = std::fma(-q, b, a.h) + a.l;
+  return dd_fast(q, r / b);
+}
+long long q62(DD v) {
+  const double x = std::ldexp(v.h, 62), f = std::floor(x);
+  return (long long)f + std::llround((x - f) + std::ldexp(v.l, 62));
+}
+// cos and sin of 2 pi t / N (0 <= t < N), by quadrant, the Taylor series in [0, pi/4]
+void q62_cos_sin(int t, int N, long long* c, long long* s) {
+  const int quad = (int)((4LL * t) / N);
+  int rem = (int)(4LL * t - (long long)quad * N);   // angle = (pi / 2) (quad + rem / N)
+  const bool swap = 2 * rem > N;
+  if (swap) rem = N - rem;
+  const DD half_pi{1.5707963267948966, 6.123233995736766e-17};
+  const DD x = dd_div(dd_mul(half_pi, {(double)rem, 0.0}), (double)N);
+  DD term{1.0, 0.0}, cs{0.0, 0.0}, sn{0.0, 0.0};
+  for (int k = 0; k <= 26; ++k) {   // term = x^k / k!
+    if (k > 0) term = dd_div(dd_mul(term, x), k);
+    DD& acc = (k & 1) ? sn : cs;
+    acc = dd_add(acc, (k & 2) ? DD{-term.h, -term.l} : term);
+  }
+  const long long a = q62(swap ? sn : cs), b = q62(swap ? cs : sn);
+  const long long cc[4] = {a, -b, -a, b}, ss[4] = {b, a, -b, -a};
+  *c = cc[quad];
+  *s = ss[quad];
+}
+// v = h 2^32 + l with |l| < 2^31, as w[0] = h, w[1] = l
+void q_halves(long long v, int* w) {
+  if ((int)v == INT32_MIN) ++v;
+  w[1] = (int)v;
+  w[0] = (int)((v - w[1]) >> 32);
 }
 
 // ---------------------------------------------------------------------------
@@ -659,7 +715,7 @@ static rbc_status upload_tables(rbc_t h) {
   }
   Mat Wn = lobatto_interp(N, thn);
 
-  add(zinv); add(zfwd); add(cc); add(tw); add(s2); add(s4); add(mp);
+  add(zinv); add(zfwd); add(cc); add(s2); add(s4); add(mp);
   add(Tb); add(Td); add(TDi); add(TL); add(Ti);
   add(Pb); add(Pd); add(PDi); add(PL); add(Pi);
   add(Ub); add(Ud); add(UDi); add(UL_); add(Ui);
@@ -684,6 +740,22 @@ static rbc_status upload_tables(rbc_t h) {
     add(packed);
   };
   add_f32(zinv); add_f32(zfwd); add_f32(tw);
+  {
+    // fixed-point twiddles of the FP64 mode's x FFTs and 2 / k of the x-means
+    std::vector<double> twfx(g.mixed ? 0 : (size_t)2 * g.Mx);
+    for (int t = 0; t < (int)twfx.size() / 2; ++t) {
+      long long cq, sq;
+      q62_cos_sin(t, g.Mx, &cq, &sq);
+      int w[4];
+      q_halves(cq, w);
+      q_halves(-sq, w + 2);
+      memcpy(&twfx[(size_t)2 * t], w, sizeof(w));
+    }
+    add(twfx);
+    std::vector<double> rk(nm, 0.0);
+    for (int m = 1; m < nm; ++m) rk[m] = 2.0 / (g.kfac * m);
+    add(rk);
+  }
   add(Tinv); add(Pinv); add(Uinv);
   // tensor-core z-inverse operator images (mixed precision only)
   const bool tc = g.mixed && tc_zinv_supported(g);
@@ -717,7 +789,6 @@ static rbc_status upload_tables(rbc_t h) {
   T.zinv = b + offs[i++];
   T.zfwd = b + offs[i++];
   T.cc = b + offs[i++];
-  T.tw = reinterpret_cast<const double2*>(b + offs[i++]);
   T.s2 = b + offs[i++];
   T.s4 = b + offs[i++];
   T.mp = b + offs[i++];
@@ -733,6 +804,8 @@ static rbc_status upload_tables(rbc_t h) {
   T.zinv32 = reinterpret_cast<const float*>(b + offs[i++]);
   T.zfwd32 = reinterpret_cast<const float*>(b + offs[i++]);
   T.tw32 = reinterpret_cast<const float2*>(b + offs[i++]);
+  T.twfx = reinterpret_cast<const int4*>(b + offs[i++]);
+  T.rk = b + offs[i++];
   T.T_inv = dense ? b + offs[i] : nullptr;
   ++i;
   T.P_inv = dense ? b + offs[i] : nullptr;

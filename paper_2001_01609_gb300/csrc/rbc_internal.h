@@ -51,7 +51,6 @@ struct Tables {
   const double* zinv;   // [4][Mz][Nz]  d^q T_n / ds^q at the padded Lobatto points, q = 0..3
   const double* zfwd;   // [Nz][Mz]     padded Lobatto values -> T coefficients n < Nz
   const double* cc;     // [Mz]         Clenshaw-Curtis weights on the padded points
-  const double2* tw;    // [Mx]         exp(-2 pi i t / Mx)
   const double* s2;     // [2][nq][3]   C^(2) conversion S1 S0, tau row t, columns q = t..t+2
   const double* s4;     // [2][nq][5]   C^(4) conversion S3 S2 S1 S0, columns q = t..t+4
   const double* mp;     // [2][nq][5][nm] psi mass operator lap_k in C^(4)
@@ -76,7 +75,11 @@ struct Tables {
   // FP32 copies of the transform tables (RBC_MIXED)
   const float* zinv32;  // [4][Mz][Nz]
   const float* zfwd32;  // [Nz][Mz]
-  const float2* tw32;   // [Mx]
+  const float2* tw32;   // [Mx]         exp(-2 pi i t / Mx)
+  // x FFTs of the FP64 mode: the same twiddles with 62 fractional bits, each part
+  // as signed 32-bit halves (re hi, re lo, im hi, im lo; part = hi 2^32 + lo)
+  const int4* twfx;     // [Mx]
+  const double* rk;     // [nm]         2 / k_m (0 for m = 0): Parseval sums of the x-means
   // tensor-core z-inverse operands (RBC_MIXED): TF32 hi/lo images of the
   // interleaved operator rows, pre-swizzled per 128-row tile and 32-wide K-chunk
   const float *tcA_psi_hi, *tcA_psi_lo, *tcA_T_hi, *tcA_T_lo;
@@ -118,9 +121,9 @@ struct Shapes {
   int solve_tms = 0;   // Fourier modes per k_solve block (power of two, <= 16)
   int zfwd_tm = 0;     // Fourier modes per k_zfwd block (power of two, <= 32)
   int zfwd_nch = 0;    // chunks of the n range per k_zfwd block (1, 2, 4, 8)
-  int rows_cl = -1;    // 1: the clustered row kernel, 0: one block per row
-  int rows_threads = 0;   // threads of a k_rows block (256, 512 or 1024)
-  int rows_lean = -1;  // 1: k_rows with 5 + 3 shared rows, 0: 5 + 5 (where either fits)
+  int rows_cl = -1;    // 1: the clustered row kernel (FP64: one row per block), 0: one block per row (FP64: full blocks)
+  int rows_threads = 0;   // threads of a k_rows block (256, 512 or 1024; FP64: at most 384 are used)
+  int rows_lean = -1;  // 1: k_rows with 5 + 3 shared rows, 0: 5 + 5 (where either fits; FP64: one layout)
 };
 
 // Per-call workspace pointers (capacity >= B states).
@@ -128,7 +131,7 @@ struct Work {
   double* Xs;      // stage state, B states
   double* F;       // explicit-term coefficients, B states
   double* R;       // RK accumulators, [B][4] states (tau rows in the coefficient slots)
-  double* Z;       // z-inverse output, [B][9][Mz][nm] complex (FP64, or FP32 in the first half)
+  double* Z;       // z-inverse output, [B][6][Mz][nm] complex in FP64, [B][9][Mz][nm] in FP32 (mixed)
   double* Q;       // row-kernel output, [B][2][Mz][nm] complex (FP64 or FP32)
   double* wT;      // [B][Mz] x-mean of w T
   int* maxs;       // [1] max over nsteps, right before nsteps (copied with it)
@@ -185,7 +188,9 @@ inline cudaError_t launch_pdl(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 blo
 #define RBC_HD
 #endif
 RBC_HD inline size_t state_doubles(const Grid& g) { return (size_t)2 * g.Nz * g.nm * 2; }
-RBC_HD inline size_t z_doubles(const Grid& g) { return (size_t)9 * g.Mz * g.nm * 2; }
+// z-inverse output: six FP64 fields (u, w, d_x omega, d_z omega, d_x T, d_z T); the nine
+// FP32 fields of the mixed mode take less
+RBC_HD inline size_t z_doubles(const Grid& g) { return (size_t)6 * g.Mz * g.nm * 2; }
 RBC_HD inline size_t q_doubles(const Grid& g) { return (size_t)2 * g.Mz * g.nm * 2; }
 
 // ---- launchers (rbc_kernels.cu) ----
@@ -227,7 +232,9 @@ int correct_norm_blocks(const Grid& gf);
 cudaError_t launch_correct_norm(const Grid& gf, const Grid& gc, const Tables& tf, int mode, const double* Ff,
                                 const double* Gnew, double* Gold, double* C, const double* Uprev, double* U,
                                 double* Fnext, double* partial, unsigned* counter, double* norms, cudaStream_t s);
-size_t rows_smem_bytes(const Grid& g);
+// row kernel of the FP64 mode (rbc_rows_fx.cu)
+cudaError_t configure_rows_fx(const Grid& g);
+cudaError_t launch_rows_fx(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
 // whether a launch shape can run on this grid (shared memory, threads)
 bool shapes_valid(const Grid& g, const Shapes& sh, size_t es);
 size_t static_scratch_doubles_needed(const Grid& g);

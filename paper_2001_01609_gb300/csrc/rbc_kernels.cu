@@ -185,18 +185,21 @@ __device__ __forceinline__ C2<T> zinv_field(int f, int m, T k, const C2<T>* P, C
 }
 
 // Fields of one output row (j, m); half = 0: fields 0-3, 1: fields 4-8, -1: all.
+// FP32 keeps all nine; FP64 keeps 0-3, d_x T (diag: T itself) and d_z T, which
+// are all that its row kernel (diag: the averages of Sec. 2.2) reads.
 template <typename T>
 __device__ __forceinline__ void zinv_store(const Grid& g, T* Zb, int j, int m, T k, const C2<T>* P, C2<T> t0,
-                                           C2<T> t1, int half) {
+                                           C2<T> t1, int half, bool diag) {
   const size_t fs = (size_t)g.Mz * g.nm * 2;
   T* zb = Zb + ((size_t)j * g.nm + m) * 2;
-  const int f0 = half == 1 ? 4 : 0, f1 = half == 0 ? 4 : 9;
-  for (int f = f0; f < f1; ++f) stc<T>(zb + f * fs, zinv_field<T>(f, m, k, P, t0, t1));
+  const int f0 = half == 1 ? 4 : 0, f1 = half == 0 ? 4 : sizeof(T) == 8 ? 6 : 9;
+  for (int f = f0; f < f1; ++f)
+    stc<T>(zb + f * fs, zinv_field<T>(sizeof(T) == 4 || f < 4 ? f : f == 5 ? 8 : diag ? 6 : 7, m, k, P, t0, t1));
 }
 
 template <typename T>
 __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
-                          T* __restrict__ Z, int B, const int* nsteps, int stepidx, int blk, int kp) {
+                          T* __restrict__ Z, int B, const int* nsteps, int stepidx, int blk, int kp, bool diag) {
   using V = C2<T>;
   extern __shared__ __align__(16) unsigned char zsm[];
   V* part = reinterpret_cast<V*>(zsm);                 // [kp][12][32] when kp > 1
@@ -246,7 +249,7 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
     }
   }
   const T k = (T)(g.kfac * m);
-  T* Zb = Z + (size_t)b * 9 * g.Mz * g.nm * 2;
+  T* Zb = Z + (size_t)b * (sizeof(T) == 8 ? 6 : 9) * g.Mz * g.nm * 2;
   const int jr = g.Mz - 1 - j;
   if (kp > 1) {
     if (wact) {
@@ -281,11 +284,11 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
       if (row == 0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) P[q] = Ev[q] + Ov[q];
-        zinv_store<T>(g, Zb, j, m, k, P, Ev[4] + Ov[4], Ev[5] + Ov[5], half);
+        zinv_store<T>(g, Zb, j, m, k, P, Ev[4] + Ov[4], Ev[5] + Ov[5], half, diag);
       } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q) P[q] = ((q & 1) ? (T)-1 : (T)1) * (Ev[q] - Ov[q]);
-        zinv_store<T>(g, Zb, jr, m, k, P, Ev[4] - Ov[4], (T)-1 * (Ev[5] - Ov[5]), half);
+        zinv_store<T>(g, Zb, jr, m, k, P, Ev[4] - Ov[4], (T)-1 * (Ev[5] - Ov[5]), half, diag);
       }
     }
     return;
@@ -294,19 +297,19 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
   V P[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) P[q] = E[q] + O[q];
-  zinv_store<T>(g, Zb, j, m, k, P, E[4] + O[4], E[5] + O[5], -1);
+  zinv_store<T>(g, Zb, j, m, k, P, E[4] + O[4], E[5] + O[5], -1, diag);
   if (jr != j) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) P[q] = ((q & 1) ? (T)-1 : (T)1) * (E[q] - O[q]);
-    zinv_store<T>(g, Zb, jr, m, k, P, E[4] - O[4], (T)-1 * (E[5] - O[5]), -1);
+    zinv_store<T>(g, Zb, jr, m, k, P, E[4] - O[4], (T)-1 * (E[5] - O[5]), -1, diag);
   }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_zinv(Grid g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
-                                              T* __restrict__ Z, int B, const int* nsteps, const int* step) {
+                                              T* __restrict__ Z, int B, const int* nsteps, const int* step, bool diag) {
   pdl_wait();
-  zinv_item<T>(g, Bz, X, S, Z, B, nsteps, nsteps ? *step : 0, blockIdx.x, blockDim.x / 32);
+  zinv_item<T>(g, Bz, X, S, Z, B, nsteps, nsteps ? *step : 0, blockIdx.x, blockDim.x / 32, diag);
 }
 
 // Warps sharing the coefficient sum of one k_zinv row pair.  It fixes the order
@@ -400,7 +403,6 @@ static bool rows_batched(const Grid& g, size_t es) { return rows_bytes_batched(g
 static size_t rows_smem_for(const Grid& g, size_t es, bool lean) {
   return rows_batched(g, es) ? (lean ? rows_bytes_lean(g, es) : rows_bytes_batched(g, es)) : rows_bytes_serial(g, es);
 }
-size_t rows_smem_bytes(const Grid& g) { return rows_smem_for(g, 8, false); }
 // The lean layout by default where the full one leaves room for a single block
 // per SM and the lean one for two.
 static bool rows_lean_default(const Grid& g, size_t es) {
@@ -1308,14 +1310,16 @@ void Prof::end(int k, cudaStream_t s, double fl, double by) {
 
 // Algorithmic work of one launch over B slices (all active).
 static double zinv_flops(const Grid& g, int B) { return 24.0 * B * ((g.Mz + 1) / 2) * g.nm * g.Nz; }
-static double zinv_bytes(const Grid& g, int B, size_t es = 8) {
-  return 8.0 * B * state_doubles(g) + (double)es * B * z_doubles(g);
+// (nf z-inverse fields of es-byte reals; nfft x FFTs per row)
+static double z_reals(const Grid& g, int nf) { return 2.0 * nf * g.Mz * g.nm; }
+static double zinv_bytes(const Grid& g, int B, int nf, size_t es) {
+  return 8.0 * B * state_doubles(g) + (double)es * B * z_reals(g, nf);
 }
-static double rows_flops(const Grid& g, int B) {
-  return (double)B * g.Mz * (6.0 * 5.0 * g.Mx * std::log2((double)g.Mx) + 10.0 * g.Mx);
+static double rows_flops(const Grid& g, int B, int nfft) {
+  return (double)B * g.Mz * (nfft * 5.0 * g.Mx * std::log2((double)g.Mx) + 10.0 * g.Mx);
 }
-static double rows_bytes(const Grid& g, int B, size_t es = 8) {
-  return (double)es * B * (z_doubles(g) + q_doubles(g)) + 8.0 * B * g.Mz;
+static double rows_bytes(const Grid& g, int B, int nf, size_t es) {
+  return (double)es * B * (z_reals(g, nf) + q_doubles(g)) + 8.0 * B * g.Mz;
 }
 static double zfwd_flops(const Grid& g, int B) { return 4.0 * B * g.Nz * g.nm * ((g.Mz + 1) / 2) * 2.0; }
 static double zfwd_bytes(const Grid& g, int B, size_t es = 8) {
@@ -1339,12 +1343,9 @@ static cudaError_t allow_smem(F* fn, int need, int& allowed) {
 }
 
 cudaError_t configure_kernels(const Grid& g) {
-  static int a_rows_d = 48 * 1024, a_rows_f = 48 * 1024, a_solve = 48 * 1024;
-  static int a_zfwd_d = 48 * 1024, a_zfwd_f = 48 * 1024;
-  static int a_rcl_d = 48 * 1024, a_rcl_f = 48 * 1024;
-  cudaError_t e = allow_smem(k_rows<double>, (int)rows_smem_for(g, 8, false), a_rows_d);
-  if (e == cudaSuccess && rows_cl_bytes(g, 8) <= 200 * 1024)
-    e = allow_smem(k_rows_cl<double>, (int)rows_cl_bytes(g, 8), a_rcl_d);
+  static int a_rows_f = 48 * 1024, a_solve = 48 * 1024, a_zfwd_d = 48 * 1024, a_zfwd_f = 48 * 1024;
+  static int a_rcl_f = 48 * 1024;
+  cudaError_t e = g.mixed ? cudaSuccess : configure_rows_fx(g);
   if (e == cudaSuccess && rows_cl_bytes(g, 4) <= 200 * 1024)
     e = allow_smem(k_rows_cl<float>, (int)rows_cl_bytes(g, 4), a_rcl_f);
   if (e == cudaSuccess) e = allow_smem(k_rows<float>, (int)rows_smem_for(g, 4, false), a_rows_f);
@@ -1357,31 +1358,44 @@ cudaError_t configure_kernels(const Grid& g) {
   return e;
 }
 
-template <typename T>
-static void launch_transforms_in(const Grid& g, const Tables& t, const T* Bz, const C2<T>* tw, const Work& w,
-                                 const double* X, int B, const int* ns, Prof* pf, cudaStream_t s) {
-  const size_t S = state_doubles(g);
+// FP32 transforms (mixed): z inverse and row kernel.
+static void launch_transforms_f32(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
+                                  Prof* pf, cudaStream_t s) {
   const int kp = zinv_warps(g);
   const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
-  T* Z = reinterpret_cast<T*>(w.Z);
-  T* Q = reinterpret_cast<T*>(w.Q);
+  float* Z = reinterpret_cast<float*>(w.Z);
+  float* Q = reinterpret_cast<float*>(w.Q);
+  const size_t es = sizeof(float);
   if (pf) pf->begin(RBC_KERNEL_ZINV, s);
-  if (sizeof(T) == 4 && t.tcA_psi_hi != nullptr)
+  if (t.tcA_psi_hi != nullptr)
     launch_zinv_tc(g, t, w, X, B, ns, s);              // tensor cores, TF32 with split compensation
   else
-    launch_pdl(w.pdl != 0, k_zinv<T>, zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * sizeof(T) : 0, s, g, Bz, X,
-               S, Z, B, ns, w.step);
-  if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, sizeof(T)));
-  const size_t es = sizeof(T);
+    launch_pdl(w.pdl != 0, k_zinv<float>, zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * es : 0, s, g, t.zinv32, X,
+               state_doubles(g), Z, B, ns, w.step, false);
+  if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 9, es));
   if (pf) pf->begin(RBC_KERNEL_ROWS, s);
   if (rows_cl_of(g, w, B, es))
-    launch_pdl(w.pdl != 0, k_rows_cl<T>, (unsigned)(B * g.Mz * kRowsCluster), kRowsThreads, rows_cl_bytes(g, es), s,
-               g, tw, Z, Q, w.wT, B, ns, w.step);
+    launch_pdl(w.pdl != 0, k_rows_cl<float>, (unsigned)(B * g.Mz * kRowsCluster), kRowsThreads, rows_cl_bytes(g, es), s,
+               g, t.tw32, Z, Q, w.wT, B, ns, w.step);
   else
-    launch_pdl(w.pdl != 0, k_rows<T>, (unsigned)(B * g.Mz), rows_threads_of(w),
-               rows_smem_for(g, es, rows_lean_of(g, w, es)), s, g, tw, Z, Q, w.wT, B, rows_batched(g, es) ? 1 : 0,
+    launch_pdl(w.pdl != 0, k_rows<float>, (unsigned)(B * g.Mz), rows_threads_of(w),
+               rows_smem_for(g, es, rows_lean_of(g, w, es)), s, g, t.tw32, Z, Q, w.wT, B, rows_batched(g, es) ? 1 : 0,
                rows_lean_of(g, w, es) ? 1 : 0, ns, w.step);
-  if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B), rows_bytes(g, B, sizeof(T)));
+  if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B, 6), rows_bytes(g, B, 9, es));
+}
+
+// FP64: z inverse, and the row kernel in fixed point (three inverse FFTs and one forward).
+static void launch_transforms_f64(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
+                                  Prof* pf, cudaStream_t s) {
+  const int kp = zinv_warps(g);
+  const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
+  if (pf) pf->begin(RBC_KERNEL_ZINV, s);
+  launch_pdl(w.pdl != 0, k_zinv<double>, zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * sizeof(double) : 0, s, g,
+             t.zinv, X, state_doubles(g), w.Z, B, ns, w.step, false);
+  if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 6, sizeof(double)));
+  if (pf) pf->begin(RBC_KERNEL_ROWS, s);
+  launch_rows_fx(g, t, w, B, ns, s);
+  if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B, 4), rows_bytes(g, B, 6, sizeof(double)));
 }
 
 cudaError_t launch_explicit(const Grid& g, const Tables& t, const Work& w, const double* X, int B, bool all_active,
@@ -1389,9 +1403,9 @@ cudaError_t launch_explicit(const Grid& g, const Tables& t, const Work& w, const
   const int* ns = all_active ? nullptr : w.nsteps;
   Prof* pf = (w.prof && w.prof->on && !all_active) ? w.prof : nullptr;
   if (g.mixed)
-    launch_transforms_in<float>(g, t, t.zinv32, t.tw32, w, X, B, ns, pf, s);
+    launch_transforms_f32(g, t, w, X, B, ns, pf, s);
   else
-    launch_transforms_in<double>(g, t, t.zinv, t.tw, w, X, B, ns, pf, s);
+    launch_transforms_f64(g, t, w, X, B, ns, pf, s);
   count(2);
   return cudaGetLastError();
 }
@@ -1499,8 +1513,7 @@ cudaError_t launch_nusselt(const Grid& g, const Tables& t, const Work& w, const 
 }
 
 // Consistency-check averages of Sec. 2.2, pass 1.  Z holds the FP64 z inverse
-// of every state (fields u, w, d_x omega, d_z omega, ..., T, ... at the padded
-// rows).  Block per (state, padded row j): x-means by Parseval over the kept
+// of every state (fields u, w, d_x omega, d_z omega, T at the padded rows).  Block per (state, padded row j): x-means by Parseval over the kept
 // modes (weight 1 for m = 0, 2 otherwise; Re(a conj b) for a pair of fields):
 //   u^2 + w^2,   u.lap u = -u d_z omega + w d_x omega,   w T,
 //   (T - <T>_x)^2 (modes m >= 1),   <T>_x = Re T_0(s_j).
@@ -1509,13 +1522,13 @@ __global__ void __launch_bounds__(128) k_diag_rows(Grid g, const double* __restr
   __shared__ double red[128];
   const int b = blockIdx.x / g.Mz, j = blockIdx.x - b * g.Mz;
   const size_t fs = (size_t)g.Mz * g.nm * 2;
-  const double* zb = Z + (size_t)b * 9 * fs + (size_t)j * g.nm * 2;
+  const double* zb = Z + (size_t)b * 6 * fs + (size_t)j * g.nm * 2;
   double ke = 0.0, ep = 0.0, wt = 0.0, tv = 0.0;
   for (int m = threadIdx.x; m < g.nm; m += blockDim.x) {
     const double c = m == 0 ? 1.0 : 2.0;
     const double2 u = ld2(zb + 2 * m), w = ld2(zb + fs + 2 * m);
     const double2 dxo = ld2(zb + 2 * fs + 2 * m), dzo = ld2(zb + 3 * fs + 2 * m);
-    const double2 t = ld2(zb + 6 * fs + 2 * m);
+    const double2 t = ld2(zb + 4 * fs + 2 * m);
     ke += c * (u.x * u.x + u.y * u.y + w.x * w.x + w.y * w.y);
     ep += c * (w.x * dxo.x + w.y * dxo.y - u.x * dzo.x - u.y * dzo.y);
     wt += c * (w.x * t.x + w.y * t.y);
@@ -1531,7 +1544,7 @@ __global__ void __launch_bounds__(128) k_diag_rows(Grid g, const double* __restr
     r[g.Mz] = ep;
     r[2 * g.Mz] = wt;
     r[3 * g.Mz] = tv;
-    r[4 * g.Mz] = zb[6 * fs];
+    r[4 * g.Mz] = zb[4 * fs];
   }
 }
 
@@ -1584,7 +1597,7 @@ cudaError_t launch_diagnostics(const Grid& g, const Tables& t, const Work& w, co
   const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
   // FP64 z inverse of all states (no step mask), whatever the handle's precision
   k_zinv<double><<<zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * sizeof(double) : 0, s>>>(
-      g, t.zinv, X, state_doubles(g), w.Z, B, nullptr, w.step);
+      g, t.zinv, X, state_doubles(g), w.Z, B, nullptr, w.step, true);
   k_diag_rows<<<(unsigned)(B * g.Mz), 128, 0, s>>>(g, w.Z, w.Q);
   k_diag_final<<<(unsigned)B, 128, 0, s>>>(g, t.cc, X, w.Q, out);
   count(3);
@@ -1999,8 +2012,10 @@ static std::atomic<double*> g_static_ptr[kMaxDevices] = {};
 
 // Layout: Z, Q, the <wT>_x profile (Mz rounded up to even), then 8 doubles:
 // the three Nusselt numbers and, in the fifth, the int error bits of the call.
+// The admission bound counts nine FP64 z-inverse fields (the header's 132 Nx Nz
+// bytes), so the grids it refuses do not depend on how many the kernels keep.
 size_t static_scratch_doubles_needed(const Grid& g) {
-  return z_doubles(g) + q_doubles(g) + (size_t)((g.Mz + 1) & ~1) + 8;
+  return z_doubles(g) / 6 * 9 + q_doubles(g) + (size_t)((g.Mz + 1) & ~1) + 8;
 }
 
 cudaError_t launch_nusselt_static(const Grid& g, const Tables& t, const double* X, double* host_out3,

@@ -1,0 +1,51 @@
+"""The transform kernels at the edges of their sizes, against the FP64 oracle.
+
+One step of every row length (Nx = 4 .. 1024: one, two and three passes per
+FFT) and batch size (several rows per block, a ragged last block).
+Tolerances: FP64 1e-12 relative to the largest coefficient, ten times the
+largest difference of the two implementations' roundings seen on these grids;
+FP32 products 1e-5, the bound of the mixed mode's parity tests.
+"""
+import numpy as np
+import pytest
+
+from layout import from_abi, max_rel_diff, to_abi
+from oracle.rbc import RBC
+from paper_2001_01609_gb300.inputs import initial_temperature
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore::DeprecationWarning")]
+
+
+@pytest.fixture(scope="module")
+def rbc():
+    from paper_2001_01609_gb300 import build
+    build.build()
+    from paper_2001_01609_gb300 import rbc as r
+    r.load()
+    return r
+
+
+def nonlinear_state(o, seed):
+    X = o.from_grid(initial_temperature(o.Nx, o.Nz, seed=seed, amplitude=0.3, Lx=o.Lx))
+    X, _ = o.step(X)
+    return X
+
+
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-5)])
+@pytest.mark.parametrize("Nx", [4, 8, 16, 32, 64, 128, 256, 512, 1024])
+def test_every_row_length_matches_oracle(rbc, Nx, precision, tol):
+    Nz, Ra, dt = 10, 1e5, 1e-4
+    o = RBC(Ra, 1.0, 2.0, Nx, Nz, dt)
+    F = rbc.Propagator(Ra, 1.0, 2.0, Nx, Nz, dt, precision)
+    Xs = [nonlinear_state(o, s) for s in range(3)]
+    st = F.new_states(3)
+    for b, X in enumerate(Xs):
+        st[b].copy_(torch.from_numpy(to_abi(X)))
+    nu = torch.zeros(3, dtype=torch.float64, device="cuda")
+    F.step_batch(st, [2, 0, 1], nu)
+    assert F.check_diverged() == rbc.RBC_OK
+    for b, n in enumerate([2, 0, 1]):
+        ref, integ = o.run(Xs[b], n)
+        assert max_rel_diff(from_abi(st[b].cpu().numpy()), ref) < tol
+        assert abs(nu[b].item() - integ) <= tol * max(abs(integ), 1e-30)
