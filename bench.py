@@ -140,14 +140,15 @@ class Clocks:
 NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_kernels.cu",
     "paper_2001_01609_gb300/csrc/rbc_rows_fx.cu",
+    "paper_2001_01609_gb300/csrc/rbc_zfx.cu",
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "14b5cb7099fd2f3c67d58d101e9c8d4854ffc574521d322c5bde380c822e2e24"
+NCU_TRAFFIC_SHA256 = "9bb111593476e43ea3b14d93377113fdd3c47d447289a7c490818b9979c4d1ef"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 127437, "coarse:k_rows": 400026, "coarse:k_zfwd": 118144, "coarse:k_solve": 827264,
-    "fine:k_zinv@32": 8581376, "fine:k_rows@32": 37900288, "fine:k_zfwd@32": 12622080, "fine:k_solve@32": 23538880,
-    "fine:k_zinv@2": 662118, "fine:k_rows@2": 2501325, "fine:k_zfwd@2": 821376, "fine:k_solve@2": 2441728,
+    "coarse:k_zinv": 122573, "coarse:k_rows": 398541, "coarse:k_zfwd": 118848, "coarse:k_solve": 826944,
+    "fine:k_zinv@32": 8598016, "fine:k_rows@32": 37895424, "fine:k_zfwd@32": 12627776, "fine:k_solve@32": 23542784,
+    "fine:k_zinv@2": 653517, "fine:k_rows@2": 2506701, "fine:k_zfwd@2": 826368, "fine:k_solve@2": 2442368,
 }
 
 

@@ -143,24 +143,34 @@ long long q62(DD v) {
   const double x = std::ldexp(v.h, 62), f = std::floor(x);
   return (long long)f + std::llround((x - f) + std::ldexp(v.l, 62));
 }
-// cos and sin of 2 pi t / N (0 <= t < N), by quadrant, the Taylor series in [0, pi/4]
-void q62_cos_sin(int t, int N, long long* c, long long* s) {
-  const int quad = (int)((4LL * t) / N);
-  int rem = (int)(4LL * t - (long long)quad * N);   // angle = (pi / 2) (quad + rem / N)
-  const bool swap = 2 * rem > N;
-  if (swap) rem = N - rem;
-  const DD half_pi{1.5707963267948966, 6.123233995736766e-17};
-  const DD x = dd_div(dd_mul(half_pi, {(double)rem, 0.0}), (double)N);
+// cos and sin of (pi / 2) rem / N, 0 <= rem <= N / 2, by the Taylor series
+void q62_octant(int rem, int N, long long* c, long long* s) {
+  const DD x = dd_div(dd_mul({1.5707963267948966, 6.123233995736766e-17}, {(double)rem, 0.0}), (double)N);
   DD term{1.0, 0.0}, cs{0.0, 0.0}, sn{0.0, 0.0};
-  for (int k = 0; k <= 26; ++k) {   // term = x^k / k!
+  for (int k = 0; k <= 20; ++k) {   // term = x^k / k!, below 2^-70 at k = 21
     if (k > 0) term = dd_div(dd_mul(term, x), k);
     DD& acc = (k & 1) ? sn : cs;
     acc = dd_add(acc, (k & 2) ? DD{-term.h, -term.l} : term);
   }
-  const long long a = q62(swap ? sn : cs), b = q62(swap ? cs : sn);
-  const long long cc[4] = {a, -b, -a, b}, ss[4] = {b, a, -b, -a};
-  *c = cc[quad];
-  *s = ss[quad];
+  *c = q62(cs);
+  *s = q62(sn);
+}
+// cos and sin of 2 pi t / N, 0 <= t < N, interleaved
+std::vector<long long> q62_circle(int N) {
+  std::vector<long long> out((size_t)2 * N), oct((size_t)2 * (N / 2 + 1), -1);   // cos >= 0 once known
+  for (int t = 0; t < N; ++t) {
+    const int quad = (int)((4LL * t) / N);
+    int rem = (int)(4LL * t - (long long)quad * N);   // angle = (pi / 2) (quad + rem / N)
+    const bool swap = 2 * rem > N;
+    if (swap) rem = N - rem;
+    long long* o = &oct[(size_t)2 * rem];
+    if (o[0] < 0) q62_octant(rem, N, o, o + 1);
+    const long long a = o[swap ? 1 : 0], b = o[swap ? 0 : 1];
+    const long long cc[4] = {a, -b, -a, b}, ss[4] = {b, a, -b, -a};
+    out[2 * t] = cc[quad];
+    out[2 * t + 1] = ss[quad];
+  }
+  return out;
 }
 // v = h 2^32 + l with |l| < 2^31, as w[0] = h, w[1] = l
 void q_halves(long long v, int* w) {
@@ -715,7 +725,7 @@ static rbc_status upload_tables(rbc_t h) {
   }
   Mat Wn = lobatto_interp(N, thn);
 
-  add(zinv); add(zfwd); add(cc); add(s2); add(s4); add(mp);
+  add(cc); add(s2); add(s4); add(mp);
   add(Tb); add(Td); add(TDi); add(TL); add(Ti);
   add(Pb); add(Pd); add(PDi); add(PL); add(Pi);
   add(Ub); add(Ud); add(UDi); add(UL_); add(Ui);
@@ -743,18 +753,27 @@ static rbc_status upload_tables(rbc_t h) {
   {
     // fixed-point twiddles of the FP64 mode's x FFTs and 2 / k of the x-means
     std::vector<double> twfx(g.mixed ? 0 : (size_t)2 * g.Mx);
-    for (int t = 0; t < (int)twfx.size() / 2; ++t) {
-      long long cq, sq;
-      q62_cos_sin(t, g.Mx, &cq, &sq);
+    const std::vector<long long> cs = q62_circle(g.mixed ? 0 : g.Mx);
+    for (size_t t = 0; t < cs.size() / 2; ++t) {
       int w[4];
-      q_halves(cq, w);
-      q_halves(-sq, w + 2);
-      memcpy(&twfx[(size_t)2 * t], w, sizeof(w));
+      q_halves(cs[2 * t], w);
+      q_halves(-cs[2 * t + 1], w + 2);
+      memcpy(&twfx[2 * t], w, sizeof(w));
     }
     add(twfx);
     std::vector<double> rk(nm, 0.0);
     for (int m = 1; m < nm; ++m) rk[m] = 2.0 / (g.kfac * m);
     add(rk);
+  }
+  {
+    // fixed-point z transforms
+    std::vector<int> A, Ae, G, W, We;
+    zfx_build(g, zinv.data(), zfwd.data(), A, Ae, G, W, We);
+    for (const std::vector<int>* v : {&A, &Ae, &G, &W, &We}) {
+      std::vector<double> packed((v->size() + 1) / 2, 0.0);
+      memcpy(packed.data(), v->data(), v->size() * sizeof(int));
+      add(packed);
+    }
   }
   add(Tinv); add(Pinv); add(Uinv);
   // tensor-core z-inverse operator images (mixed precision only)
@@ -786,8 +805,6 @@ static rbc_status upload_tables(rbc_t h) {
   const double* b = h->d_tables;
   int i = 0;
   Tables& T = h->t;
-  T.zinv = b + offs[i++];
-  T.zfwd = b + offs[i++];
   T.cc = b + offs[i++];
   T.s2 = b + offs[i++];
   T.s4 = b + offs[i++];
@@ -806,6 +823,11 @@ static rbc_status upload_tables(rbc_t h) {
   T.tw32 = reinterpret_cast<const float2*>(b + offs[i++]);
   T.twfx = reinterpret_cast<const int4*>(b + offs[i++]);
   T.rk = b + offs[i++];
+  T.zfxA = reinterpret_cast<const int2*>(b + offs[i++]);
+  T.zfxAe = reinterpret_cast<const int*>(b + offs[i++]);
+  T.zfxG = reinterpret_cast<const int4*>(b + offs[i++]);
+  T.zfxW = reinterpret_cast<const int2*>(b + offs[i++]);
+  T.zfxWe = reinterpret_cast<const int*>(b + offs[i++]);
   T.T_inv = dense ? b + offs[i] : nullptr;
   ++i;
   T.P_inv = dense ? b + offs[i] : nullptr;

@@ -48,8 +48,14 @@ inline double t_wall_rhs(const Grid& g, int p) {
 // Parity-split tables are laid out [p][row][j][m] so that threads with
 // consecutive Fourier index m read consecutive addresses.
 struct Tables {
-  const double* zinv;   // [4][Mz][Nz]  d^q T_n / ds^q at the padded Lobatto points, q = 0..3
-  const double* zfwd;   // [Nz][Mz]     padded Lobatto values -> T coefficients n < Nz
+  // z transforms of the FP64 mode (and of the Sec. 2.2 averages) in fixed point,
+  // see rbc_zfx.cu: entries as halves (h, l), h 2^30 + l; Kp, Kh: nq and
+  // ceil(Mz/2) padded to a multiple of eight, Mh = ceil(Mz/2)
+  const int2* zfxA;     // [Mh][2][Kp][4]  d^q T_n / ds^q 2^-G_q(n) at the padded points, n = 2 k + parity
+  const int* zfxAe;     // [4][Mh]         exponent of each row
+  const int4* zfxG;     // [Nz]            G_q(n), q = 0..3
+  const int2* zfxW;     // [Nz][Kh]        padded Lobatto values -> T coefficients
+  const int* zfxWe;     // [Nz]            exponent of each row
   const double* cc;     // [Mz]         Clenshaw-Curtis weights on the padded points
   const double* s2;     // [2][nq][3]   C^(2) conversion S1 S0, tau row t, columns q = t..t+2
   const double* s4;     // [2][nq][5]   C^(4) conversion S3 S2 S1 S0, columns q = t..t+4
@@ -253,6 +259,14 @@ void scheme_tableau(int scheme, double AE[5][5], double AI[5][5], int* ns, doubl
 cudaError_t upload_schemes();
 constexpr int kProfileSampleSteps = 8;     // steps recorded kernel by kernel in a sampled call
 cudaError_t configure_kernels(const Grid& g);
+// z transforms in fixed point (rbc_zfx.cu); diag: T in place of d_x T
+cudaError_t configure_zfx(const Grid& g);
+cudaError_t launch_zinv_fx(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
+                           bool diag, cudaStream_t s);
+cudaError_t launch_zfwd_fx(const Grid& g, const Tables& t, const Work& w, int B, cudaStream_t s);
+// tables from the FP64 matrices zinv[4][Mz][Nz] and zfwd[Nz][Mz], as ints in the layouts of Tables
+void zfx_build(const Grid& g, const double* zinv, const double* zfwd, std::vector<int>& A, std::vector<int>& Ae,
+               std::vector<int>& G, std::vector<int>& W, std::vector<int>& We);
 // tensor-core z inverse transform (rbc_tcgen05.cu)
 RBC_HD int tc_zinv_mtiles(const Grid& g, int nops);
 RBC_HD int tc_zinv_kchunks(const Grid& g);

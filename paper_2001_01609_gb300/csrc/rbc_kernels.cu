@@ -185,21 +185,18 @@ __device__ __forceinline__ C2<T> zinv_field(int f, int m, T k, const C2<T>* P, C
 }
 
 // Fields of one output row (j, m); half = 0: fields 0-3, 1: fields 4-8, -1: all.
-// FP32 keeps all nine; FP64 keeps 0-3, d_x T (diag: T itself) and d_z T, which
-// are all that its row kernel (diag: the averages of Sec. 2.2) reads.
 template <typename T>
 __device__ __forceinline__ void zinv_store(const Grid& g, T* Zb, int j, int m, T k, const C2<T>* P, C2<T> t0,
-                                           C2<T> t1, int half, bool diag) {
+                                           C2<T> t1, int half) {
   const size_t fs = (size_t)g.Mz * g.nm * 2;
   T* zb = Zb + ((size_t)j * g.nm + m) * 2;
-  const int f0 = half == 1 ? 4 : 0, f1 = half == 0 ? 4 : sizeof(T) == 8 ? 6 : 9;
-  for (int f = f0; f < f1; ++f)
-    stc<T>(zb + f * fs, zinv_field<T>(sizeof(T) == 4 || f < 4 ? f : f == 5 ? 8 : diag ? 6 : 7, m, k, P, t0, t1));
+  const int f0 = half == 1 ? 4 : 0, f1 = half == 0 ? 4 : 9;
+  for (int f = f0; f < f1; ++f) stc<T>(zb + f * fs, zinv_field<T>(f, m, k, P, t0, t1));
 }
 
 template <typename T>
 __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
-                          T* __restrict__ Z, int B, const int* nsteps, int stepidx, int blk, int kp, bool diag) {
+                          T* __restrict__ Z, int B, const int* nsteps, int stepidx, int blk, int kp) {
   using V = C2<T>;
   extern __shared__ __align__(16) unsigned char zsm[];
   V* part = reinterpret_cast<V*>(zsm);                 // [kp][12][32] when kp > 1
@@ -249,7 +246,7 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
     }
   }
   const T k = (T)(g.kfac * m);
-  T* Zb = Z + (size_t)b * (sizeof(T) == 8 ? 6 : 9) * g.Mz * g.nm * 2;
+  T* Zb = Z + (size_t)b * 9 * g.Mz * g.nm * 2;
   const int jr = g.Mz - 1 - j;
   if (kp > 1) {
     if (wact) {
@@ -284,11 +281,11 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
       if (row == 0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) P[q] = Ev[q] + Ov[q];
-        zinv_store<T>(g, Zb, j, m, k, P, Ev[4] + Ov[4], Ev[5] + Ov[5], half, diag);
+        zinv_store<T>(g, Zb, j, m, k, P, Ev[4] + Ov[4], Ev[5] + Ov[5], half);
       } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q) P[q] = ((q & 1) ? (T)-1 : (T)1) * (Ev[q] - Ov[q]);
-        zinv_store<T>(g, Zb, jr, m, k, P, Ev[4] - Ov[4], (T)-1 * (Ev[5] - Ov[5]), half, diag);
+        zinv_store<T>(g, Zb, jr, m, k, P, Ev[4] - Ov[4], (T)-1 * (Ev[5] - Ov[5]), half);
       }
     }
     return;
@@ -297,19 +294,19 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
   V P[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) P[q] = E[q] + O[q];
-  zinv_store<T>(g, Zb, j, m, k, P, E[4] + O[4], E[5] + O[5], -1, diag);
+  zinv_store<T>(g, Zb, j, m, k, P, E[4] + O[4], E[5] + O[5], -1);
   if (jr != j) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) P[q] = ((q & 1) ? (T)-1 : (T)1) * (E[q] - O[q]);
-    zinv_store<T>(g, Zb, jr, m, k, P, E[4] - O[4], (T)-1 * (E[5] - O[5]), -1, diag);
+    zinv_store<T>(g, Zb, jr, m, k, P, E[4] - O[4], (T)-1 * (E[5] - O[5]), -1);
   }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_zinv(Grid g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
-                                              T* __restrict__ Z, int B, const int* nsteps, const int* step, bool diag) {
+                                              T* __restrict__ Z, int B, const int* nsteps, const int* step) {
   pdl_wait();
-  zinv_item<T>(g, Bz, X, S, Z, B, nsteps, nsteps ? *step : 0, blockIdx.x, blockDim.x / 32, diag);
+  zinv_item<T>(g, Bz, X, S, Z, B, nsteps, nsteps ? *step : 0, blockIdx.x, blockDim.x / 32);
 }
 
 // Warps sharing the coefficient sum of one k_zinv row pair.  It fixes the order
@@ -1343,16 +1340,15 @@ static cudaError_t allow_smem(F* fn, int need, int& allowed) {
 }
 
 cudaError_t configure_kernels(const Grid& g) {
-  static int a_rows_f = 48 * 1024, a_solve = 48 * 1024, a_zfwd_d = 48 * 1024, a_zfwd_f = 48 * 1024;
+  static int a_rows_f = 48 * 1024, a_solve = 48 * 1024, a_zfwd_f = 48 * 1024;
   static int a_rcl_f = 48 * 1024;
-  cudaError_t e = g.mixed ? cudaSuccess : configure_rows_fx(g);
+  cudaError_t e = configure_zfx(g);   // also the averages of Sec. 2.2 of a mixed handle
+  if (e == cudaSuccess && !g.mixed) e = configure_rows_fx(g);
   if (e == cudaSuccess && rows_cl_bytes(g, 4) <= 200 * 1024)
     e = allow_smem(k_rows_cl<float>, (int)rows_cl_bytes(g, 4), a_rcl_f);
   if (e == cudaSuccess) e = allow_smem(k_rows<float>, (int)rows_smem_for(g, 4, false), a_rows_f);
   if (e == cudaSuccess)
     e = allow_smem(k_solve, (int)std::max(solve_smem(g, 1), solve_smem(g, 1 << 20)), a_solve);
-  if (e == cudaSuccess)
-    e = allow_smem(k_zfwd<double>, (int)std::max(zfwd_smem(g, 1, 8), zfwd_smem(g, 1 << 20, 8)), a_zfwd_d);
   if (e == cudaSuccess)
     e = allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f);
   return e;
@@ -1371,7 +1367,7 @@ static void launch_transforms_f32(const Grid& g, const Tables& t, const Work& w,
     launch_zinv_tc(g, t, w, X, B, ns, s);              // tensor cores, TF32 with split compensation
   else
     launch_pdl(w.pdl != 0, k_zinv<float>, zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * es : 0, s, g, t.zinv32, X,
-               state_doubles(g), Z, B, ns, w.step, false);
+               state_doubles(g), Z, B, ns, w.step);
   if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 9, es));
   if (pf) pf->begin(RBC_KERNEL_ROWS, s);
   if (rows_cl_of(g, w, B, es))
@@ -1384,14 +1380,11 @@ static void launch_transforms_f32(const Grid& g, const Tables& t, const Work& w,
   if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B, 6), rows_bytes(g, B, 9, es));
 }
 
-// FP64: z inverse, and the row kernel in fixed point (three inverse FFTs and one forward).
+// FP64: the transforms and products in fixed point (three inverse FFTs and one forward).
 static void launch_transforms_f64(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
                                   Prof* pf, cudaStream_t s) {
-  const int kp = zinv_warps(g);
-  const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
   if (pf) pf->begin(RBC_KERNEL_ZINV, s);
-  launch_pdl(w.pdl != 0, k_zinv<double>, zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * sizeof(double) : 0, s, g,
-             t.zinv, X, state_doubles(g), w.Z, B, ns, w.step, false);
+  launch_zinv_fx(g, t, w, X, B, ns, false, s);
   if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 6, sizeof(double)));
   if (pf) pf->begin(RBC_KERNEL_ROWS, s);
   launch_rows_fx(g, t, w, B, ns, s);
@@ -1410,17 +1403,14 @@ cudaError_t launch_explicit(const Grid& g, const Tables& t, const Work& w, const
   return cudaGetLastError();
 }
 
-template <typename T>
-static void launch_zfwd(const Grid& g, const T* W, const Work& w, int B, Prof* pf, cudaStream_t s) {
-  const size_t S = state_doubles(g), es = sizeof(T);
+static void launch_zfwd_f32(const Grid& g, const Tables& t, const Work& w, int B, cudaStream_t s) {
+  const size_t S = state_doubles(g), es = sizeof(float);
   const int tm = zfwd_tm_of(g, w, B, es);
   const int mt = (g.nm + tm - 1) / tm;
   const int nch = zfwd_nch_of(g, w, B, tm);
   const size_t smem = (size_t)2 * ((g.Mz + 1) / 2) * tm * 2 * es;
-  if (pf) pf->begin(RBC_KERNEL_ZFWD, s);
-  launch_pdl(w.pdl != 0, k_zfwd<T>, (unsigned)(B * 2 * mt * nch), 128, smem, s, g, W, reinterpret_cast<const T*>(w.Q),
-             w.F, S, B, tm, nch, w.nsteps, w.step);
-  if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, es));
+  launch_pdl(w.pdl != 0, k_zfwd<float>, (unsigned)(B * 2 * mt * nch), 128, smem, s, g, t.zfwd32,
+             reinterpret_cast<const float*>(w.Q), w.F, S, B, tm, nch, w.nsteps, w.step);
 }
 
 cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* X, int B, int stage, double* nu,
@@ -1430,15 +1420,14 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   cudaError_t e = launch_explicit(g, t, w, Xin, B, false, s);
   if (e != cudaSuccess) return e;
   Prof* pf = (w.prof && w.prof->on) ? w.prof : nullptr;
-  if (g.mixed && t.tcW_hi[0] != nullptr) {
-    // tensor cores, TF32 with split compensation
-    if (pf) pf->begin(RBC_KERNEL_ZFWD, s);
-    launch_zfwd_tc(g, t, w, B, s);
-    if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, 4));
-  } else if (g.mixed)
-    launch_zfwd<float>(g, t.zfwd32, w, B, pf, s);
+  if (pf) pf->begin(RBC_KERNEL_ZFWD, s);
+  if (g.mixed && t.tcW_hi[0] != nullptr)
+    launch_zfwd_tc(g, t, w, B, s);                     // tensor cores, TF32 with split compensation
+  else if (g.mixed)
+    launch_zfwd_f32(g, t, w, B, s);
   else
-    launch_zfwd<double>(g, t.zfwd, w, B, pf, s);
+    launch_zfwd_fx(g, t, w, B, s);
+  if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, g.mixed ? 4 : 8));
   const int tms = solve_tms_of(g, w, B);
   const int mtiles = (g.nm + tms - 1) / tms;
   if (pf) pf->begin(RBC_KERNEL_SOLVE, s);
@@ -1593,11 +1582,9 @@ __global__ void __launch_bounds__(128) k_diag_final(Grid g, const double* __rest
 cudaError_t launch_diagnostics(const Grid& g, const Tables& t, const Work& w, const double* X, int B, double* out,
                                cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
-  const int kp = zinv_warps(g);
-  const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
   // FP64 z inverse of all states (no step mask), whatever the handle's precision
-  k_zinv<double><<<zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * sizeof(double) : 0, s>>>(
-      g, t.zinv, X, state_doubles(g), w.Z, B, nullptr, w.step, true);
+  cudaError_t e = launch_zinv_fx(g, t, w, X, B, nullptr, true, s);
+  if (e != cudaSuccess) return e;
   k_diag_rows<<<(unsigned)(B * g.Mz), 128, 0, s>>>(g, w.Z, w.Q);
   k_diag_final<<<(unsigned)B, 128, 0, s>>>(g, t.cc, X, w.Q, out);
   count(3);
