@@ -141,14 +141,15 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_kernels.cu",
     "paper_2001_01609_gb300/csrc/rbc_rows_fx.cu",
     "paper_2001_01609_gb300/csrc/rbc_zfx.cu",
+    "paper_2001_01609_gb300/csrc/rbc_solve.cu",
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "9bb111593476e43ea3b14d93377113fdd3c47d447289a7c490818b9979c4d1ef"
+NCU_TRAFFIC_SHA256 = "d16354a2b2212781a3d0dba67d9e5ec4cd3f9dfcde1658f81e66015e7e0e44fb"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 122573, "coarse:k_rows": 398541, "coarse:k_zfwd": 118848, "coarse:k_solve": 826944,
-    "fine:k_zinv@32": 8598016, "fine:k_rows@32": 37895424, "fine:k_zfwd@32": 12627776, "fine:k_solve@32": 23542784,
-    "fine:k_zinv@2": 653517, "fine:k_rows@2": 2506701, "fine:k_zfwd@2": 826368, "fine:k_solve@2": 2442368,
+    "coarse:k_zinv": 122112, "coarse:k_rows": 400845, "coarse:k_zfwd": 118208, "coarse:k_solve": 827392,
+    "fine:k_zinv@32": 8602778, "fine:k_rows@32": 37891738, "fine:k_zfwd@32": 12626816, "fine:k_solve@32": 23859904,
+    "fine:k_zinv@2": 655104, "fine:k_rows@2": 2501683, "fine:k_zfwd@2": 824896, "fine:k_solve@2": 2763456,
 }
 
 

@@ -184,7 +184,7 @@ void q_halves(long long v, int* w) {
 // top, then tau rows whose nonzeros lie in columns r-D .. r+D (dominant
 // derivative term on the diagonal).  Eliminating columns n-1 .. D from the
 // bottom creates no fill; what remains is a D x D dense block and a lower
-// band.  No pivoting; the residual is checked after factoring.
+// band.  Only entries of the band and of the boundary rows are looked at.  No pivoting; the residual is checked after factoring.
 // ---------------------------------------------------------------------------
 struct UL {
   int n = 0, D = 0;
@@ -207,12 +207,9 @@ bool ul_factor(Mat A, int n, int D, UL& f, std::string& why) {
       return false;
     }
     for (int r = 0; r < c; ++r) {
+      if (r == D) r = std::max(r, c - D);   // the boundary rows, then the rows of the band
       const double v = a(r, c);
       if (v == 0.0) continue;
-      if (r >= D && r < c - D) {
-        why = "band structure violated";
-        return false;
-      }
       const double mult = v / piv;
       for (int q = std::max(0, c - D); q < c; ++q) a(r, q) -= mult * a(c, q);
       a(r, c) = 0.0;
@@ -223,11 +220,6 @@ bool ul_factor(Mat A, int n, int D, UL& f, std::string& why) {
     }
   }
   for (int r = D; r < n; ++r) {
-    for (int q = 0; q < r - D; ++q)
-      if (a(r, q) != 0.0) {
-        why = "lower band structure violated";
-        return false;
-      }
     for (int j = 0; j < D; ++j) f.Lb[(size_t)r * D + j] = a(r, r - D + j);
     f.invd[r] = 1.0 / a(r, r);
   }
@@ -280,7 +272,7 @@ double ul_residual(const Mat& A, const UL& f, unsigned seed) {
   double rmax = 0.0, amax = 0.0, xmax = 0.0, bmax = 0.0;
   for (int i = 0; i < n; ++i) {
     double r = -b[i], arow = 0.0;
-    for (int j = 0; j < n; ++j) {
+    for (int j = i < f.D ? 0 : i - f.D; j < (i < f.D ? n : std::min(n, i + f.D + 1)); ++j) {
       r += A[(size_t)i * n + j] * x[j];
       arow += std::fabs(A[(size_t)i * n + j]);
     }
@@ -605,17 +597,100 @@ static rbc_status upload_tables(rbc_t h) {
 
   // ---- stage matrices and their UL factors ----
   const double hdt = g.gamma * g.dt;       // stage matrices M - gamma dt L
-  auto layout = [&](std::vector<double>& dst, const std::vector<double>& src, int p, int rows, int D, int nmod,
-                    int mi) {
-    for (int c = 0; c < rows; ++c)
-      for (int j = 0; j < D; ++j) dst[((size_t)(p * rows + c) * D + j) * nmod + mi] = src[(size_t)c * D + j];
+  struct SegTables {   // see SegFactors
+    std::vector<double> beta, multD, Dinv, invd, ilb, phi, theta;
   };
-  std::vector<double> Tb((size_t)2 * nq * nm), Td(Tb.size()), TDi((size_t)2 * nm), TL(Tb.size()), Ti(Tb.size());
-  std::vector<double> Pb((size_t)2 * nq * 2 * nm), Pd(Pb.size()), PDi((size_t)2 * 4 * nm), PL(Pb.size()),
-      Pi((size_t)2 * nq * nm);
-  std::vector<double> Ub((size_t)2 * nq), Ud(Ub.size()), UDi(2), UL_(Ub.size()), Ui(Ub.size());
+  const bool dense = nq <= kDenseSolveMaxNq, seg = solve_segmented(g);
+  // mixed precision: the factors as they are, [p][row][j][m]
+  struct UlTables {
+    std::vector<double> multB, multD, Dinv, Lb, invd;
+  };
+  UlTables uT, uP, uU;
+  auto ul_store = [&](UlTables& t, const UL& f, int p, int nmod, int mi) {
+    if (dense || seg) return;
+    const int D = f.D;
+    if (t.invd.empty()) {
+      for (auto* v : {&t.multB, &t.multD, &t.Lb}) v->assign((size_t)2 * nq * D * nmod, 0.0);
+      t.Dinv.assign((size_t)2 * D * D * nmod, 0.0);
+      t.invd.assign((size_t)2 * nq * nmod, 0.0);
+    }
+    for (int r = 0; r < nq; ++r) {
+      for (int j = 0; j < D; ++j) {
+        const size_t at = ((size_t)(p * nq + r) * D + j) * nmod + mi;
+        t.multB[at] = f.multB[(size_t)r * D + j];
+        t.multD[at] = f.multD[(size_t)r * D + j];
+        t.Lb[at] = f.Lb[(size_t)r * D + j];
+      }
+      t.invd[(size_t)(p * nq + r) * nmod + mi] = f.invd[r];
+    }
+    for (int e = 0; e < D * D; ++e) t.Dinv[((size_t)p * D * D + e) * nmod + mi] = f.Dinv[e];
+  };
+  const int LR = solve_seg_rows(nq), NR = (nq + LR - 1) / LR * LR;
+  SegTables sT, sP, sU;
+  auto seg_alloc = [&](SegTables& t, int D, int nmod) {
+    if (!seg) return;
+    for (auto* v : {&t.beta, &t.multD, &t.ilb, &t.phi, &t.theta}) v->assign((size_t)2 * NR * D * nmod, 0.0);
+    t.Dinv.assign((size_t)2 * D * D * nmod, 0.0);
+    t.invd.assign((size_t)2 * NR * nmod, 0.0);
+  };
+  seg_alloc(sT, 1, nm);
+  seg_alloc(sP, 2, nm);
+  seg_alloc(sU, 1, 1);
+  auto seg_store = [&](SegTables& t, const UL& f, int p, int nmod, int mi) {
+    if (!seg) return;
+    const int D = f.D;
+    auto at = [&](int r, int j) { return ((size_t)(p * NR + r) * D + j) * nmod + mi; };
+    std::vector<double> ilb((size_t)nq * D), v(nq + D + LR, 0.0);
+    for (int r = 0; r < nq; ++r) {
+      t.invd[(size_t)(p * NR + r) * nmod + mi] = r < D ? 0.0 : f.invd[r];
+      for (int j = 0; j < D; ++j) {
+        // row r gets -multB[r + 1 + j][D - 1 - j] times row r + 1 + j
+        const int c = r + 1 + j;
+        if (r >= D && c < nq && c / LR == r / LR) t.beta[at(r, j)] = f.multB[(size_t)c * D + D - 1 - j];
+        t.multD[at(r, j)] = f.multD[(size_t)r * D + j];
+        t.ilb[at(r, j)] = ilb[(size_t)r * D + j] = f.invd[r] * f.Lb[(size_t)r * D + j];
+      }
+    }
+    for (int e = 0; e < D * D; ++e) t.Dinv[((size_t)p * D * D + e) * nmod + mi] = f.Dinv[e];
+    for (int r0 = 0; r0 < nq; r0 += LR) {
+      const int e = r0 + LR;
+      for (int j = 0; j < D; ++j) {
+        if (e + j < nq) {   // backward: a unit value at row e + j
+          for (int i = 0; i < D; ++i) v[e + i] = i == j ? 1.0 : 0.0;
+          for (int c = e - 1; c >= std::max(r0, D); --c) {
+            double a = 0.0;
+            for (int i = 1; i <= D; ++i)
+              if (c + i < nq && c + i < e + D) a = std::fma(-f.multB[(size_t)(c + i) * D + D - i], v[c + i], a);
+            v[c] = a;
+            t.phi[at(c, j)] = a;
+          }
+        }
+        const int b0 = r0 == 0 ? 0 : r0 - D;   // forward: a unit value at row b0 + j
+        for (int i = 0; i < D; ++i) v[b0 + i] = i == j ? 1.0 : 0.0;
+        if (r0 == 0)
+          for (int i = 0; i < D; ++i) t.theta[at(i, j)] = v[i];
+        for (int r = std::max(r0, D); r < std::min(nq, e); ++r) {
+          double a = 0.0;
+          for (int i = 0; i < D; ++i) a = std::fma(-ilb[(size_t)r * D + i], v[r - D + i], a);
+          v[r] = a;
+          t.theta[at(r, j)] = a;
+        }
+      }
+    }
+  };
+  // taps by matrix row
+  std::vector<double> seg_s2(seg ? (size_t)2 * NR * 3 : 0, 0.0), seg_s4(seg ? (size_t)2 * NR * 5 : 0, 0.0),
+      seg_mp(seg ? (size_t)2 * NR * 5 * nm : 0, 0.0);
+  for (int p = 0; p < 2 && seg; ++p)
+    for (int t = 0; t < nq - 1; ++t) {
+      for (int j = 0; j < 3; ++j) seg_s2[(size_t)(p * NR + t + 1) * 3 + j] = s2[(p * nq + t) * 3 + j];
+      for (int j = 0; j < 5 && t < nq - 2; ++j) {
+        seg_s4[(size_t)(p * NR + t + 2) * 5 + j] = s4[(p * nq + t) * 5 + j];
+        for (int m = 0; m < nm; ++m)
+          seg_mp[((size_t)(p * NR + t + 2) * 5 + j) * nm + m] = mp[((size_t)(p * nq + t) * 5 + j) * nm + m];
+      }
+    }
   // explicit inverses of the parity systems of small grids, [p][r][q][m]
-  const bool dense = nq <= kDenseSolveMaxNq;
   const size_t ninv = dense ? (size_t)2 * nq * nq : 0;
   std::vector<double> Tinv(ninv * nm), Pinv(ninv * nm), Uinv(ninv);
   auto inverse_into = [&](const UL& f, std::vector<double>& dst, int p, int nmod, int mi) {
@@ -639,37 +714,31 @@ static rbc_status upload_tables(rbc_t h) {
         const double n = 2 * q + p;
         A[q] = (g.bc == RBC_FIXED_FLUX) ? n * n : 1.0;
       }
-      for (int t = 0; t + 1 < nq; ++t)
-        for (int q = 0; q < nq; ++q) {
+      for (int t = 0; t + 1 < nq; ++t)   // (couplings: columns t .. t + 2)
+        for (int q = t; q < std::min(nq, t + 3); ++q) {
           const int r = 2 * t + p, c = 2 * q + p;
           A[(size_t)(1 + t) * nq + q] = el(S2, r, c) - hdt * (4.0 * el(D2, r, c) - k * k * el(S2, r, c));
         }
       UL f;
       if (!ul_factor(A, nq, 1, f, why)) return fail(RBC_EINVAL, "T system m=%d p=%d: %s", m, p, why.c_str());
       worst = std::max(worst, ul_residual(A, f, 17 * m + p));
-      layout(Tb, f.multB, p, nq, 1, nm, m);
-      layout(Td, f.multD, p, nq, 1, nm, m);
-      layout(TL, f.Lb, p, nq, 1, nm, m);
-      for (int r = 0; r < nq; ++r) Ti[(size_t)(p * nq + r) * nm + m] = f.invd[r];
-      TDi[(size_t)p * nm + m] = f.Dinv[0];
+      seg_store(sT, f, p, nm, m);
+      ul_store(uT, f, p, nm, m);
       if (dense) inverse_into(f, Tinv, p, nm, m);
       if (m == 0) {
         // mean flow: S2 - h 4 Pr D2
         Mat U((size_t)nq * nq, 0.0);
         for (int q = 0; q < nq; ++q) U[q] = 1.0;
         for (int t = 0; t + 1 < nq; ++t)
-          for (int q = 0; q < nq; ++q) {
+          for (int q = t; q < std::min(nq, t + 3); ++q) {
             const int r = 2 * t + p, c = 2 * q + p;
             U[(size_t)(1 + t) * nq + q] = el(S2, r, c) - hdt * 4.0 * g.Pr * el(D2, r, c);
           }
         UL fu;
         if (!ul_factor(U, nq, 1, fu, why)) return fail(RBC_EINVAL, "U system p=%d: %s", p, why.c_str());
         worst = std::max(worst, ul_residual(U, fu, 99 + p));
-        layout(Ub, fu.multB, p, nq, 1, 1, 0);
-        layout(Ud, fu.multD, p, nq, 1, 1, 0);
-        layout(UL_, fu.Lb, p, nq, 1, 1, 0);
-        for (int r = 0; r < nq; ++r) Ui[(size_t)p * nq + r] = fu.invd[r];
-        UDi[p] = fu.Dinv[0];
+        seg_store(sU, fu, p, 1, 0);
+        ul_store(uU, fu, p, 1, 0);
         if (dense) inverse_into(fu, Uinv, p, 1, 0);
       } else {
         // streamfunction: BC rows (ones, n^2), tau rows of M - h L in C^(4)
@@ -679,8 +748,8 @@ static rbc_status upload_tables(rbc_t h) {
           P[q] = 1.0;
           P[(size_t)nq + q] = n * n;
         }
-        for (int t = 0; t + 2 < nq; ++t)
-          for (int q = 0; q < nq; ++q) {
+        for (int t = 0; t + 2 < nq; ++t)   // (columns t .. t + 4)
+          for (int q = t; q < std::min(nq, t + 5); ++q) {
             const int r = 2 * t + p, c = 2 * q + p;
             const double M = 4.0 * el(S4D2, r, c) - k * k * el(S4, r, c);
             const double L =
@@ -690,11 +759,8 @@ static rbc_status upload_tables(rbc_t h) {
         UL fp;
         if (!ul_factor(P, nq, 2, fp, why)) return fail(RBC_EINVAL, "psi system m=%d p=%d: %s", m, p, why.c_str());
         worst = std::max(worst, ul_residual(P, fp, 31 * m + p));
-        layout(Pb, fp.multB, p, nq, 2, nm, m);
-        layout(Pd, fp.multD, p, nq, 2, nm, m);
-        layout(PL, fp.Lb, p, nq, 2, nm, m);
-        for (int r = 0; r < nq; ++r) Pi[(size_t)(p * nq + r) * nm + m] = fp.invd[r];
-        for (int e = 0; e < 4; ++e) PDi[((size_t)p * 4 + e) * nm + m] = fp.Dinv[e];
+        seg_store(sP, fp, p, nm, m);
+        ul_store(uP, fp, p, nm, m);
         if (dense) inverse_into(fp, Pinv, p, nm, m);
       }
     }
@@ -725,25 +791,33 @@ static rbc_status upload_tables(rbc_t h) {
   }
   Mat Wn = lobatto_interp(N, thn);
 
+  if (seg) mp.clear();   // (laid out by matrix row in seg_mp)
   add(cc); add(s2); add(s4); add(mp);
-  add(Tb); add(Td); add(TDi); add(TL); add(Ti);
-  add(Pb); add(Pd); add(PDi); add(PL); add(Pi);
-  add(Ub); add(Ud); add(UDi); add(UL_); add(Ui);
+  for (UlTables* t : {&uT, &uP, &uU}) {
+    add(t->multB); add(t->multD); add(t->Dinv); add(t->Lb); add(t->invd);
+  }
+  for (SegTables* t : {&sT, &sP, &sU})
+    for (auto* v : {&t->beta, &t->multD, &t->Dinv, &t->invd, &t->ilb, &t->phi, &t->theta}) add(*v);
+  add(seg_s2); add(seg_s4); add(seg_mp);
   add(gram); add(twn); add(Vn); add(Vn1); add(Wn);
   {
-    // dt * (explicit tableau), then (gamma dt) Pr: the same IEEE products the
-    // stage solve would form per element
+    // dt * (explicit tableau), (gamma dt) Pr, (implicit tableau) / gamma: products
+    // the stage solve would otherwise form per element
     double ae[5][5], ai[5][5], gm;
     int ns;
     scheme_tableau(g.scheme, ae, ai, &ns, &gm);
-    std::vector<double> dtae(26);
+    std::vector<double> dtae(51);
     for (int i = 0; i < 5; ++i)
-      for (int j = 0; j < 5; ++j) dtae[i * 5 + j] = g.dt * ae[i][j];
+      for (int j = 0; j < 5; ++j) {
+        dtae[i * 5 + j] = g.dt * ae[i][j];
+        dtae[26 + i * 5 + j] = g.inv_gamma * ai[i][j];
+      }
     dtae[25] = (g.gamma * g.dt) * g.Pr;
     add(dtae);
   }
-  // FP32 copies of the transform tables, packed two floats per double slot
+  // FP32 copies of the transform tables (mixed precision), packed two floats per double slot
   auto add_f32 = [&](const std::vector<double>& v) {
+    if (!g.mixed) return add({});
     std::vector<double> packed((v.size() + 1) / 2, 0.0);
     float* f = reinterpret_cast<float*>(packed.data());
     for (size_t i = 0; i < v.size(); ++i) f[i] = (float)v[i];
@@ -809,9 +883,14 @@ static rbc_status upload_tables(rbc_t h) {
   T.s2 = b + offs[i++];
   T.s4 = b + offs[i++];
   T.mp = b + offs[i++];
-  T.T_multB = b + offs[i++]; T.T_multD = b + offs[i++]; T.T_Dinv = b + offs[i++]; T.T_Lb = b + offs[i++]; T.T_invd = b + offs[i++];
-  T.P_multB = b + offs[i++]; T.P_multD = b + offs[i++]; T.P_Dinv = b + offs[i++]; T.P_Lb = b + offs[i++]; T.P_invd = b + offs[i++];
-  T.U_multB = b + offs[i++]; T.U_multD = b + offs[i++]; T.U_Dinv = b + offs[i++]; T.U_Lb = b + offs[i++]; T.U_invd = b + offs[i++];
+  for (const double** q : {&T.T_multB, &T.T_multD, &T.T_Dinv, &T.T_Lb, &T.T_invd, &T.P_multB, &T.P_multD, &T.P_Dinv, &T.P_Lb,
+                           &T.P_invd, &T.U_multB, &T.U_multD, &T.U_Dinv, &T.U_Lb, &T.U_invd})
+    *q = b + offs[i++];
+  for (SegFactors* f : {&T.segT, &T.segP, &T.segU})
+    for (const double** q : {&f->beta, &f->multD, &f->Dinv, &f->invd, &f->ilb, &f->phi, &f->theta}) *q = b + offs[i++];
+  T.seg_s2 = b + offs[i++];
+  T.seg_s4 = b + offs[i++];
+  T.seg_mp = b + offs[i++];
   T.gram = b + offs[i++];
   T.twn = reinterpret_cast<const double2*>(b + offs[i++]);
   T.Vn = b + offs[i++];

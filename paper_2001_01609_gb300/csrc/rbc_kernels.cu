@@ -808,7 +808,8 @@ static size_t zfwd_smem(const Grid& g, int B, size_t es) {
 }
 
 // ---------------------------------------------------------------------------
-// Stage solve (k_solve).  Block per (slice, Chebyshev parity p, tile of tms
+// Stage solve (k_solve) of the mixed mode and of small grids (the FP64 mode's
+// larger grids: rbc_solve.cu).  Block per (slice, Chebyshev parity p, tile of tms
 // Fourier modes); a column is one (mode m, real/imaginary part c) pair -- the
 // stage matrices are real, so the two parts are independent systems except for
 // the implicit buoyancy coupling -i k Pr Ra T (the imaginary part of T feeds
@@ -1347,7 +1348,8 @@ cudaError_t configure_kernels(const Grid& g) {
   if (e == cudaSuccess && rows_cl_bytes(g, 4) <= 200 * 1024)
     e = allow_smem(k_rows_cl<float>, (int)rows_cl_bytes(g, 4), a_rcl_f);
   if (e == cudaSuccess) e = allow_smem(k_rows<float>, (int)rows_smem_for(g, 4, false), a_rows_f);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
+  if (e == cudaSuccess && !solve_segmented(g))
     e = allow_smem(k_solve, (int)std::max(solve_smem(g, 1), solve_smem(g, 1 << 20)), a_solve);
   if (e == cudaSuccess)
     e = allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f);
@@ -1428,11 +1430,16 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   else
     launch_zfwd_fx(g, t, w, B, s);
   if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, g.mixed ? 4 : 8));
-  const int tms = solve_tms_of(g, w, B);
-  const int mtiles = (g.nm + tms - 1) / tms;
   if (pf) pf->begin(RBC_KERNEL_SOLVE, s);
-  launch_pdl(w.pdl != 0, k_solve, (unsigned)(B * 2 * mtiles), solve_threads(g, tms), solve_smem_tms(g, tms), s, g, t,
-             X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
+  if (solve_segmented(g)) {
+    e = launch_solve_seg(g, t, w, X, B, stage, nu, s);
+  } else {
+    const int tms = solve_tms_of(g, w, B);
+    const int mtiles = (g.nm + tms - 1) / tms;
+    e = launch_pdl(w.pdl != 0, k_solve, (unsigned)(B * 2 * mtiles), solve_threads(g, tms), solve_smem_tms(g, tms), s, g,
+                   t, X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
+  }
+  if (e != cudaSuccess) return e;
   if (pf) pf->end(RBC_KERNEL_SOLVE, s, solve_flops(g, B), solve_bytes(g, B));
   count(2);
   return cudaGetLastError();
