@@ -145,11 +145,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "d16354a2b2212781a3d0dba67d9e5ec4cd3f9dfcde1658f81e66015e7e0e44fb"
+NCU_TRAFFIC_SHA256 = "f3c30ce161899ad87a7a5080491aa1e5c97bd5b294ac18b34306673340789cde"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 122112, "coarse:k_rows": 400845, "coarse:k_zfwd": 118208, "coarse:k_solve": 827392,
-    "fine:k_zinv@32": 8602778, "fine:k_rows@32": 37891738, "fine:k_zfwd@32": 12626816, "fine:k_solve@32": 23859904,
-    "fine:k_zinv@2": 655104, "fine:k_rows@2": 2501683, "fine:k_zfwd@2": 824896, "fine:k_solve@2": 2763456,
+    "coarse:k_zinv": 120166, "coarse:k_rows": 389018, "coarse:k_zfwd": 118272, "coarse:k_solve": 827456,
+    "fine:k_zinv@32": 8609894, "fine:k_rows@32": 37881037, "fine:k_zfwd@32": 12627200, "fine:k_solve@32": 23855488,
+    "fine:k_zinv@2": 653875, "fine:k_rows@2": 2490778, "fine:k_zfwd@2": 827584, "fine:k_solve@2": 2764608,
 }
 
 

@@ -19,15 +19,16 @@
 // x = 3 a + b, b = 0, 1, 2): G_b[k] = w^(k b) C[k] + w^((k-L) b) C[k - L], and
 // of the forward combination only the kept outputs are formed.  L = R M: the
 // butterflies run in registers (radix up to 16), exchanging through shared
-// memory once per pass; the last inverse pass, the products and the first
-// forward pass act on the same points and stay in one thread's registers.
+// memory once per pass; the products and the first forward pass act on the
+// same points and stay in one thread's registers.
 //   P0  modes -> exponents, packed spectra C, D (shared), terms of the x-means
 //   P1  G_b and the M-point transforms (P1b: the second half of M = 32, 64)
-//   P2  R-point inverse, products, R-point forward (registers)
+//   P2  R-point inverse transforms
+//   P3  products, R-point forward transforms
 //   PB  M-point forward transforms
 //   PF  sum over b, unpacking, x-means, store
-// Block: RB rows, any number of threads that covers the P2 items; items are
-// flattened over the block's rows.
+// Block: RB rows, at least one thread per P3 item; items are flattened over the
+// block's rows.
 //
 // Fixed point: each row and field gets the exponent of its summed mode moduli
 // (an upper bound of the grid values), so grid values are integers below 2^59
@@ -42,8 +43,11 @@
 // 64 clocks, a 32x32->64 multiply-add for 4 and a 64-bit add for 2, so the
 // same FFT costs about a tenth.  Measured (GB300, per launch, against five
 // FP64 FFTs in radix-4 passes through shared memory): 256 x 64, 32 states
-// 491 -> 127 us; 512 x 128, 3 states 207 -> 60 us; 64 x 32, 23 states
-// 41 -> 21 us; 128 x 32, one state 20.4 -> 19.6 us (latency: the barriers).
+// 491 -> 108 us; 512 x 128, 3 states 207 -> 59 us; 64 x 32, 23 states
+// 41 -> 17 us; 128 x 32, one state 20.4 -> 18.3 us (latency: the barriers).
+// One thread keeping the points of all three inverse FFTs in registers (P2 and
+// P3 in one pass, 166 registers, C and D in a place of their own) took 127, 60,
+// 22 and 19.8 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -246,8 +250,13 @@ template <int L> struct Plan {
   static constexpr int FS = M * (R + 1);
   static constexpr int kSum1 = (L + 7) / 8, kSum2 = (kSum1 + 7) / 8, kSum3 = (kSum2 + 7) / 8;
   static constexpr int kSums = 2 * (L + kSum1 + kSum2 + kSum3);
+  // with a single first pass (M2 = 1) each of its items belongs to one thread,
+  // which reads its spectra before any is overwritten: C, D share H's place
+  static constexpr bool kAlias = M2 == 1;
   static constexpr size_t row_bytes =
-      ((6 * (size_t)L + 9 * (size_t)FS) * sizeof(C) + (size_t)kSums * 8 + 15) / 16 * 16;
+      (((kAlias ? 0 : 6 * (size_t)L) + 9 * (size_t)FS) * sizeof(C) + (size_t)kSums * 8 + 15) / 16 * 16;
+  // threads of a block of rb rows: one per P2 item, and per P1 item where those are single
+  static constexpr int threads(int rb) { return (rb * (kAlias && 9 * R > 3 * M ? 9 * R : 3 * M) + 31) / 32 * 32; }
   static constexpr int kSH = 2;                                    // each forward twiddle halves twice
   static constexpr int kShift = kSH * (M2 > 1 ? 3 : 2);
 };
@@ -263,7 +272,7 @@ struct RowMeta {
 };
 
 template <int L>
-__global__ void __launch_bounds__(384) k_rows_fx(Grid g, const W* __restrict__ TW, const double* __restrict__ rk,
+__global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ? 2 : 1) k_rows_fx(Grid g, const W* __restrict__ TW, const double* __restrict__ rk,
                                                  const double* __restrict__ Z, double* __restrict__ Q,
                                                  double* __restrict__ wT, int nrows, int RB, const int* nsteps,
                                                  const int* step) {
@@ -288,7 +297,7 @@ __global__ void __launch_bounds__(384) k_rows_fx(Grid g, const W* __restrict__ T
   }
   auto Cb = [&](int r) { return reinterpret_cast<C*>(rsm + (size_t)r * P::row_bytes); };
   auto Db = [&](int r) { return Cb(r) + 3 * L; };
-  auto Hb = [&](int r) { return Cb(r) + 6 * L; };
+  auto Hb = [&](int r) { return Cb(r) + (P::kAlias ? 0 : 6 * L); };
   auto Sb = [&](int r) { return reinterpret_cast<double*>(Hb(r) + 9 * FS); };
   const size_t fs = (size_t)g.Mz * L * 2;
   auto zrow = [&](int r) {
@@ -399,29 +408,53 @@ __global__ void __launch_bounds__(384) k_rows_fx(Grid g, const W* __restrict__ T
   constexpr int s1 = 2 * L, s2 = s1 + 2 * P::kSum1, s3 = s2 + 2 * P::kSum2;
 
   // ---- P1: G_b and the first inverse pass; item (b, row, pair, j, s), s fastest
-  for (int i = tid; i < RB * 9 * R * M2; i += T) {
-    const int b = i / (RB * 3 * R * M2), i1 = i - b * RB * 3 * R * M2;
-    const int r = i1 / (3 * R * M2), i2 = i1 - r * 3 * R * M2;
-    const int pr = i2 / (R * M2), i3 = i2 - pr * R * M2;
-    const int j = i3 / R, s = i3 - j * R;
-    if (!meta[r].act) continue;
-    const C* c = Cb(r) + pr * L;
-    const C* d = Db(r) + pr * L;
+  {
     C x[M1];
+    int b, r, pr, j, sx;
+    auto item = [&](int i) {
+      b = i / (RB * 3 * R * M2);
+      const int i1 = i - b * RB * 3 * R * M2;
+      r = i1 / (3 * R * M2);
+      const int i2 = i1 - r * 3 * R * M2;
+      pr = i2 / (R * M2);
+      const int i3 = i2 - pr * R * M2;
+      j = i3 / R;
+      sx = i3 - j * R;
+    };
+    auto gather = [&] {
+      const C* c = Cb(r) + pr * L;
+      const C* d = Db(r) + pr * L;
 #pragma unroll
-    for (int a = 0; a < M1; ++a) {
-      const int k = R * (M2 * a + j) + s;
-      if (b == 0)
-        x[a] = add(c[k], d[k]);
-      else
-        x[a] = cmul2c(c[k], tw(k * b), d[k], tw(k * b + (3 - b) * L));
-    }
-    dft<M1, 1>(x);
-    C* h = Hb(r) + (pr * 3 + b) * FS + s;
+      for (int a = 0; a < M1; ++a) {
+        const int k = R * (M2 * a + j) + sx;
+        if (b == 0)
+          x[a] = add(c[k], d[k]);
+        else
+          x[a] = cmul2c(c[k], tw(k * b), d[k], tw(k * b + (3 - b) * L));
+      }
+    };
+    auto transform = [&] {
+      dft<M1, 1>(x);
+      C* h = Hb(r) + (pr * 3 + b) * FS + sx;
 #pragma unroll
-    for (int u = 0; u < M1; ++u) {
-      if (M2 > 1 && u > 0) x[u] = cmulw<true, 0>(x[u], tw(3 * R * u * j));
-      h[(u + M1 * j) * (R + 1)] = x[u];
+      for (int u = 0; u < M1; ++u) {
+        if (M2 > 1 && u > 0) x[u] = cmulw<true, 0>(x[u], tw(3 * R * u * j));
+        h[(u + M1 * j) * (R + 1)] = x[u];
+      }
+    };
+    if constexpr (P::kAlias) {
+      item(tid);
+      const bool on = tid < RB * 9 * R && meta[min(r, RB - 1)].act;
+      if (on) gather();
+      __syncthreads();
+      if (on) transform();
+    } else {
+      for (int i = tid; i < RB * 9 * R * M2; i += T) {
+        item(i);
+        if (!meta[r].act) continue;
+        gather();
+        transform();
+      }
     }
   }
   tree(0, L, s1, P::kSum1);
@@ -443,52 +476,62 @@ __global__ void __launch_bounds__(384) k_rows_fx(Grid g, const W* __restrict__ T
     __syncthreads();
   }
 
-  // ---- P2: last inverse pass, products, first forward pass; one item (row, b, q) per thread
+  // ---- P2: last inverse pass, in place; item (row, pair, b, q), q fastest
+  for (int i = tid; i < RB * 9 * M; i += T) {
+    const int r = i / (9 * M), i1 = i - r * 9 * M;
+    const int ff = i1 / M, q = i1 - ff * M;
+    if (!meta[r].act) continue;
+    C* h = Hb(r) + ff * FS + q * (R + 1);
+    C x[R];
+#pragma unroll
+    for (int s = 0; s < R; ++s) x[s] = h[s];
+#pragma unroll
+    for (int s = 1; s < R; ++s)
+      if (M > 1) x[s] = cmulw<true, 0>(x[s], tw(3 * s * q));
+    dft<R, 1>(x);
+#pragma unroll
+    for (int t = 0; t < R; ++t) h[t] = x[t];
+  }
+  if (P::kSum1 > 1) tree(s1, P::kSum1, s2, P::kSum2);
+  __syncthreads();
+
+  // ---- P3: products and the first forward pass; one item (row, b, q) per thread,
+  // the points t of the P2 item at (b, q)
   {
     const int r = tid / (3 * M), i1 = tid - r * 3 * M;
     const int b = i1 / M, q = i1 - b * M;
     const bool on = tid < RB * 3 * M && meta[min(r, RB - 1)].act;
     C* h = Hb(on ? r : 0) + b * FS + q * (R + 1);
     C x[R];
-    auto inverse = [&](int pr) {
-#pragma unroll
-      for (int s = 0; s < R; ++s) x[s] = h[pr * 3 * FS + s];
-#pragma unroll
-      for (int s = 1; s < R; ++s)
-        if (M > 1) x[s] = cmulw<true, 0>(x[s], tw(3 * s * q));
-      dft<R, 1>(x);
-    };
     i64 vh[2][R];        // N_T, N_omega: 96-bit values vh 2^32 + vl
     unsigned vl[2][R];
     if (on) {
-      int uh[R], ul[R], wh[R], wl[R];
-      inverse(0);
+      i64 acc[2] = {0, 0};
+      unsigned accl[2] = {0, 0};
 #pragma unroll
       for (int t = 0; t < R; ++t) {
-        fx::split32(x[t].x, uh[t], ul[t]);
-        fx::split32(x[t].y, wh[t], wl[t]);
-      }
+        const C uw = h[t];
+        int uh, ul, wh, wl;
+        fx::split32(uw.x, uh, ul);
+        fx::split32(uw.y, wh, wl);
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        inverse(2 - k);   // k = 0: d_x T, d_z T; k = 1: d_x omega, d_z omega
-        i64 acc = 0;
-        unsigned accl = 0;
-#pragma unroll
-        for (int t = 0; t < R; ++t) {
+        for (int k = 0; k < 2; ++k) {
+          const C ab = h[(2 - k) * 3 * FS + t];   // k = 0: d_x T, d_z T; k = 1: d_x omega, d_z omega
           int ah, al, bh, bl;
-          fx::split32(x[t].x, ah, al);
-          fx::split32(x[t].y, bh, bl);
-          const i64 ph = fx::madw(uh[t], ah, (i64)wh[t] * bh);
-          const i64 pm = fx::madw(uh[t], al, fx::madw(ul[t], ah, fx::madw(wh[t], bl, (i64)wl[t] * bh)));
+          fx::split32(ab.x, ah, al);
+          fx::split32(ab.y, bh, bl);
+          const i64 ph = fx::madw(uh, ah, (i64)wh * bh);
+          const i64 pm = fx::madw(uh, al, fx::madw(ul, ah, fx::madw(wh, bl, (i64)wl * bh)));
           const i64 v = ph + (pm >> 32);
           vh[k][t] = v;
           vl[k][t] = (unsigned)pm;
-          acc |= v ^ (v >> 63);
-          accl |= (unsigned)pm ^ (unsigned)(v >> 63);
+          acc[k] |= v ^ (v >> 63);
+          accl[k] |= (unsigned)pm ^ (unsigned)(v >> 63);
         }
-        const int bits = acc ? 96 - __clzll(acc) : 32 - __clz((int)accl);
-        atomicMax(&meta[r].bits[k], bits);
       }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        atomicMax(&meta[r].bits[k], acc[k] ? 96 - __clzll(acc[k]) : 32 - __clz((int)accl[k]));
     }
     __syncthreads();
     if (on) {
@@ -517,7 +560,7 @@ __global__ void __launch_bounds__(384) k_rows_fx(Grid g, const W* __restrict__ T
       for (int s = 0; s < R; ++s) h[s] = cmulw<false, P::kSH>(x[s], tw(3 * s * q));
     }
   }
-  if (P::kSum1 > 1) tree(s1, P::kSum1, s2, P::kSum2);
+  if (P::kSum2 > 1) tree(s2, P::kSum2, s3, P::kSum3);
   __syncthreads();
 
   // ---- PB: M-point forward transforms of the three sub-rows, in place
@@ -551,7 +594,6 @@ __global__ void __launch_bounds__(384) k_rows_fx(Grid g, const W* __restrict__ T
     for (int a = 0; a < M1; ++a)
       h[a * (R + 1)] = cmulw<false, P::kSH>(x[a], tw((R * (M2 * a + j) + s) * b));
   }
-  if (P::kSum2 > 1) tree(s2, P::kSum2, s3, P::kSum3);
   __syncthreads();
 
   // ---- PF: C[m] = Y_0 + Y_1 + Y_2, C[N - m] = Y_0 + w Y_1 + w^2 Y_2 (w = exp(2 pi i / 3))
@@ -610,17 +652,17 @@ struct RowsShape {
 
 template <int L> RowsShape rows_shape(const Work& w, int nrows) {
   using P = Plan<L>;
-  const int cap = (w.shapes && w.shapes->rows_threads > 0) ? std::min(384, w.shapes->rows_threads) : 192;
+  const int cap = (w.shapes && w.shapes->rows_threads > 0) ? std::min(320, w.shapes->rows_threads) : 192;
   int rb = 1;
-  while (rb < kMaxRB && 2 * rb * 3 * P::M <= cap && 2 * rb * P::row_bytes <= 100 * 1024) rb *= 2;
+  while (rb < kMaxRB && P::threads(2 * rb) <= cap && 2 * rb * P::row_bytes <= 100 * 1024) rb *= 2;
   const int form = w.shapes ? w.shapes->rows_cl : -1;
   if (form == 1)
     rb = 1;
   else if (form < 0)
     while (rb > 1 && (long)nrows < 2L * 152 * rb) rb /= 2;
-  int th = (rb * 3 * P::M + 31) / 32 * 32;
-  th = std::max(th, std::min(128, (rb * 9 * P::R * P::M2 + 31) / 32 * 32));
-  return {rb, std::min(th, 384), rb * P::row_bytes};
+  // a row alone: threads for the other passes' items too
+  const int th = std::max(P::threads(rb), std::min(128, (rb * 9 * P::R * P::M2 + 31) / 32 * 32));
+  return {rb, th, rb * P::row_bytes};
 }
 
 template <int L> cudaError_t launch_rows_L(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s) {
