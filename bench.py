@@ -145,11 +145,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "f3c30ce161899ad87a7a5080491aa1e5c97bd5b294ac18b34306673340789cde"
+NCU_TRAFFIC_SHA256 = "98aabc57f56584e86a11977fe4f4508c01e4ffbb8b08b36a190f0df361bf26bf"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 120166, "coarse:k_rows": 389018, "coarse:k_zfwd": 118272, "coarse:k_solve": 827456,
-    "fine:k_zinv@32": 8609894, "fine:k_rows@32": 37881037, "fine:k_zfwd@32": 12627200, "fine:k_solve@32": 23855488,
-    "fine:k_zinv@2": 653875, "fine:k_rows@2": 2490778, "fine:k_zfwd@2": 827584, "fine:k_solve@2": 2764608,
+    "coarse:k_zinv": 135731, "coarse:k_rows": 386560, "coarse:k_zfwd": 123584, "coarse:k_solve": 828992,
+    "fine:k_zinv@32": 10443366, "fine:k_rows@32": 37903309, "fine:k_zfwd@32": 12628864, "fine:k_solve@32": 23856064,
+    "fine:k_zinv@2": 667648, "fine:k_rows@2": 2491136, "fine:k_zfwd@2": 830144, "fine:k_solve@2": 2762880,
 }
 
 

@@ -1,7 +1,9 @@
 """The transform kernels at the edges of their sizes, against the FP64 oracle.
 
 One step of every row length (Nx = 4 .. 1024: one, two and three passes per
-FFT) and batch size (several rows per block, a ragged last block).
+FFT) and batch size (several rows per block, a ragged last block), and of the
+column lengths around the groups, chunks and segments of the z sums and stage
+solves, in batches that take each split of a row pair, alone and together.
 Tolerances: FP64 1e-12 relative to the largest coefficient, ten times the
 largest difference of the two implementations' roundings seen on these grids;
 FP32 products 1e-5, the bound of the mixed mode's parity tests.
@@ -49,3 +51,24 @@ def test_every_row_length_matches_oracle(rbc, Nx, precision, tol):
         ref, integ = o.run(Xs[b], n)
         assert max_rel_diff(from_abi(st[b].cpu().numpy()), ref) < tol
         assert abs(nu[b].item() - integ) <= tol * max(abs(integ), 1e-30)
+
+
+@pytest.mark.parametrize("Nz", [8, 16, 18, 32, 34, 36, 64, 66, 128, 130, 258])
+def test_column_lengths_match_oracle_and_batches_agree(rbc, Nz, Nx=8):
+    Ra, dt = 1e4, 1e-5
+    o = RBC(Ra, 1.0, 2.0, Nx, Nz, dt)
+    F = rbc.Propagator(Ra, 1.0, 2.0, Nx, Nz, dt, 0)
+    X0 = nonlinear_state(o, 7)
+    alone = F.new_states(1)
+    alone[0].copy_(torch.from_numpy(to_abi(X0)))
+    states = {B: alone[:1].repeat(B, 1, 1, 1, 1) for B in (3, 40, 100)}
+    nu = torch.zeros(100, dtype=torch.float64, device="cuda")
+    F.step_batch(alone, 1, nu[:1])
+    ref, integ = o.run(X0, 1)
+    assert max_rel_diff(from_abi(alone[0].cpu().numpy()), ref) < 1e-12
+    assert abs(nu[0].item() - integ) <= 1e-12 * abs(integ)
+    for B, st in states.items():
+        nub = torch.zeros(B, dtype=torch.float64, device="cuda")
+        F.step_batch(st, 1, nub)
+        assert torch.equal(st, alone.expand_as(st)) and torch.equal(nub, nu[:1].expand(B)), B
+    assert F.check_diverged() == rbc.RBC_OK
