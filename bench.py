@@ -145,11 +145,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "98aabc57f56584e86a11977fe4f4508c01e4ffbb8b08b36a190f0df361bf26bf"
+NCU_TRAFFIC_SHA256 = "e4d4f340df89c3a063fe6c7233afb778166f1a53035ac2093c58342aaa741b6a"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 135731, "coarse:k_rows": 386560, "coarse:k_zfwd": 123584, "coarse:k_solve": 828992,
-    "fine:k_zinv@32": 10443366, "fine:k_rows@32": 37903309, "fine:k_zfwd@32": 12628864, "fine:k_solve@32": 23856064,
-    "fine:k_zinv@2": 667648, "fine:k_rows@2": 2491136, "fine:k_zfwd@2": 830144, "fine:k_solve@2": 2762880,
+    "coarse:k_zinv": 135219, "coarse:k_rows": 386406, "coarse:k_zfwd": 123328, "coarse:k_solve": 826624,
+    "fine:k_zinv@32": 10443213, "fine:k_rows@32": 37880678, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23855232,
+    "fine:k_zinv@2": 667136, "fine:k_rows@2": 2490266, "fine:k_zfwd@2": 829952, "fine:k_solve@2": 2764928,
 }
 
 

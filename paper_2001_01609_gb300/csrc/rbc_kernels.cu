@@ -1306,6 +1306,11 @@ void Prof::end(int k, cudaStream_t s, double fl, double by) {
   bytes[k] += by;
 }
 
+// Tiles and threads of the L2 norms (see k_l2_diff).
+constexpr int kCorrTile = 8;
+constexpr int kCorrThreads = 256;
+__global__ void k_l2_diff(Grid g, const double* __restrict__ gram, const double* A, const double* Bm, double* out, int ncta);
+
 // Algorithmic work of one launch over B slices (all active).
 static double zinv_flops(const Grid& g, int B) { return 24.0 * B * ((g.Mz + 1) / 2) * g.nm * g.Nz; }
 // (nf z-inverse fields of es-byte reals; nfft x FFTs per row)
@@ -1341,6 +1346,11 @@ static cudaError_t allow_smem(F* fn, int need, int& allowed) {
 }
 
 cudaError_t configure_kernels(const Grid& g) {
+  // k_l2_diff: tiles of up to 512 coefficients, clusters of up to 16 blocks
+  cudaError_t l2 = cudaFuncSetAttribute(k_l2_diff, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        kCorrTile * 512 * (int)sizeof(double2));
+  if (l2 == cudaSuccess) l2 = cudaFuncSetAttribute(k_l2_diff, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (l2 != cudaSuccess) return l2;
   static int a_rows_f = 48 * 1024, a_solve = 48 * 1024, a_zfwd_f = 48 * 1024;
   static int a_rcl_f = 48 * 1024;
   cudaError_t e = configure_zfx(g);   // also the averages of Sec. 2.2 of a mixed handle
@@ -1657,8 +1667,6 @@ cudaError_t launch_add(double* a, const double* b, int n, cudaStream_t s) {
 // order, each tile's terms summed by the block in a fixed order, with explicit
 // roundings; rbc_l2_diff and the fused Parareal correction share this order,
 // so both give the same bits.
-constexpr int kCorrTile = 8;
-constexpr int kCorrThreads = 256;
 
 // w Re(conj(di) . s) added to acc, s = sum_j gram_ij d_j
 __device__ __forceinline__ double l2_term(double acc, double w, double2 di, double2 s) {
@@ -1669,41 +1677,80 @@ __device__ __forceinline__ double2 gram_acc(double2 s, double gij, double2 dj) {
 }
 
 // ||A_b - B_b||^2 (or ||A_b||^2 when Bm is null) of the temperature field of nst
-// states, block (kCorrThreads threads) per state.
-__global__ void __launch_bounds__(kCorrThreads) k_l2_diff(Grid g, const double* gram, const double* A, const double* Bm,
-                                                          double* out) {
+// states.  A cluster of ncta blocks per state: block c sums the tiles c, c + ncta,
+// ... (differences staged once in shared memory) and leaves each tile's sum in
+// the first block, which adds them in tile order.  The result does not depend
+// on ncta, and no scratch outlives the call.
+// Bound: the FP64 pipe, Nz / 2 complex-by-real multiply-adds per coefficient (15 us
+// for 16 states of 256 x 64).  One block per state that walked over all tiles and
+// formed each difference Nz / 2 times left 136 of 152 SMs idle: the two norms,
+// correction and restriction of 16 such states took 729 us together, now 76.
+constexpr int kMaxTiles = 64;   // nm <= 512
+__global__ void __launch_bounds__(kCorrThreads) k_l2_diff(Grid g, const double* __restrict__ gram, const double* A,
+                                                          const double* Bm, double* out, int ncta) {
+  namespace cg = cooperative_groups;
+  extern __shared__ double2 sd[];             // [kCorrTile][Nz]: the tile's modes
   __shared__ double red[kCorrThreads];
-  const int b = blockIdx.x;
+  __shared__ double tile_sum[kMaxTiles];      // the first block's holds all tiles
+  cg::cluster_group cl = cg::this_cluster();
+  const int b = blockIdx.x / ncta, c = blockIdx.x - b * ncta;
   const size_t S = state_doubles(g);
   const double* a = A + (size_t)b * S;
   const double* bb = Bm ? Bm + (size_t)b * S : nullptr;
-  double tot = 0.0;
-  for (int m0 = 0; m0 < g.nm; m0 += kCorrTile) {
-    const int tm = min(kCorrTile, g.nm - m0);
+  double* sums = cl.map_shared_rank(tile_sum, 0);
+  const int tiles = (g.nm + kCorrTile - 1) / kCorrTile;
+  cl.sync();                                  // every block runs before its memory is written
+  for (int t = c; t < tiles; t += ncta) {
+    const int m0 = t * kCorrTile, tm = min(kCorrTile, g.nm - m0);
+    for (int it = threadIdx.x; it < tm * g.Nz; it += blockDim.x) {
+      const int dm = it % tm, i = it / tm;
+      double2 d = ld2(a + soff(g, 0, i, m0 + dm));
+      if (bb) d = d - ld2(bb + soff(g, 0, i, m0 + dm));
+      sd[dm * g.Nz + i] = d;
+    }
+    __syncthreads();
     double acc = 0.0;
     for (int it = threadIdx.x; it < tm * g.Nz; it += blockDim.x) {
-      const int dm = it % tm, i = it / tm, m = m0 + dm;
-      double2 di = ld2(a + soff(g, 0, i, m));
-      if (bb) di = di - ld2(bb + soff(g, 0, i, m));
+      const int dm = it % tm, i = it / tm;
+      const double2* d = sd + dm * g.Nz;
       double2 s = {0.0, 0.0};
-      for (int jn = (i & 1); jn < g.Nz; jn += 2) {
-        double2 dj = ld2(a + soff(g, 0, jn, m));
-        if (bb) dj = dj - ld2(bb + soff(g, 0, jn, m));
-        s = gram_acc(s, __ldg(gram + (size_t)i * g.Nz + jn), dj);
-      }
-      acc = l2_term(acc, m == 0 ? 1.0 : 2.0, di, s);
+#pragma unroll 4
+      for (int jn = (i & 1); jn < g.Nz; jn += 2) s = gram_acc(s, __ldg(gram + (size_t)i * g.Nz + jn), d[jn]);
+      acc = l2_term(acc, m0 + dm == 0 ? 1.0 : 2.0, d[i], s);
     }
-    tot += block_sum(acc, red);
+    acc = block_sum(acc, red);                // (ends with a barrier: sd may be rewritten)
+    if (threadIdx.x == 0) sums[t] = acc;
   }
-  if (threadIdx.x == 0) out[b] = 0.5 * g.Lx * tot;
+  cl.sync();
+  if (c == 0 && threadIdx.x == 0) {
+    double tot = 0.0;
+    for (int t = 0; t < tiles; ++t) tot += tile_sum[t];
+    out[b] = 0.5 * g.Lx * tot;
+  }
 }
 
+// Blocks per state: one per tile up to a cluster of 16, eight (the portable size)
+// from 38 states on, where 38 x 8 already makes two blocks per SM.
 cudaError_t launch_l2_diff(const Grid& g, const Tables& t, const double* A, const double* Bm, int nst, double* out,
                            cudaStream_t s) {
   if (nst <= 0) return cudaSuccess;
-  k_l2_diff<<<nst, kCorrThreads, 0, s>>>(g, t.gram, A, Bm, out);
+  const int tiles = (g.nm + kCorrTile - 1) / kCorrTile;
+  int ncta = 1;
+  while (2 * ncta <= std::min(tiles, nst >= 38 ? 8 : 16)) ncta *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = (unsigned)(nst * ncta);
+  cfg.blockDim = kCorrThreads;
+  cfg.dynamicSmemBytes = (size_t)kCorrTile * g.Nz * sizeof(double2);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)ncta;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_l2_diff, g, t.gram, A, Bm, out, ncta);
   count();
-  return cudaGetLastError();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // ---------------------------------------------------------------------------

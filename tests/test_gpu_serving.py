@@ -13,6 +13,7 @@ import numpy as np
 import pytest
 
 from layout import from_abi, max_rel_diff, to_abi
+from oracle.ultraspherical import cheb_gram
 from oracle.rbc import RBC, prolong as o_prolong, restrict as o_restrict
 from paper_2001_01609_gb300.inputs import initial_temperature
 
@@ -112,6 +113,26 @@ def test_parareal_building_blocks_match_oracle(rbc):
         np.testing.assert_allclose(out2[b].item(), d, rtol=1e-10, atol=1e-14)
     with pytest.raises(rbc.RBCError):
         rbc.restrict(G, F, coarse, fine)                 # "coarse" finer than "fine"
+
+
+@pytest.mark.parametrize("Nx,Nz", [(4, 8), (16, 10), (32, 512), (64, 10), (256, 12), (1024, 8)])
+def test_l2_norms_of_every_cluster_size(rbc, Nx, Nz):
+    """1 .. 64 tiles of eight modes, one to 16 blocks per state (eight from 38 states on): FP64 rounding bounds, and
+    the bits of a state alone."""
+    F = rbc.Propagator(1e4, 1.0, 2.0, Nx, Nz, 1e-5, 0)
+    G = cheb_gram(Nz)
+    g = torch.Generator(device="cuda").manual_seed(Nx + Nz)
+    A, Bm = (torch.randn((39,) + F.state_shape, dtype=torch.float64, device="cuda", generator=g) for _ in range(2))
+    out = {n: torch.zeros(n, dtype=torch.float64, device="cuda") for n in (1, 37, 39)}
+    for n, o in out.items():
+        rbc.l2_diff(F, A[:n], Bm[:n], o)
+    d = (A - Bm)[:, 0].cpu().numpy().reshape(39, Nz, Nx // 2, 2)
+    w = np.where(np.arange(Nx // 2) == 0, 1.0, 2.0)
+    ref = np.einsum("bnmc,nk,bkmc,m->b", d, G, d, w, optimize=True)
+    terms = np.einsum("bnmc,nk,bkmc,m->b", abs(d), abs(G), abs(d), w, optimize=True)
+    bound = 2.0 ** -52 * (2 * Nz + Nx) * terms      # additions in a row, at most, on either side
+    assert (abs(out[39].cpu().numpy() - ref) <= bound).all()      # Lx / 2 = 1
+    assert torch.equal(out[37], out[39][:37]) and torch.equal(out[1], out[39][:1])
 
 
 def small_classes(Nx, Nz, precision):
