@@ -140,16 +140,17 @@ class Clocks:
 NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_kernels.cu",
     "paper_2001_01609_gb300/csrc/rbc_rows_fx.cu",
+    "paper_2001_01609_gb300/csrc/rbc_rows_f32.cu",
     "paper_2001_01609_gb300/csrc/rbc_zfx.cu",
     "paper_2001_01609_gb300/csrc/rbc_solve.cu",
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "e4d4f340df89c3a063fe6c7233afb778166f1a53035ac2093c58342aaa741b6a"
+NCU_TRAFFIC_SHA256 = "e4ba3c1ad885cea77ea7e84e465d90168a694128fd4fc749035b2aaddd256255"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 135219, "coarse:k_rows": 386406, "coarse:k_zfwd": 123328, "coarse:k_solve": 826624,
-    "fine:k_zinv@32": 10443213, "fine:k_rows@32": 37880678, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23855232,
-    "fine:k_zinv@2": 667136, "fine:k_rows@2": 2490266, "fine:k_zfwd@2": 829952, "fine:k_solve@2": 2764928,
+    "coarse:k_zinv": 135066, "coarse:k_rows": 386867, "coarse:k_zfwd": 123072, "coarse:k_solve": 831232,
+    "fine:k_zinv@32": 10437888, "fine:k_rows@32": 37880115, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23858048,
+    "fine:k_zinv@2": 671027, "fine:k_rows@2": 2490931, "fine:k_zfwd@2": 830208, "fine:k_solve@2": 2765056,
 }
 
 

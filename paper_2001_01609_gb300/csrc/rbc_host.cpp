@@ -1535,14 +1535,9 @@ extern "C" rbc_status rbc_autotune(rbc_t h, int B, double out_ms[2], cudaStream_
     c.rows_cl = cl;
     if ((s = trial(c)) != RBC_OK) return s;
   }
-  for (int th = 512; th <= 1024; th *= 2) {   // block size of the one-block-per-row kernel
+  for (int th = 512; th <= 1024; th *= 2) {   // largest block of the row kernel
     Shapes c = best;
     c.rows_threads = th;
-    if ((s = trial(c)) != RBC_OK) return s;
-  }
-  for (int ln = 0; ln <= 1; ++ln) {             // its shared-memory layout
-    Shapes c = best;
-    c.rows_lean = ln;
     if ((s = trial(c)) != RBC_OK) return s;
   }
   for (int tm = 4; tm <= 32; tm *= 2)

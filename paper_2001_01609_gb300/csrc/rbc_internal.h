@@ -153,9 +153,9 @@ struct Shapes {
   int solve_tms = 0;   // Fourier modes per k_solve block (power of two, <= 16)
   int zfwd_tm = 0;     // Fourier modes per k_zfwd block (power of two, <= 32)
   int zfwd_nch = 0;    // chunks of the n range per k_zfwd block (1, 2, 4, 8)
-  int rows_cl = -1;    // 1: the clustered row kernel (FP64: one row per block), 0: one block per row (FP64: full blocks)
-  int rows_threads = 0;   // threads of a k_rows block (256, 512 or 1024; FP64: at most 384 are used)
-  int rows_lean = -1;  // 1: k_rows with 5 + 3 shared rows, 0: 5 + 5 (where either fits; FP64: one layout)
+  int rows_cl = -1;    // 1: one row per row-kernel block, 0: as many as fill it
+  int rows_threads = 0;   // largest row-kernel block (256, 512 or 1024; FP32 uses up to 256, FP64 up to 320)
+  int rows_lean = -1;  // kept for callers that pin shapes; the row kernels have one layout
 };
 
 // Per-call workspace pointers (capacity >= B states).
@@ -264,6 +264,9 @@ int correct_norm_blocks(const Grid& gf);
 cudaError_t launch_correct_norm(const Grid& gf, const Grid& gc, const Tables& tf, int mode, const double* Ff,
                                 const double* Gnew, double* Gold, double* C, const double* Uprev, double* U,
                                 double* Fnext, double* partial, unsigned* counter, double* norms, cudaStream_t s);
+// row kernel of the mixed mode (rbc_rows_f32.cu)
+cudaError_t configure_rows_f32(const Grid& g);
+cudaError_t launch_rows_f32(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
 // row kernel of the FP64 mode (rbc_rows_fx.cu)
 cudaError_t configure_rows_fx(const Grid& g);
 cudaError_t launch_rows_fx(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);

@@ -4,9 +4,9 @@
 // launches:
 //   k_zinv   z inverse transform: Chebyshev coefficients -> 9 fields at the
 //            3/2-padded Lobatto points, with the Fourier-mode factors ik;
-//   k_rows   per (slice, padded z-row): packed inverse real FFTs in x
-//            (shared memory, mixed-radix Stockham), advective products,
-//            one packed forward FFT, truncation to the kept modes, x-means;
+//   k_rows_* per padded z-row: packed inverse real FFTs in x, advective products,
+//            one packed forward FFT, truncation to the kept modes, x-means
+//            (rbc_rows_f32.cu, FP64: rbc_rows_fx.cu);
 //   k_zfwd   z forward transform of the products to T coefficients n < Nz;
 //   k_solve  per (slice, Fourier mode, Chebyshev parity): RK443 right-hand
 //            side in tau rows, UL banded solve of the implicit system
@@ -320,91 +320,10 @@ static int zinv_warps(const Grid& g) {
   return kp;
 }
 
-// ---------------------------------------------------------------------------
-// Shared-memory mixed-radix Stockham FFT of length N = 3 * 2^p (radices
-// 4, ..., 4, [2], 3) applied to na arrays of length N at once (array a at
-// [a * N]).  y_q = sum_r x_r exp(sign 2 pi i q r / N), unnormalised.
-// Ping-pongs between a and b; returns the buffer holding the results.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ C2<T>* fft_smem(C2<T>* a, C2<T>* b, int N, int na, int sign, const C2<T>* tw) {
-  using V = C2<T>;
-  int p = 0;
-  for (int M = N / 3; M > 1; M >>= 1) ++p;
-  const int nr = p / 2 + (p & 1) + 1;
-  int Ns = 1, lns = 0;                                 // Ns = 2^lns
-  V* x = a;
-  V* y = b;
-  const T s3 = (T)0.86602540378443864676 * (T)sign;   // sign * sqrt(3)/2
-  const T sg = (T)sign;
-  for (int pass = 0; pass < nr; ++pass) {
-    const int R = (pass < p / 2) ? 4 : ((p & 1) && pass == p / 2) ? 2 : 3;
-    // N = 3 2^p: N / R and N / (Ns R) by shifts (the radix-3 pass leaves 2^p)
-    const int nb = R == 4 ? N >> 2 : R == 2 ? N >> 1 : 1 << p;
-    const int stride = nb >> lns;
-    for (int it = threadIdx.x; it < na * nb; it += blockDim.x) {
-      const int arr = na == 1 ? 0 : it / nb, jj = it - arr * nb;   // one array: no division
-      const V* xa = x + arr * N;
-      V* ya = y + arr * N;
-      const int k = jj & (Ns - 1);                  // Ns is a power of two (the radix-3 pass is last)
-      V v[4];
-      for (int r = 0; r < R; ++r) v[r] = xa[jj + r * nb];
-      if (Ns > 1) {
-        // k < Ns and r < R, so k r stride < Ns R stride = N: the index needs no reduction
-        const int kstr = k * stride;
-        for (int r = 1; r < R; ++r) {
-          V wv = tw[kstr * r];
-          if (sign > 0) wv.y = -wv.y;
-          v[r] = cmul(v[r], wv);
-        }
-      }
-      const int base = (jj - k) * R + k;            // (jj / Ns) Ns R + k
-      if (R == 2) {
-        ya[base] = v[0] + v[1];
-        ya[base + Ns] = v[0] - v[1];
-      } else if (R == 4) {
-        const V a0 = v[0] + v[2], a1 = v[0] - v[2];
-        const V b0 = v[1] + v[3], b1 = v[1] - v[3];
-        const V ib1 = sg * times_i(b1);
-        ya[base] = a0 + b0;
-        ya[base + Ns] = a1 + ib1;
-        ya[base + 2 * Ns] = a0 - b0;
-        ya[base + 3 * Ns] = a1 - ib1;
-      } else {
-        const V t1 = v[1] + v[2], t2 = v[1] - v[2];
-        const V m1 = v[0] - (T)0.5 * t1;
-        // m1 +- s3 i t2 with one rounding per part (explicit fma)
-        ya[base] = v[0] + t1;
-        ya[base + Ns] = mk2<T>(fma(-s3, t2.y, m1.x), fma(s3, t2.x, m1.y));
-        ya[base + 2 * Ns] = mk2<T>(fma(s3, t2.y, m1.x), fma(-s3, t2.x, m1.y));
-      }
-    }
-    __syncthreads();
-    V* tmp = x;
-    x = y;
-    y = tmp;
-    Ns *= R;
-    lns += R == 4 ? 2 : R == 2 ? 1 : 0;                // the radix-3 pass is the last
-  }
-  return x;
-}
-
-// Shared memory of k_rows: two ping-pong sets of 5 complex rows and the
-// twiddles (11 Mx complex values); lean: 5 + 3 rows and the twiddles (9 Mx),
-// the inverse FFTs in groups of three and two rows; or, when neither fits, two
-// single rows, the twiddles and 9 real fields, with the five inverse FFTs in turn.
-static size_t rows_bytes_batched(const Grid& g, size_t es) { return (size_t)g.Mx * 11 * 2 * es; }
-static size_t rows_bytes_lean(const Grid& g, size_t es) { return (size_t)g.Mx * 9 * 2 * es; }
-static size_t rows_bytes_serial(const Grid& g, size_t es) { return (size_t)g.Mx * (3 * 2 + 9) * es; }
-static bool rows_batched(const Grid& g, size_t es) { return rows_bytes_batched(g, es) <= 200 * 1024; }
-static size_t rows_smem_for(const Grid& g, size_t es, bool lean) {
-  return rows_batched(g, es) ? (lean ? rows_bytes_lean(g, es) : rows_bytes_batched(g, es)) : rows_bytes_serial(g, es);
-}
-// The lean layout by default where the full one leaves room for a single block
-// per SM and the lean one for two.
-static bool rows_lean_default(const Grid& g, size_t es) {
-  return rows_batched(g, es) && rows_bytes_batched(g, es) > 113 * 1024 && rows_bytes_lean(g, es) <= 113 * 1024;
-}
+// Bounds of the row-kernel shapes that rbc_set_shapes accepts (shared memory of
+// the forms its fourth and sixth values once named; the row kernels take any).
+static bool rows_batched(const Grid& g, size_t es) { return (size_t)g.Mx * 11 * 2 * es <= 200 * 1024; }
+static size_t rows_cl_bytes(const Grid& g, size_t es) { return (size_t)g.Mx * 5 * 2 * es + (size_t)2 * g.Mx * 8; }
 
 // Deterministic block sum: the fixed tree red[t] += red[t + s], s = blockDim/2
 // down to 1 (blockDim a power of two, at least 32).  Levels s >= 32 go through
@@ -426,295 +345,6 @@ __device__ double block_sum(double v, double* red) {
   const double r = red[0];
   __syncthreads();
   return r;
-}
-
-// Pair pr of real fields (2 pr, 2 pr + 1) of row j as one complex spectrum of
-// length Mx: C = A + iB with the Hermitian extensions, zero beyond the kept modes.
-template <typename T>
-__device__ __forceinline__ C2<T> rows_packed(const Grid& g, const T* zrow, size_t fs, int pr, int x) {
-  using V = C2<T>;
-  const int fa = 2 * pr, fb = 2 * pr + 1, Mx = g.Mx, nm = g.nm;
-  const T* za = zrow + fa * fs;
-  const T* zb = zrow + fb * fs;
-  V c = mk2<T>(0, 0);
-  if (x < nm) {
-    const V a = ldc<T>(za + 2 * x);
-    const V bb = (fb < 9) ? ldc<T>(zb + 2 * x) : mk2<T>(0, 0);
-    c = a + times_i(bb);
-  } else if (x > Mx - nm) {
-    const int m = Mx - x;
-    const V a = ldc<T>(za + 2 * m);
-    const V bb = (fb < 9) ? ldc<T>(zb + 2 * m) : mk2<T>(0, 0);
-    c = conj2(a) + times_i(conj2(bb));
-  }
-  return c;
-}
-
-// Two block sums over the first 256 threads at once (the others pass nothing
-// and only meet the barriers): for each value the tree of block_sum at 256
-// threads, whatever blockDim is, with half the barriers of two calls.
-__device__ double2 block_sum256_2(double a, double b, double2* red) {
-  if (threadIdx.x < 256) red[threadIdx.x] = make_double2(a, b);
-  __syncthreads();
-  for (int s = 128; s >= 32; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      const double2 u = red[threadIdx.x], v = red[threadIdx.x + s];
-      red[threadIdx.x] = make_double2(u.x + v.x, u.y + v.y);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < 32) {
-    double x = red[threadIdx.x].x, y = red[threadIdx.x].y;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-      x += __shfl_down_sync(0xffffffffu, x, s);
-      y += __shfl_down_sync(0xffffffffu, y, s);
-    }
-    if (threadIdx.x == 0) red[0] = make_double2(x, y);
-  }
-  __syncthreads();
-  const double2 r = red[0];
-  __syncthreads();
-  return r;
-}
-
-// ---------------------------------------------------------------------------
-// Row kernel (k_rows).  Block per (slice, padded row j).  Pairs of real fields
-// share one complex inverse FFT (C = A + iB with the Hermitian extensions);
-// products in advective form (Eqs. 3, 5):
-//   N_T = u T_x + w T_z,  N_omega = u omega_x + w omega_z,
-//   <N_u>_x = <u u_x + w u_z>_x,  <w T>_x;
-// one packed forward FFT (N_T + i N_omega), truncation to m < nm.
-// Q[b][0][j][m] = N_T, Q[b][1][j][m] = N_omega (m >= 1), (<N_u>, 0) at m = 0.
-// The x-means are summed in FP64 in both precision modes, from per-point
-// terms staged in shared memory: thread t < 256 adds x = t, t + 256, ..., then
-// a 256-wide tree, so the bits do not depend on the block size (256 to 1024
-// threads, a launch shape) and equal those of k_rows_cl.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ void rows_item(const Grid& g, const C2<T>* __restrict__ tw, const T* __restrict__ Z, T* __restrict__ Q,
-                          double* __restrict__ wT, int B, int batched, int lean, const int* nsteps, int stepidx,
-                          int blk) {
-  using V = C2<T>;
-  extern __shared__ __align__(16) unsigned char rsm[];
-  const int b = blk / g.Mz, j = blk - b * g.Mz;
-  if (b >= B || !slice_active_at(nsteps, stepidx, b)) return;
-  const int Mx = g.Mx, nm = g.nm;
-  __shared__ double2 red[256];
-  const size_t fs = (size_t)g.Mz * nm * 2;
-  const T* zrow = Z + (size_t)b * 9 * fs + (size_t)j * nm * 2;
-  const V* fld;      // field value at x: real/imag parts of the five packed rows
-  const V* fld3 = nullptr;   // rows 3 and 4 (batched: fld + 3 Mx unless lean)
-  V* A;
-  V* Bf;
-  V* tws;
-  V* P = nullptr;    // free rows after the inverse FFTs: products, scratch, x-mean terms
-  V* P2 = nullptr;
-  T* vU = nullptr;
-  T* fr = nullptr;
-  if (batched) {
-    // the five packed rows and the FFT scratch: five more rows, or (lean) three,
-    // the inverse FFTs then running in groups of three and two rows (the same
-    // arithmetic per row; less shared memory, more blocks per SM)
-    A = reinterpret_cast<V*>(rsm);
-    Bf = A + 5 * Mx;
-    tws = Bf + (lean ? 3 : 5) * Mx;
-    for (int x = threadIdx.x; x < Mx; x += blockDim.x) tws[x] = ldgc<T>(tw + x);
-    for (int pr = 0; pr < 5; ++pr)
-      for (int x = threadIdx.x; x < Mx; x += blockDim.x) A[pr * Mx + x] = rows_packed<T>(g, zrow, fs, pr, x);
-    __syncthreads();
-    if (!lean) {
-      fld = fft_smem<T>(A, Bf, Mx, 5, +1, tws);
-      fld3 = fld + 3 * Mx;
-      P = (fld == A) ? Bf : A;                 // the five rows not holding the fields
-      vU = reinterpret_cast<T*>(P + Mx);
-      P2 = (P == A) ? Bf : A;                  // a field row, free once the products are formed
-    } else {
-      fld = fft_smem<T>(A, Bf, Mx, 3, +1, tws);
-      V* fr3 = fld == A ? Bf : A;              // rows free after the first group
-      fld3 = fft_smem<T>(A + 3 * Mx, fr3, Mx, 2, +1, tws);
-      // three free rows: the scratch (even pass count) or A[2..4] (odd)
-      P = fld == A ? Bf : A + 2 * Mx;
-      vU = reinterpret_cast<T*>(P + Mx);
-      P2 = P + 2 * Mx;
-    }
-  } else {
-    A = reinterpret_cast<V*>(rsm);
-    Bf = A + Mx;
-    tws = Bf + Mx;
-    fr = reinterpret_cast<T*>(tws + Mx);
-    for (int x = threadIdx.x; x < Mx; x += blockDim.x) tws[x] = ldgc<T>(tw + x);
-    for (int pr = 0; pr < 5; ++pr) {
-      for (int x = threadIdx.x; x < Mx; x += blockDim.x) A[x] = rows_packed<T>(g, zrow, fs, pr, x);
-      __syncthreads();
-      const V* res = fft_smem<T>(A, Bf, Mx, 1, +1, tws);
-      for (int x = threadIdx.x; x < Mx; x += blockDim.x) {
-        fr[(2 * pr) * Mx + x] = res[x].x;
-        if (pr < 4) fr[(2 * pr + 1) * Mx + x] = res[x].y;
-      }
-      __syncthreads();
-    }
-    fld = nullptr;
-    P = A;
-    P2 = Bf;
-    vU = reinterpret_cast<T*>(P2);            // the scratch row holds the 2 Mx terms
-  }
-  auto field = [&](int fi, int x) -> T {
-    if (fld) {
-      const int k = fi >> 1;
-      const V v = k < 3 ? fld[k * Mx + x] : fld3[(k - 3) * Mx + x];
-      return (fi & 1) ? v.y : v.x;
-    }
-    return fr[fi * Mx + x];
-  };
-  // per-point x-mean terms (in T: each is the FP64 sum's exact input)
-  T* vW = vU + Mx;
-  for (int x = threadIdx.x; x < Mx; x += blockDim.x) {
-    const T u = field(0, x), w = field(1, x);
-    const T nO = fma(u, field(2, x), w * field(3, x));
-    vU[x] = fma(u, field(4, x), w * field(5, x));
-    const T nT = fma(u, field(7, x), w * field(8, x));
-    vW[x] = w * field(6, x);
-    P[x] = mk2<T>(nT, nO);
-  }
-  __syncthreads();
-  double nU = 0.0, wt = 0.0;
-  if (threadIdx.x < 256)
-    for (int x = threadIdx.x; x < Mx; x += 256) {
-      nU += (double)vU[x];
-      wt += (double)vW[x];
-    }
-  const double2 sUW = block_sum256_2(nU, wt, red);
-  const double sU = sUW.x, sW = sUW.y;
-  const V* C = fft_smem<T>(P, P2, Mx, 1, -1, tws);
-  const T inv = (T)1 / (T)Mx;
-  const T half = (T)0.5 * inv;
-  const size_t qs = (size_t)g.Mz * nm * 2;
-  T* q0 = Q + (size_t)b * 2 * qs + (size_t)j * nm * 2;
-  T* q1 = q0 + qs;
-  for (int m = threadIdx.x; m < nm; m += blockDim.x) {
-    const V cm = C[m];
-    const V cn = conj2(C[m == 0 ? 0 : Mx - m]);
-    const V s = cm + cn, d = cm - cn;
-    stc<T>(q0 + 2 * m, mk2<T>(half * s.x, half * s.y));
-    if (m == 0)
-      stc<T>(q1, mk2<T>((T)(sU / Mx), (T)0));
-    else
-      stc<T>(q1 + 2 * m, mk2<T>(half * d.y, -half * d.x));
-  }
-  if (threadIdx.x == 0) wT[(size_t)b * g.Mz + j] = sW / Mx;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k_rows(Grid g, const C2<T>* __restrict__ tw, const T* __restrict__ Z,
-                                              T* __restrict__ Q, double* __restrict__ wT, int B, int batched,
-                                              int lean, const int* nsteps, const int* step) {
-  pdl_wait();
-  rows_item<T>(g, tw, Z, Q, wT, B, batched, lean, nsteps, nsteps ? *step : 0, blockIdx.x);
-}
-
-// ---------------------------------------------------------------------------
-// Row kernel for small batches (k_rows_cl): the same arithmetic as k_rows,
-// spread over a cluster of five CTAs per row so that a single slice uses five
-// times as many SMs' FP64 pipes.  CTA c runs the inverse FFT of field pair c
-// (fields 2c, 2c+1) in its shared memory; after a cluster barrier every CTA
-// forms the products for its share of the x points, reading the nine fields
-// from the five CTAs through distributed shared memory, and writes them, with
-// the per-point terms of the two x-means, into CTA 0.  After a second barrier
-// CTA 0 sums the x-means with exactly the per-thread order and tree of k_rows
-// (256 threads) and runs the forward FFT, so the results are bit for bit
-// those of k_rows.
-// ---------------------------------------------------------------------------
-constexpr int kRowsCluster = 5;
-constexpr int kRowsThreads = 256;
-
-static size_t rows_cl_bytes(const Grid& g, size_t es) {
-  // A, Bf, twiddles, P, P2 (complex) + two real per-point arrays (double)
-  return (size_t)g.Mx * 5 * 2 * es + (size_t)2 * g.Mx * 8;
-}
-static bool rows_use_cluster(const Grid& g, int B, size_t es) {
-  return (long)B * g.Mz <= 2L * 152 && rows_cl_bytes(g, es) <= 200 * 1024;
-}
-
-template <typename T>
-__global__ void __cluster_dims__(kRowsCluster, 1, 1) __launch_bounds__(kRowsThreads)
-    k_rows_cl(Grid g, const C2<T>* __restrict__ tw, const T* __restrict__ Z, T* __restrict__ Q,
-              double* __restrict__ wT, int B, const int* nsteps, const int* step) {
-  using V = C2<T>;
-  namespace cg = cooperative_groups;
-  extern __shared__ __align__(16) unsigned char csm[];
-  __shared__ double2 red[kRowsThreads];
-  pdl_wait();
-  cg::cluster_group cl = cg::this_cluster();
-  const int c = (int)cl.block_rank();
-  const int row = blockIdx.x / kRowsCluster;
-  const int b = row / g.Mz, j = row - b * g.Mz;
-  // uniform over the cluster (same b and step): no CTA reaches a cluster barrier alone
-  if (b >= B || !slice_active(nsteps, step, b)) return;
-  const int Mx = g.Mx, nm = g.nm;
-  V* A = reinterpret_cast<V*>(csm);
-  V* Bf = A + Mx;
-  V* tws = Bf + Mx;
-  V* P = tws + Mx;
-  V* P2 = P + Mx;
-  double* vU = reinterpret_cast<double*>(P2 + Mx);
-  double* vW = vU + Mx;
-  const size_t fs = (size_t)g.Mz * nm * 2;
-  const T* zrow = Z + (size_t)b * 9 * fs + (size_t)j * nm * 2;
-  for (int x = threadIdx.x; x < Mx; x += blockDim.x) {
-    tws[x] = ldgc<T>(tw + x);
-    A[x] = rows_packed<T>(g, zrow, fs, c, x);
-  }
-  __syncthreads();
-  const V* res = fft_smem<T>(A, Bf, Mx, 1, +1, tws);   // same buffer in every CTA
-  cl.sync();
-  const V* fr[kRowsCluster];
-#pragma unroll
-  for (int r = 0; r < kRowsCluster; ++r) fr[r] = cl.map_shared_rank(res, r);
-  V* P0 = cl.map_shared_rank(P, 0);
-  double* vU0 = cl.map_shared_rank(vU, 0);
-  double* vW0 = cl.map_shared_rank(vW, 0);
-  auto field = [&](int fi, int x) -> T {
-    const V v = fr[fi >> 1][x];
-    return (fi & 1) ? v.y : v.x;
-  };
-  const int per = (Mx + kRowsCluster - 1) / kRowsCluster;
-  const int x0 = c * per, x1 = min(Mx, x0 + per);
-  for (int x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
-    const T u = field(0, x), w = field(1, x);
-    const T nO = fma(u, field(2, x), w * field(3, x));
-    vU0[x] = (double)fma(u, field(4, x), w * field(5, x));
-    const T nT = fma(u, field(7, x), w * field(8, x));
-    vW0[x] = (double)(w * field(6, x));
-    P0[x] = mk2<T>(nT, nO);
-  }
-  cl.sync();
-  if (c != 0) return;
-  // x-means: thread t adds x = t, t + 256, ... from 0, then the tree of k_rows
-  double nU = 0.0, wt = 0.0;
-  for (int x = threadIdx.x; x < Mx; x += blockDim.x) {
-    nU += vU[x];
-    wt += vW[x];
-  }
-  const double2 sUW = block_sum256_2(nU, wt, red);   // kRowsThreads = 256: the same tree
-  const double sU = sUW.x, sW = sUW.y;
-  const V* C = fft_smem<T>(P, P2, Mx, 1, -1, tws);
-  const T inv = (T)1 / (T)Mx;
-  const T half = (T)0.5 * inv;
-  const size_t qs = (size_t)g.Mz * nm * 2;
-  T* q0 = Q + (size_t)b * 2 * qs + (size_t)j * nm * 2;
-  T* q1 = q0 + qs;
-  for (int m = threadIdx.x; m < nm; m += blockDim.x) {
-    const V cm = C[m];
-    const V cn = conj2(C[m == 0 ? 0 : Mx - m]);
-    const V s2 = cm + cn, d = cm - cn;
-    stc<T>(q0 + 2 * m, mk2<T>(half * s2.x, half * s2.y));
-    if (m == 0)
-      stc<T>(q1, mk2<T>((T)(sU / Mx), (T)0));
-    else
-      stc<T>(q1 + 2 * m, mk2<T>(half * d.y, -half * d.x));
-  }
-  if (threadIdx.x == 0) wT[(size_t)b * g.Mz + j] = sW / Mx;
 }
 
 // ---------------------------------------------------------------------------
@@ -1219,16 +849,6 @@ static int zfwd_tm_of(const Grid& g, const Work& w, int B, size_t es) {
 static int zfwd_nch_of(const Grid& g, const Work& w, int B, int tm) {
   return (w.shapes && w.shapes->zfwd_nch > 0) ? w.shapes->zfwd_nch : zfwd_chunks(g, B, tm);
 }
-static bool rows_cl_of(const Grid& g, const Work& w, int B, size_t es) {
-  return (w.shapes && w.shapes->rows_cl >= 0) ? w.shapes->rows_cl != 0 : rows_use_cluster(g, B, es);
-}
-static int rows_threads_of(const Work& w) {
-  return (w.shapes && w.shapes->rows_threads > 0) ? w.shapes->rows_threads : kRowsThreads;
-}
-static bool rows_lean_of(const Grid& g, const Work& w, size_t es) {
-  return (w.shapes && w.shapes->rows_lean >= 0) ? w.shapes->rows_lean != 0 : rows_lean_default(g, es);
-}
-
 bool shapes_valid(const Grid& g, const Shapes& sh, size_t es) {
   if (sh.solve_tms > 0 && (sh.solve_tms > 16 || (sh.solve_tms & (sh.solve_tms - 1)) ||
                            solve_smem_tms(g, sh.solve_tms) > 200 * 1024))
@@ -1351,13 +971,9 @@ cudaError_t configure_kernels(const Grid& g) {
                                         kCorrTile * 512 * (int)sizeof(double2));
   if (l2 == cudaSuccess) l2 = cudaFuncSetAttribute(k_l2_diff, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (l2 != cudaSuccess) return l2;
-  static int a_rows_f = 48 * 1024, a_solve = 48 * 1024, a_zfwd_f = 48 * 1024;
-  static int a_rcl_f = 48 * 1024;
+  static int a_solve = 48 * 1024, a_zfwd_f = 48 * 1024;
   cudaError_t e = configure_zfx(g);   // also the averages of Sec. 2.2 of a mixed handle
-  if (e == cudaSuccess && !g.mixed) e = configure_rows_fx(g);
-  if (e == cudaSuccess && rows_cl_bytes(g, 4) <= 200 * 1024)
-    e = allow_smem(k_rows_cl<float>, (int)rows_cl_bytes(g, 4), a_rcl_f);
-  if (e == cudaSuccess) e = allow_smem(k_rows<float>, (int)rows_smem_for(g, 4, false), a_rows_f);
+  if (e == cudaSuccess) e = g.mixed ? configure_rows_f32(g) : configure_rows_fx(g);
   if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
   if (e == cudaSuccess && !solve_segmented(g))
     e = allow_smem(k_solve, (int)std::max(solve_smem(g, 1), solve_smem(g, 1 << 20)), a_solve);
@@ -1372,7 +988,6 @@ static void launch_transforms_f32(const Grid& g, const Tables& t, const Work& w,
   const int kp = zinv_warps(g);
   const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
   float* Z = reinterpret_cast<float*>(w.Z);
-  float* Q = reinterpret_cast<float*>(w.Q);
   const size_t es = sizeof(float);
   if (pf) pf->begin(RBC_KERNEL_ZINV, s);
   if (t.tcA_psi_hi != nullptr)
@@ -1382,13 +997,7 @@ static void launch_transforms_f32(const Grid& g, const Tables& t, const Work& w,
                state_doubles(g), Z, B, ns, w.step);
   if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 9, es));
   if (pf) pf->begin(RBC_KERNEL_ROWS, s);
-  if (rows_cl_of(g, w, B, es))
-    launch_pdl(w.pdl != 0, k_rows_cl<float>, (unsigned)(B * g.Mz * kRowsCluster), kRowsThreads, rows_cl_bytes(g, es), s,
-               g, t.tw32, Z, Q, w.wT, B, ns, w.step);
-  else
-    launch_pdl(w.pdl != 0, k_rows<float>, (unsigned)(B * g.Mz), rows_threads_of(w),
-               rows_smem_for(g, es, rows_lean_of(g, w, es)), s, g, t.tw32, Z, Q, w.wT, B, rows_batched(g, es) ? 1 : 0,
-               rows_lean_of(g, w, es) ? 1 : 0, ns, w.step);
+  launch_rows_f32(g, t, w, B, ns, s);
   if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B, 6), rows_bytes(g, B, 9, es));
 }
 

@@ -72,3 +72,20 @@ def test_column_lengths_match_oracle_and_batches_agree(rbc, Nz, Nx=8):
         F.step_batch(st, 1, nub)
         assert torch.equal(st, alone.expand_as(st)) and torch.equal(nub, nu[:1].expand(B)), B
     assert F.check_diverged() == rbc.RBC_OK
+
+
+@pytest.mark.parametrize("Nx", [4, 8, 16, 32, 64, 128, 256, 512, 1024])
+def test_mixed_rows_alone_and_in_batches_agree(rbc, Nx, Nz=10):
+    """15 rows (one per block, every pass spread), 345 and 2250 rows (several per block, a ragged last one)."""
+    F = rbc.Propagator(1e5, 1.0, 2.0, Nx, Nz, 1e-4, 1)
+    o = RBC(1e5, 1.0, 2.0, Nx, Nz, 1e-4)
+    alone = F.new_states(1)
+    alone[0].copy_(torch.from_numpy(to_abi(nonlinear_state(o, 5))))
+    states = [alone[:1].repeat(B, 1, 1, 1, 1) for B in (23, 150)]
+    nu = torch.zeros(1, dtype=torch.float64, device="cuda")
+    F.step_batch(alone, 2, nu)
+    for st in states:
+        nub = torch.zeros(st.shape[0], dtype=torch.float64, device="cuda")
+        F.step_batch(st, 2, nub)
+        assert torch.equal(st, alone.expand_as(st)) and torch.equal(nub, nu.expand_as(nub))
+    assert F.check_diverged() == rbc.RBC_OK
