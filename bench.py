@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "e4ba3c1ad885cea77ea7e84e465d90168a694128fd4fc749035b2aaddd256255"
+NCU_TRAFFIC_SHA256 = "712c3f0afa35826772be67cda2aa0f6489b694b99e9564565dc3b7371299a7ad"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 135066, "coarse:k_rows": 386867, "coarse:k_zfwd": 123072, "coarse:k_solve": 831232,
-    "fine:k_zinv@32": 10437888, "fine:k_rows@32": 37880115, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23858048,
-    "fine:k_zinv@2": 671027, "fine:k_rows@2": 2490931, "fine:k_zfwd@2": 830208, "fine:k_solve@2": 2765056,
+    "coarse:k_zinv": 135066, "coarse:k_rows": 386458, "coarse:k_zfwd": 123456, "coarse:k_solve": 802688,
+    "fine:k_zinv@32": 10447206, "fine:k_rows@32": 37880269, "fine:k_zfwd@32": 12631040, "fine:k_solve@32": 23876224,
+    "fine:k_zinv@2": 671488, "fine:k_rows@2": 2492672, "fine:k_zfwd@2": 832768, "fine:k_solve@2": 2769408,
 }
 
 

@@ -20,6 +20,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "rbc_internal.h"
 
@@ -462,7 +463,7 @@ struct SolveSmem {
   const double* X;   // step-start state of this slice (global; stage 1)
   double* y;    // [nq][W] right-hand side, then solution
   double* r;    // [nq][W] r_i of the tau rows
-  double* T;    // [nq][W] T_i, kept for the psi coupling; the dense path's solution of each system
+  double* T;    // [nq][W] T_i, kept for the psi coupling
   int W;        // columns = 2 * tms
   double Ra;    // Rayleigh number of this slice
   double cpl;   // ((gamma dt) Pr) Ra of this slice
@@ -637,42 +638,17 @@ __device__ __forceinline__ bool solve_recurrence(const Grid& g, const Tables& tb
   return ok;
 }
 
-// phases 2-3 for small grids: x_r = sum_q Ainv[r][q] b_q for one (row r, column
-// col); b holds the boundary values in rows 0 .. D-1 and the tau right-hand
-// sides below them.
-template <int KIND>
-__device__ __forceinline__ bool solve_dense(const Grid& g, const Tables& tb, int p, int m, int c, int r, int col,
-                                            const SolveSmem& sm, double* __restrict__ Xo) {
-  const int nq = g.nq, W = sm.W;
-  const int f = (KIND == KT) ? 0 : 1;
-  const int nmod = (KIND == KU) ? 1 : g.nm;
-  const int mi = (KIND == KU) ? 0 : m;
-  const double* inv = (KIND == KT) ? tb.T_inv : (KIND == KP) ? tb.P_inv : tb.U_inv;
-  const double* row = inv + ((size_t)p * nq + r) * nq * nmod + mi;
-  double acc0 = 0.0, acc1 = 0.0;                       // two partial sums: shorter chain
-  for (int q = 0; q + 1 < nq; q += 2) {
-    acc0 = fma(__ldg(row + (size_t)q * nmod), sm.y[q * W + col], acc0);
-    acc1 = fma(__ldg(row + (size_t)(q + 1) * nmod), sm.y[(q + 1) * W + col], acc1);
-  }
-  if (nq & 1) acc0 = fma(__ldg(row + (size_t)(nq - 1) * nmod), sm.y[(nq - 1) * W + col], acc0);
-  const double x = acc0 + acc1;
-  sm.T[r * W + col] = x;
-  Xo[soff(g, f, 2 * r + p, m) + c] = x;
-  return isfinite(x);
-}
-
 // phase 4 for one (tau row t, column col)
 template <int KIND>
 __device__ __forceinline__ void solve_lx(const Grid& g, const Tables& tb, int stage, int p, int m, int c, int t,
-                                         int col, const SolveSmem& sm, const double* xs, double* __restrict__ R,
-                                         size_t S) {
+                                         int col, const SolveSmem& sm, double* __restrict__ R, size_t S) {
   using SY = Sys<KIND>;
   const int nq = g.nq, W = sm.W;
   const int f = (KIND == KT) ? 0 : 1;
   double mx = 0.0;
 #pragma unroll
   for (int j = 0; j <= SY::LAM; ++j)
-    if (t + j < nq) mx = fma(SY::tapM(g, tb, p, t, j, m), xs[(t + j) * W + col], mx);
+    if (t + j < nq) mx = fma(SY::tapM(g, tb, p, t, j, m), sm.y[(t + j) * W + col], mx);
   const double lx2 = g.inv_gamma * (mx - sm.r[t * W + col]);   // dt (L X_i + coupling)
   const size_t ro = soff(g, f, 2 * t + p, m) + c;
 #pragma unroll
@@ -681,6 +657,27 @@ __device__ __forceinline__ void solve_lx(const Grid& g, const Tables& tb, int st
       double* Rl = R + (size_t)(l + 1) * S + ro;
       *Rl = fma(c_AI[g.scheme][l + 2][stage], lx2, *(Rl));
     }
+}
+
+// Nu_V(t_n) (Eq. 9) of the step-start state: wall temperature difference of
+// the mean profile + Clenshaw-Curtis integral of <wT>_x; trapezoid weight.
+// The first warp of the block of the odd coefficients of mode 0 sums it: each
+// lane a strided share of both sums, then a fixed shuffle tree (the order
+// depends on the grid only).  That block overwrites these coefficients only
+// after its barriers (a one-stage scheme writes X0 itself).
+__device__ __forceinline__ void nu_integral(const Grid& g, const Tables& tb, const double* X0, const double* wT,
+                                            double* nu, int b, int stepidx) {
+  if (threadIdx.x >= 32 || nu == nullptr) return;
+  const int lane = threadIdx.x;
+  double cond = 0.0, adv = 0.0;
+  for (int n = 2 * lane + 1; n < g.Nz; n += 64) cond -= 2.0 * *(X0 + soff(g, 0, n, 0));
+  for (int jz = lane; jz < g.Mz; jz += 32) adv = fma(__ldg(tb.cc + jz), *(wT + (size_t)b * g.Mz + jz), adv);
+#pragma unroll
+  for (int sh = 16; sh > 0; sh >>= 1) {
+    cond += __shfl_down_sync(0xffffffffu, cond, sh);
+    adv += __shfl_down_sync(0xffffffffu, adv, sh);
+  }
+  if (lane == 0) nu[b] += ((stepidx == 0) ? 0.5 : 1.0) * g.dt * (cond + 0.5 * adv);
 }
 
 __device__ void solve_item(const Grid& g, const Tables& tb, double* X, double* Xs, const double* F, double* R,
@@ -713,27 +710,9 @@ __device__ void solve_item(const Grid& g, const Tables& tb, double* X, double* X
   sm.F = Fb;
   sm.X = X0;
   double* Rb = R + (size_t)b * 4 * S;
-  if (stage == 1 && m0 == 0 && p == 1 && threadIdx.x < 32 && nu != nullptr) {
-    // Nu_V(t_n) (Eq. 9) of the step-start state: wall temperature difference of
-    // the mean profile + Clenshaw-Curtis integral of <wT>_x; trapezoid weight.
-    // The first warp sums it: each lane a strided share of both sums, then a
-    // fixed shuffle tree (the order depends on the grid only). The odd
-    // coefficients read here belong to this block, which overwrites them only
-    // after the barriers below (a one-stage scheme writes X0 here).
-    const int lane = threadIdx.x;
-    double cond = 0.0, adv = 0.0;
-    for (int n = 2 * lane + 1; n < g.Nz; n += 64) cond -= 2.0 * *(X0 + soff(g, 0, n, 0));
-    for (int jz = lane; jz < g.Mz; jz += 32) adv = fma(__ldg(tb.cc + jz), *(wT + (size_t)b * g.Mz + jz), adv);
-#pragma unroll
-    for (int sh = 16; sh > 0; sh >>= 1) {
-      cond += __shfl_down_sync(0xffffffffu, cond, sh);
-      adv += __shfl_down_sync(0xffffffffu, adv, sh);
-    }
-    if (lane == 0) nu[b] += ((stepidx == 0) ? 0.5 : 1.0) * g.dt * (cond + 0.5 * adv);
-  }
+  if (stage == 1 && m0 == 0 && p == 1) nu_integral(g, tb, X0, wT, nu, b, stepidx);
   bool ok = true;
-  for (int sys = 0; sys < 2; ++sys) {
-    const int f = sys;                               // field 0 = T, 1 = psi / U
+  for (int sys = 0; sys < 2; ++sys) {   // T, then psi / U
     // phase 1
     const int ntmax = nq - 1;
     for (int it = threadIdx.x; it < ntmax * W; it += blockDim.x) {
@@ -748,33 +727,7 @@ __device__ void solve_item(const Grid& g, const Tables& tb, double* X, double* X
         solve_rhs<KP>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
     }
     __syncthreads();
-    const bool dense = g.nq <= kDenseSolveMaxNq;
-    if (dense) {
-      // boundary rows of b: the mean temperature's wall values (Eq. 6) or
-      // slopes (Eq. 7) in parity combinations; zero for T at m >= 1, psi and U
-      for (int it = threadIdx.x; it < 2 * W; it += blockDim.x) {
-        const int r = it >> lw, col = it & (W - 1);
-        if (col >= ncol) continue;
-        const int m = m0 + col / 2, c = col & 1;
-        const int D = (sys == 1 && m != 0) ? 2 : 1;
-        if (r >= D) continue;
-        sm.y[r * W + col] = (sys == 0 && m == 0 && c == 0) ? t_wall_rhs(g, p) : 0.0;
-      }
-      __syncthreads();
-      for (int it = threadIdx.x; it < nq * W; it += blockDim.x) {
-        const int r = it >> lw, col = it & (W - 1);
-        if (col >= ncol) continue;
-        const int m = m0 + col / 2, c = col & 1;
-        bool o2;
-        if (sys == 0)
-          o2 = solve_dense<KT>(g, tb, p, m, c, r, col, sm, Xo);
-        else if (m == 0)
-          o2 = solve_dense<KU>(g, tb, p, m, c, r, col, sm, Xo);
-        else
-          o2 = solve_dense<KP>(g, tb, p, m, c, r, col, sm, Xo);
-        ok = ok && o2;
-      }
-    } else if ((int)threadIdx.x < ncol) {
+    if ((int)threadIdx.x < ncol) {
       // phases 2, 3: one column per thread, columns packed into the fewest warps
       // (an FP64 warp instruction occupies its sub-partition's FP64 pipe for the
       // same time however many lanes are active, so packing is cheapest)
@@ -789,7 +742,6 @@ __device__ void solve_item(const Grid& g, const Tables& tb, double* X, double* X
       ok = ok && o2;
     }
     __syncthreads();
-    const double* xs = dense ? sm.T : sm.y;
     // phase 4
     if (stage < g.ns) {
       for (int it = threadIdx.x; it < ntmax * W; it += blockDim.x) {
@@ -797,11 +749,11 @@ __device__ void solve_item(const Grid& g, const Tables& tb, double* X, double* X
         if (col >= ncol) continue;
         const int m = m0 + col / 2, c = col & 1;
         if (sys == 0)
-          solve_lx<KT>(g, tb, stage, p, m, c, t, col, sm, xs, Rb, S);
+          solve_lx<KT>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
         else if (m == 0)
-          solve_lx<KU>(g, tb, stage, p, m, c, t, col, sm, xs, Rb, S);
+          solve_lx<KU>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
         else if (t < nq - 2)
-          solve_lx<KP>(g, tb, stage, p, m, c, t, col, sm, xs, Rb, S);
+          solve_lx<KP>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
       }
     }
     __syncthreads();
@@ -818,6 +770,174 @@ __global__ void __launch_bounds__(256) k_solve(Grid g, Tables tb, double* X, dou
                                                const int* step) {
   pdl_wait();
   solve_item(g, tb, X, Xs, F, R, S, wT, nu, flags, err, B, stage, tms, ra, nsteps, nsteps ? *step : 0, blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// Stage solve of small grids (k_solve_dense, nq <= kDenseSolveMaxNq), both modes:
+// x = Ainv b with the dense inverses, one thread per (row r, column), which is
+// tau row r of the right-hand side, row r of the product and tau row r of
+// dt L X_i in turn.  Everything a thread needs from global memory is fetched at
+// the start, the rows of Ainv before the launch before it has finished; r_i and
+// the later accumulators stay in registers between the right-hand side and
+// dt L X_i.
+// Bound: latency (one trip to memory, then about 50 FP64 instructions in a
+// row; blocks of one mode leave one warp per sub-partition).  Measured (GB300,
+// a whole stage; as phases of k_solve, each with its own trips to memory,
+// before): 128 x 32, one state 33.6 -> 31.3 us in FP64, 25.7 -> 23.2 us in mixed
+// precision; 64 x 32, 23 states 49.5 -> 46.1 us and 41.0 -> 37.3 us.
+// ---------------------------------------------------------------------------
+constexpr int kDenseThreads = 256;   // rows times columns of a tile
+
+// finite, from the exponent bits (an FP64 comparison would occupy the FP64 pipe)
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+__global__ void __launch_bounds__(kDenseThreads) k_solve_dense(Grid g, Tables tb, double* X, double* Xs, const double* F,
+                                                               double* R, size_t S, const double* wT, double* nu,
+                                                               int* flags, int* err, int B, int stage, int tms,
+                                                               const double* ra, const int* nsteps, const int* step) {
+  constexpr int NQ = kDenseSolveMaxNq;
+  __shared__ double y[kDenseThreads], xT[kDenseThreads];   // [nq][W]: right-hand side; solution
+  const int nq = g.nq, W = 2 * tms, lw = __ffs(W) - 1, mt = (g.nm + tms - 1) / tms;
+  const int b = blockIdx.x / (2 * mt), rem = blockIdx.x - b * 2 * mt, p = rem / mt, m0 = (rem - p * mt) * tms;
+  const int t = threadIdx.x >> lw, col = threadIdx.x & (W - 1), m = m0 + col / 2, c = col & 1;
+  const bool on = t < nq && m < g.nm;
+  double a[NQ];
+  auto fetch_inv = [&](const double* inv, int nmod, int mi) {
+    const double* row = inv + ((size_t)p * nq + t) * nq * nmod + mi;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) a[q] = (on && q < nq) ? __ldg(row + (size_t)q * nmod) : 0.0;
+  };
+  fetch_inv(tb.T_inv, g.nm, m);
+  pdl_wait();
+  const int stepidx = nsteps ? *step : 0;
+  if (b >= B || !slice_active_at(nsteps, stepidx, b)) return;   // uniform per block
+  if (flags[b] & kFlagTimeout) return;                          // as in solve_item
+  double* X0 = X + (size_t)b * S;
+  double* Xo = (stage == g.ns) ? X0 : Xs + (size_t)b * S;
+  const double* Fb = F + (size_t)b * S;
+  double* Rb = R + (size_t)b * 4 * S;
+  const double Ra = ra ? ra[b] : g.Ra;
+  const double cpl = (c == 0 ? __ldg(tb.dtae + 25) * Ra : -(__ldg(tb.dtae + 25) * Ra)) * (g.kfac * m);
+  const int ns = g.ns;
+
+  // tau row t of field f: taps of F, of X (stage 1) or the accumulated r_i, later accumulators
+  struct Row {
+    double f[5], x[5], R[3];
+  } rows[2];
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    const int lam = f == 1 && m != 0 ? 4 : 2, nt = nq - lam / 2;
+    Row& w = rows[f];
+    const bool mine = on && t < nt;
+    const size_t ro = soff(g, f, 2 * t + p, m) + c;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      const bool in = mine && j <= lam && t + j < nq;
+      w.f[j] = in ? Fb[soff(g, f, 2 * (t + j) + p, m) + c] : 0.0;
+      w.x[j] = in && stage == 1 ? X0[soff(g, f, 2 * (t + j) + p, m) + c] : 0.0;
+    }
+    if (stage > 1 && mine) w.x[0] = Rb[(size_t)(stage - 1) * S + ro];
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+      w.R[l] = (mine && stage > 1 && l + 2 > stage && l + 2 <= ns) ? Rb[(size_t)(l + 1) * S + ro] : 0.0;
+  }
+  if (stage == 1 && m0 == 0 && p == 1) nu_integral(g, tb, X0, wT, nu, b, stepidx);
+
+  bool ok = true;
+  auto system = [&](auto kind, int f) {
+    constexpr int KIND = decltype(kind)::value;
+    using SY = Sys<KIND>;
+    Row& w = rows[f];
+    const bool mine = on && t < nq - SY::D;
+    double r = 0.0;
+    if (mine) {
+      double fv = 0.0;
+#pragma unroll
+      for (int j = 0; j <= SY::LAM; ++j)
+        if (t + j < nq) fv = fma(SY::tapF(g, tb, p, t, j), w.f[j], fv);
+      if (KIND != KP) fv = -fv;
+      if (stage == 1) {
+        double mx = 0.0;
+#pragma unroll
+        for (int j = 0; j <= SY::LAM; ++j)
+          if (t + j < nq) mx = fma(SY::tapM(g, tb, p, t, j, m), w.x[j], mx);
+        r = fma(__ldg(tb.dtae + 5), fv, mx);
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+          if (l + 2 <= ns) w.R[l] = fma(__ldg(tb.dtae + (l + 2) * 5), fv, mx);
+      } else {
+        r = fma(__ldg(tb.dtae + stage * 5 + stage - 1), fv, w.x[0]);
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+          if (l + 2 > stage && l + 2 <= ns) w.R[l] = fma(__ldg(tb.dtae + (l + 2) * 5 + stage - 1), fv, w.R[l]);
+      }
+      double bv = r;
+      if (KIND == KP) {
+        double st = 0.0;
+#pragma unroll
+        for (int j = 0; j <= 4; ++j)
+          if (t + j < nq) st = fma(__ldg(tb.s4 + (p * nq + t) * 5 + j), xT[(t + j) * W + (col ^ 1)], st);
+        bv = fma(cpl, st, bv);
+      }
+      y[(t + SY::D) * W + col] = bv;
+    }
+    // boundary rows of b: the mean temperature's wall values (Eq. 6) or slopes
+    // (Eq. 7) in parity combinations; zero for T at m >= 1, psi and U
+    if (on && t < SY::D) y[t * W + col] = (KIND == KT && m == 0 && c == 0) ? t_wall_rhs(g, p) : 0.0;
+    return r;
+  };
+  // rows of the product, dt L X_i into the later accumulators
+  auto finish = [&](auto kind, int f, double r) {
+    constexpr int KIND = decltype(kind)::value;
+    using SY = Sys<KIND>;
+    if (!(on && t < nq - SY::D && stage < ns)) return;
+    double mx = 0.0;
+#pragma unroll
+    for (int j = 0; j <= SY::LAM; ++j)
+      if (t + j < nq) mx = fma(SY::tapM(g, tb, p, t, j, m), xT[(t + j) * W + col], mx);
+    const double lx2 = g.inv_gamma * (mx - r);
+    const size_t ro = soff(g, f, 2 * t + p, m) + c;
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+      if (l + 2 > stage && l + 2 <= ns) Rb[(size_t)(l + 1) * S + ro] = fma(c_AI[g.scheme][l + 2][stage], lx2, rows[f].R[l]);
+  };
+  auto product = [&](int f) {
+    if (!on) return;
+    double acc0 = 0.0, acc1 = 0.0;                       // two partial sums: shorter chain
+#pragma unroll
+    for (int q = 0; q < NQ; q += 2) {
+      if (q < nq) acc0 = fma(a[q], y[q * W + col], acc0);
+      if (q + 1 < nq) acc1 = fma(a[q + 1], y[(q + 1) * W + col], acc1);
+    }
+    const double x = acc0 + acc1;
+    xT[t * W + col] = x;
+    Xo[soff(g, f, 2 * t + p, m) + c] = x;
+    ok = ok && finite_bits(x);
+  };
+  using T_ = std::integral_constant<int, KT>;
+  using P_ = std::integral_constant<int, KP>;
+  using U_ = std::integral_constant<int, KU>;
+  const double rT = system(T_(), 0);
+  __syncthreads();
+  product(0);
+  if (m == 0)
+    fetch_inv(tb.U_inv, 1, 0);
+  else
+    fetch_inv(tb.P_inv, g.nm, m);
+  __syncthreads();
+  finish(T_(), 0, rT);
+  const double rP = m == 0 ? system(U_(), 1) : system(P_(), 1);
+  __syncthreads();
+  product(1);
+  __syncthreads();
+  if (m == 0)
+    finish(U_(), 1, rP);
+  else
+    finish(P_(), 1, rP);
+  if (!ok) {
+    atomicOr(flags + b, kFlagNonFinite);
+    atomicOr(err, kFlagNonFinite);
+  }
 }
 
 // Modes per k_solve block.  Every column's arithmetic is independent of the
@@ -1053,9 +1173,12 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   if (solve_segmented(g)) {
     e = launch_solve_seg(g, t, w, X, B, stage, nu, s);
   } else {
-    const int tms = solve_tms_of(g, w, B);
+    const bool dense = g.nq <= kDenseSolveMaxNq;
+    int tms = solve_tms_of(g, w, B);
+    while (dense && g.nq * 2 * tms > kDenseThreads) tms >>= 1;
     const int mtiles = (g.nm + tms - 1) / tms;
-    e = launch_pdl(w.pdl != 0, k_solve, (unsigned)(B * 2 * mtiles), solve_threads(g, tms), solve_smem_tms(g, tms), s, g,
+    e = launch_pdl(w.pdl != 0, dense ? k_solve_dense : k_solve, (unsigned)(B * 2 * mtiles),
+                   dense ? (g.nq * 2 * tms + 31) / 32 * 32 : solve_threads(g, tms), dense ? 0 : solve_smem_tms(g, tms), s, g,
                    t, X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
   }
   if (e != cudaSuccess) return e;
