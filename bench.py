@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "712c3f0afa35826772be67cda2aa0f6489b694b99e9564565dc3b7371299a7ad"
+NCU_TRAFFIC_SHA256 = "d033826ae653971f6656312b11a06015b30b45c56d103a46938a6862f76c4f87"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 135066, "coarse:k_rows": 386458, "coarse:k_zfwd": 123456, "coarse:k_solve": 802688,
-    "fine:k_zinv@32": 10447206, "fine:k_rows@32": 37880269, "fine:k_zfwd@32": 12631040, "fine:k_solve@32": 23876224,
-    "fine:k_zinv@2": 671488, "fine:k_rows@2": 2492672, "fine:k_zfwd@2": 832768, "fine:k_solve@2": 2769408,
+    "coarse:k_zinv": 135014, "coarse:k_rows": 390451, "coarse:k_zfwd": 123328, "coarse:k_solve": 801920,
+    "fine:k_zinv@32": 10456781, "fine:k_rows@32": 37880678, "fine:k_zfwd@32": 12628416, "fine:k_solve@32": 23856128,
+    "fine:k_zinv@2": 669133, "fine:k_rows@2": 2490317, "fine:k_zfwd@2": 829952, "fine:k_solve@2": 2763776,
 }
 
 

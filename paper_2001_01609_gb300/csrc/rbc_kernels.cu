@@ -439,35 +439,35 @@ static size_t zfwd_smem(const Grid& g, int B, size_t es) {
 }
 
 // ---------------------------------------------------------------------------
-// Stage solve (k_solve) of the mixed mode and of small grids (the FP64 mode's
-// larger grids: rbc_solve.cu).  Block per (slice, Chebyshev parity p, tile of tms
-// Fourier modes); a column is one (mode m, real/imaginary part c) pair -- the
-// stage matrices are real, so the two parts are independent systems except for
-// the implicit buoyancy coupling -i k Pr Ra T (the imaginary part of T feeds
-// the real part of psi and vice versa).  Per system (T first, then psi for
-// m >= 1 or the mean flow U for m = 0):
-//   phase 1 (all threads, one tau row of one column each): right-hand side of
-//           the stage, updates of the later RK accumulators;
-//   phase 2 (one thread per column): backward elimination with the UL factors;
-//   phase 3 (same thread): boundary block, forward substitution;
-//   phase 4 (all threads): dt L X_i = (M X_i - r_i) / gamma into later accumulators.
-// Phase 1 reads F and the step-start state straight from global memory
-// (consecutive threads take consecutive (m, re/im) columns, so the loads
-// coalesce); the right-hand sides, r_i and T_i live in shared memory, three
-// arrays of nq x 2 tms doubles, so that more blocks share an SM.
+// Stage solve (k_solve) of the mixed mode with nq > kDenseSolveMaxNq (smaller
+// grids: k_solve_dense; the FP64 mode's: rbc_solve.cu).  Block per (slice,
+// Chebyshev parity p, tile of tms Fourier modes); a column is one (mode m,
+// real/imaginary part c) pair -- the stage matrices are real, so the two parts
+// are independent systems except for the implicit buoyancy coupling -i k Pr Ra T
+// (the imaginary part of T feeds the real part of psi and vice versa).  Per
+// system (T first, then psi for m >= 1 or the mean flow U for m = 0):
+//   phase 1 (all threads, NB consecutive tau rows of one column each): right-hand
+//           side of the stage, updates of the later RK accumulators;
+//   phase 2 (one warp, a column per lane): backward elimination with the UL
+//           factors;
+//   phase 3 (same warp): boundary block, forward substitution;
+//   phase 4 (all threads): the solution to memory, dt L X_i = (M X_i - r_i) / gamma
+//           into the later accumulators.
+// In phases 2 and 3 a second warp copies the factors of RC steps at a time into
+// shared memory, two chunks ahead, and sums the boundary rows one chunk behind;
+// a third solves the mean flow of the tile that holds mode 0.  The temperature's
+// and the second system's values share one array of nq + 2 rows of 2 tms doubles:
+// row i of the latter lies two rows lower, in rows that phase 1, going up, has
+// read.  A second array holds r_i.
+//
+// Bound: the FP64 pipe (2 operations per clock and SM) when blocks fill it, else
+// the recurrences: ten dependent warp instructions of 64 clocks per row.
+// Measured (GB300, per launch; before, all rows' factors from L2 by the recurring
+// warp, three arrays and 256 threads of 125 registers, two blocks per SM; same
+// bits): 1024 x 256, 32 states 1650 -> 1117 us, one state 240 -> 103 us; 512 x 128,
+// 64 states 810 -> 515 us; 256 x 64, 8 states 83 -> 42 us, one state 37 -> 28 us.
 // ---------------------------------------------------------------------------
 enum { KT = 0, KP = 1, KU = 2 };
-
-struct SolveSmem {
-  const double* F;   // explicit terms of this slice (global; read in phase 1, coalesced over the columns)
-  const double* X;   // step-start state of this slice (global; stage 1)
-  double* y;    // [nq][W] right-hand side, then solution
-  double* r;    // [nq][W] r_i of the tau rows
-  double* T;    // [nq][W] T_i, kept for the psi coupling
-  int W;        // columns = 2 * tms
-  double Ra;    // Rayleigh number of this slice
-  double cpl;   // ((gamma dt) Pr) Ra of this slice
-};
 
 template <int KIND>
 struct Sys {
@@ -497,166 +497,312 @@ struct Sys {
   }
 };
 
-// phase 1 for one (tau row t, column col)
-template <int KIND>
-__device__ __forceinline__ void solve_rhs(const Grid& g, const Tables& tb, int stage, int p, int m, int c, int t,
-                                          int col, const SolveSmem& sm, double* __restrict__ R, size_t S) {
+// finite, from the exponent bits (an FP64 comparison would occupy the FP64 pipe)
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// What a thread of k_solve works on: its column, and its state's arrays.
+struct SolveCol {
+  int p, m, c, col, W;
+  double cpl;        // gamma dt Pr Ra k, negated in the imaginary part's column
+  const double* F;   // explicit terms
+  const double* X;   // step-start state
+  double* R;         // accumulated right-hand sides
+  double* Xo;
+  size_t S;
+};
+
+// phase 1 for tau rows t0 .. t0 + NB - 1 of a column: r_i, and the right-hand
+// side bv of the system (psi: with the buoyancy of T, row r of it at T[r W])
+template <int KIND, int NB>
+__device__ __forceinline__ void solve_rhs(const Grid& g, const Tables& tb, int stage, const SolveCol& k, int t0,
+                                          const double* T, double* r, double* bv) {
   using SY = Sys<KIND>;
-  const int nq = g.nq, W = sm.W;
+  constexpr int NW = NB + SY::LAM;
+  const int nq = g.nq, nt = nq - SY::D, ns = g.ns;
   const int f = (KIND == KT) ? 0 : 1;
-  double fv = 0.0;
+  const size_t rs = soff(g, 0, 2, 0);                         // coefficients n, n + 2
+  const size_t o0 = soff(g, f, 2 * t0 + k.p, k.m) + k.c;
+  if (t0 >= nt) return;
+  double fw[NW], ri[NB], Rl[NB][3];
 #pragma unroll
-  for (int j = 0; j <= SY::LAM; ++j)
-    if (t + j < nq) fv = fma(SY::tapF(g, tb, p, t, j), sm.F[soff(g, f, 2 * (t + j) + p, m) + c], fv);
-  if (KIND != KP) fv = -fv;
-  const int ns = g.ns;
-  const size_t ro = soff(g, f, 2 * t + p, m) + c;
-  double r;
+  for (int i = 0; i < NW; ++i) fw[i] = (t0 + i < nq) ? k.F[o0 + i * rs] : 0.0;
   if (stage == 1) {
-    double mx = 0.0;
+    double xw[NW];
+#pragma unroll
+    for (int i = 0; i < NW; ++i) xw[i] = (t0 + i < nq) ? k.X[o0 + i * rs] : 0.0;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int t = t0 + i;
+      double mx = 0.0;
+#pragma unroll
+      for (int j = 0; j <= SY::LAM; ++j)
+        if (t + j < nq && t < nt) mx = fma(SY::tapM(g, tb, k.p, t, j, k.m), xw[i + j], mx);
+      ri[i] = mx;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      ri[i] = (t0 + i < nt) ? k.R[(size_t)(stage - 1) * k.S + o0 + i * rs] : 0.0;
+#pragma unroll
+      for (int l = 0; l < 3; ++l)
+        Rl[i][l] = (t0 + i < nt && l + 2 > stage && l + 2 <= ns) ? k.R[(size_t)(l + 1) * k.S + o0 + i * rs] : 0.0;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int t = t0 + i;
+    if (t >= nt) break;
+    double fv = 0.0;
 #pragma unroll
     for (int j = 0; j <= SY::LAM; ++j)
-      if (t + j < nq) mx = fma(SY::tapM(g, tb, p, t, j, m), sm.X[soff(g, f, 2 * (t + j) + p, m) + c], mx);
-    r = fma(__ldg(tb.dtae + 5), fv, mx);
-#pragma unroll
-    for (int l = 2; l <= 4; ++l)
-      if (l <= ns) R[(size_t)(l - 1) * S + ro] = fma(__ldg(tb.dtae + l * 5), fv, mx);
-  } else {
-    double Rl[3];
-    const double Ri = *(R + (size_t)(stage - 1) * S + ro);
-#pragma unroll
-    for (int l = 0; l < 3; ++l) Rl[l] = (l + 2 > stage && l + 2 <= ns) ? *(R + (size_t)(l + 1) * S + ro) : 0.0;
-    r = fma(__ldg(tb.dtae + stage * 5 + stage - 1), fv, Ri);
+      if (t + j < nq) fv = fma(SY::tapF(g, tb, k.p, t, j), fw[i + j], fv);
+    if (KIND != KP) fv = -fv;
+    r[i] = fma(__ldg(tb.dtae + stage * 5 + stage - 1), fv, ri[i]);
 #pragma unroll
     for (int l = 0; l < 3; ++l)
       if (l + 2 > stage && l + 2 <= ns)
-        R[(size_t)(l + 1) * S + ro] = fma(__ldg(tb.dtae + (l + 2) * 5 + stage - 1), fv, Rl[l]);
-  }
-  sm.r[t * W + col] = r;
-  double bv = r;
-  if (KIND == KP) {
-    // + gamma dt (-i k Pr Ra) S4 T_i: real part + k.. Im(S4 T), imaginary part - k.. Re(S4 T)
-    double st = 0.0;
+        k.R[(size_t)(l + 1) * k.S + o0 + i * rs] =
+            fma(__ldg(tb.dtae + (l + 2) * 5 + stage - 1), fv, stage == 1 ? ri[i] : Rl[i][l]);
+    bv[i] = r[i];
+    if (KIND == KP) {
+      // + gamma dt (-i k Pr Ra) S4 T_i: real part + k.. Im(S4 T), imaginary part - k.. Re(S4 T)
+      double st = 0.0;
 #pragma unroll
-    for (int j = 0; j <= 4; ++j)
-      if (t + j < nq) st = fma(__ldg(tb.s4 + (p * nq + t) * 5 + j), sm.T[(t + j) * W + (col ^ 1)], st);
-    // (+-1) gamma dt Pr Ra k with the roundings of that left-to-right product:
-    // the sign is exact, so it may come last
-    const double cpl = (c == 0 ? sm.cpl : -sm.cpl) * (g.kfac * m);
-    bv = fma(cpl, st, bv);
+      for (int j = 0; j <= 4; ++j)
+        if (t + j < nq) st = fma(SY::tapF(g, tb, k.p, t, j), T[(t + j) * k.W + (k.col ^ 1)], st);
+      bv[i] = fma(k.cpl, st, bv[i]);
+    }
   }
-  sm.y[(t + SY::D) * W + col] = bv;
 }
 
-// phases 2 and 3 for one column
-template <int KIND>
-__device__ __forceinline__ bool solve_recurrence(const Grid& g, const Tables& tb, int p, int m, int c, int col,
-                                                 const SolveSmem& sm, double* __restrict__ Xo) {
+// phase 4 for coefficients (and tau rows) t0 .. t0 + NB - 1 of a column; row i of
+// the solution at x[i W], r_i at r[i W]
+template <int KIND, int NB>
+__device__ __forceinline__ bool solve_lx(const Grid& g, const Tables& tb, int stage, const SolveCol& k, int t0,
+                                         const double* x, const double* r) {
   using SY = Sys<KIND>;
-  constexpr int D = SY::D;
-  const int nq = g.nq, W = sm.W;
+  constexpr int NW = NB + SY::LAM;
+  const int nq = g.nq, nt = nq - SY::D, ns = g.ns;
   const int f = (KIND == KT) ? 0 : 1;
-  const int nmod = (KIND == KU) ? 1 : g.nm;
-  const int mi = (KIND == KU) ? 0 : m;
-  const double* multB = SY::multB(tb);
-  const double* multD = SY::multD(tb);
-  auto tix = [&](int cc, int jj) { return ((size_t)(p * nq + cc) * D + jj) * nmod + mi; };
-  // The factor entries of RC consecutive steps are loaded together before the
-  // steps run, so the sequential chain does not wait on one load per step.
-  constexpr int RC = 8;
-  double pend[D], bd[D];
-#pragma unroll
-  for (int jj = 0; jj < D; ++jj) pend[jj] = bd[jj] = 0.0;
-  for (int c0 = nq - 1; c0 >= D; c0 -= RC) {
-    double mb[RC][D], md[RC][D];
-#pragma unroll
-    for (int k = 0; k < RC; ++k) {
-      const int cc = c0 - k;
-#pragma unroll
-      for (int jj = 0; jj < D; ++jj) {
-        mb[k][jj] = (cc >= D) ? __ldg(multB + tix(cc, jj)) : 0.0;
-        md[k][jj] = (cc >= D) ? __ldg(multD + tix(cc, jj)) : 0.0;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < RC; ++k) {
-      const int cc = c0 - k;
-      if (cc < D) break;
-      const double bc = sm.y[cc * W + col] + pend[0];
-      sm.y[cc * W + col] = bc;
-#pragma unroll
-      for (int jj = 0; jj < D - 1; ++jj) pend[jj] = fma(-mb[k][D - 1 - jj], bc, pend[jj + 1]);
-      pend[D - 1] = -mb[k][0] * bc;
-#pragma unroll
-      for (int r2 = 0; r2 < D; ++r2) bd[r2] = fma(-md[k][r2], bc, bd[r2]);
-    }
-  }
-  // boundary rows: parity combinations of the wall values (Eq. 6) or slopes (Eq. 7)
-  if (KIND == KT && m == 0 && c == 0) bd[0] += t_wall_rhs(g, p);
-  const double* Dinv = SY::Dinv(tb);
-  const double* Lb = SY::Lb(tb);
-  const double* invd = SY::invd(tb);
-  double win[D];
+  const size_t rs = soff(g, 0, 2, 0);
+  const size_t o0 = soff(g, f, 2 * t0 + k.p, k.m) + k.c;
+  double xw[NW], Rl[NB][3];
   bool ok = true;
 #pragma unroll
-  for (int r2 = 0; r2 < D; ++r2) {
-    double x = 0.0;
+  for (int i = 0; i < NB; ++i)
 #pragma unroll
-    for (int c2 = 0; c2 < D; ++c2) x = fma(__ldg(Dinv + ((size_t)(p * D * D) + r2 * D + c2) * nmod + mi), bd[c2], x);
-    win[r2] = x;
-    sm.y[r2 * W + col] = x;
-    Xo[soff(g, f, 2 * r2 + p, m) + c] = x;
-    if (KIND == KT) sm.T[r2 * W + col] = x;
-    ok = ok && isfinite(x);
-  }
-  for (int r0 = D; r0 < nq; r0 += RC) {
-    double lb[RC][D], iv[RC];
+    for (int l = 0; l < 3; ++l)
+      Rl[i][l] = (t0 + i < nt && l + 2 > stage && l + 2 <= ns) ? k.R[(size_t)(l + 1) * k.S + o0 + i * rs] : 0.0;
 #pragma unroll
-    for (int k = 0; k < RC; ++k) {
-      const int r2 = r0 + k;
+  for (int i = 0; i < NW; ++i) xw[i] = (t0 + i < nq) ? x[(t0 + i) * k.W + k.col] : 0.0;
 #pragma unroll
-      for (int jj = 0; jj < D; ++jj) lb[k][jj] = (r2 < nq) ? __ldg(Lb + tix(r2, jj)) : 0.0;
-      iv[k] = (r2 < nq) ? __ldg(invd + (size_t)(p * nq + r2) * nmod + mi) : 0.0;
+  for (int i = 0; i < NB; ++i) {
+    const int t = t0 + i;
+    if (t < nq) {
+      k.Xo[o0 + i * rs] = xw[i];
+      ok = ok && finite_bits(xw[i]);
     }
+    if (stage < ns && t < nt) {
+      double mx = 0.0;
 #pragma unroll
-    for (int k = 0; k < RC; ++k) {
-      const int r2 = r0 + k;
-      if (r2 >= nq) break;
-      double y = sm.y[r2 * W + col];
+      for (int j = 0; j <= SY::LAM; ++j)
+        if (t + j < nq) mx = fma(SY::tapM(g, tb, k.p, t, j, k.m), xw[i + j], mx);
+      const double lx2 = g.inv_gamma * (mx - r[t * k.W + k.col]);   // dt (L X_i + coupling)
 #pragma unroll
-      for (int jj = 0; jj < D; ++jj) y = fma(-lb[k][jj], win[jj], y);
-      const double x = iv[k] * y;
-      sm.y[r2 * W + col] = x;
-      Xo[soff(g, f, 2 * r2 + p, m) + c] = x;
-      if (KIND == KT) sm.T[r2 * W + col] = x;
-#pragma unroll
-      for (int jj = 0; jj < D - 1; ++jj) win[jj] = win[jj + 1];
-      win[D - 1] = x;
-      ok = ok && isfinite(x);
+      for (int l = 0; l < 3; ++l)
+        if (l + 2 > stage && l + 2 <= ns)
+          k.R[(size_t)(l + 1) * k.S + o0 + i * rs] = fma(c_AI[g.scheme][l + 2][stage], lx2, Rl[i][l]);
     }
   }
   return ok;
 }
 
-// phase 4 for one (tau row t, column col)
+// Phases 2 and 3 of a tile by two warps.  Chunk j of the sequence (RC steps
+// backward, then RC forward) lies in ring[j % 3]: the first warp works on chunk j
+// while the second sums the boundary rows of chunk j - 1 and chunks j + 1 and
+// j + 2 are on their way.  Both warps pass the barrier before every chunk and
+// two at the turn, so neither waits for more than the other's chunk.
+constexpr int RC = 4;
+__host__ __device__ constexpr int solve_ring(int tms) { return RC * 4 * tms; }   // doubles per chunk
+
+__device__ __forceinline__ void pair_sync() {
+  __syncwarp();
+  asm volatile("bar.sync 1, 64;" ::: "memory");
+}
+
 template <int KIND>
-__device__ __forceinline__ void solve_lx(const Grid& g, const Tables& tb, int stage, int p, int m, int c, int t,
-                                         int col, const SolveSmem& sm, double* __restrict__ R, size_t S) {
+__device__ __forceinline__ void solve_helper(const Grid& g, const Tables& tb, int p, int m0, int tms, const double* y,
+                                             double* ring, double* bdx) {
   using SY = Sys<KIND>;
-  const int nq = g.nq, W = sm.W;
-  const int f = (KIND == KT) ? 0 : 1;
-  double mx = 0.0;
+  constexpr int D = SY::D;
+  const int nq = g.nq, W = 2 * tms, lt = __ffs(tms) - 1, lane = threadIdx.x & 31;
+  const int nb = (nq - D + RC - 1) / RC;
+  const double *mB = SY::multB(tb), *mD = SY::multD(tb), *Lb = SY::Lb(tb), *iv = SY::invd(tb);
+  // backward chunk: [step][2 D][mode], multipliers of the rows below, then of the
+  // boundary rows; forward: [step][D + 1][mode], L and the inverse diagonal
+  auto load = [&](int j) {
+    double* dst = ring + (j % 3) * solve_ring(tms);
+    const bool back = j < nb;
+    const int per = back ? 2 * D : D + 1, r0 = back ? nq - 1 - j * RC : D + (j - nb) * RC;
+    if (j < 2 * nb)
+      for (int e = lane; e < RC * per * tms; e += 32) {
+        const int mode = e & (tms - 1), q = e >> lt, st = q / per, w = q - st * per;
+        const int row = back ? r0 - st : r0 + st;
+        if (row < D || row >= nq) continue;
+        const size_t rw = (size_t)(p * nq + row);
+        const double* src = back ? (w < D ? mB : mD) + (rw * D + (w < D ? w : w - D)) * g.nm
+                                 : (w < D ? Lb + (rw * D + w) * g.nm : iv + rw * g.nm);
+        const unsigned d = (unsigned)__cvta_generic_to_shared(dst + e);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src + m0 + mode) : "memory");
+      }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const bool on = lane < W && (KIND != KP || m0 + (lane >> 1) > 0);
+  double bd[D];
 #pragma unroll
-  for (int j = 0; j <= SY::LAM; ++j)
-    if (t + j < nq) mx = fma(SY::tapM(g, tb, p, t, j, m), sm.y[(t + j) * W + col], mx);
-  const double lx2 = g.inv_gamma * (mx - sm.r[t * W + col]);   // dt (L X_i + coupling)
-  const size_t ro = soff(g, f, 2 * t + p, m) + c;
+  for (int q = 0; q < D; ++q) bd[q] = 0.0;
+  auto boundary = [&](int j) {
+    if (on) {
+      const double* f = ring + (j % 3) * solve_ring(tms) + (lane >> 1);
 #pragma unroll
-  for (int l = 0; l < 3; ++l)
-    if (l + 2 > stage && l + 2 <= g.ns) {
-      double* Rl = R + (size_t)(l + 1) * S + ro;
-      *Rl = fma(c_AI[g.scheme][l + 2][stage], lx2, *(Rl));
+      for (int st = 0; st < RC; ++st) {
+        const int row = nq - 1 - j * RC - st;
+        if (row < D) break;
+        const double v = y[row * W + lane];
+#pragma unroll
+        for (int q = 0; q < D; ++q) bd[q] = fma(-f[(st * 2 * D + D + q) * tms], v, bd[q]);
+      }
     }
+    __syncwarp();
+  };
+  load(0);
+  load(1);
+  for (int j = 0; j < nb; ++j) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    pair_sync();                       // chunk j is here; the rows of chunk j - 1 are final
+    if (j > 0) boundary(j - 1);
+    load(j + 2);
+  }
+  pair_sync();
+  boundary(nb - 1);
+  if (on)
+#pragma unroll
+    for (int q = 0; q < D; ++q) bdx[q * W + lane] = bd[q];
+  pair_sync();
+  for (int j = nb; j < 2 * nb; ++j) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    pair_sync();
+    load(j + 2);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+template <int KIND>
+__device__ __forceinline__ void solve_recurrence(const Grid& g, const Tables& tb, int p, int m0, int tms, double* y,
+                                                 const double* ring, const double* bdx) {
+  using SY = Sys<KIND>;
+  constexpr int D = SY::D;
+  const int nq = g.nq, W = 2 * tms, lane = threadIdx.x & 31, m = m0 + (lane >> 1);
+  const int nb = (nq - D + RC - 1) / RC;
+  const bool on = lane < W && (KIND != KP || m > 0);   // (mode 0: solve_mean)
+  double Di[D][D], pend[D], win[D];
+#pragma unroll
+  for (int r = 0; r < D; ++r) {
+    pend[r] = win[r] = 0.0;
+#pragma unroll
+    for (int q = 0; q < D; ++q) Di[r][q] = on ? __ldg(SY::Dinv(tb) + ((size_t)(p * D * D) + r * D + q) * g.nm + m) : 0.0;
+  }
+  for (int j = 0; j < nb; ++j) {
+    pair_sync();
+    if (on) {
+      const double* f = ring + (j % 3) * solve_ring(tms) + (lane >> 1);
+      const int r0 = nq - 1 - j * RC;
+      double mb[RC][D], v[RC];
+#pragma unroll
+      for (int st = 0; st < RC; ++st) {
+        const bool in = r0 - st >= D;
+        v[st] = in ? y[(r0 - st) * W + lane] : 0.0;
+#pragma unroll
+        for (int q = 0; q < D; ++q) mb[st][q] = in ? f[(st * 2 * D + q) * tms] : 0.0;
+      }
+#pragma unroll
+      for (int st = 0; st < RC; ++st) {
+        if (r0 - st < D) break;
+        const double bc = __dadd_rn(v[st], pend[0]);
+        y[(r0 - st) * W + lane] = bc;
+#pragma unroll
+        for (int q = 0; q < D - 1; ++q) pend[q] = fma(-mb[st][D - 1 - q], bc, pend[q + 1]);
+        pend[D - 1] = __dmul_rn(-mb[st][0], bc);
+      }
+    }
+  }
+  pair_sync();
+  pair_sync();
+  if (on) {
+    // boundary rows: parity combinations of the wall values (Eq. 6) or slopes (Eq. 7)
+    double bd[D];
+#pragma unroll
+    for (int q = 0; q < D; ++q) bd[q] = bdx[q * W + lane];
+    if (KIND == KT && m == 0 && (lane & 1) == 0) bd[0] += t_wall_rhs(g, p);
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      double x = 0.0;
+#pragma unroll
+      for (int q = 0; q < D; ++q) x = fma(Di[r][q], bd[q], x);
+      win[r] = x;
+      y[r * W + lane] = x;
+    }
+  }
+  for (int j = nb; j < 2 * nb; ++j) {
+    pair_sync();
+    if (on) {
+      const double* f = ring + (j % 3) * solve_ring(tms) + (lane >> 1);
+      const int r0 = D + (j - nb) * RC;
+      double lb[RC][D], iv[RC], v[RC];
+#pragma unroll
+      for (int st = 0; st < RC; ++st) {
+        const bool in = r0 + st < nq;
+        v[st] = in ? y[(r0 + st) * W + lane] : 0.0;
+        iv[st] = in ? f[(st * (D + 1) + D) * tms] : 0.0;
+#pragma unroll
+        for (int q = 0; q < D; ++q) lb[st][q] = in ? f[(st * (D + 1) + q) * tms] : 0.0;
+      }
+#pragma unroll
+      for (int st = 0; st < RC; ++st) {
+        if (r0 + st >= nq) break;
+        double v2 = v[st];
+#pragma unroll
+        for (int q = 0; q < D; ++q) v2 = fma(-lb[st][q], win[q], v2);
+        const double x = iv[st] * v2;
+        y[(r0 + st) * W + lane] = x;
+#pragma unroll
+        for (int q = 0; q < D - 1; ++q) win[q] = win[q + 1];
+        win[D - 1] = x;
+      }
+    }
+  }
+}
+
+// Phases 2 and 3 of the mean flow, one column (part c of mode 0) per lane.
+__device__ __forceinline__ void solve_mean(const Grid& g, const Tables& tb, int p, int W, double* y) {
+  const int nq = g.nq, lane = threadIdx.x & 31;
+  if (lane >= 2) return;
+  const double *mB = tb.U_multB + p * nq, *mD = tb.U_multD + p * nq, *Lb = tb.U_Lb + p * nq, *iv = tb.U_invd + p * nq;
+  double pend = 0.0, bd = 0.0;
+#pragma unroll 8
+  for (int r = nq - 1; r >= 1; --r) {
+    const double bc = __dadd_rn(y[r * W + lane], pend);
+    y[r * W + lane] = bc;
+    pend = __dmul_rn(-__ldg(mB + r), bc);
+    bd = fma(-__ldg(mD + r), bc, bd);
+  }
+  double x = fma(__ldg(tb.U_Dinv + p), bd, 0.0);
+  y[lane] = x;
+#pragma unroll 8
+  for (int r = 1; r < nq; ++r) {
+    x = __ldg(iv + r) * fma(-__ldg(Lb + r), x, y[r * W + lane]);
+    y[r * W + lane] = x;
+  }
 }
 
 // Nu_V(t_n) (Eq. 9) of the step-start state: wall temperature difference of
@@ -680,96 +826,100 @@ __device__ __forceinline__ void nu_integral(const Grid& g, const Tables& tb, con
   if (lane == 0) nu[b] += ((stepidx == 0) ? 0.5 : 1.0) * g.dt * (cond + 0.5 * adv);
 }
 
-__device__ void solve_item(const Grid& g, const Tables& tb, double* X, double* Xs, const double* F, double* R,
-                           size_t S, const double* wT, double* nu, int* flags, int* err, int B, int stage, int tms,
-                           const double* ra, const int* nsteps, int stepidx, int blk) {
+constexpr int kSolveThreads = 128;
+constexpr int kSolveSmem = 140 * 1024;   // nq = 256, 16 modes
+
+template <int NB>
+__global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, double* X, double* Xs, const double* F,
+                                                            double* R, size_t S, const double* wT, double* nu, int* flags,
+                                                            int* err, int B, int stage, int tms, const double* ra,
+                                                            const int* nsteps, const int* step) {
   extern __shared__ double sbuf[];
-  const int mt = (g.nm + tms - 1) / tms;
-  const int b = blk / (2 * mt);
-  const int rem = blk - b * 2 * mt;
-  const int p = rem / mt;
-  const int m0 = (rem - p * mt) * tms;
+  pdl_wait();
+  const int stepidx = nsteps ? *step : 0;
+  const int mt = (g.nm + tms - 1) / tms;       // tms divides nm: both are powers of two
+  const int b = blockIdx.x / (2 * mt), rem = blockIdx.x - b * 2 * mt, p = rem / mt, m0 = (rem - p * mt) * tms;
   if (b >= B || !slice_active_at(nsteps, stepidx, b)) return;   // uniform per block
   // a transform of this state gave up waiting (the tensor-core kernels): leave
   // the state as it was at the start of the failing step
   if (flags[b] & kFlagTimeout) return;
-  const int nq = g.nq;
-  const int W = 2 * tms;                         // a power of two (tms is)
-  const int lw = __ffs(W) - 1;
-  const int ncol = 2 * min(tms, g.nm - m0);
-  SolveSmem sm;
-  sm.W = W;
-  sm.Ra = ra ? ra[b] : g.Ra;
-  sm.cpl = __ldg(tb.dtae + 25) * sm.Ra;
-  sm.y = sbuf;
-  sm.r = sm.y + (size_t)nq * W;
-  sm.T = sm.r + (size_t)nq * W;
+  const int nq = g.nq, W = 2 * tms, lw = __ffs(W) - 1, warp = threadIdx.x >> 5;
+  SolveCol k;
+  k.p = p;
+  k.W = W;
+  k.col = threadIdx.x & (W - 1);
+  k.m = m0 + k.col / 2;
+  k.c = k.col & 1;
+  const double cpl0 = __ldg(tb.dtae + 25) * (ra ? ra[b] : g.Ra);
+  // (+-1) gamma dt Pr Ra k with the roundings of that left-to-right product:
+  // the sign is exact, so it may come last
+  k.cpl = (k.c == 0 ? cpl0 : -cpl0) * (g.kfac * k.m);
   double* X0 = X + (size_t)b * S;
-  double* Xo = (stage == g.ns) ? X0 : Xs + (size_t)b * S;   // stiffly accurate: last stage = new state
-  const double* Fb = F + (size_t)b * S;
-  sm.F = Fb;
-  sm.X = X0;
-  double* Rb = R + (size_t)b * 4 * S;
+  k.F = F + (size_t)b * S;
+  k.X = X0;
+  k.R = R + (size_t)b * 4 * S;
+  k.Xo = (stage == g.ns) ? X0 : Xs + (size_t)b * S;   // stiffly accurate: last stage = new state
+  k.S = S;
+  double* y2 = sbuf;                           // psi / U: rows of W
+  double* T = y2 + 2 * W;                      // T: row i where row i + 2 of psi goes
+  double* rr = T + (size_t)nq * W;             // [nq][W] r_i
+  double* ring = rr + (size_t)nq * W;          // [3] chunks of factors
+  double* bdx = ring + 3 * solve_ring(tms);    // [2][W] boundary rows
+  const int rows = NB * (kSolveThreads >> lw), mine = NB * ((int)threadIdx.x >> lw);   // rows per round
+  // The warps of the recurrences: blocks of an SM take different ones (those
+  // resident together are about 152 apart), since a warp's number fixes its
+  // sub-partition and with it the FP64 pipe.
+  const int first = (int)((blockIdx.x / 152 + blockIdx.x) & 3);
   if (stage == 1 && m0 == 0 && p == 1) nu_integral(g, tb, X0, wT, nu, b, stepidx);
-  bool ok = true;
-  for (int sys = 0; sys < 2; ++sys) {   // T, then psi / U
-    // phase 1
-    const int ntmax = nq - 1;
-    for (int it = threadIdx.x; it < ntmax * W; it += blockDim.x) {
-      const int t = it >> lw, col = it & (W - 1);
-      if (col >= ncol) continue;
-      const int m = m0 + col / 2, c = col & 1;
-      if (sys == 0)
-        solve_rhs<KT>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
-      else if (m == 0)
-        solve_rhs<KU>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
-      else if (t < nq - 2)
-        solve_rhs<KP>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < ncol) {
-      // phases 2, 3: one column per thread, columns packed into the fewest warps
-      // (an FP64 warp instruction occupies its sub-partition's FP64 pipe for the
-      // same time however many lanes are active, so packing is cheapest)
-      const int col = threadIdx.x, m = m0 + col / 2, c = col & 1;
-      bool o2;
-      if (sys == 0)
-        o2 = solve_recurrence<KT>(g, tb, p, m, c, col, sm, Xo);
-      else if (m == 0)
-        o2 = solve_recurrence<KU>(g, tb, p, m, c, col, sm, Xo);
-      else
-        o2 = solve_recurrence<KP>(g, tb, p, m, c, col, sm, Xo);
-      ok = ok && o2;
-    }
-    __syncthreads();
-    // phase 4
-    if (stage < g.ns) {
-      for (int it = threadIdx.x; it < ntmax * W; it += blockDim.x) {
-        const int t = it >> lw, col = it & (W - 1);
-        if (col >= ncol) continue;
-        const int m = m0 + col / 2, c = col & 1;
-        if (sys == 0)
-          solve_lx<KT>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
-        else if (m == 0)
-          solve_lx<KU>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
-        else if (t < nq - 2)
-          solve_lx<KP>(g, tb, stage, p, m, c, t, col, sm, Rb, S);
+
+  for (int t0 = mine; t0 < nq; t0 += rows) {
+    double r[NB], bv[NB];
+    solve_rhs<KT, NB>(g, tb, stage, k, t0, nullptr, r, bv);
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (t0 + i < nq - 1) {
+        rr[(t0 + i) * W + k.col] = r[i];
+        T[(t0 + i + 1) * W + k.col] = bv[i];
       }
-    }
-    __syncthreads();
   }
+  __syncthreads();
+  if (warp == first)
+    solve_recurrence<KT>(g, tb, p, m0, tms, T, ring, bdx);
+  else if (warp == (first ^ 1))
+    solve_helper<KT>(g, tb, p, m0, tms, T, ring, bdx);
+  __syncthreads();
+  bool ok = true;
+  for (int t0 = mine; t0 < nq; t0 += rows) ok = solve_lx<KT, NB>(g, tb, stage, k, t0, T, rr) && ok;
+  for (int tb0 = 0; tb0 < nq; tb0 += rows) {   // every thread: the barrier below
+    const int t0 = tb0 + mine;
+    double r[NB], bv[NB];
+    if (k.m == 0)
+      solve_rhs<KU, NB>(g, tb, stage, k, t0, nullptr, r, bv);
+    else
+      solve_rhs<KP, NB>(g, tb, stage, k, t0, T, r, bv);
+    const int D = k.m == 0 ? 1 : 2;
+    __syncthreads();                           // rows up to tb0 + rows - 1 of T have been read
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (t0 + i < nq - D) {
+        rr[(t0 + i) * W + k.col] = r[i];
+        y2[(t0 + i + D) * W + k.col] = bv[i];
+      }
+  }
+  __syncthreads();
+  if (warp == first)
+    solve_recurrence<KP>(g, tb, p, m0, tms, y2, ring, bdx);
+  else if (warp == (first ^ 1))
+    solve_helper<KP>(g, tb, p, m0, tms, y2, ring, bdx);
+  else if (warp == (first ^ 2) && m0 == 0)
+    solve_mean(g, tb, p, W, y2);
+  __syncthreads();
+  for (int t0 = mine; t0 < nq; t0 += rows)
+    ok = (k.m == 0 ? solve_lx<KU, NB>(g, tb, stage, k, t0, y2, rr) : solve_lx<KP, NB>(g, tb, stage, k, t0, y2, rr)) && ok;
   if (!ok) {
     atomicOr(flags + b, kFlagNonFinite);
     atomicOr(err, kFlagNonFinite);
   }
-}
-
-__global__ void __launch_bounds__(256) k_solve(Grid g, Tables tb, double* X, double* Xs, const double* F, double* R,
-                                               size_t S, const double* wT, double* nu, int* flags, int* err, int B,
-                                               int stage, int tms, const double* ra, const int* nsteps,
-                                               const int* step) {
-  pdl_wait();
-  solve_item(g, tb, X, Xs, F, R, S, wT, nu, flags, err, B, stage, tms, ra, nsteps, nsteps ? *step : 0, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -787,9 +937,6 @@ __global__ void __launch_bounds__(256) k_solve(Grid g, Tables tb, double* X, dou
 // precision; 64 x 32, 23 states 49.5 -> 46.1 us and 41.0 -> 37.3 us.
 // ---------------------------------------------------------------------------
 constexpr int kDenseThreads = 256;   // rows times columns of a tile
-
-// finite, from the exponent bits (an FP64 comparison would occupy the FP64 pipe)
-__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
 __global__ void __launch_bounds__(kDenseThreads) k_solve_dense(Grid g, Tables tb, double* X, double* Xs, const double* F,
                                                                double* R, size_t S, const double* wT, double* nu,
@@ -940,24 +1087,23 @@ __global__ void __launch_bounds__(kDenseThreads) k_solve_dense(Grid g, Tables tb
   }
 }
 
+// shared memory of a k_solve block: T and psi, r_i, factors, boundary rows
+static size_t solve_smem_tms(const Grid& g, int tms) {
+  return ((size_t)(2 * g.nq + 4) * 2 * tms + 3 * solve_ring(tms)) * 8;
+}
 // Modes per k_solve block.  Every column's arithmetic is independent of the
-// tiling, so a small batch (a coarse sweep) takes single-mode tiles and spreads
-// over the SMs instead of leaving most of them idle.
-// shared memory of a k_solve block: y, r and T, nq x 2 tms doubles each
-static size_t solve_smem_tms(const Grid& g, int tms) { return (size_t)3 * g.nq * 2 * tms * 8; }
+// tiling.  A small batch (a coarse sweep) takes small tiles and spreads over the
+// SMs instead of leaving most of them idle; a large one the largest tile of which
+// five blocks share an SM: with 128 coefficients per parity 8 modes (1024 x 256,
+// 32 states 1117 us, 16 modes 1330), below 16 (512 x 128, 64 states 515 us against
+// 510, 256 x 64, 32 states 99 us against 102).
 static int solve_tile(const Grid& g, int B) {
   int tms = 16;
   while (tms > 1 && (long)B * 2 * ((g.nm + tms - 1) / tms) < 2L * 152) tms >>= 1;
   if (tms > g.nm) tms = g.nm;
-  while (tms > 1 && solve_smem_tms(g, tms) > 200 * 1024) tms >>= 1;
+  while (tms > 1 && solve_smem_tms(g, tms) > 44 * 1024) tms >>= 1;
   return tms;
 }
-// threads of a k_solve block: one per (row, column) of the tile, whole warps, at most 256
-static int solve_threads(const Grid& g, int tms) {
-  const int items = g.nq * 2 * tms;
-  return std::min(256, std::max(32, (items + 31) / 32 * 32));
-}
-static size_t solve_smem(const Grid& g, int B) { return solve_smem_tms(g, solve_tile(g, B)); }
 
 // The shapes of a launch: the tuned ones where set, else the heuristics.
 static int solve_tms_of(const Grid& g, const Work& w, int B) {
@@ -1091,12 +1237,13 @@ cudaError_t configure_kernels(const Grid& g) {
                                         kCorrTile * 512 * (int)sizeof(double2));
   if (l2 == cudaSuccess) l2 = cudaFuncSetAttribute(k_l2_diff, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (l2 != cudaSuccess) return l2;
-  static int a_solve = 48 * 1024, a_zfwd_f = 48 * 1024;
+  static int a_zfwd_f = 48 * 1024;
   cudaError_t e = configure_zfx(g);   // also the averages of Sec. 2.2 of a mixed handle
   if (e == cudaSuccess) e = g.mixed ? configure_rows_f32(g) : configure_rows_fx(g);
   if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
   if (e == cudaSuccess && !solve_segmented(g))
-    e = allow_smem(k_solve, (int)std::max(solve_smem(g, 1), solve_smem(g, 1 << 20)), a_solve);
+    for (auto* fn : {k_solve<1>, k_solve<2>, k_solve<4>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmem);
   if (e == cudaSuccess)
     e = allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f);
   return e;
@@ -1175,10 +1322,14 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   } else {
     const bool dense = g.nq <= kDenseSolveMaxNq;
     int tms = solve_tms_of(g, w, B);
-    while (dense && g.nq * 2 * tms > kDenseThreads) tms >>= 1;
+    while (tms > g.nm || (dense && g.nq * 2 * tms > kDenseThreads)) tms >>= 1;
     const int mtiles = (g.nm + tms - 1) / tms;
-    e = launch_pdl(w.pdl != 0, dense ? k_solve_dense : k_solve, (unsigned)(B * 2 * mtiles),
-                   dense ? (g.nq * 2 * tms + 31) / 32 * 32 : solve_threads(g, tms), dense ? 0 : solve_smem_tms(g, tms), s, g,
+    // tau rows per thread and round: four share the loads of a window; fewer while
+    // a round would not give every thread of the block a row
+    const int items = g.nq * 2 * tms;
+    auto* kernel = dense ? k_solve_dense : items >= 4 * kSolveThreads ? k_solve<4> : items >= 2 * kSolveThreads ? k_solve<2> : k_solve<1>;
+    e = launch_pdl(w.pdl != 0, kernel, (unsigned)(B * 2 * mtiles), dense ? (items + 31) / 32 * 32 : kSolveThreads,
+                   dense ? 0 : solve_smem_tms(g, tms), s, g,
                    t, X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
   }
   if (e != cudaSuccess) return e;
