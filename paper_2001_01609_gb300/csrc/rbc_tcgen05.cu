@@ -11,14 +11,11 @@
 // which keeps about FP32 accuracy (the mixed mode computes the transforms and
 // products in FP32).
 //
-// CTA per (slice, tile of 64 columns, 128-row tile of one field's operator
-// rows).  Thread 0 starts bulk (TMA) copies of the operator images' K-chunks
-// (pre-swizzled on the host, 16 KB each, hi and lo) into a ring of up to four
-// shared-memory stages, while all threads convert the X tile (all K) from FP64
-// into hi/lo TF32 operands; thread 0 then issues the MMAs of each chunk as it
-// lands and refills a stage once its MMAs are done, and the four warps read
-// the 128 x 64 FP32 accumulator from tensor memory and form the fields of the
-// z-inverse output with the ik factors (the epilogue of k_zinv).
+// CTA per (slice, tile of 64 columns, row tiles of one field's operators): the X
+// tile (all K) becomes hi/lo operands in shared memory, the operator images'
+// K-chunks (pre-swizzled on the host, 16 KB each, hi and lo) stream in by bulk
+// (TMA) copies, and the fields of the z-inverse output are formed from the
+// 128 x 64 FP32 accumulators with the ik factors (the epilogue of k_zinv).
 // Operands are K-major with the 128-byte swizzle; every mbarrier wait is bounded
 // and reports through the slice's error flag, and nothing (MMA or copy) is in
 // flight when a kernel frees its tensor memory.
@@ -44,6 +41,11 @@ constexpr int kChunkFloats = kTileM * 32;   // one 128-row image chunk of 128-by
 // so that kTcGroups times as many stores are in flight as with four warps
 constexpr int kTcGroups = 2;
 constexpr int kTcThreads = 128 * kTcGroups;
+constexpr int kZinvTcThreads = kTcThreads + 64;   // and the issuing and the copying warp of k_zinv_tc
+// columns and row stride (floats) of the staged accumulator in k_zinv_tc's
+// epilogue (16-byte rows whose 128-bit accesses meet no bank twice)
+constexpr int kEpiCols = 32, kEpiStride = kEpiCols + 4;
+constexpr int kEpiBytes = kTileM * kEpiStride * 4;
 constexpr long long kWaitLimit = 1LL << 24;   // default spin limit of a bounded wait
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -180,6 +182,130 @@ __device__ __forceinline__ void store_c(float* Zb, const Grid& g, int field, int
 // on (set by tc_set_wait_limit; tests lower it to make the waits give up).
 __device__ long long g_wait_limit = kWaitLimit;
 
+// 4 K-steps x 3 MMAs (hi*hi, hi*lo, lo*hi) of one chunk: descriptors of the hi
+// operands; the lo ones lie a fixed distance behind (addresses / 16 below 2^14,
+// so sums stay in the descriptors' address field)
+template <bool BF>
+__device__ __forceinline__ void mma_chunk(uint32_t tmem, uint64_t a, uint64_t x, uint64_t xlo, uint32_t idesc, bool more) {
+  constexpr uint64_t alo = kTileM * 128 >> 4;
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks) {            // four 32-byte K-steps per 128-byte row
+    const uint64_t o = 2 * ks;
+    const uint32_t acc0 = (more || ks > 0) ? 1u : 0u;
+    if (BF) {
+      mma_bf16(tmem, a + o, x + o, idesc, acc0);
+      mma_bf16(tmem, a + o, x + xlo + o, idesc, 1u);
+      mma_bf16(tmem, a + alo + o, x + o, idesc, 1u);
+    } else {
+      mma_tf32(tmem, a + o, x + o, idesc, acc0);
+      mma_tf32(tmem, a + o, x + xlo + o, idesc, 1u);
+      mma_tf32(tmem, a + alo + o, x + o, idesc, 1u);
+    }
+  }
+}
+
+// barriers of the eight converting warps of k_zinv_tc
+__device__ __forceinline__ void group_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTcThreads) : "memory"); }
+__device__ __forceinline__ bool group_and(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)v), "n"(kTcThreads)
+      : "memory");
+  return r != 0;
+}
+
+// X tile of k_zinv_tc: columns c0 .. c0 + 63 of field rows x[n][2 nm] as hi/lo operands
+template <bool BF>
+__device__ __forceinline__ void convert_tile(const Grid& g, const double* x, int c0, int kc, int tid,
+                                             unsigned char* hi, unsigned char* lo) {
+  constexpr int PER = BF ? 8 : 4, KE = BF ? 64 : 32;   // operands per 16 bytes, per 128-byte row
+  const int col = tid & (kTileN - 1), gc = c0 + col, w = 2 * g.nm;
+#pragma unroll(BF ? 2 : 4)
+  for (int kg = tid / kTileN; kg < kc * 8; kg += kTcThreads / kTileN) {
+    const int n0 = kg * PER;
+    float v[PER];
+#pragma unroll
+    for (int e = 0; e < PER; ++e) v[e] = (gc < w && n0 + e < g.Nz) ? (float)__ldg(x + (size_t)(n0 + e) * w + gc) : 0.f;
+    const uint32_t o = (uint32_t)(n0 / KE) * kTileN * 128 + swz_b(col, (n0 % KE) * (16 / PER));
+    uint32_t h[4], l[4];
+    if (BF) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * e]), h1 = __float2bfloat16_rn(v[2 * e + 1]);
+        const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * e] - __bfloat162float(h0));
+        const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * e + 1] - __bfloat162float(h1));
+        h[e] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+        l[e] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        h[e] = to_tf32(v[e]);
+        l[e] = to_tf32(v[e] - __uint_as_float(h[e]));
+      }
+    }
+    *reinterpret_cast<uint4*>(hi + o) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(lo + o) = make_uint4(l[0], l[1], l[2], l[3]);
+  }
+}
+
+// Fields of row tile t, columns c0 .. c0 + 63, from the accumulator at tmem,
+// kEpiCols columns at a time: its rows go to shared memory, and each half-warp
+// forms the fields of one j at 16 modes, so that every store is one 128-byte
+// segment.  All eight warps.
+__device__ __forceinline__ void zinv_fields(const Grid& g, uint32_t tmem, float* epi, const float* kf, float* Zb,
+                                            int nops, int t, int c0, int warp, int lane) {
+  const int r = (warp & 3) * 32 + lane;       // tile row = TMEM lane
+  const int lj = nops == 4 ? 2 : 1, jper = kTileM >> lj;
+  for (int cb = 0; cb < kTileN; cb += kEpiCols) {
+    const int cw = (warp >> 2) * (kEpiCols / kTcGroups);   // this warp's 16 of them
+    float v[16];
+    tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb + cw, v);
+    float4* dst = reinterpret_cast<float4*>(epi + r * kEpiStride + cw);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    group_sync();
+    const int ml = lane & 15, m = ((c0 + cb) >> 1) + ml;
+    if (m < g.nm) {
+      const float k = kf[cb / 2 + ml];
+      for (int jl = warp * 2 + (lane >> 4); jl < jper; jl += 2 * (kTcThreads / 32)) {
+        const int j = t * jper + jl;
+        if (j >= g.Mz) break;
+        const float* e = epi + (jl << lj) * kEpiStride + 2 * ml;
+        const float2 P0 = *reinterpret_cast<const float2*>(e), P1 = *reinterpret_cast<const float2*>(e + kEpiStride);
+        if (nops == 4) {
+          // P[q] = (re, im) of d^q psi/ds^q (m = 0: of U)
+          const float2 P2 = *reinterpret_cast<const float2*>(e + 2 * kEpiStride);
+          const float2 P3 = *reinterpret_cast<const float2*>(e + 3 * kEpiStride);
+          if (m == 0) {
+            store_c(Zb, g, 0, j, 0, P0.x, 0.f);            // u = U
+            store_c(Zb, g, 1, j, 0, 0.f, 0.f);             // w
+            store_c(Zb, g, 2, j, 0, 0.f, 0.f);             // d_x omega
+            store_c(Zb, g, 3, j, 0, -4.f * P2.x, 0.f);     // d_z omega = -U_zz
+            store_c(Zb, g, 4, j, 0, 0.f, 0.f);             // d_x u
+            store_c(Zb, g, 5, j, 0, 2.f * P1.x, 0.f);      // d_z u = U_z
+          } else {
+            const float omr = k * k * P0.x - 4.f * P2.x, omi = k * k * P0.y - 4.f * P2.y;
+            store_c(Zb, g, 0, j, m, 2.f * P1.x, 2.f * P1.y);   // u = d_z psi
+            store_c(Zb, g, 1, j, m, k * P0.y, -k * P0.x);      // w = -ik psi
+            store_c(Zb, g, 2, j, m, -k * omi, k * omr);        // d_x omega = ik omega
+            store_c(Zb, g, 3, j, m, 2.f * k * k * P1.x - 8.f * P3.x, 2.f * k * k * P1.y - 8.f * P3.y);
+            store_c(Zb, g, 4, j, m, -k * 2.f * P1.y, k * 2.f * P1.x);   // d_x u = ik u
+            store_c(Zb, g, 5, j, m, 4.f * P2.x, 4.f * P2.y);            // d_z u
+          }
+        } else {
+          store_c(Zb, g, 6, j, m, P0.x, P0.y);                          // T
+          store_c(Zb, g, 7, j, m, m == 0 ? 0.f : -k * P0.y, m == 0 ? 0.f : k * P0.x);   // d_x T
+          store_c(Zb, g, 8, j, m, 2.f * P1.x, 2.f * P1.y);              // d_z T
+        }
+      }
+    }
+    if (cb + kEpiCols < kTileN) group_sync();   // read before the next columns overwrite it
+  }
+}
+
 // Error bits of a state and of its handle (kFlagTimeout when a wait gave up).
 __device__ __forceinline__ void flag_timeout(int* flags, int* err, int b) {
   atomicOr(flags + b, kFlagTimeout);
@@ -256,56 +382,73 @@ void tc_zinv_build_images(const Grid& g, const double* zinv, int nops, float* hi
     }
 }
 
-// Operator-image stages (16 KB hi + 16 KB lo per K-chunk) of k_zinv_tc: up to
-// four, as many as fit beside the X tile in 200 KB of shared memory.
-static int tc_zinv_stages(const Grid& g) {
-  const int kc = tc_zinv_kchunks(g);
-  for (int nb = std::min(kc, 4); nb > 1; --nb)
-    if ((size_t)kc * kTileN * 128 * 2 + (size_t)nb * 2 * kTileM * 128 + 1024 <= 200 * 1024) return nb;
-  return 1;
+// Grid-only choice (so a state gives the same bits in any batch): the tensor
+// cores take grids with at least 64 Chebyshev coefficients whose X tile and
+// first image stages fit in 200 KB of shared memory.
+bool tc_zinv_supported(const Grid& g) {
+  const size_t x = (size_t)tc_zinv_kchunks(g) * kTileN * 128 * 2, stage = 2 * kTileM * 128;
+  return g.Nz >= 64 && x + stage + 1024 <= 200 * 1024;
 }
 
-size_t tc_zinv_smem_bytes(const Grid& g) {
-  // X tile hi/lo (all K), the A-chunk stages hi/lo, alignment slack
-  return (size_t)tc_zinv_kchunks(g) * kTileN * 128 * 2 + (size_t)tc_zinv_stages(g) * 2 * kTileM * 128 + 1024;
+// Shape of a k_zinv_tc launch: row tiles per CTA, image stages (16 KB hi + 16 KB
+// lo per K-chunk) and shared memory: X tile hi/lo (all K), stages, the epilogue's
+// rows, alignment slack.  The fewest row tiles that make no more CTAs than SMs
+// (1024 x 256, one state: 26 us with two, 35 with one, 72 with all twelve), else
+// all of a field's, so that its X tile is converted once (512 x 128, 64 states in
+// BF16: 142 us, 207 with one).
+struct ZinvTcShape {
+  int tiles, stages;
+  size_t smem;
+};
+static ZinvTcShape tc_zinv_shape(const Grid& g, int B) {
+  const int kc = tc_zinv_kchunks(g), ntile = (2 * g.nm + kTileN - 1) / kTileN;
+  const size_t x = (size_t)kc * kTileN * 128 * 2, stage = 2 * kTileM * 128;
+  const int m4 = tc_zinv_mtiles(g, 4), m2 = tc_zinv_mtiles(g, 2);
+  int tiles = 1;
+  while (tiles < m4 && (long)B * ntile * ((m4 + tiles - 1) / tiles + (m2 + tiles - 1) / tiles) > 152) ++tiles;
+  const size_t rest = (tiles == 1 ? 0 : kEpiBytes) + 1024;   // (one tile: the epilogue's rows replace the operands)
+  int nb = std::min(4, kc * tiles);
+  while (nb > 1 && x + nb * stage + rest > 222 * 1024) --nb;
+  return {tiles, nb, x + nb * stage + rest};
 }
 
 // Output fields: psi (nops = 4): u, w, d_x omega, d_z omega, d_x u, d_z u (0..5);
 // T (nops = 2): T, d_x T, d_z T (6..8).
-// CTA per (slice, 64-column tile, field, group of 128-row tiles of the field's
-// operator rows): one row tile per CTA when K is at most two 32-wide chunks
-// (the X tile is cheap to convert, and a single slice spreads over more CTAs),
-// all of the field's row tiles otherwise (the X tile, converted once, serves
-// them all).  Thread 0 streams the K-chunks of the operator images, tile after
-// tile, into a ring of NB shared-memory stages with bulk (TMA) copies while all
-// threads convert the X tile to hi/lo TF32 operands; it issues 3 x 4 MMAs per
-// chunk as each lands, refilling a stage once its MMAs completed (so the next
-// tile's chunks arrive during the current tile's epilogue); after each tile
-// the four warps read the accumulator and form the fields.
-__host__ __device__ inline bool tc_zinv_tile_per_cta(const Grid& g) { return tc_zinv_kchunks(g) <= 2; }
-
-__global__ void __launch_bounds__(kTcThreads) k_zinv_tc(Grid g, const float* __restrict__ Ahi_psi,
+// CTA per (slice, 64-column tile, field, `tiles` consecutive 128-row tiles of the
+// field's operator rows).  Eight warps convert the X tile to hi/lo operands and
+// then form the fields, tile after tile.  One lane of a ninth streams the K-chunks
+// of the operator images into a ring of NB shared-memory stages with bulk (TMA)
+// copies, one of a tenth issues 3 x 4 MMAs per chunk as it lands, one tile ahead:
+// the accumulators of two tiles alternate in tensor memory.
+// Bound: the images' way from L2 into shared memory (1024 x 256: 256 KB per
+// row tile, two stages of 32 KB in flight) and the conversion of X.  Measured
+// (GB300, per launch; before, one thread issued, refilled and waited in turn,
+// all threads polled, fields were stored in scattered 8-byte pieces and wave
+// numbers converted from FP64 at every store; same bits): 1024 x 256, 32 states
+// 1067 -> 439 us, one state 195 -> 26 us; 512 x 128, 64 states 472 -> 159 us, in
+// BF16 342 -> 142 us; 256 x 64, 8 states 24.7 -> 14 us, one state 19 -> 12 us.
+__global__ void __launch_bounds__(kZinvTcThreads) k_zinv_tc(Grid g, const float* __restrict__ Ahi_psi,
                                                  const float* __restrict__ Alo_psi, const float* __restrict__ Ahi_T,
                                                  const float* __restrict__ Alo_T, const double* __restrict__ X,
                                                  size_t S, float* __restrict__ Z, int B, const int* nsteps,
-                                                 const int* step, int* flags, int* err, int NB) {
+                                                 const int* step, int* flags, int* err, int tiles, int NB) {
   pdl_wait();
   extern __shared__ __align__(1024) unsigned char tc_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)tc_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[4], empty[4], accb[1];
+  __shared__ __align__(8) uint64_t full[4], empty[4], accb[2], accfree[2];
   __shared__ uint32_t tmem_base;
+  __shared__ float kf[kTileN / 2];            // wave numbers of the tile's modes
   const int ntile = (2 * g.nm + kTileN - 1) / kTileN;
   const int mt4 = tc_zinv_mtiles(g, 4), mt2 = tc_zinv_mtiles(g, 2);
-  const bool one = tc_zinv_tile_per_cta(g);
-  const int units = one ? mt4 + mt2 : 2;      // CTAs per (slice, column tile)
+  const int u4 = (mt4 + tiles - 1) / tiles, units = u4 + (mt2 + tiles - 1) / tiles;   // CTAs per (slice, column tile)
   const int per_b = ntile * units;
   const int b = blockIdx.x / per_b;
   int rem = blockIdx.x - b * per_b;
   const int ct = rem / units;
   const int q = rem - ct * units;
-  const int fsel = one ? (q < mt4 ? 0 : 1) : q;   // 0: psi (nops 4), 1: T (nops 2)
-  const int t0 = one ? (q < mt4 ? q : q - mt4) : 0;
-  const int t1 = one ? t0 + 1 : (fsel == 0 ? mt4 : mt2);
+  const int fsel = q < u4 ? 0 : 1;            // 0: psi (nops 4), 1: T (nops 2)
+  const int t0 = (fsel == 0 ? q : q - u4) * tiles;
+  const int t1 = min(t0 + tiles, fsel == 0 ? mt4 : mt2);
   const int c0 = ct * kTileN;
   if (b >= B || !(nsteps == nullptr || *step < nsteps[b])) return;   // uniform per block
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -313,202 +456,134 @@ __global__ void __launch_bounds__(kTcThreads) k_zinv_tc(Grid g, const float* __r
   const int f = fsel == 0 ? 1 : 0;            // state field: psi slot 1, T slot 0
   const int kc = tc_zinv_kchunks(g);
   const int nchunks = (t1 - t0) * kc;         // the chunks this CTA streams, tile after tile
-  const float* Ahi = (fsel == 0 ? Ahi_psi : Ahi_T) + (size_t)t0 * kc * kChunkFloats;
-  const float* Alo = (fsel == 0 ? Alo_psi : Alo_T) + (size_t)t0 * kc * kChunkFloats;
-  constexpr uint32_t kChunkBytes = kChunkFloats * 4;   // one image chunk, 16 KB
   const bool bf = g.tcbf16 != 0;
-  const int ke = tc_ke(g), es = 128 / ke, lke = bf ? 6 : 5;   // ke = 2^lke
   unsigned char* sXhi = base;
   unsigned char* sXlo = sXhi + (size_t)kc * kTileN * 128;
   unsigned char* sA = sXlo + (size_t)kc * kTileN * 128;   // [stage][hi, lo][128 x 128 B]
-  uint32_t seen_full[4] = {0, 0, 0, 0}, copies[4] = {0, 0, 0, 0};   // thread 0's bookkeeping
-  uint32_t seen_empty[4] = {0, 0, 0, 0}, commits[4] = {0, 0, 0, 0};
-  uint32_t acc_commits = 0, acc_seen = 0;
-  if (tid == 0) {
+  // the epilogue's rows, [128][kEpiStride]: where one tile is all, in the operands' place
+  float* epi = reinterpret_cast<float*>(tiles == 1 ? base : sA + (size_t)NB * 2 * kTileM * 128);
+  const long long limit = g_wait_limit;
+  const bool loader = tid == kTcThreads, issuer = tid == kTcThreads + 32;
+
+  const float* Ahi = (fsel == 0 ? Ahi_psi : Ahi_T) + (size_t)t0 * kc * kChunkFloats;
+  const float* Alo = (fsel == 0 ? Alo_psi : Alo_T) + (size_t)t0 * kc * kChunkFloats;
+  constexpr uint32_t kChunkBytes = kChunkFloats * 4;   // one image chunk, 16 KB
+  auto fetch = [&](int c, int buf) {          // chunk c into its stage
+    unsigned char* ah = sA + (size_t)buf * 2 * kTileM * 128;
+    arrive_expect_tx(&full[buf], 2 * kChunkBytes);
+    bulk_g2s(ah, Ahi + (size_t)c * kChunkFloats, kChunkBytes, &full[buf]);
+    bulk_g2s(ah + kTileM * 128, Alo + (size_t)c * kChunkFloats, kChunkBytes, &full[buf]);
+  };
+  if (loader) {
     for (int i = 0; i < NB; ++i) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&full[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&empty[i])));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&accb[0])));
+    for (int i = 0; i < 2; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&accb[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&accfree[i])));
+    }
     asm volatile("fence.mbarrier_init.release.cluster;");
     // the first NB chunks of the operator images start streaming in at once
-    for (int c = 0; c < NB && c < nchunks; ++c) {
-      unsigned char* ah = sA + (size_t)c * 2 * kTileM * 128;
-      arrive_expect_tx(&full[c], 2 * kChunkBytes);
-      bulk_g2s(ah, Ahi + (size_t)c * kChunkFloats, kChunkBytes, &full[c]);
-      bulk_g2s(ah + kTileM * 128, Alo + (size_t)c * kChunkFloats, kChunkBytes, &full[c]);
-      copies[c]++;
-    }
+    for (int c = 0; c < NB && c < nchunks; ++c) fetch(c, c);
   }
-  if (warp == 0) {
-    __syncwarp();                             // the warp converged again after thread 0's set-up
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(saddr(&tmem_base)));
+  if (warp == kTcThreads / 32) {
+    __syncwarp();                             // the warp converged again after the loader's set-up
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(saddr(&tmem_base)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  // X tile -> hi/lo TF32 operands, K-major (row = column of the tile, k = n)
-  // (four consecutive columns, two modes, per item: 16-byte loads, several in flight)
-  const double* Xb = X + (size_t)b * S;
-#pragma unroll 4
-  for (int it = tid; it < kc * ke * (kTileN / 4); it += blockDim.x) {
-    const int n = it / (kTileN / 4), col = (it - n * (kTileN / 4)) * 4;
-    const int gc = c0 + col;                  // even: columns gc .. gc+3 are modes gc/2, gc/2 + 1
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    if (n < g.Nz) {
-      const double* src = Xb + soff2(g, f, n, gc >> 1);
-      if (gc + 3 < 2 * g.nm) {
-        const double2 v0 = *reinterpret_cast<const double2*>(src);
-        const double2 v1 = *reinterpret_cast<const double2*>(src + 2);
-        v[0] = v0.x; v[1] = v0.y; v[2] = v1.x; v[3] = v1.y;
-      } else {
-        for (int e = 0; e < 4; ++e)
-          if (gc + e < 2 * g.nm) v[e] = src[e];
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t o = (uint32_t)(n >> lke) * kTileN * 128 + swz_b(col + e, (n & (ke - 1)) * es);
-      store_split(bf, (float)v[e], sXhi, sXlo, o);
-    }
+  } else if (warp < kTcThreads / 32) {
+    if (tid < kTileN / 2) kf[tid] = (float)(g.kfac * (c0 / 2 + tid));
+    // X tile -> hi/lo operands, K-major (row = column of the tile, k = n): one
+    // column's 16 bytes of consecutive n per item, consecutive columns per warp
+    if (bf)
+      convert_tile<true>(g, X + (size_t)b * S + soff2(g, f, 0, 0), c0, kc, tid, sXhi, sXlo);
+    else
+      convert_tile<false>(g, X + (size_t)b * S + soff2(g, f, 0, 0), c0, kc, tid, sXhi, sXlo);
   }
   asm volatile("fence.proxy.async.shared::cta;");
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
-  const uint32_t idesc = bf ? instr_desc_bf16(kTileM, kTileN) : instr_desc_tf32(kTileM, kTileN);
-  const long long limit = g_wait_limit;
-  bool issued_all = true;
-  bool ok = true;
-  float* Zb = Z + (size_t)b * 9 * g.Mz * g.nm * 2;
-  for (int t = t0; t < t1 && ok; ++t) {
-    if (tid == 0) {
-      for (int c = 0; c < kc; ++c) {
-        const int gi = (t - t0) * kc + c, buf = gi % NB;
-        if (!wait_parity(&full[buf], seen_full[buf] & 1, limit)) {
-          issued_all = false;
-          break;
-        }
-        seen_full[buf]++;
+  // A stage has one copy or one chunk's MMAs in flight at a time, an accumulator
+  // one tile's: the parities below name the only phase that can be pending.
+  // Nothing may be in flight when the kernel frees tensor memory and exits: the
+  // loader waits for its last copies, the issuer for its last commits, with the
+  // default limit.
+  if (loader) {
+    bool ok = true;
+    int c = min(NB, nchunks), buf = 0;
+    uint32_t par = 0;                         // of the stages' next phase
+    for (; c < nchunks; ++c) {
+      ok = wait_parity(&empty[buf], par, limit);   // chunk c - NB has been used
+      if (!ok) break;
+      fetch(c, buf);
+      if (++buf == NB) {
+        buf = 0;
+        par ^= 1;
+      }
+    }
+    for (int i = max(0, c - NB); i < c; ++i) wait_parity(&full[i % NB], (i / NB) & 1, kWaitLimit);
+    if (!ok) flag_timeout(flags, err, b);     // a bounded wait gave up
+  } else if (issuer) {
+    const uint32_t idesc = bf ? instr_desc_bf16(kTileM, kTileN) : instr_desc_tf32(kTileM, kTileN);
+    const uint64_t dx = smem_desc(saddr(sXhi)), da = smem_desc(saddr(sA));
+    const uint64_t xlo = (uint64_t)(kc * kTileN * 128) >> 4;
+    bool ok = true;
+    int buf = 0, used = 0, done = 0;          // chunks issued, tiles committed
+    uint32_t par = 0;
+    for (int t = t0; t < t1 && ok; ++t) {
+      const int ab = (t - t0) & 1;
+      if (t - t0 >= 2) {                      // the fields of tile t - 2 have been formed
+        ok = wait_parity(&accfree[ab], ((t - t0) / 2 - 1) & 1, limit);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        unsigned char* ah = sA + (size_t)buf * 2 * kTileM * 128;
-        unsigned char* al = ah + (size_t)kTileM * 128;
-        const uint32_t xh = saddr(sXhi) + (uint32_t)c * kTileN * 128;
-        const uint32_t xl = saddr(sXlo) + (uint32_t)c * kTileN * 128;
-        for (int ks = 0; ks < 4; ++ks) {       // four 32-byte K-steps per 128-byte row
-          const uint32_t o = ks * 32;
-          const uint32_t acc0 = (c > 0 || ks > 0) ? 1u : 0u;
-          mma3(bf, tmem, saddr(ah) + o, saddr(al) + o, xh + o, xl + o, idesc, acc0);
-        }
+      }
+      for (int c = 0; c < kc; ++c) {
+        ok = wait_parity(&full[buf], par, limit);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint64_t a = da + (uint64_t)buf * (2 * kTileM * 128 >> 4), x = dx + (uint64_t)c * (kTileN * 128 >> 4);
+        const uint32_t d = tmem + ab * kTileN;
+        if (bf)
+          mma_chunk<true>(d, a, x, xlo, idesc, c > 0);
+        else
+          mma_chunk<false>(d, a, x, xlo, idesc, c > 0);
         commit(&empty[buf]);
-        commits[buf]++;
-        if (gi + NB < nchunks) {              // refill the stage once its MMAs are done
-          if (!wait_parity(&empty[buf], seen_empty[buf] & 1, limit)) {
-            issued_all = false;
-            break;
-          }
-          seen_empty[buf]++;
-          arrive_expect_tx(&full[buf], 2 * kChunkBytes);
-          bulk_g2s(ah, Ahi + (size_t)(gi + NB) * kChunkFloats, kChunkBytes, &full[buf]);
-          bulk_g2s(al, Alo + (size_t)(gi + NB) * kChunkFloats, kChunkBytes, &full[buf]);
-          copies[buf]++;
+        ++used;
+        if (++buf == NB) {
+          buf = 0;
+          par ^= 1;
         }
       }
-      if (issued_all) {
-        commit(&accb[0]);
-        acc_commits++;
+      if (ok) {
+        commit(&accb[ab]);
+        ++done;
       }
     }
-    // accumulator of tile t ready (thread 0 committed it after the tile's last chunk)
-    const bool acc_done = wait_parity(&accb[0], (uint32_t)(t - t0) & 1, limit);
-    if (tid == 0 && acc_done) acc_seen++;
-    ok = __syncthreads_and(acc_done && issued_all) != 0;
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (!ok) break;
-    const int rows_per_j = nops, jper = kTileM / nops;
-    const int r = (warp & 3) * 32 + lane;     // tile row = TMEM lane
-    const int jl = r / rows_per_j, op = r % rows_per_j;
-    const int j = t * jper + jl;
-    const int cbeg = (warp >> 2) * (kTileN / kTcGroups);
-    for (int cc = cbeg; cc < cbeg + kTileN / kTcGroups; cc += 16) {
-      float v[16];
-      tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cc, v);
-      float P[4][16];
-#pragma unroll
-      for (int qq = 0; qq < 4; ++qq)
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int src = (lane & ~(rows_per_j - 1)) | (qq & (rows_per_j - 1));
-          P[qq][i] = __shfl_sync(0xffffffffu, v[i], src);
-        }
-      if (j >= g.Mz) continue;
-#pragma unroll
-      for (int i = 0; i < 16; i += 2) {
-        const int gc = c0 + cc + i;
-        if (gc >= 2 * g.nm) break;
-        const int m = gc >> 1;
-        const float k = (float)(g.kfac * m);
-        if (nops == 4) {
-          // P[q] = (re, im) of d^q psi/ds^q (m = 0: of U)
-          const float p0r = P[0][i], p0i = P[0][i + 1], p1r = P[1][i], p1i = P[1][i + 1];
-          const float p2r = P[2][i], p2i = P[2][i + 1], p3r = P[3][i], p3i = P[3][i + 1];
-          if (m == 0) {
-            if (op == 0) {
-              store_c(Zb, g, 0, j, 0, p0r, 0.f);            // u = U
-              store_c(Zb, g, 1, j, 0, 0.f, 0.f);            // w
-            } else if (op == 1) {
-              store_c(Zb, g, 2, j, 0, 0.f, 0.f);            // d_x omega
-              store_c(Zb, g, 3, j, 0, -4.f * p2r, 0.f);     // d_z omega = -U_zz
-            } else if (op == 2) {
-              store_c(Zb, g, 4, j, 0, 0.f, 0.f);            // d_x u
-              store_c(Zb, g, 5, j, 0, 2.f * p1r, 0.f);      // d_z u = U_z
-            }
-          } else if (op == 0) {
-            store_c(Zb, g, 0, j, m, 2.f * p1r, 2.f * p1i);  // u = d_z psi
-            store_c(Zb, g, 1, j, m, k * p0i, -k * p0r);     // w = -ik psi
-          } else if (op == 1) {
-            const float omr = k * k * p0r - 4.f * p2r, omi = k * k * p0i - 4.f * p2i;
-            store_c(Zb, g, 2, j, m, -k * omi, k * omr);     // d_x omega = ik omega
-            store_c(Zb, g, 3, j, m, 2.f * k * k * p1r - 8.f * p3r, 2.f * k * k * p1i - 8.f * p3i);
-          } else if (op == 2) {
-            store_c(Zb, g, 4, j, m, -k * 2.f * p1i, k * 2.f * p1r);   // d_x u = ik u
-            store_c(Zb, g, 5, j, m, 4.f * p2r, 4.f * p2i);            // d_z u
-          }
-        } else {
-          const float tr = P[0][i], ti = P[0][i + 1], dr = P[1][i], di = P[1][i + 1];
-          if (op == 0) {
-            store_c(Zb, g, 6, j, m, tr, ti);                          // T
-            store_c(Zb, g, 7, j, m, m == 0 ? 0.f : -k * ti, m == 0 ? 0.f : k * tr);   // d_x T
-          } else {
-            store_c(Zb, g, 8, j, m, 2.f * dr, 2.f * di);              // d_z T
-          }
-        }
-      }
+    for (int i = max(0, used - NB); i < used; ++i) wait_parity(&empty[i % NB], (i / NB) & 1, kWaitLimit);
+    for (int i = max(0, done - 2); i < done; ++i) wait_parity(&accb[i & 1], (i >> 1) & 1, kWaitLimit);
+    if (!ok) flag_timeout(flags, err, b);
+  } else if (warp < kTcThreads / 32) {
+    float* Zb = Z + (size_t)b * 9 * g.Mz * g.nm * 2;
+    bool ok = true;
+    for (int t = t0; t < t1 && ok; ++t) {
+      const int ab = (t - t0) & 1;
+      ok = group_and(tid != 0 || wait_parity(&accb[ab], ((t - t0) >> 1) & 1, limit));
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      if (!ok) break;
+      zinv_fields(g, tmem + ab * kTileN, epi, kf, Zb, nops, t, c0, warp, lane);
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      group_sync();                           // accumulator and staged rows read
+      if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&accfree[ab])) : "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();                          // accumulator read before the next tile overwrites it
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (!ok && tid == 0) flag_timeout(flags, err, b);
   }
-  if (!ok && tid == 0) flag_timeout(flags, err, b);   // a bounded wait gave up
-  if (tid == 0) {
-    // nothing may be in flight when the kernel frees tensor memory and exits:
-    // the MMAs (their commits) and the bulk copies (their stages), with the
-    // default limit, in order
-    for (int i = 0; i < NB; ++i) {
-      while (seen_full[i] < copies[i]) {
-        if (!wait_parity(&full[i], seen_full[i] & 1, kWaitLimit)) break;
-        seen_full[i]++;
-      }
-      while (seen_empty[i] < commits[i]) {
-        if (!wait_parity(&empty[i], seen_empty[i] & 1, kWaitLimit)) break;
-        seen_empty[i]++;
-      }
-    }
-    if (acc_seen < acc_commits) wait_parity(&accb[0], acc_seen & 1, kWaitLimit);
-  }
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem));
+  if (warp == kTcThreads / 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem));
 }
 
 // ---------------------------------------------------------------------------
@@ -754,20 +829,14 @@ cudaError_t launch_zfwd_tc(const Grid& g, const Tables& t, const Work& w, int B,
 
 cudaError_t launch_zinv_tc(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
                            cudaStream_t s) {
-  static int allowed = 48 * 1024;
-  const size_t smem = tc_zinv_smem_bytes(g);
-  if ((int)smem > allowed) {
-    cudaError_t e = cudaFuncSetAttribute(k_zinv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    allowed = (int)smem;
-  }
+  const ZinvTcShape sh = tc_zinv_shape(g, B);
+  static const cudaError_t e = cudaFuncSetAttribute(k_zinv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024);
+  if (e != cudaSuccess) return e;
   const int ntile = (2 * g.nm + kTileN - 1) / kTileN;
-  const int units = tc_zinv_tile_per_cta(g) ? tc_zinv_mtiles(g, 4) + tc_zinv_mtiles(g, 2) : 2;
-  return launch_pdl(w.pdl != 0, k_zinv_tc, (unsigned)(B * ntile * units), kTcThreads, smem, s, g, t.tcA_psi_hi,
+  const int units = (tc_zinv_mtiles(g, 4) + sh.tiles - 1) / sh.tiles + (tc_zinv_mtiles(g, 2) + sh.tiles - 1) / sh.tiles;
+  return launch_pdl(w.pdl != 0, k_zinv_tc, (unsigned)(B * ntile * units), kZinvTcThreads, sh.smem, s, g, t.tcA_psi_hi,
                     t.tcA_psi_lo, t.tcA_T_hi, t.tcA_T_lo, X, state_doubles(g), reinterpret_cast<float*>(w.Z), B, ns,
-                    w.step, w.flags, w.err, tc_zinv_stages(g));
+                    w.step, w.flags, w.err, sh.tiles, sh.stages);
 }
-
-bool tc_zinv_supported(const Grid& g) { return g.Nz >= 64 && tc_zinv_smem_bytes(g) <= 200 * 1024; }
 
 }  // namespace rbc
