@@ -41,7 +41,7 @@ constexpr int kChunkFloats = kTileM * 32;   // one 128-row image chunk of 128-by
 // so that kTcGroups times as many stores are in flight as with four warps
 constexpr int kTcGroups = 2;
 constexpr int kTcThreads = 128 * kTcGroups;
-constexpr int kZinvTcThreads = kTcThreads + 64;   // and the issuing and the copying warp of k_zinv_tc
+constexpr int kWsThreads = kTcThreads + 64;   // and the copying and the issuing warp
 // columns and row stride (floats) of the staged accumulator in k_zinv_tc's
 // epilogue (16-byte rows whose 128-bit accesses meet no bank twice)
 constexpr int kEpiCols = 32, kEpiStride = kEpiCols + 4;
@@ -93,36 +93,6 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t ad, uint64_t bd
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-}
-
-// 3 MMAs (hi*hi, hi*lo, lo*hi) of one 32-byte K-step of the A and X operands
-__device__ __forceinline__ void mma3(bool bf, uint32_t tmem, uint32_t ah, uint32_t al, uint32_t xh, uint32_t xl,
-                                     uint32_t idesc, uint32_t acc0) {
-  if (bf) {
-    mma_bf16(tmem, smem_desc(ah), smem_desc(xh), idesc, acc0);
-    mma_bf16(tmem, smem_desc(ah), smem_desc(xl), idesc, 1u);
-    mma_bf16(tmem, smem_desc(al), smem_desc(xh), idesc, 1u);
-  } else {
-    mma_tf32(tmem, smem_desc(ah), smem_desc(xh), idesc, acc0);
-    mma_tf32(tmem, smem_desc(ah), smem_desc(xl), idesc, 1u);
-    mma_tf32(tmem, smem_desc(al), smem_desc(xh), idesc, 1u);
-  }
-}
-
-// hi/lo split of an FP32 value x into the operand type, stored at byte offset
-// o of the hi and lo tiles: TF32 (cvt.rna) or BF16 (round to nearest even)
-__device__ __forceinline__ void store_split(bool bf, float x, unsigned char* hi, unsigned char* lo, uint32_t o) {
-  if (bf) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(x);
-    const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
-    *reinterpret_cast<__nv_bfloat16*>(hi + o) = h;
-    *reinterpret_cast<__nv_bfloat16*>(lo + o) = l;
-  } else {
-    const uint32_t h = to_tf32(x);
-    const uint32_t l = to_tf32(x - __uint_as_float(h));
-    *reinterpret_cast<uint32_t*>(hi + o) = h;
-    *reinterpret_cast<uint32_t*>(lo + o) = l;
-  }
 }
 
 __device__ __forceinline__ void commit(uint64_t* mbar) {
@@ -204,7 +174,7 @@ __device__ __forceinline__ void mma_chunk(uint32_t tmem, uint64_t a, uint64_t x,
   }
 }
 
-// barriers of the eight converting warps of k_zinv_tc
+// barriers of the eight converting warps
 __device__ __forceinline__ void group_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTcThreads) : "memory"); }
 __device__ __forceinline__ bool group_and(bool v) {
   uint32_t r;
@@ -216,39 +186,137 @@ __device__ __forceinline__ bool group_and(bool v) {
   return r != 0;
 }
 
-// X tile of k_zinv_tc: columns c0 .. c0 + 63 of field rows x[n][2 nm] as hi/lo operands
-template <bool BF>
-__device__ __forceinline__ void convert_tile(const Grid& g, const double* x, int c0, int kc, int tid,
-                                             unsigned char* hi, unsigned char* lo) {
+// FP32 -> FP64 on the integer pipe (a conversion instruction holds its
+// sub-partition's FP64 pipe for 64 clocks); denormals, infinities and NaN take the
+// instruction.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t u = __float_as_uint(v), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u) return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+  if (a == 0) return __hiloint2double((int)u, 0);
+  return (double)v;
+}
+
+// Values val(raw(k)), k < kc K-chunks, of column tid % 64 of the tile as hi/lo
+// operands, K-major (row = column of the tile): 16 bytes of consecutive k per
+// item.  raw() loads without a branch, and the loads of several items are in flight
+// together (item by item, a tile of 1024 x 256 took three times as long to convert
+// as to multiply).
+template <bool BF, int ITEMS, typename Raw, typename Load, typename Val>
+__device__ __forceinline__ void convert_tile(Load&& raw, Val&& val, int kc, int tid, unsigned char* hi, unsigned char* lo) {
   constexpr int PER = BF ? 8 : 4, KE = BF ? 64 : 32;   // operands per 16 bytes, per 128-byte row
-  const int col = tid & (kTileN - 1), gc = c0 + col, w = 2 * g.nm;
-#pragma unroll(BF ? 2 : 4)
-  for (int kg = tid / kTileN; kg < kc * 8; kg += kTcThreads / kTileN) {
-    const int n0 = kg * PER;
-    float v[PER];
+  constexpr int U = BF ? ITEMS / 2 : ITEMS, STEP = kTcThreads / kTileN;
+  const int col = tid & (kTileN - 1);
+  for (int kb = tid / kTileN; kb < kc * 8; kb += U * STEP) {
+    Raw in[U][PER];
 #pragma unroll
-    for (int e = 0; e < PER; ++e) v[e] = (gc < w && n0 + e < g.Nz) ? (float)__ldg(x + (size_t)(n0 + e) * w + gc) : 0.f;
-    const uint32_t o = (uint32_t)(n0 / KE) * kTileN * 128 + swz_b(col, (n0 % KE) * (16 / PER));
-    uint32_t h[4], l[4];
-    if (BF) {
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * e]), h1 = __float2bfloat16_rn(v[2 * e + 1]);
-        const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * e] - __bfloat162float(h0));
-        const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * e + 1] - __bfloat162float(h1));
-        h[e] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-        l[e] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+      for (int e = 0; e < PER; ++e) in[u][e] = raw((kb + u * STEP) * PER + e);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k0 = (kb + u * STEP) * PER;
+      if (k0 >= kc * KE) break;
+      float v[PER];
+#pragma unroll
+      for (int e = 0; e < PER; ++e) v[e] = val(in[u][e], k0 + e);
+      const uint32_t o = (uint32_t)(k0 / KE) * kTileN * 128 + swz_b(col, (k0 % KE) * (16 / PER));
+      uint32_t h[4], l[4];
+      if (BF) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * e]), h1 = __float2bfloat16_rn(v[2 * e + 1]);
+          const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * e] - __bfloat162float(h0));
+          const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * e + 1] - __bfloat162float(h1));
+          h[e] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+          l[e] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          h[e] = to_tf32(v[e]);
+          l[e] = to_tf32(v[e] - __uint_as_float(h[e]));
+        }
       }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        h[e] = to_tf32(v[e]);
-        l[e] = to_tf32(v[e] - __uint_as_float(h[e]));
-      }
+      *reinterpret_cast<uint4*>(hi + o) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(lo + o) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    *reinterpret_cast<uint4*>(hi + o) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(lo + o) = make_uint4(l[0], l[1], l[2], l[3]);
   }
+}
+
+// K-chunk c of the images (hi, lo) into stage buf
+__device__ __forceinline__ void fetch_chunk(unsigned char* sA, const float* Ahi, const float* Alo, int c, int buf,
+                                            uint64_t* full) {
+  constexpr uint32_t bytes = kChunkFloats * 4;   // 16 KB
+  unsigned char* ah = sA + (size_t)buf * 2 * bytes;
+  arrive_expect_tx(full, 2 * bytes);
+  bulk_g2s(ah, Ahi + (size_t)c * kChunkFloats, bytes, full);
+  bulk_g2s(ah + bytes, Alo + (size_t)c * kChunkFloats, bytes, full);
+}
+
+// The loader: chunks NB .. n - 1, each once its stage is free; false if a wait gave
+// up.  A stage has one copy or one chunk's MMAs in flight at a time, so the
+// parities below name the only phase that can be pending.  Returns with no copy
+// in flight.
+__device__ __forceinline__ bool stream_chunks(unsigned char* sA, const float* Ahi, const float* Alo, int n, int NB,
+                                              uint64_t* full, uint64_t* empty, long long limit) {
+  bool ok = true;
+  int c = min(NB, n), buf = 0;
+  uint32_t par = 0;                           // of the stages' next phase
+  for (; c < n; ++c) {
+    ok = wait_parity(&empty[buf], par, limit);   // chunk c - NB has been used
+    if (!ok) break;
+    fetch_chunk(sA, Ahi, Alo, c, buf, &full[buf]);
+    if (++buf == NB) {
+      buf = 0;
+      par ^= 1;
+    }
+  }
+  for (int i = max(0, c - NB); i < c; ++i) wait_parity(&full[i % NB], (i / NB) & 1, kWaitLimit);
+  return ok;
+}
+
+// The issuer's place in the ring, chunks issued so far.
+struct Ring {
+  int buf;
+  uint32_t par;
+  int used;
+};
+
+// The MMAs of one row tile (kc chunks) as they land; false if a wait gave up.
+__device__ __forceinline__ bool issue_tile(bool bf, uint32_t tmem, unsigned char* sA, unsigned char* sXhi, int kc, int NB,
+                                           Ring& ring, uint64_t* full, uint64_t* empty, uint32_t idesc, long long limit) {
+  const uint64_t da = smem_desc(saddr(sA)), dx = smem_desc(saddr(sXhi)), xlo = (uint64_t)(kc * kTileN * 128) >> 4;
+  for (int c = 0; c < kc; ++c) {
+    if (!wait_parity(&full[ring.buf], ring.par, limit)) return false;
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint64_t a = da + (uint64_t)ring.buf * (2 * kTileM * 128 >> 4), x = dx + (uint64_t)c * (kTileN * 128 >> 4);
+    if (bf)
+      mma_chunk<true>(tmem, a, x, xlo, idesc, c > 0);
+    else
+      mma_chunk<false>(tmem, a, x, xlo, idesc, c > 0);
+    commit(&empty[ring.buf]);
+    ++ring.used;
+    if (++ring.buf == NB) {
+      ring.buf = 0;
+      ring.par ^= 1;
+    }
+  }
+  return true;
+}
+// waits for the MMAs of the last chunks issued
+__device__ __forceinline__ void drain_ring(int used, int NB, uint64_t* empty) {
+  for (int i = max(0, used - NB); i < used; ++i) wait_parity(&empty[i % NB], (i / NB) & 1, kWaitLimit);
+}
+
+// kEpiCols columns of the accumulator, from column cb on, to shared memory
+__device__ __forceinline__ void stage_rows(uint32_t tmem, float* epi, int cb, int warp, int lane) {
+  const int r = (warp & 3) * 32 + lane;       // tile row = TMEM lane
+  const int cw = (warp >> 2) * (kEpiCols / kTcGroups);   // this warp's 16 of them
+  float v[16];
+  tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb + cw, v);
+  float4* dst = reinterpret_cast<float4*>(epi + r * kEpiStride + cw);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
 }
 
 // Fields of row tile t, columns c0 .. c0 + 63, from the accumulator at tmem,
@@ -257,15 +325,9 @@ __device__ __forceinline__ void convert_tile(const Grid& g, const double* x, int
 // segment.  All eight warps.
 __device__ __forceinline__ void zinv_fields(const Grid& g, uint32_t tmem, float* epi, const float* kf, float* Zb,
                                             int nops, int t, int c0, int warp, int lane) {
-  const int r = (warp & 3) * 32 + lane;       // tile row = TMEM lane
   const int lj = nops == 4 ? 2 : 1, jper = kTileM >> lj;
   for (int cb = 0; cb < kTileN; cb += kEpiCols) {
-    const int cw = (warp >> 2) * (kEpiCols / kTcGroups);   // this warp's 16 of them
-    float v[16];
-    tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb + cw, v);
-    float4* dst = reinterpret_cast<float4*>(epi + r * kEpiStride + cw);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    stage_rows(tmem, epi, cb, warp, lane);
     group_sync();
     const int ml = lane & 15, m = ((c0 + cb) >> 1) + ml;
     if (m < g.nm) {
@@ -427,7 +489,7 @@ static ZinvTcShape tc_zinv_shape(const Grid& g, int B) {
 // numbers converted from FP64 at every store; same bits): 1024 x 256, 32 states
 // 1067 -> 439 us, one state 195 -> 26 us; 512 x 128, 64 states 472 -> 159 us, in
 // BF16 342 -> 142 us; 256 x 64, 8 states 24.7 -> 14 us, one state 19 -> 12 us.
-__global__ void __launch_bounds__(kZinvTcThreads) k_zinv_tc(Grid g, const float* __restrict__ Ahi_psi,
+__global__ void __launch_bounds__(kWsThreads) k_zinv_tc(Grid g, const float* __restrict__ Ahi_psi,
                                                  const float* __restrict__ Alo_psi, const float* __restrict__ Ahi_T,
                                                  const float* __restrict__ Alo_T, const double* __restrict__ X,
                                                  size_t S, float* __restrict__ Z, int B, const int* nsteps,
@@ -467,13 +529,6 @@ __global__ void __launch_bounds__(kZinvTcThreads) k_zinv_tc(Grid g, const float*
 
   const float* Ahi = (fsel == 0 ? Ahi_psi : Ahi_T) + (size_t)t0 * kc * kChunkFloats;
   const float* Alo = (fsel == 0 ? Alo_psi : Alo_T) + (size_t)t0 * kc * kChunkFloats;
-  constexpr uint32_t kChunkBytes = kChunkFloats * 4;   // one image chunk, 16 KB
-  auto fetch = [&](int c, int buf) {          // chunk c into its stage
-    unsigned char* ah = sA + (size_t)buf * 2 * kTileM * 128;
-    arrive_expect_tx(&full[buf], 2 * kChunkBytes);
-    bulk_g2s(ah, Ahi + (size_t)c * kChunkFloats, kChunkBytes, &full[buf]);
-    bulk_g2s(ah + kTileM * 128, Alo + (size_t)c * kChunkFloats, kChunkBytes, &full[buf]);
-  };
   if (loader) {
     for (int i = 0; i < NB; ++i) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&full[i])));
@@ -485,7 +540,7 @@ __global__ void __launch_bounds__(kZinvTcThreads) k_zinv_tc(Grid g, const float*
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
     // the first NB chunks of the operator images start streaming in at once
-    for (int c = 0; c < NB && c < nchunks; ++c) fetch(c, c);
+    for (int c = 0; c < NB && c < nchunks; ++c) fetch_chunk(sA, Ahi, Alo, c, c, &full[c]);
   }
   if (warp == kTcThreads / 32) {
     __syncwarp();                             // the warp converged again after the loader's set-up
@@ -493,75 +548,45 @@ __global__ void __launch_bounds__(kZinvTcThreads) k_zinv_tc(Grid g, const float*
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   } else if (warp < kTcThreads / 32) {
     if (tid < kTileN / 2) kf[tid] = (float)(g.kfac * (c0 / 2 + tid));
-    // X tile -> hi/lo operands, K-major (row = column of the tile, k = n): one
-    // column's 16 bytes of consecutive n per item, consecutive columns per warp
+    // X tile -> hi/lo operands, K-major (row = column of the tile, k = n)
+    const int w = 2 * g.nm, gc = c0 + (tid & (kTileN - 1));
+    const double* x = X + (size_t)b * S + soff2(g, f, 0, 0) + min(gc, w - 1);
+    auto coef = [&](int n) { return __ldg(x + (size_t)min(n, g.Nz - 1) * w); };
+    auto real = [&](double v, int n) { return gc < w && n < g.Nz ? (float)v : 0.f; };
     if (bf)
-      convert_tile<true>(g, X + (size_t)b * S + soff2(g, f, 0, 0), c0, kc, tid, sXhi, sXlo);
+      convert_tile<true, 8, double>(coef, real, kc, tid, sXhi, sXlo);
     else
-      convert_tile<false>(g, X + (size_t)b * S + soff2(g, f, 0, 0), c0, kc, tid, sXhi, sXlo);
+      convert_tile<false, 8, double>(coef, real, kc, tid, sXhi, sXlo);
   }
   asm volatile("fence.proxy.async.shared::cta;");
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
-  // A stage has one copy or one chunk's MMAs in flight at a time, an accumulator
-  // one tile's: the parities below name the only phase that can be pending.
   // Nothing may be in flight when the kernel frees tensor memory and exits: the
   // loader waits for its last copies, the issuer for its last commits, with the
-  // default limit.
+  // default limit.  An accumulator has one tile's MMAs in flight at a time.
   if (loader) {
-    bool ok = true;
-    int c = min(NB, nchunks), buf = 0;
-    uint32_t par = 0;                         // of the stages' next phase
-    for (; c < nchunks; ++c) {
-      ok = wait_parity(&empty[buf], par, limit);   // chunk c - NB has been used
-      if (!ok) break;
-      fetch(c, buf);
-      if (++buf == NB) {
-        buf = 0;
-        par ^= 1;
-      }
-    }
-    for (int i = max(0, c - NB); i < c; ++i) wait_parity(&full[i % NB], (i / NB) & 1, kWaitLimit);
+    const bool ok = stream_chunks(sA, Ahi, Alo, nchunks, NB, full, empty, limit);
     if (!ok) flag_timeout(flags, err, b);     // a bounded wait gave up
   } else if (issuer) {
     const uint32_t idesc = bf ? instr_desc_bf16(kTileM, kTileN) : instr_desc_tf32(kTileM, kTileN);
-    const uint64_t dx = smem_desc(saddr(sXhi)), da = smem_desc(saddr(sA));
-    const uint64_t xlo = (uint64_t)(kc * kTileN * 128) >> 4;
     bool ok = true;
-    int buf = 0, used = 0, done = 0;          // chunks issued, tiles committed
-    uint32_t par = 0;
-    for (int t = t0; t < t1 && ok; ++t) {
-      const int ab = (t - t0) & 1;
-      if (t - t0 >= 2) {                      // the fields of tile t - 2 have been formed
-        ok = wait_parity(&accfree[ab], ((t - t0) / 2 - 1) & 1, limit);
+    Ring ring = {0, 0, 0};
+    int done = 0;                             // tiles committed
+    for (int t = t0; t < t1; ++t) {
+      const int ab = done & 1;
+      if (done >= 2) {                        // the fields of tile t - 2 have been formed
+        ok = wait_parity(&accfree[ab], (done / 2 - 1) & 1, limit);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
       }
-      for (int c = 0; c < kc; ++c) {
-        ok = wait_parity(&full[buf], par, limit);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint64_t a = da + (uint64_t)buf * (2 * kTileM * 128 >> 4), x = dx + (uint64_t)c * (kTileN * 128 >> 4);
-        const uint32_t d = tmem + ab * kTileN;
-        if (bf)
-          mma_chunk<true>(d, a, x, xlo, idesc, c > 0);
-        else
-          mma_chunk<false>(d, a, x, xlo, idesc, c > 0);
-        commit(&empty[buf]);
-        ++used;
-        if (++buf == NB) {
-          buf = 0;
-          par ^= 1;
-        }
-      }
-      if (ok) {
-        commit(&accb[ab]);
-        ++done;
-      }
+      ok = issue_tile(bf, tmem + ab * kTileN, sA, sXhi, kc, NB, ring, full, empty, idesc, limit);
+      if (!ok) break;
+      commit(&accb[ab]);
+      ++done;
     }
-    for (int i = max(0, used - NB); i < used; ++i) wait_parity(&empty[i % NB], (i / NB) & 1, kWaitLimit);
+    drain_ring(ring.used, NB, empty);
     for (int i = max(0, done - 2); i < done; ++i) wait_parity(&accb[i & 1], (i >> 1) & 1, kWaitLimit);
     if (!ok) flag_timeout(flags, err, b);
   } else if (warp < kTcThreads / 32) {
@@ -639,7 +664,16 @@ bool tc_zfwd_supported(const Grid& g) { return g.Nz >= 64 && tc_zfwd_smem_bytes(
 
 // CTA per (slice, field, parity, 64-column tile, 128-row tile of W's rows of
 // that parity); the images stream in through the bulk-copy ring of k_zinv_tc.
-__global__ void __launch_bounds__(kTcThreads) k_zfwd_tc(Grid g, const float* __restrict__ Whi0, const float* __restrict__ Wlo0,
+// Roles as in k_zinv_tc.
+// Bound: latency of a CTA's chain (folds, images, MMAs, stores), one or two CTAs
+// per SM.  Measured (GB300, per launch; one thread issuing, copying and waiting,
+// loads item by item and scattered 16-byte stores before; same bits): 1024 x 256,
+// 32 states 319 -> 232 us, in BF16 262 -> 168 us; 512 x 128, 64 states 170 -> 136
+// us, in BF16 104 -> 66 us; 256 x 64, 8 states 14.4 -> 10.8 us.
+// ITEMS (K-major 16-byte items per thread in flight): 8 where shared memory leaves
+// one CTA per SM, 4 (fewer registers) where two fit.
+template <int ITEMS>
+__global__ void __launch_bounds__(kWsThreads, ITEMS == 4 ? 2 : 1) k_zfwd_tc(Grid g, const float* __restrict__ Whi0, const float* __restrict__ Wlo0,
                                                  const float* __restrict__ Whi1, const float* __restrict__ Wlo1,
                                                  const float* __restrict__ Q, double* __restrict__ F, size_t S, int B,
                                                  const int* nsteps, const int* step, int* flags, int* err, int NB) {
@@ -661,168 +695,106 @@ __global__ void __launch_bounds__(kTcThreads) k_zfwd_tc(Grid g, const float* __r
   const int c0 = ct * kTileN;
   if (b >= B || !(nsteps == nullptr || *step < nsteps[b])) return;   // uniform per block
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int kc = tc_zfwd_kchunks(g), Mh = (g.Mz + 1) / 2;
-  const float* Ahi = (p == 0 ? Whi0 : Whi1) + (size_t)t * kc * kChunkFloats;
-  const float* Alo = (p == 0 ? Wlo0 : Wlo1) + (size_t)t * kc * kChunkFloats;
-  constexpr uint32_t kChunkBytes = kChunkFloats * 4;
+  const int kc = tc_zfwd_kchunks(g);
   const bool bf = g.tcbf16 != 0;
-  const int ke = tc_ke(g), es = 128 / ke, lke = bf ? 6 : 5;   // ke = 2^lke
   unsigned char* sXhi = base;
   unsigned char* sXlo = sXhi + (size_t)kc * kTileN * 128;
   unsigned char* sA = sXlo + (size_t)kc * kTileN * 128;   // [stage][hi, lo][128 x 128 B]
-  uint32_t seen_full[4] = {0, 0, 0, 0}, copies[4] = {0, 0, 0, 0};
-  uint32_t seen_empty[4] = {0, 0, 0, 0}, commits[4] = {0, 0, 0, 0};
-  uint32_t acc_commits = 0, acc_seen = 0;
-  if (tid == 0) {
+  float* epi = reinterpret_cast<float*>(base);            // the epilogue's rows replace the operands
+  const long long limit = g_wait_limit;
+  const bool loader = tid == kTcThreads, issuer = tid == kTcThreads + 32;
+  const float* Ahi = (p == 0 ? Whi0 : Whi1) + (size_t)t * kc * kChunkFloats;
+  const float* Alo = (p == 0 ? Wlo0 : Wlo1) + (size_t)t * kc * kChunkFloats;
+  if (loader) {
     for (int i = 0; i < NB; ++i) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&full[i])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&empty[i])));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&accb[0])));
     asm volatile("fence.mbarrier_init.release.cluster;");
-    for (int c = 0; c < NB && c < kc; ++c) {
-      unsigned char* ah = sA + (size_t)c * 2 * kTileM * 128;
-      arrive_expect_tx(&full[c], 2 * kChunkBytes);
-      bulk_g2s(ah, Ahi + (size_t)c * kChunkFloats, kChunkBytes, &full[c]);
-      bulk_g2s(ah + kTileM * 128, Alo + (size_t)c * kChunkFloats, kChunkBytes, &full[c]);
-      copies[c]++;
-    }
+    for (int c = 0; c < NB && c < kc; ++c) fetch_chunk(sA, Ahi, Alo, c, c, &full[c]);
   }
-  if (warp == 0) {
-    __syncwarp();                             // the warp converged again after thread 0's set-up
+  if (warp == kTcThreads / 32) {
+    __syncwarp();                             // the warp converged again after the loader's set-up
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(saddr(&tmem_base)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  // folds of parity p -> hi/lo TF32 operands, K-major (row = column of the tile, k = jh)
-  // (four consecutive columns per item: 16-byte loads, several in flight)
-  const float* q = Q + (size_t)(b * 2 + f) * g.Mz * g.nm * 2;
-  const bool vec = (2 * g.nm) % 4 == 0;
-#pragma unroll 4
-  for (int it = tid; it < kc * ke * (kTileN / 4); it += blockDim.x) {
-    const int jh = it / (kTileN / 4), col = (it - jh * (kTileN / 4)) * 4;
-    const int jr = g.Mz - 1 - jh;
-    float a[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
-    if (jh < Mh) {
-      const float* ra = q + (size_t)jh * g.nm * 2 + c0 + col;
-      const float* rc = q + (size_t)jr * g.nm * 2 + c0 + col;
-      if (vec && c0 + col + 3 < 2 * g.nm) {
-        const float4 va = *reinterpret_cast<const float4*>(ra);
-        a[0] = va.x; a[1] = va.y; a[2] = va.z; a[3] = va.w;
-        if (jr != jh) {
-          const float4 vc = *reinterpret_cast<const float4*>(rc);
-          c[0] = vc.x; c[1] = vc.y; c[2] = vc.z; c[3] = vc.w;
-        }
-      } else {
-        for (int e = 0; e < 4; ++e)
-          if (c0 + col + e < 2 * g.nm) {
-            a[e] = ra[e];
-            if (jr != jh) c[e] = rc[e];
-          }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float x = 0.f;
-      if (jh < Mh && c0 + col + e < 2 * g.nm) x = (jr != jh) ? (p == 0 ? a[e] + c[e] : a[e] - c[e]) : (p == 0 ? a[e] : 0.f);
-      const uint32_t o = (uint32_t)(jh >> lke) * kTileN * 128 + swz_b(col + e, (jh & (ke - 1)) * es);
-      store_split(bf, x, sXhi, sXlo, o);
-    }
+  } else if (warp < kTcThreads / 32) {
+    // folds of parity p -> hi/lo operands, K-major (row = column of the tile, k = jh)
+    const float* q = Q + (size_t)(b * 2 + f) * g.Mz * g.nm * 2;
+    const int w = 2 * g.nm, Mh = (g.Mz + 1) / 2, gc = c0 + (tid & (kTileN - 1));
+    const float* qc = q + min(gc, w - 1);
+    auto pair = [&](int jh) {
+      const int j = min(jh, Mh - 1);
+      return make_float2(__ldg(qc + (size_t)j * w), __ldg(qc + (size_t)(g.Mz - 1 - j) * w));
+    };
+    auto fold = [&](float2 v, int jh) {
+      const bool twice = g.Mz - 1 - jh != jh;
+      const float x = p == 0 ? (twice ? v.x + v.y : v.x) : (twice ? v.x - v.y : 0.f);
+      return gc < w && jh < Mh ? x : 0.f;
+    };
+    if (bf)
+      convert_tile<true, ITEMS, float2>(pair, fold, kc, tid, sXhi, sXlo);
+    else
+      convert_tile<false, ITEMS, float2>(pair, fold, kc, tid, sXhi, sXlo);
   }
   asm volatile("fence.proxy.async.shared::cta;");
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_base;
-  const uint32_t idesc = bf ? instr_desc_bf16(kTileM, kTileN) : instr_desc_tf32(kTileM, kTileN);
-  const long long limit = g_wait_limit;
-  bool issued_all = true;
-  if (tid == 0) {
-    for (int c = 0; c < kc; ++c) {
-      const int buf = c % NB;
-      if (!wait_parity(&full[buf], seen_full[buf] & 1, limit)) {
-        issued_all = false;
-        break;
+  // (one phase per stage and pass over the ring, one of the accumulator: see k_zinv_tc)
+  if (loader) {
+    const bool ok = stream_chunks(sA, Ahi, Alo, kc, NB, full, empty, limit);
+    if (!ok) flag_timeout(flags, err, b);     // a bounded wait gave up
+  } else if (issuer) {
+    const uint32_t idesc = bf ? instr_desc_bf16(kTileM, kTileN) : instr_desc_tf32(kTileM, kTileN);
+    Ring ring = {0, 0, 0};
+    const bool ok = issue_tile(bf, tmem, sA, sXhi, kc, NB, ring, full, empty, idesc, limit);
+    if (ok) commit(&accb[0]);
+    drain_ring(ring.used, NB, empty);
+    if (ok)
+      wait_parity(&accb[0], 0, kWaitLimit);
+    else
+      flag_timeout(flags, err, b);
+  } else if (warp < kTcThreads / 32) {
+    const bool ok = group_and(tid != 0 || wait_parity(&accb[0], 0, limit));
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (ok) {
+      // kEpiCols columns at a time through shared memory: each half-warp widens
+      // and stores 32 of them, 256 bytes, of one row
+      double* Fb = F + (size_t)b * S;
+      for (int cb = 0; cb < kTileN; cb += kEpiCols) {
+        stage_rows(tmem, epi, cb, warp, lane);
+        group_sync();
+        const int m = ((c0 + cb) >> 1) + (lane & 15);
+        if (m < g.nm)
+          for (int r = warp * 2 + (lane >> 4); r < kTileM; r += 2 * (kTcThreads / 32)) {
+            const int n = 2 * (t * kTileM + r) + p;
+            if (n >= g.Nz) break;
+            const float2 v = *reinterpret_cast<const float2*>(epi + r * kEpiStride + 2 * (lane & 15));
+            *reinterpret_cast<double2*>(Fb + soff2(g, f, n, m)) = make_double2(widen(v.x), widen(v.y));
+          }
+        if (cb + kEpiCols < kTileN) group_sync();
       }
-      seen_full[buf]++;
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      unsigned char* ah = sA + (size_t)buf * 2 * kTileM * 128;
-      unsigned char* al = ah + (size_t)kTileM * 128;
-      const uint32_t xh = saddr(sXhi) + (uint32_t)c * kTileN * 128;
-      const uint32_t xl = saddr(sXlo) + (uint32_t)c * kTileN * 128;
-      for (int ks = 0; ks < 4; ++ks) {         // four 32-byte K-steps per 128-byte row
-        const uint32_t o = ks * 32;
-        const uint32_t acc0 = (c > 0 || ks > 0) ? 1u : 0u;
-        mma3(bf, tmem, saddr(ah) + o, saddr(al) + o, xh + o, xl + o, idesc, acc0);
-      }
-      commit(&empty[buf]);
-      commits[buf]++;
-      if (c + NB < kc) {
-        if (!wait_parity(&empty[buf], seen_empty[buf] & 1, limit)) {
-          issued_all = false;
-          break;
-        }
-        seen_empty[buf]++;
-        arrive_expect_tx(&full[buf], 2 * kChunkBytes);
-        bulk_g2s(ah, Ahi + (size_t)(c + NB) * kChunkFloats, kChunkBytes, &full[buf]);
-        bulk_g2s(al, Alo + (size_t)(c + NB) * kChunkFloats, kChunkBytes, &full[buf]);
-        copies[buf]++;
-      }
-    }
-    if (issued_all) {
-      commit(&accb[0]);
-      acc_commits = 1;
+    } else if (tid == 0) {
+      flag_timeout(flags, err, b);
     }
   }
-  const bool acc_done = wait_parity(&accb[0], 0, limit);
-  if (tid == 0 && acc_done) acc_seen = 1;
-  const bool ok = __syncthreads_and(acc_done && issued_all) != 0;
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (ok) {
-    double* Fb = F + (size_t)b * S;
-    const int n = 2 * (t * kTileM + (warp & 3) * 32 + lane) + p;   // tile row = TMEM lane
-    const int cbeg = (warp >> 2) * (kTileN / kTcGroups);
-    for (int cc = cbeg; cc < cbeg + kTileN / kTcGroups; cc += 16) {
-      float v[16];
-      tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cc, v);
-      if (n >= g.Nz) continue;
-#pragma unroll
-      for (int i = 0; i < 16; i += 2) {
-        const int gc = c0 + cc + i;
-        if (gc >= 2 * g.nm) break;
-        *reinterpret_cast<double2*>(Fb + soff2(g, f, n, gc >> 1)) = make_double2((double)v[i], (double)v[i + 1]);
-      }
-    }
-  }
-  if (!ok && tid == 0) flag_timeout(flags, err, b);   // a bounded wait gave up
-  if (tid == 0) {
-    for (int i = 0; i < NB; ++i) {
-      while (seen_full[i] < copies[i]) {
-        if (!wait_parity(&full[i], seen_full[i] & 1, kWaitLimit)) break;
-        seen_full[i]++;
-      }
-      while (seen_empty[i] < commits[i]) {
-        if (!wait_parity(&empty[i], seen_empty[i] & 1, kWaitLimit)) break;
-        seen_empty[i]++;
-      }
-    }
-    if (acc_seen < acc_commits) wait_parity(&accb[0], 0, kWaitLimit);
-  }
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem));
+  if (warp == kTcThreads / 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem));
 }
 
 cudaError_t launch_zfwd_tc(const Grid& g, const Tables& t, const Work& w, int B, cudaStream_t s) {
-  static int allowed = 48 * 1024;
   const size_t smem = tc_zfwd_smem_bytes(g);
-  if ((int)smem > allowed) {
-    cudaError_t e = cudaFuncSetAttribute(k_zfwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    allowed = (int)smem;
-  }
+  auto* kernel = smem > 112 * 1024 ? k_zfwd_tc<8> : k_zfwd_tc<4>;
+  static const cudaError_t e8 = cudaFuncSetAttribute(k_zfwd_tc<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  static const cudaError_t e4 = cudaFuncSetAttribute(k_zfwd_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e8 != cudaSuccess || e4 != cudaSuccess) return e8 != cudaSuccess ? e8 : e4;
   const int ntile = (2 * g.nm + kTileN - 1) / kTileN;
-  return launch_pdl(w.pdl != 0, k_zfwd_tc, (unsigned)(B * 2 * 2 * ntile * tc_zfwd_mtiles(g)), kTcThreads, smem, s, g,
+  return launch_pdl(w.pdl != 0, kernel, (unsigned)(B * 2 * 2 * ntile * tc_zfwd_mtiles(g)), kWsThreads, smem, s, g,
                     t.tcW_hi[0], t.tcW_lo[0], t.tcW_hi[1], t.tcW_lo[1], reinterpret_cast<const float*>(w.Q), w.F,
                     state_doubles(g), B, w.nsteps, w.step, w.flags, w.err, tc_zfwd_stages(g));
 }
@@ -834,7 +806,7 @@ cudaError_t launch_zinv_tc(const Grid& g, const Tables& t, const Work& w, const 
   if (e != cudaSuccess) return e;
   const int ntile = (2 * g.nm + kTileN - 1) / kTileN;
   const int units = (tc_zinv_mtiles(g, 4) + sh.tiles - 1) / sh.tiles + (tc_zinv_mtiles(g, 2) + sh.tiles - 1) / sh.tiles;
-  return launch_pdl(w.pdl != 0, k_zinv_tc, (unsigned)(B * ntile * units), kZinvTcThreads, sh.smem, s, g, t.tcA_psi_hi,
+  return launch_pdl(w.pdl != 0, k_zinv_tc, (unsigned)(B * ntile * units), kWsThreads, sh.smem, s, g, t.tcA_psi_hi,
                     t.tcA_psi_lo, t.tcA_T_hi, t.tcA_T_lo, X, state_doubles(g), reinterpret_cast<float*>(w.Z), B, ns,
                     w.step, w.flags, w.err, sh.tiles, sh.stages);
 }

@@ -89,3 +89,26 @@ def test_mixed_rows_alone_and_in_batches_agree(rbc, Nx, Nz=10):
         F.step_batch(st, 2, nub)
         assert torch.equal(st, alone.expand_as(st)) and torch.equal(nub, nu.expand_as(nub))
     assert F.check_diverged() == rbc.RBC_OK
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("Nz", [34, 62, 64, 66, 96, 128, 130, 256, 258])
+def test_mixed_column_lengths_match_oracle_and_batches_agree(rbc, Nz, precision, Nx=16):
+    """K-chunks and row tiles of the tensor-core transforms (one per CTA alone, all of a field's in batches), rows per
+    thread and chunks of the stage solve; above Nz = 256 the FP32 CUDA-core transforms."""
+    Ra, dt = 1e4, 1e-5
+    o = RBC(Ra, 1.0, 2.0, Nx, Nz, dt)
+    F = rbc.Propagator(Ra, 1.0, 2.0, Nx, Nz, dt, precision)
+    X0 = nonlinear_state(o, 3)
+    alone = F.new_states(1)
+    alone[0].copy_(torch.from_numpy(to_abi(X0)))
+    states = [alone[:1].repeat(B, 1, 1, 1, 1) for B in (5, 60, 170)]
+    nu = torch.zeros(1, dtype=torch.float64, device="cuda")
+    F.step_batch(alone, 1, nu)
+    ref, integ = o.run(X0, 1)
+    assert max_rel_diff(from_abi(alone[0].cpu().numpy()), ref) < 1e-5
+    for st in states:
+        nub = torch.zeros(st.shape[0], dtype=torch.float64, device="cuda")
+        F.step_batch(st, 1, nub)
+        assert torch.equal(st, alone.expand_as(st)) and torch.equal(nub, nu.expand_as(nub))
+    assert F.check_diverged() == rbc.RBC_OK
