@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "d033826ae653971f6656312b11a06015b30b45c56d103a46938a6862f76c4f87"
+NCU_TRAFFIC_SHA256 = "ee4c1830b5a919e0bbc34ada01a5c987e6a2c6bbd90519294753dca2c3e97c0c"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 135014, "coarse:k_rows": 390451, "coarse:k_zfwd": 123328, "coarse:k_solve": 801920,
-    "fine:k_zinv@32": 10456781, "fine:k_rows@32": 37880678, "fine:k_zfwd@32": 12628416, "fine:k_solve@32": 23856128,
-    "fine:k_zinv@2": 669133, "fine:k_rows@2": 2490317, "fine:k_zfwd@2": 829952, "fine:k_solve@2": 2763776,
+    "coarse:k_zinv": 141722, "coarse:k_rows": 386202, "coarse:k_zfwd": 123072, "coarse:k_solve": 801792,
+    "fine:k_zinv@32": 10432410, "fine:k_rows@32": 37881088, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23855872,
+    "fine:k_zinv@2": 673946, "fine:k_rows@2": 2490470, "fine:k_zfwd@2": 830720, "fine:k_solve@2": 2764800,
 }
 
 

@@ -43,6 +43,22 @@ __device__ __forceinline__ double pow2(int e) {
   return e > 1023 ? __hiloint2double(0x7ff00000, 0) : e < -1022 ? 0.0 : __hiloint2double((e + 1023) << 20, 0);
 }
 
+// v 2^e rounded to nearest even, for a result in the normal range or zero
+// (others: the FP64 instructions).  About 20 integer instructions; a conversion
+// and a multiplication hold the sub-partition's FP64 pipe for 64 clocks each.
+__device__ __forceinline__ double to_double(i64 v, int e) {
+  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << (lz & 63);
+  const int be = 1023 + 63 - lz + e;          // of a value in [2^(63 - lz + e), 2^(64 - lz + e))
+  const unsigned long long q = m >> 11;
+  const unsigned up = (((unsigned)m & 0x7ffu) + 0x3ffu + ((unsigned)q & 1u)) >> 11;
+  unsigned long long r = ((unsigned long long)(unsigned)(be - 1) << 52) + q + up;   // q holds the leading 1
+  if (a == 0) r = 0;
+  else if ((unsigned)(be - 1) >= 2045u) return (double)v * pow2(e);
+  return __longlong_as_double((long long)(r | (v < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
 // a = h 2^32 + l, -2^31 <= l < 2^31.
 __device__ __forceinline__ void split32(i64 a, int& h, int& l) {
   l = (int)a;

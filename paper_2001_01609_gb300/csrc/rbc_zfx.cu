@@ -14,8 +14,8 @@
 // Bound: integer issue, 13 clocks of a sub-partition per term and warp (12 of
 // them the multiply-adds) against 64 for an FP64 multiply-add.
 // Measured (GB300, per launch, FP64 sums before): inverse, 256 x 64, 32 states
-// 301 -> 129 us, 8 states 82 -> 44 us, one state 40 -> 15 us; 512 x 128, 3 states
-// 215 -> 99 us; 64 x 32, 23 states 26.5 -> 16.5 us.  Forward: 100 -> 38 us,
+// 301 -> 121 us, 8 states 82 -> 41 us, one state 40 -> 15 us; 512 x 128, 3 states
+// 215 -> 95 us; 64 x 32, 23 states 26.5 -> 16.5 us.  Forward: 100 -> 38 us,
 // 30 -> 16.5 us, 12.4 -> 10.3 us, 83 -> 33 us, 10.8 -> 9.4 us.  (128 x 32, one
 // state: 13.3 -> 10.3 and 9.3 -> 8.3 us, of which about 7 are the launch as timed.)
 // Against 64-bit plain torch the temperature after a few steps is 2 to 3 times
@@ -52,9 +52,14 @@ __device__ __forceinline__ void mac30(int2 a, int2 x, i64& hi, i64& mid) {
   mid = fx::madw(a.x, x.y, fx::madw(a.y, x.x, mid));
 }
 constexpr i64 kHalf = 1ll << 29;
-// 2^e v for a column exponent that may mark a non-finite column
+// 2^e v for a column exponent that may mark a non-finite column; INT: on the integer
+// pipe.  The inverse, whose blocks alternate between sums on the integer pipe and
+// fields on the FP64 pipe, gains (128 -> 121 us at 256 x 64, 32 states); the
+// forward sums, two instructions of 64 clocks against 20, do not (37.7 -> 38.9 us).
+template <bool INT>
 __device__ __forceinline__ double scaled(i64 v, int ecol, int e) {
-  return ecol >= kNaN ? __hiloint2double(0x7ff80000, 0) : (double)v * fx::pow2(ecol - 1022 + e);
+  if (ecol >= kNaN) return __hiloint2double(0x7ff80000, 0);
+  return INT ? fx::to_double(v, ecol - 1022 + e) : (double)v * fx::pow2(ecol - 1022 + e);
 }
 
 }  // namespace
@@ -188,16 +193,17 @@ __device__ __forceinline__ void zinv_block(const Grid& g, const int2* __restrict
 #pragma unroll
       for (int q = 0; q < NQ; ++q) hi[r][q] += mid[r][q] >> 30;
   };
-  const double k = g.kfac * m;
+  const double k = g.kfac * m, kk = k * k;
   const size_t fs = (size_t)g.Mz * g.nm * 2;
   double* Zc = Zb + (NQ == 4 ? 0 : 4 * fs) + (size_t)2 * (valid ? m : 0) + c;
   // fields of padded row j from the sums of its row pair jp (sg = -1: the mirrored row)
   auto emit = [&](int jp, int j, int sg, const i64* E, const i64* O) {
+    // 2^q times the q-th sum: the factors of two of the fields below (exact)
     double P[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const i64 v = sg > 0 ? E[q] + O[q] : (q & 1) ? O[q] - E[q] : E[q] - O[q];
-      P[q] = scaled(v, ec[q], __ldg(Ea + q * Mh + jp) - 60);
+      P[q] = scaled<true>(v, ec[q], __ldg(Ea + q * Mh + jp) - 60 + q);
     }
     // i z of a complex value: the partner lane's part, negated in the real lane
     auto timesi = [&](double v) {
@@ -208,18 +214,18 @@ __device__ __forceinline__ void zinv_block(const Grid& g, const int2* __restrict
     double* z = Zc + (size_t)j * g.nm * 2;
     if constexpr (NQ == 4) {
       const double ip = timesi(P[0]);
-      const double om = fma(k * k, P[0], -4.0 * P[2]);          // omega = k^2 psi - 4 d2(psi)
+      const double om = fma(kk, P[0], -P[2]);                   // omega = k^2 psi - 4 d2(psi)
       const double io = timesi(om);
       if (!valid) return;
-      z[0] = m0 ? (c == 0 ? P[0] : 0.0) : 2.0 * P[1];           // u = d_z psi (m = 0: U)
+      z[0] = m0 ? (c == 0 ? P[0] : 0.0) : P[1];                 // u = d_z psi (m = 0: U)
       z[fs] = m0 ? 0.0 : -k * ip;                               // w = -ik psi
       z[2 * fs] = m0 ? 0.0 : k * io;                            // d_x omega
-      z[3 * fs] = m0 ? (c == 0 ? -4.0 * P[2] : 0.0) : fma((2.0 * k) * k, P[1], -8.0 * P[3]);   // d_z omega
+      z[3 * fs] = m0 ? (c == 0 ? -P[2] : 0.0) : fma(kk, P[1], -P[3]);   // d_z omega = 2 k^2 d1 - 8 d3
     } else {
       const double it = timesi(P[0]);
       if (!valid) return;
       z[0] = diag ? P[0] : m0 ? 0.0 : k * it;                   // d_x T (the averages of Sec. 2.2: T)
-      z[fs] = 2.0 * P[1];                                       // d_z T
+      z[fs] = P[1];                                             // d_z T
     }
   };
   const int rounds = (Mh + jblocks * JB - 1) / (jblocks * JB);
@@ -489,7 +495,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_zfwd_fx(Grid g, const int2* __r
     for (int i = 0; i < NI; ++i)
       if (valid && r0 + i < g.nq) {
         const int n = 2 * (r0 + i) + p;
-        Fb[n * rs] = scaled(hi[i], em, __ldg(We + n) - 59);
+        Fb[n * rs] = scaled<false>(hi[i], em, __ldg(We + n) - 59);
       }
   }
 }
