@@ -146,7 +146,7 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "ee4c1830b5a919e0bbc34ada01a5c987e6a2c6bbd90519294753dca2c3e97c0c"
+NCU_TRAFFIC_SHA256 = "8257f368db763ba4576ff6c7dd5ea5f7f08216e61d6c6e814d30b112a106d05a"
 NCU_TRAFFIC = {
     "coarse:k_zinv": 141722, "coarse:k_rows": 386202, "coarse:k_zfwd": 123072, "coarse:k_solve": 801792,
     "fine:k_zinv@32": 10432410, "fine:k_rows@32": 37881088, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23855872,

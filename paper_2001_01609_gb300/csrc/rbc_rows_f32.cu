@@ -34,7 +34,7 @@
 // Bound: issue slots, about 350 instructions per point, of them 220 FP32
 // arithmetic; with few rows the chain of passes.  Measured (GB300, per launch; one
 // radix-4 step per pass with twiddles and operands in shared memory, 18 barriers,
-// before; the bits are the same): 1024 x 256, 32 states 1560 -> 725 us; 512 x 128,
+// before; the bits are the same): 1024 x 256, 32 states 1560 -> 568 us; 512 x 128,
 // 64 states 568 -> 263 us; 256 x 64, 8 states 32.9 -> 16.4 us, one state 16.7 ->
 // 12.4 us; 128 x 32, one state 12.3 -> 12.2 us, six 20.8 -> 12.4 us.
 #include <cuda_runtime.h>
@@ -193,7 +193,7 @@ constexpr int kMaxRows = 16;
 constexpr int kSplitThreads = 640;   // SPLIT: the five FFTs' C items of 128 points
 
 template <int P, bool SPLIT>
-__global__ void __launch_bounds__(SPLIT ? kSplitThreads : 256) k_rows_f32(Grid g, const C* __restrict__ TW, const float* __restrict__ Z,
+__global__ void __launch_bounds__(SPLIT ? kSplitThreads : 512) k_rows_f32(Grid g, const C* __restrict__ TW, const float* __restrict__ Z,
                                                   float* __restrict__ Q, double* __restrict__ wT, int nrows, int NR,
                                                   const int* nsteps, const int* step) {
   using PL = Plan32<P>;
@@ -432,7 +432,9 @@ cudaError_t launch_rows_P(const Grid& g, const Tables& t, const Work& w, int B, 
     return launch_pdl(w.pdl != 0, k_rows_f32<P, true>, blocks, th, PL::row_bytes, s, g, t.tw32, Z, Q, w.wT, nrows, nr,
                       ns, w.step);
   }
-  const int th = std::max((nr * PL::NK + 31) / 32 * 32, std::min(256, (nr * 5 * PL::GA + 31) / 32 * 32));
+  // 1024 x 256, 32 states: 568 us with a thread per item of passes A and B (480 per
+  // row), 722 with 256; shorter rows, several to a block, are slower beyond 256
+  const int th = P == 9 ? 512 : std::max((nr * PL::NK + 31) / 32 * 32, std::min(256, (nr * 5 * PL::GA + 31) / 32 * 32));
   return launch_pdl(w.pdl != 0, k_rows_f32<P, false>, blocks, th, nr * PL::row_bytes, s, g, t.tw32, Z, Q, w.wT, nrows,
                     nr, ns, w.step);
 }
