@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "8257f368db763ba4576ff6c7dd5ea5f7f08216e61d6c6e814d30b112a106d05a"
+NCU_TRAFFIC_SHA256 = "7a5004801afed779c26d9bc67571fb85560c895e9b082776578fd4d1b5fb1bf1"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 141722, "coarse:k_rows": 386202, "coarse:k_zfwd": 123072, "coarse:k_solve": 801792,
-    "fine:k_zinv@32": 10432410, "fine:k_rows@32": 37881088, "fine:k_zfwd@32": 12628544, "fine:k_solve@32": 23855872,
-    "fine:k_zinv@2": 673946, "fine:k_rows@2": 2490470, "fine:k_zfwd@2": 830720, "fine:k_solve@2": 2764800,
+    "coarse:k_zinv": 141619, "coarse:k_rows": 386406, "coarse:k_zfwd": 123520, "coarse:k_solve": 802112,
+    "fine:k_zinv@32": 10434611, "fine:k_rows@32": 37881037, "fine:k_zfwd@32": 12629120, "fine:k_solve@32": 23858176,
+    "fine:k_zinv@2": 673741, "fine:k_rows@2": 2491034, "fine:k_zfwd@2": 831168, "fine:k_solve@2": 2763328,
 }
 
 

@@ -43,7 +43,7 @@
 // 64 clocks, a 32x32->64 multiply-add for 4 and a 64-bit add for 2, so the
 // same FFT costs about a tenth.  Measured (GB300, per launch, against five
 // FP64 FFTs in radix-4 passes through shared memory): 256 x 64, 32 states
-// 491 -> 108 us; 512 x 128, 3 states 207 -> 59 us; 64 x 32, 23 states
+// 491 -> 108 us; 512 x 128, 3 states 207 -> 48 us; 64 x 32, 23 states
 // 41 -> 17 us; 128 x 32, one state 20.4 -> 18.3 us (latency: the barriers).
 // One thread keeping the points of all three inverse FFTs in registers (P2 and
 // P3 in one pass, 166 registers, C and D in a place of their own) took 127, 60,
@@ -660,8 +660,14 @@ template <int L> RowsShape rows_shape(const Work& w, int nrows) {
     rb = 1;
   else if (form < 0)
     while (rb > 1 && (long)nrows < 2L * 152 * rb) rb /= 2;
-  // a row alone: threads for the other passes' items too
-  const int th = std::max(P::threads(rb), std::min(128, (rb * 9 * P::R * P::M2 + 31) / 32 * 32));
+  // threads for the other passes' items too: a row alone has 9 R M2 in its first
+  // pass and unpacks L modes.  With few rows per SM they shorten its chain (256 x 64,
+  // one state 29.0 -> 24.8 us; 512 x 128, 3 states 59.6 -> 47.9 us); with more the
+  // rows hide each other's (512 x 128, 16 states 226 us either way), except at
+  // L = 512, where shared memory holds two (1024 x 256, 8 states 684 -> 561 us).
+  const int items = rb > 1 ? rb * 9 * P::R * P::M2 : std::max(9 * P::R * P::M2, L + 32);
+  const int most = rb > 1 ? 128 : L == 512 ? 320 : nrows <= 4 * 152 ? 256 : 128;
+  const int th = std::max(P::threads(rb), std::min(most, (items + 31) / 32 * 32));
   return {rb, th, rb * P::row_bytes};
 }
 
