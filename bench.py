@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "7a5004801afed779c26d9bc67571fb85560c895e9b082776578fd4d1b5fb1bf1"
+NCU_TRAFFIC_SHA256 = "44402ecaddc0dccc236be580331677e986e7aa4de25b57b131975c1b2ab39fa9"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 141619, "coarse:k_rows": 386406, "coarse:k_zfwd": 123520, "coarse:k_solve": 802112,
-    "fine:k_zinv@32": 10434611, "fine:k_rows@32": 37881037, "fine:k_zfwd@32": 12629120, "fine:k_solve@32": 23858176,
-    "fine:k_zinv@2": 673741, "fine:k_rows@2": 2491034, "fine:k_zfwd@2": 831168, "fine:k_solve@2": 2763328,
+    "coarse:k_zinv": 141773, "coarse:k_rows": 386509, "coarse:k_zfwd": 123200, "coarse:k_solve": 802432,
+    "fine:k_zinv@32": 10430771, "fine:k_rows@32": 37885747, "fine:k_zfwd@32": 12628864, "fine:k_solve@32": 23856704,
+    "fine:k_zinv@2": 673792, "fine:k_rows@2": 2490675, "fine:k_zfwd@2": 830016, "fine:k_solve@2": 2764608,
 }
 
 

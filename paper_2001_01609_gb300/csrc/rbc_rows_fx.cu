@@ -43,8 +43,8 @@
 // 64 clocks, a 32x32->64 multiply-add for 4 and a 64-bit add for 2, so the
 // same FFT costs about a tenth.  Measured (GB300, per launch, against five
 // FP64 FFTs in radix-4 passes through shared memory): 256 x 64, 32 states
-// 491 -> 108 us; 512 x 128, 3 states 207 -> 48 us; 64 x 32, 23 states
-// 41 -> 17 us; 128 x 32, one state 20.4 -> 18.3 us (latency: the barriers).
+// 491 -> 108 us; 512 x 128, 3 states 207 -> 46 us; 64 x 32, 23 states
+// 41 -> 16.5 us; 128 x 32, one state 20.4 -> 16.6 us (latency: the barriers).
 // One thread keeping the points of all three inverse FFTs in registers (P2 and
 // P3 in one pass, 166 registers, C and D in a place of their own) took 127, 60,
 // 22 and 19.8 us.
@@ -282,6 +282,12 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
   __shared__ RowMeta meta[kMaxRB];
   const int tid = threadIdx.x, T = blockDim.x;
   const int row0 = blockIdx.x * RB;
+  // twiddles into L1 while the launch before this one finishes: the passes' first
+  // uses, one after another, would each wait for L2
+  for (int i = tid * 8; i < N; i += T * 8) {
+    int a, b, c, d;
+    asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "l"(TW + i));
+  }
   pdl_wait();
   const int stepidx = nsteps ? *step : 0;
   if (tid < RB) {
@@ -309,13 +315,17 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
   __syncthreads();
 
   // ---- P0: packed spectra and the terms of the x-means
+  double2 v[6];                     // a thread's item, kept where it has only one
+  const bool once = RB * L <= T;
+  auto load_item = [&](int r, int m) {
+    const double* z = zrow(r);
+#pragma unroll
+    for (int f = 0; f < 6; ++f) v[f] = ld(z, f, m);
+  };
   for (int i = tid; i < RB * L; i += T) {
     const int r = i / L, m = i - r * L;
     if (!meta[r].act) continue;
-    const double* z = zrow(r);
-    double2 v[6];
-#pragma unroll
-    for (int f = 0; f < 6; ++f) v[f] = ld(z, f, m);
+    load_item(r, m);
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       int e = max(fx::hi_abs(v[f].x), fx::hi_abs(v[f].y)) >> 20;
@@ -335,15 +345,14 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
   for (int i = tid; i < RB * L; i += T) {
     const int r = i / L, m = i - r * L;
     if (!meta[r].act) continue;
-    const double* z = zrow(r);
+    if (!once) load_item(r, m);
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
-      const double2 v = ld(z, f, m);
       const int em = meta[r].emax[f];
       unsigned t = 0;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        const double x = c ? v.y : v.x;
+        const double x = c ? v[f].y : v[f].x;
         const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
         t += (((unsigned)(hi & 0xfffff) | 0x100000u) >> min(em - e + 4, 31)) + 1u;
       }
@@ -376,14 +385,14 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
   for (int i = tid; i < RB * L; i += T) {
     const int r = i / L, m = i - r * L;
     if (!meta[r].act) continue;
-    const double* z = zrow(r);
+    if (!once) load_item(r, m);
     C* c = Cb(r);
     C* d = Db(r);
     int E[6];
     exponents(r, E);
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
-      const double2 a = ld(z, 2 * p, m), b = ld(z, 2 * p + 1, m);
+      const double2 a = v[2 * p], b = v[2 * p + 1];
       const i64 ax = fx::from_double<59>(a.x, E[2 * p] + 1022), ay = fx::from_double<59>(a.y, E[2 * p] + 1022);
       const i64 bx = fx::from_double<59>(b.x, E[2 * p + 1] + 1022), by = fx::from_double<59>(b.y, E[2 * p + 1] + 1022);
       c[p * L + m] = make_longlong2(ax - by, ay + bx);
@@ -662,7 +671,7 @@ template <int L> RowsShape rows_shape(const Work& w, int nrows) {
     while (rb > 1 && (long)nrows < 2L * 152 * rb) rb /= 2;
   // threads for the other passes' items too: a row alone has 9 R M2 in its first
   // pass and unpacks L modes.  With few rows per SM they shorten its chain (256 x 64,
-  // one state 29.0 -> 24.8 us; 512 x 128, 3 states 59.6 -> 47.9 us); with more the
+  // one state 29.0 -> 24.6 us; 512 x 128, 3 states 59.6 -> 48 us); with more the
   // rows hide each other's (512 x 128, 16 states 226 us either way), except at
   // L = 512, where shared memory holds two (1024 x 256, 8 states 684 -> 561 us).
   const int items = rb > 1 ? rb * 9 * P::R * P::M2 : std::max(9 * P::R * P::M2, L + 32);
