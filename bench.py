@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "44402ecaddc0dccc236be580331677e986e7aa4de25b57b131975c1b2ab39fa9"
+NCU_TRAFFIC_SHA256 = "68d748b1607440b3a638a3ee8950820a45c61811f29c16a12ed21edb4d445e2b"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 141773, "coarse:k_rows": 386509, "coarse:k_zfwd": 123200, "coarse:k_solve": 802432,
-    "fine:k_zinv@32": 10430771, "fine:k_rows@32": 37885747, "fine:k_zfwd@32": 12628864, "fine:k_solve@32": 23856704,
-    "fine:k_zinv@2": 673792, "fine:k_rows@2": 2490675, "fine:k_zfwd@2": 830016, "fine:k_solve@2": 2764608,
+    "coarse:k_zinv": 143514, "coarse:k_rows": 388147, "coarse:k_zfwd": 123456, "coarse:k_solve": 802816,
+    "fine:k_zinv@32": 9590067, "fine:k_rows@32": 37881856, "fine:k_zfwd@32": 12628608, "fine:k_solve@32": 23861888,
+    "fine:k_zinv@2": 677990, "fine:k_rows@2": 2492314, "fine:k_zfwd@2": 830272, "fine:k_solve@2": 2763648,
 }
 
 

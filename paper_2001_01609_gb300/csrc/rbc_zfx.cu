@@ -14,8 +14,8 @@
 // Bound: integer issue, 13 clocks of a sub-partition per term and warp (12 of
 // them the multiply-adds) against 64 for an FP64 multiply-add.
 // Measured (GB300, per launch, FP64 sums before): inverse, 256 x 64, 32 states
-// 301 -> 121 us, 8 states 82 -> 41 us, one state 40 -> 15 us; 512 x 128, 3 states
-// 215 -> 95 us; 64 x 32, 23 states 26.5 -> 16.5 us.  Forward: 100 -> 38 us,
+// 301 -> 116 us, 8 states 82 -> 39 us, one state 40 -> 14 us; 512 x 128, 3 states
+// 215 -> 89 us; 64 x 32, 23 states 26.5 -> 16.5 us.  Forward: 100 -> 38 us,
 // 30 -> 16.5 us, 12.4 -> 10.3 us, 83 -> 33 us, 10.8 -> 9.4 us.  (128 x 32, one
 // state: 13.3 -> 10.3 and 9.3 -> 8.3 us, of which about 7 are the launch as timed.)
 // Against 64-bit plain torch the temperature after a few steps is 2 to 3 times
@@ -99,7 +99,7 @@ __device__ __forceinline__ void zinv_block(const Grid& g, const int2* __restrict
   const size_t xs = (size_t)g.nm * 2;                                       // coefficient stride
   const double* x0 = Xb + (NQ == 4 ? g.Nz * xs : 0) + (size_t)2 * (valid ? m : 0) + c;
   constexpr int JW = KS == 1 ? 2 : 1;                                       // row pairs per warp
-  int2* XS = reinterpret_cast<int2*>(zsm);                                  // [chunk][NQ][32]
+  int4* XS = reinterpret_cast<int4*>(zsm);                                  // [chunk][NQ / 2][32], two operators each
   i64* part = reinterpret_cast<i64*>(zsm + (size_t)chunk * NQ * kCols * sizeof(int2));   // [8][NQ][32], KS > 1
   // Table rows of the warp's JW row pairs, up to kSub entries at a time, on
   // their way through registers while the entries before them are summed.
@@ -158,34 +158,38 @@ __device__ __forceinline__ void zinv_block(const Grid& g, const int2* __restrict
 #pragma unroll 2
     for (int i = i0 + warp; i < i1; i += kWarps) {
       const int p = i / Kp, n = 2 * (i - p * Kp) + p;
-      int2* dst = XS + (size_t)(i - i0) * NQ * kCols + lane;
+      int4* dst = XS + (size_t)(i - i0) * (NQ / 2) * kCols + lane;
       const double v = valid && n < g.Nz ? __ldg(x0 + n * xs) : 0.0;
       const int4 gq = __ldg(gexp + (n < g.Nz ? n : 0));
       const int gs[4] = {gq.x, gq.y, gq.z, gq.w};
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) dst[q * kCols] = halves30(fx::from_double<60>(v, ec[q] - gs[q]));
+      for (int h = 0; h < NQ / 2; ++h) {
+        const int2 a = halves30(fx::from_double<60>(v, ec[2 * h] - gs[2 * h]));
+        const int2 b = halves30(fx::from_double<60>(v, ec[2 * h + 1] - gs[2 * h + 1]));
+        dst[h * kCols] = make_int4(a.x, a.y, b.x, b.y);
+      }
     }
   };
   // one group of eight terms, entries e0 .. e0 + 7 of arow against staged columns x0s ..
   auto group = [&](int e0, int x0s, i64 (*hi)[NQ]) {
-    const int2* x = XS + (size_t)x0s * NQ * kCols + lane;
+    const int4* x = XS + (size_t)x0s * (NQ / 2) * kCols + lane;
     i64 mid[JW][NQ];
 #pragma unroll
     for (int r = 0; r < JW; ++r)
 #pragma unroll
       for (int q = 0; q < NQ; ++q) mid[r][q] = kHalf;
-#pragma unroll 4
-    for (int e = 0; e < kGroup; ++e) {
-      int2 xv[NQ];
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) xv[q] = x[(e * NQ + q) * kCols];
+    for (int e = 0; e < kGroup; ++e) {
+      int4 xv[NQ / 2];
+#pragma unroll
+      for (int h = 0; h < NQ / 2; ++h) xv[h] = x[(e * (NQ / 2) + h) * kCols];
 #pragma unroll
       for (int r = 0; r < JW; ++r)
 #pragma unroll
         for (int h = 0; h < NQ / 2; ++h) {
-          const int4 v = arow[(r * kSub + e0 + e) * (NQ / 2) + h];
-          mac30(make_int2(v.x, v.y), xv[2 * h], hi[r][2 * h], mid[r][2 * h]);
-          mac30(make_int2(v.z, v.w), xv[2 * h + 1], hi[r][2 * h + 1], mid[r][2 * h + 1]);
+          const int4 v = arow[(r * kSub + e0 + e) * (NQ / 2) + h], w = xv[h];
+          mac30(make_int2(v.x, v.y), make_int2(w.x, w.y), hi[r][2 * h], mid[r][2 * h]);
+          mac30(make_int2(v.z, v.w), make_int2(w.z, w.w), hi[r][2 * h + 1], mid[r][2 * h + 1]);
         }
     }
 #pragma unroll
