@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "68d748b1607440b3a638a3ee8950820a45c61811f29c16a12ed21edb4d445e2b"
+NCU_TRAFFIC_SHA256 = "f417f48b8d134202b5215ab53aa969a8f28ed60e4ad65f9b2729a128b2f29b85"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 143514, "coarse:k_rows": 388147, "coarse:k_zfwd": 123456, "coarse:k_solve": 802816,
-    "fine:k_zinv@32": 9590067, "fine:k_rows@32": 37881856, "fine:k_zfwd@32": 12628608, "fine:k_solve@32": 23861888,
-    "fine:k_zinv@2": 677990, "fine:k_rows@2": 2492314, "fine:k_zfwd@2": 830272, "fine:k_solve@2": 2763648,
+    "coarse:k_zinv": 143565, "coarse:k_rows": 386918, "coarse:k_zfwd": 125056, "coarse:k_solve": 803328,
+    "fine:k_zinv@32": 9585357, "fine:k_rows@32": 37886003, "fine:k_zfwd@32": 12636416, "fine:k_solve@32": 23856064,
+    "fine:k_zinv@2": 675123, "fine:k_rows@2": 2491290, "fine:k_zfwd@2": 830016, "fine:k_solve@2": 2763456,
 }
 
 

@@ -458,13 +458,14 @@ static size_t zfwd_smem(const Grid& g, int B, size_t es) {
 // a third solves the mean flow of the tile that holds mode 0.  The temperature's
 // and the second system's values share one array of nq + 2 rows of 2 tms doubles:
 // row i of the latter lies two rows lower, in rows that phase 1, going up, has
-// read.  A second array holds r_i.
+// read.  A second array, or (RG) this stage's accumulator, which phase 1 has read,
+// holds r_i.
 //
 // Bound: the FP64 pipe (2 operations per clock and SM) when blocks fill it, else
 // the recurrences: ten dependent warp instructions of 64 clocks per row.
 // Measured (GB300, per launch; before, all rows' factors from L2 by the recurring
 // warp, three arrays and 256 threads of 125 registers, two blocks per SM; same
-// bits): 1024 x 256, 32 states 1650 -> 1117 us, one state 240 -> 103 us; 512 x 128,
+// bits): 1024 x 256, 32 states 1650 -> 1042 us, one state 240 -> 103 us; 512 x 128,
 // 64 states 810 -> 515 us; 256 x 64, 8 states 83 -> 42 us, one state 37 -> 28 us.
 // ---------------------------------------------------------------------------
 enum { KT = 0, KP = 1, KU = 2 };
@@ -576,8 +577,8 @@ __device__ __forceinline__ void solve_rhs(const Grid& g, const Tables& tb, int s
 }
 
 // phase 4 for coefficients (and tau rows) t0 .. t0 + NB - 1 of a column; row i of
-// the solution at x[i W], r_i at r[i W]
-template <int KIND, int NB>
+// the solution at x[i W], r_i at r[i W] or (RG) in the accumulator of this stage
+template <int KIND, int NB, bool RG>
 __device__ __forceinline__ bool solve_lx(const Grid& g, const Tables& tb, int stage, const SolveCol& k, int t0,
                                          const double* x, const double* r) {
   using SY = Sys<KIND>;
@@ -586,13 +587,15 @@ __device__ __forceinline__ bool solve_lx(const Grid& g, const Tables& tb, int st
   const int f = (KIND == KT) ? 0 : 1;
   const size_t rs = soff(g, 0, 2, 0);
   const size_t o0 = soff(g, f, 2 * t0 + k.p, k.m) + k.c;
-  double xw[NW], Rl[NB][3];
+  double xw[NW], Rl[NB][3], rg[NB];
   bool ok = true;
 #pragma unroll
-  for (int i = 0; i < NB; ++i)
+  for (int i = 0; i < NB; ++i) {
+    if (RG) rg[i] = (t0 + i < nt && stage < ns) ? k.R[(size_t)(stage - 1) * k.S + o0 + i * rs] : 0.0;
 #pragma unroll
     for (int l = 0; l < 3; ++l)
       Rl[i][l] = (t0 + i < nt && l + 2 > stage && l + 2 <= ns) ? k.R[(size_t)(l + 1) * k.S + o0 + i * rs] : 0.0;
+  }
 #pragma unroll
   for (int i = 0; i < NW; ++i) xw[i] = (t0 + i < nq) ? x[(t0 + i) * k.W + k.col] : 0.0;
 #pragma unroll
@@ -607,7 +610,7 @@ __device__ __forceinline__ bool solve_lx(const Grid& g, const Tables& tb, int st
 #pragma unroll
       for (int j = 0; j <= SY::LAM; ++j)
         if (t + j < nq) mx = fma(SY::tapM(g, tb, k.p, t, j, k.m), xw[i + j], mx);
-      const double lx2 = g.inv_gamma * (mx - r[t * k.W + k.col]);   // dt (L X_i + coupling)
+      const double lx2 = g.inv_gamma * (mx - (RG ? rg[i] : r[t * k.W + k.col]));   // dt (L X_i + coupling)
 #pragma unroll
       for (int l = 0; l < 3; ++l)
         if (l + 2 > stage && l + 2 <= ns)
@@ -829,7 +832,7 @@ __device__ __forceinline__ void nu_integral(const Grid& g, const Tables& tb, con
 constexpr int kSolveThreads = 128;
 constexpr int kSolveSmem = 140 * 1024;   // nq = 256, 16 modes
 
-template <int NB>
+template <int NB, bool RG>
 __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, double* X, double* Xs, const double* F,
                                                             double* R, size_t S, const double* wT, double* nu, int* flags,
                                                             int* err, int B, int stage, int tms, const double* ra,
@@ -862,8 +865,8 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, d
   k.S = S;
   double* y2 = sbuf;                           // psi / U: rows of W
   double* T = y2 + 2 * W;                      // T: row i where row i + 2 of psi goes
-  double* rr = T + (size_t)nq * W;             // [nq][W] r_i
-  double* ring = rr + (size_t)nq * W;          // [3] chunks of factors
+  double* rr = T + (size_t)nq * W;             // [nq][W] r_i, if not RG
+  double* ring = rr + (RG ? 0 : (size_t)nq * W);   // [3] chunks of factors
   double* bdx = ring + 3 * solve_ring(tms);    // [2][W] boundary rows
   const int rows = NB * (kSolveThreads >> lw), mine = NB * ((int)threadIdx.x >> lw);   // rows per round
   // The warps of the recurrences: blocks of an SM take different ones (those
@@ -872,13 +875,21 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, d
   const int first = (int)((blockIdx.x / 152 + blockIdx.x) & 3);
   if (stage == 1 && m0 == 0 && p == 1) nu_integral(g, tb, X0, wT, nu, b, stepidx);
 
+  // r_i of tau row t for phase 4 (the accumulator of this stage has been read)
+  auto keep_r = [&](int f, int t, double r) {
+    if (RG)
+      k.R[(size_t)(stage - 1) * S + soff(g, f, 2 * t + p, k.m) + k.c] = r;
+    else
+      rr[t * W + k.col] = r;
+  };
+
   for (int t0 = mine; t0 < nq; t0 += rows) {
     double r[NB], bv[NB];
     solve_rhs<KT, NB>(g, tb, stage, k, t0, nullptr, r, bv);
 #pragma unroll
     for (int i = 0; i < NB; ++i)
       if (t0 + i < nq - 1) {
-        rr[(t0 + i) * W + k.col] = r[i];
+        keep_r(0, t0 + i, r[i]);
         T[(t0 + i + 1) * W + k.col] = bv[i];
       }
   }
@@ -889,7 +900,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, d
     solve_helper<KT>(g, tb, p, m0, tms, T, ring, bdx);
   __syncthreads();
   bool ok = true;
-  for (int t0 = mine; t0 < nq; t0 += rows) ok = solve_lx<KT, NB>(g, tb, stage, k, t0, T, rr) && ok;
+  for (int t0 = mine; t0 < nq; t0 += rows) ok = solve_lx<KT, NB, RG>(g, tb, stage, k, t0, T, rr) && ok;
   for (int tb0 = 0; tb0 < nq; tb0 += rows) {   // every thread: the barrier below
     const int t0 = tb0 + mine;
     double r[NB], bv[NB];
@@ -902,7 +913,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, d
 #pragma unroll
     for (int i = 0; i < NB; ++i)
       if (t0 + i < nq - D) {
-        rr[(t0 + i) * W + k.col] = r[i];
+        keep_r(1, t0 + i, r[i]);
         y2[(t0 + i + D) * W + k.col] = bv[i];
       }
   }
@@ -915,7 +926,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_solve(Grid g, Tables tb, d
     solve_mean(g, tb, p, W, y2);
   __syncthreads();
   for (int t0 = mine; t0 < nq; t0 += rows)
-    ok = (k.m == 0 ? solve_lx<KU, NB>(g, tb, stage, k, t0, y2, rr) : solve_lx<KP, NB>(g, tb, stage, k, t0, y2, rr)) && ok;
+    ok = (k.m == 0 ? solve_lx<KU, NB, RG>(g, tb, stage, k, t0, y2, rr) : solve_lx<KP, NB, RG>(g, tb, stage, k, t0, y2, rr)) && ok;
   if (!ok) {
     atomicOr(flags + b, kFlagNonFinite);
     atomicOr(err, kFlagNonFinite);
@@ -1087,21 +1098,25 @@ __global__ void __launch_bounds__(kDenseThreads) k_solve_dense(Grid g, Tables tb
   }
 }
 
-// shared memory of a k_solve block: T and psi, r_i, factors, boundary rows
-static size_t solve_smem_tms(const Grid& g, int tms) {
-  return ((size_t)(2 * g.nq + 4) * 2 * tms + 3 * solve_ring(tms)) * 8;
+// shared memory of a k_solve block: T and psi, r_i (unless rg), factors, boundary rows
+static size_t solve_smem(const Grid& g, int tms, bool rg) {
+  return ((size_t)((rg ? 1 : 2) * g.nq + 4) * 2 * tms + 3 * solve_ring(tms)) * 8;
 }
+constexpr size_t kSolveFive = 44 * 1024;   // five blocks per SM
+// r_i goes to global memory where the block would not fit five times beside it
+static bool solve_rg(const Grid& g, int tms) { return tms >= 8 && solve_smem(g, tms, false) > kSolveFive; }
 // Modes per k_solve block.  Every column's arithmetic is independent of the
 // tiling.  A small batch (a coarse sweep) takes small tiles and spreads over the
 // SMs instead of leaving most of them idle; a large one the largest tile of which
-// five blocks share an SM: with 128 coefficients per parity 8 modes (1024 x 256,
-// 32 states 1117 us, 16 modes 1330), below 16 (512 x 128, 64 states 515 us against
-// 510, 256 x 64, 32 states 99 us against 102).
+// five blocks share an SM, since a recurrence costs as much for 16 columns as for
+// 32.  With 128 coefficients per parity that takes r_i out of shared memory (1024
+// x 256, 32 states: 1042 us; kept there, 1117 with 8 modes and 1330 with 16); with
+// up to 64 it fits (512 x 128, 64 states: 515 us, in global memory 523).
 static int solve_tile(const Grid& g, int B) {
   int tms = 16;
   while (tms > 1 && (long)B * 2 * ((g.nm + tms - 1) / tms) < 2L * 152) tms >>= 1;
   if (tms > g.nm) tms = g.nm;
-  while (tms > 1 && solve_smem_tms(g, tms) > 44 * 1024) tms >>= 1;
+  while (tms > 1 && solve_smem(g, tms, solve_rg(g, tms)) > kSolveFive) tms >>= 1;
   return tms;
 }
 
@@ -1117,7 +1132,7 @@ static int zfwd_nch_of(const Grid& g, const Work& w, int B, int tm) {
 }
 bool shapes_valid(const Grid& g, const Shapes& sh, size_t es) {
   if (sh.solve_tms > 0 && (sh.solve_tms > 16 || (sh.solve_tms & (sh.solve_tms - 1)) ||
-                           solve_smem_tms(g, sh.solve_tms) > 200 * 1024))
+                           solve_smem(g, sh.solve_tms, false) > 200 * 1024))
     return false;
   if (sh.zfwd_tm > 0 && (sh.zfwd_tm > 32 || (sh.zfwd_tm & (sh.zfwd_tm - 1)) ||
                          (size_t)2 * ((g.Mz + 1) / 2) * sh.zfwd_tm * 2 * es > 200 * 1024))
@@ -1242,7 +1257,7 @@ cudaError_t configure_kernels(const Grid& g) {
   if (e == cudaSuccess) e = g.mixed ? configure_rows_f32(g) : configure_rows_fx(g);
   if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
   if (e == cudaSuccess && !solve_segmented(g))
-    for (auto* fn : {k_solve<1>, k_solve<2>, k_solve<4>})
+    for (auto* fn : {k_solve<1, false>, k_solve<2, false>, k_solve<4, false>, k_solve<4, true>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmem);
   if (e == cudaSuccess)
     e = allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f);
@@ -1327,9 +1342,14 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
     // tau rows per thread and round: four share the loads of a window; fewer while
     // a round would not give every thread of the block a row
     const int items = g.nq * 2 * tms;
-    auto* kernel = dense ? k_solve_dense : items >= 4 * kSolveThreads ? k_solve<4> : items >= 2 * kSolveThreads ? k_solve<2> : k_solve<1>;
+    const bool rg = solve_rg(g, tms);
+    auto* kernel = dense                        ? k_solve_dense
+                   : rg                         ? k_solve<4, true>
+                   : items >= 4 * kSolveThreads ? k_solve<4, false>
+                   : items >= 2 * kSolveThreads ? k_solve<2, false>
+                                                : k_solve<1, false>;
     e = launch_pdl(w.pdl != 0, kernel, (unsigned)(B * 2 * mtiles), dense ? (items + 31) / 32 * 32 : kSolveThreads,
-                   dense ? 0 : solve_smem_tms(g, tms), s, g,
+                   dense ? 0 : solve_smem(g, tms, rg), s, g,
                    t, X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
   }
   if (e != cudaSuccess) return e;
