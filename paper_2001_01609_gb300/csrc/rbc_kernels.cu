@@ -196,8 +196,8 @@ __device__ __forceinline__ void zinv_store(const Grid& g, T* Zb, int j, int m, T
 }
 
 template <typename T>
-__device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
-                          T* __restrict__ Z, int B, const int* nsteps, int stepidx, int blk, int kp) {
+__device__ __forceinline__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
+                          T* __restrict__ Z, int B, const int* nsteps, const int* step, int blk, int kp) {
   using V = C2<T>;
   extern __shared__ __align__(16) unsigned char zsm[];
   V* part = reinterpret_cast<V*>(zsm);                 // [kp][12][32] when kp > 1
@@ -206,7 +206,6 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
   const int b = blk / (Mh * mt);
   const int rem = blk - b * Mh * mt;
   const int j = rem / mt, m0 = (rem - j * mt) * 32;
-  if (b >= B || !slice_active_at(nsteps, stepidx, b)) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int m = m0 + lane;
   const bool valid = m < g.nm;
@@ -219,6 +218,14 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
   const int npair = g.Nz / 2;
   const int per = (npair + kp - 1) / kp;
   const int p0 = w * per, p1 = min(npair, p0 + per);
+  if (kp > 1 && lane < 4) {   // the warp's table entries into L1 while the launch before this one finishes
+    float t;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(t) : "l"(Bz + (size_t)(lane * g.Mz + j) * g.Nz + min(2 * p0, g.Nz - 1)));
+  }
+  pdl_wait();
+  // small grids look at whether the state is active once its values are on their way
+  const int now = nsteps ? *step : 0, last = nsteps ? nsteps[b] : 1;   // (the grid is exact: b < B)
+  if (kp == 1 && now >= last) return;
   V E[6], O[6];
 #pragma unroll
   for (int q = 0; q < 6; ++q) E[q] = O[q] = mk2<T>(0, 0);
@@ -246,6 +253,7 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
       }
     }
   }
+  if (now >= last) return;   // uniform per block
   const T k = (T)(g.kfac * m);
   T* Zb = Z + (size_t)b * 9 * g.Mz * g.nm * 2;
   const int jr = g.Mz - 1 - j;
@@ -306,8 +314,7 @@ __device__ void zinv_item(const Grid& g, const T* __restrict__ Bz, const double*
 template <typename T>
 __global__ void __launch_bounds__(256) k_zinv(Grid g, const T* __restrict__ Bz, const double* __restrict__ X, size_t S,
                                               T* __restrict__ Z, int B, const int* nsteps, const int* step) {
-  pdl_wait();
-  zinv_item<T>(g, Bz, X, S, Z, B, nsteps, nsteps ? *step : 0, blockIdx.x, blockDim.x / 32);
+  zinv_item<T>(g, Bz, X, S, Z, B, nsteps, step, blockIdx.x, blockDim.x / 32);
 }
 
 // Warps sharing the coefficient sum of one k_zinv row pair.  It fixes the order
@@ -358,8 +365,8 @@ __device__ double block_sum(double v, double* red) {
 // written in FP64 for the stage solve.
 // ---------------------------------------------------------------------------
 template <typename T>
-__device__ void zfwd_item(const Grid& g, const T* __restrict__ W, const T* __restrict__ Q, double* __restrict__ F,
-                          size_t S, int B, int tm, int nch, const int* nsteps, int stepidx, int blk) {
+__device__ __forceinline__ void zfwd_item(const Grid& g, const T* __restrict__ W, const T* __restrict__ Q, double* __restrict__ F,
+                          size_t S, int B, int tm, int nch, const int* nsteps, const int* step, int blk) {
   using V = C2<T>;
   extern __shared__ __align__(16) unsigned char fsm[];
   V* fold = reinterpret_cast<V*>(fsm);                 // [2][Mh][tm]
@@ -371,7 +378,17 @@ __device__ void zfwd_item(const Grid& g, const T* __restrict__ W, const T* __res
   const int ch = rem % nch;
   rem /= nch;
   const int f = rem / mt, m0 = (rem - f * mt) * tm;
-  if (b >= B || !slice_active_at(nsteps, stepidx, b)) return;
+  const int ng = blockDim.x >> (__ffs(tm) - 1);
+  const int mi = threadIdx.x & (tm - 1), n0 = threadIdx.x / tm;
+  const int nper = (g.Nz + nch - 1) / nch;
+  const int nlo = ch * nper, nhi = min(g.Nz, nlo + nper);
+  {   // the first table row into L1 while the launch before this one finishes
+    float t;
+    const T* wr = W + (size_t)min(nlo + n0, g.Nz - 1) * g.Mz;
+    for (int jh = mi * 32; jh < Mh; jh += tm * 32) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(t) : "l"(wr + jh));
+  }
+  pdl_wait();
+  const int now = nsteps ? *step : 0, last = nsteps ? nsteps[b] : 1;   // (the grid is exact: b < B)
   const size_t qs = (size_t)g.Mz * g.nm * 2;
   const T* q = Q + (size_t)(b * 2 + f) * qs;
   const int ltm = __ffs(tm) - 1;             // tm is a power of two
@@ -392,13 +409,10 @@ __device__ void zfwd_item(const Grid& g, const T* __restrict__ W, const T* __res
     fold[(size_t)jh * tm + mi] = ev;
     fold[(size_t)(Mh + jh) * tm + mi] = od;
   }
+  if (now >= last) return;   // uniform per block
   __syncthreads();
-  const int ng = blockDim.x >> ltm;
-  const int mi = threadIdx.x & (tm - 1), n0 = threadIdx.x >> ltm;
   const int m = m0 + mi;
   if (m >= g.nm) return;
-  const int nper = (g.Nz + nch - 1) / nch;
-  const int nlo = ch * nper, nhi = min(g.Nz, nlo + nper);
   for (int n = nlo + n0; n < nhi; n += ng) {
     const V* src = fold + (size_t)((n & 1) ? Mh : 0) * tm + mi;
     const T* wr = W + (size_t)n * g.Mz;
@@ -417,8 +431,7 @@ __device__ void zfwd_item(const Grid& g, const T* __restrict__ W, const T* __res
 template <typename T>
 __global__ void k_zfwd(Grid g, const T* __restrict__ W, const T* __restrict__ Q, double* __restrict__ F, size_t S,
                        int B, int tm, int nch, const int* nsteps, const int* step) {
-  pdl_wait();
-  zfwd_item<T>(g, W, Q, F, S, B, tm, nch, nsteps, nsteps ? *step : 0, blockIdx.x);
+  zfwd_item<T>(g, W, Q, F, S, B, tm, nch, nsteps, step, blockIdx.x);
 }
 
 static int zfwd_tile(const Grid& g, int B, size_t es) {

@@ -312,9 +312,6 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
   };
   auto ld = [&](const double* z, int f, int m) { return __ldcg(reinterpret_cast<const double2*>(z + f * fs + 2 * m)); };
   auto tw = [&](int k) -> W { return __ldg(TW + k); };
-  __syncthreads();
-
-  // ---- P0: packed spectra and the terms of the x-means
   double2 v[6];                     // a thread's item, kept where it has only one
   const bool once = RB * L <= T;
   auto load_item = [&](int r, int m) {
@@ -322,10 +319,15 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
 #pragma unroll
     for (int f = 0; f < 6; ++f) v[f] = ld(z, f, m);
   };
+  // (which rows are active is looked at once the values are on their way)
+  if (once && tid < RB * L && row0 + tid / L < nrows) load_item(tid / L, tid % L);
+  __syncthreads();
+
+  // ---- P0: packed spectra and the terms of the x-means
   for (int i = tid; i < RB * L; i += T) {
     const int r = i / L, m = i - r * L;
     if (!meta[r].act) continue;
-    load_item(r, m);
+    if (!once) load_item(r, m);
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       int e = max(fx::hi_abs(v[f].x), fx::hi_abs(v[f].y)) >> 20;

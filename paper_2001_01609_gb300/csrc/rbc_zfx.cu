@@ -16,7 +16,7 @@
 // Measured (GB300, per launch, FP64 sums before): inverse, 256 x 64, 32 states
 // 301 -> 116 us, 8 states 82 -> 39 us, one state 40 -> 14 us; 512 x 128, 3 states
 // 215 -> 89 us; 64 x 32, 23 states 26.5 -> 16.5 us.  Forward: 100 -> 38 us,
-// 30 -> 16.5 us, 12.4 -> 10.3 us, 83 -> 33 us, 10.8 -> 9.4 us.  (128 x 32, one
+// 30 -> 16.4 us, 12.4 -> 10.1 us, 83 -> 33 us, 10.8 -> 9.9 us.  (128 x 32, one
 // state: 13.3 -> 10.3 and 9.3 -> 8.3 us, of which about 7 are the launch as timed.)
 // Against 64-bit plain torch the temperature after a few steps is 2 to 3 times
 // closer than with FP64 sums, psi equally close (its solve dominates).
@@ -131,7 +131,8 @@ __device__ __forceinline__ void zinv_block(const Grid& g, const int2* __restrict
   auto share = [&](int i) { return (ks & 1) * Kp + min(i + (lane / kGroup) * every + lane % kGroup, Kp - 1) - lane; };
   fetch(jb * JB + js, KS == 1 ? 0 : share(first));
   pdl_wait();
-  if (!(nsteps == nullptr || *step < *nsteps)) return;   // uniform per block
+  // (whether the state is active is looked at once its values are on their way)
+  const int now = nsteps ? *step : 0, last = nsteps ? *nsteps : 1;
   for (int i = threadIdx.x; i < NQ * kCols; i += blockDim.x) (&ecol[0][0])[i] = 0;
   __syncthreads();
   {
@@ -147,6 +148,7 @@ __device__ __forceinline__ void zinv_block(const Grid& g, const int2* __restrict
 #pragma unroll
       for (int q = 0; q < NQ; ++q) em[q] = max(em[q], e > 0 ? v + gs[q] : 0);
     }
+    if (now >= last) return;   // uniform per block
 #pragma unroll
     for (int q = 0; q < NQ; ++q) atomicMax(&ecol[q][lane], em[q]);
   }
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_zfwd_fx(Grid g, const int2* __r
   };
   fetch(first, 0);
   pdl_wait();
-  if (b >= B || !(nsteps == nullptr || *step < nsteps[b])) return;   // uniform per block
+  const int now = nsteps ? *step : 0, last = nsteps ? nsteps[b] : 1;   // (the grid is exact: b < B)
   const int m = ct * 16 + (lane >> 1), c = lane & 1;
   const bool valid = m < g.nm;
   const size_t rs = (size_t)g.nm * 2;
@@ -450,6 +452,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_zfwd_fx(Grid g, const int2* __r
     const int e = fx::biased_exp(valid ? __ldg(q + j * rs) : 0.0);
     em = max(em, e == 0x7ff ? kNaN : e);
   }
+  if (now >= last) return;   // uniform per block
   atomicMax(&ecol[lane], em);
   __syncthreads();
   em = ecol[lane];
