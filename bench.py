@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "90383648cc772b080bf52e8322667ed0c2cef5ac92d462e4c7a493681934c892"
+NCU_TRAFFIC_SHA256 = "2288949e4959f31efe31b49944241912b9de8a42b3ad559d146f23a285025a9c"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 142848, "coarse:k_rows": 387942, "coarse:k_zfwd": 123200, "coarse:k_solve": 801792,
-    "fine:k_zinv@32": 9585357, "fine:k_rows@32": 37885184, "fine:k_zfwd@32": 12628736, "fine:k_solve@32": 23864256,
-    "fine:k_zinv@2": 675072, "fine:k_rows@2": 2496717, "fine:k_zfwd@2": 829952, "fine:k_solve@2": 2763136,
+    "coarse:k_zinv": 143155, "coarse:k_rows": 388966, "coarse:k_zfwd": 123200, "coarse:k_solve": 801920,
+    "fine:k_zinv@32": 9598925, "fine:k_rows@32": 37882829, "fine:k_zfwd@32": 12628288, "fine:k_solve@32": 23858176,
+    "fine:k_zinv@2": 674816, "fine:k_rows@2": 2492160, "fine:k_zfwd@2": 834048, "fine:k_solve@2": 2764864,
 }
 
 

@@ -1,17 +1,21 @@
-// CUDA kernels of the fine/coarse propagator (FP64 path) for sm_103a.
+// CUDA kernels of the fine/coarse propagator for sm_103a.
 //
 // One RK443 stage (Sec. 3.2, Sec. 3.6) of B batched time slices is four
 // launches:
-//   k_zinv   z inverse transform: Chebyshev coefficients -> 9 fields at the
-//            3/2-padded Lobatto points, with the Fourier-mode factors ik;
-//   k_rows_* per padded z-row: packed inverse real FFTs in x, advective products,
-//            one packed forward FFT, truncation to the kept modes, x-means
-//            (rbc_rows_f32.cu, FP64: rbc_rows_fx.cu);
-//   k_zfwd   z forward transform of the products to T coefficients n < Nz;
-//   k_solve  per (slice, Fourier mode, Chebyshev parity): RK443 right-hand
-//            side in tau rows, UL banded solve of the implicit system
-//            (temperature first, then streamfunction with the implicit
-//            buoyancy coupling), RK accumulator updates, Nu_V accumulation.
+//   z inverse  Chebyshev coefficients -> fields at the 3/2-padded Lobatto points,
+//              with the Fourier-mode factors ik (FP64: rbc_zfx.cu; mixed:
+//              rbc_tcgen05.cu from Nz = 64, else k_zinv here);
+//   rows       per padded z-row: packed inverse real FFTs in x, advective products,
+//              one packed forward FFT, truncation to the kept modes, x-means
+//              (FP64: rbc_rows_fx.cu; mixed: rbc_rows_f32.cu);
+//   z forward  the products to T coefficients n < Nz (files as the inverse; k_zfwd);
+//   solve      per (slice, Fourier mode, Chebyshev parity): RK443 right-hand
+//              side in tau rows, solve of the implicit system (temperature first,
+//              then streamfunction with the implicit buoyancy coupling), RK
+//              accumulator updates, Nu_V accumulation (small grids: k_solve_dense;
+//              FP64: rbc_solve.cu; mixed: k_solve).
+// Here also: the step loop's counters, diagnostics, statistics, transfers between
+// grids, norms and the Parareal correction.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -99,16 +103,12 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 conj2(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double2 times_i(double2 a) { return make_double2(-a.y, a.x); }
-__device__ __forceinline__ bool finite2(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 
 // Complex element (f, n, m) of a state, in doubles.
 __device__ __forceinline__ size_t soff(const Grid& g, int f, int n, int m) {
   return ((size_t)(f * g.Nz + n) * g.nm + m) * 2;
 }
 
-__device__ __forceinline__ bool slice_active(const int* nsteps, const int* step, int b) {
-  return nsteps == nullptr || *step < nsteps[b];
-}
 __device__ __forceinline__ bool slice_active_at(const int* nsteps, int stepidx, int b) {
   return nsteps == nullptr || stepidx < nsteps[b];
 }
@@ -138,7 +138,6 @@ template <> __device__ __forceinline__ double2 mk2<double>(double x, double y) {
 template <> __device__ __forceinline__ float2 mk2<float>(float x, float y) { return make_float2(x, y); }
 template <typename T> __device__ __forceinline__ C2<T> ldc(const T* p) { return *reinterpret_cast<const C2<T>*>(p); }
 template <typename T> __device__ __forceinline__ void stc(T* p, C2<T> v) { *reinterpret_cast<C2<T>*>(p) = v; }
-template <typename T> __device__ __forceinline__ C2<T> ldgc(const C2<T>* p) { return __ldg(p); }
 template <typename T> __device__ __forceinline__ C2<T> cvt2(double2 a) { return mk2<T>((T)a.x, (T)a.y); }
 
 // ---------------------------------------------------------------------------
@@ -982,7 +981,7 @@ __global__ void __launch_bounds__(kDenseThreads) k_solve_dense(Grid g, Tables tb
   pdl_wait();
   const int stepidx = nsteps ? *step : 0;
   if (b >= B || !slice_active_at(nsteps, stepidx, b)) return;   // uniform per block
-  if (flags[b] & kFlagTimeout) return;                          // as in solve_item
+  if (flags[b] & kFlagTimeout) return;                          // as in k_solve
   double* X0 = X + (size_t)b * S;
   double* Xo = (stage == g.ns) ? X0 : Xs + (size_t)b * S;
   const double* Fb = F + (size_t)b * S;
@@ -1247,8 +1246,6 @@ static double zfwd_bytes(const Grid& g, int B, size_t es = 8) {
 static double solve_flops(const Grid& g, int B) { return 120.0 * B * g.nm * 2.0 * g.nq * 2.0; }
 static double solve_bytes(const Grid& g, int B) { return 8.0 * B * state_doubles(g) * 10.0; }
 
-// The dynamic shared-memory allowance of k_rows only ever grows, so that a
-// later handle on a smaller grid does not shrink it below an earlier one's need.
 // The dynamic shared-memory allowances only ever grow, so that a later handle
 // on a smaller grid does not shrink them below an earlier one's need.
 template <typename F>
@@ -1269,10 +1266,10 @@ cudaError_t configure_kernels(const Grid& g) {
   cudaError_t e = configure_zfx(g);   // also the averages of Sec. 2.2 of a mixed handle
   if (e == cudaSuccess) e = g.mixed ? configure_rows_f32(g) : configure_rows_fx(g);
   if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
-  if (e == cudaSuccess && !solve_segmented(g))
+  if (e == cudaSuccess && g.mixed && g.nq > kDenseSolveMaxNq)
     for (auto* fn : {k_solve<1, false>, k_solve<2, false>, k_solve<4, false>, k_solve<4, true>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmem);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && g.mixed)
     e = allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f);
   return e;
 }

@@ -545,9 +545,11 @@ cudaError_t configure_zfx(const Grid& g) {
   allow(k_zinv_fx<1>, kZinvSmem);
   allow(k_zinv_fx<2>, kZinvSmem);
   allow(k_zinv_fx<4>, kZinvSmem);
-  allow(k_zfwd_fx<1>, kZfwdSmem);
-  allow(k_zfwd_fx<2>, kZfwdSmem);
-  allow(k_zfwd_fx<4>, kZfwdSmem);
+  if (!g.mixed) {
+    allow(k_zfwd_fx<1>, kZfwdSmem);
+    allow(k_zfwd_fx<2>, kZfwdSmem);
+    allow(k_zfwd_fx<4>, kZfwdSmem);
+  }
   return e;
 }
 
