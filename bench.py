@@ -146,11 +146,11 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "2288949e4959f31efe31b49944241912b9de8a42b3ad559d146f23a285025a9c"
+NCU_TRAFFIC_SHA256 = "8e467adf1e08a0b5c6ab88616c88d6fa8a39b8aa669e8d551f6a48a9848d0efe"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 143155, "coarse:k_rows": 388966, "coarse:k_zfwd": 123200, "coarse:k_solve": 801920,
-    "fine:k_zinv@32": 9598925, "fine:k_rows@32": 37882829, "fine:k_zfwd@32": 12628288, "fine:k_solve@32": 23858176,
-    "fine:k_zinv@2": 674816, "fine:k_rows@2": 2492160, "fine:k_zfwd@2": 834048, "fine:k_solve@2": 2764864,
+    "coarse:k_zinv": 143155, "coarse:k_rows": 368896, "coarse:k_zfwd": 123328, "coarse:k_solve": 803200,
+    "fine:k_zinv@32": 9588685, "fine:k_rows@32": 37884621, "fine:k_zfwd@32": 12628736, "fine:k_solve@32": 23855488,
+    "fine:k_zinv@2": 675379, "fine:k_rows@2": 2458624, "fine:k_zfwd@2": 830144, "fine:k_solve@2": 2763648,
 }
 
 

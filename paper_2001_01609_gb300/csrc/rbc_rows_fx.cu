@@ -44,7 +44,7 @@
 // same FFT costs about a tenth.  Measured (GB300, per launch, against five
 // FP64 FFTs in radix-4 passes through shared memory): 256 x 64, 32 states
 // 491 -> 108 us; 512 x 128, 3 states 207 -> 46 us; 64 x 32, 23 states
-// 41 -> 16.5 us; 128 x 32, one state 20.4 -> 16.6 us (latency: the barriers).
+// 41 -> 16.5 us; 128 x 32, one state 20.4 -> 14 us (latency: the barriers).
 // One thread keeping the points of all three inverse FFTs in registers (P2 and
 // P3 in one pass, 166 registers, C and D in a place of their own) took 127, 60,
 // 22 and 19.8 us.
@@ -271,7 +271,15 @@ struct RowMeta {
   int bits[2];      // bit lengths of the largest N_T, N_omega
 };
 
-template <int L>
+// FEW (one row per block of kFew threads, for launches of at most two blocks per
+// SM): the twiddle products before the first inverse pass and after both forward
+// passes, eight or more in a row per item otherwise, are spread over all threads
+// at the price of three barriers.  A whole stage on GB300: 128 x 32, one state
+// 29.9 -> 26.8 us, six 36.3 -> 33.6; 256 x 64, one state 55.4 -> 48.5, three 72.2 ->
+// 65.3; 64 x 32, one state 26.7 -> 25.5.
+constexpr int kFew = 288;
+
+template <int L, bool FEW>
 __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ? 2 : 1) k_rows_fx(Grid g, const W* __restrict__ TW, const double* __restrict__ rk,
                                                  const double* __restrict__ Z, double* __restrict__ Q,
                                                  double* __restrict__ wT, int nrows, int RB, const int* nsteps,
@@ -453,7 +461,35 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
         h[(u + M1 * j) * (R + 1)] = x[u];
       }
     };
-    if constexpr (P::kAlias) {
+    if constexpr (FEW) {
+      constexpr int PER = (9 * L + kFew - 1) / kFew;
+      const bool act = meta[0].act;
+      C v1[PER];
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        const int i = tid + e * kFew, pb = i / L, k = i % L, bb = pb % 3;
+        if (act && i < 9 * L) {
+          const C* c = Cb(0) + pb / 3 * L;
+          const C* d = Db(0) + pb / 3 * L;
+          v1[e] = bb == 0 ? add(c[k], d[k]) : cmul2c(c[k], tw(k * bb), d[k], tw(k * bb + (3 - bb) * L));
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < PER; ++e) {
+        const int i = tid + e * kFew, pb = i / L, k = i % L;
+        if (act && i < 9 * L) Hb(0)[pb * FS + k % R + k / R * (R + 1)] = v1[e];
+      }
+      __syncthreads();
+      if (act && tid < 9 * R) {
+        C* h = Hb(0) + tid / R * FS + tid % R;
+#pragma unroll
+        for (int a = 0; a < M1; ++a) x[a] = h[a * (R + 1)];
+        dft<M1, 1>(x);
+#pragma unroll
+        for (int u = 0; u < M1; ++u) h[u * (R + 1)] = x[u];
+      }
+    } else if constexpr (P::kAlias) {
       item(tid);
       const bool on = tid < RB * 9 * R && meta[min(r, RB - 1)].act;
       if (on) gather();
@@ -568,7 +604,15 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
     if (on) {
       dft<R, -1>(x);
 #pragma unroll
-      for (int s = 0; s < R; ++s) h[s] = cmulw<false, P::kSH>(x[s], tw(3 * s * q));
+      for (int s = 0; s < R; ++s) h[s] = FEW ? x[s] : cmulw<false, P::kSH>(x[s], tw(3 * s * q));
+    }
+  }
+  if constexpr (FEW) {
+    __syncthreads();
+    for (int i = tid; i < 3 * L && meta[0].act; i += kFew) {
+      const int b = i / L, q = i % L / R, s = i % R;
+      C* h = Hb(0) + b * FS + q * (R + 1) + s;
+      *h = cmulw<false, P::kSH>(*h, tw(3 * s * q));
     }
   }
   if (P::kSum2 > 1) tree(s2, P::kSum2, s3, P::kSum3);
@@ -603,7 +647,15 @@ __global__ void __launch_bounds__(Plan<L>::kAlias ? 320 : 384, Plan<L>::kAlias ?
     dft<M1, -1>(x);
 #pragma unroll
     for (int a = 0; a < M1; ++a)
-      h[a * (R + 1)] = cmulw<false, P::kSH>(x[a], tw((R * (M2 * a + j) + s) * b));
+      h[a * (R + 1)] = FEW ? x[a] : cmulw<false, P::kSH>(x[a], tw((R * (M2 * a + j) + s) * b));
+  }
+  if constexpr (FEW) {
+    __syncthreads();
+    for (int i = tid; i < 3 * L && meta[0].act; i += kFew) {
+      const int b = i / L, k = i % L;
+      C* h = Hb(0) + b * FS + k % R + k / R * (R + 1);
+      *h = cmulw<false, P::kSH>(*h, tw(k * b));
+    }
   }
   __syncthreads();
 
@@ -672,8 +724,8 @@ template <int L> RowsShape rows_shape(const Work& w, int nrows) {
   else if (form < 0)
     while (rb > 1 && (long)nrows < 2L * 152 * rb) rb /= 2;
   // threads for the other passes' items too: a row alone has 9 R M2 in its first
-  // pass and unpacks L modes.  With few rows per SM they shorten its chain (256 x 64,
-  // one state 29.0 -> 24.6 us; 512 x 128, 3 states 59.6 -> 48 us); with more the
+  // pass and unpacks L modes.  With few rows per SM they shorten its chain (512 x 128,
+  // 3 states 59.6 -> 48 us; up to L = 128 two rows per SM take FEW); with more the
   // rows hide each other's (512 x 128, 16 states 226 us either way), except at
   // L = 512, where shared memory holds two (1024 x 256, 8 states 684 -> 561 us).
   const int items = rb > 1 ? rb * 9 * P::R * P::M2 : std::max(9 * P::R * P::M2, L + 32);
@@ -682,17 +734,28 @@ template <int L> RowsShape rows_shape(const Work& w, int nrows) {
   return {rb, th, rb * P::row_bytes};
 }
 
+// FEW for rows of 96 to 384 points (one first pass)
+template <int L> constexpr bool kHasFew = Plan<L>::kAlias && L >= 32;
+
 template <int L> cudaError_t launch_rows_L(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s) {
   const int nrows = B * g.Mz;
   const RowsShape sh = rows_shape<L>(w, nrows);
-  return launch_pdl(w.pdl != 0, k_rows_fx<L>, (unsigned)((nrows + sh.rb - 1) / sh.rb), sh.threads, sh.smem, s, g, t.twfx,
+  if constexpr (kHasFew<L>)
+    if (sh.rb == 1 && nrows <= 2 * 152)
+      return launch_pdl(w.pdl != 0, k_rows_fx<L, true>, (unsigned)nrows, kFew, sh.smem, s, g, t.twfx, t.rk, w.Z, w.Q, w.wT,
+                        nrows, 1, ns, w.step);
+  return launch_pdl(w.pdl != 0, k_rows_fx<L, false>, (unsigned)((nrows + sh.rb - 1) / sh.rb), sh.threads, sh.smem, s, g, t.twfx,
                     t.rk, w.Z, w.Q, w.wT, nrows, sh.rb, ns, w.step);
 }
 
 template <int L> cudaError_t allow_rows_L() {
   // up to 100 KB of rows per block, or one row where that is more
   const size_t need = std::max<size_t>(100 * 1024, Plan<L>::row_bytes);
-  return cudaFuncSetAttribute(k_rows_fx<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+  if constexpr (kHasFew<L>) {
+    const cudaError_t e = cudaFuncSetAttribute(k_rows_fx<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaFuncSetAttribute(k_rows_fx<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
 }
 
 }  // namespace

@@ -74,10 +74,11 @@ def test_column_lengths_match_oracle_and_batches_agree(rbc, Nz, Nx=8):
     assert F.check_diverged() == rbc.RBC_OK
 
 
+@pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("Nx", [4, 8, 16, 32, 64, 128, 256, 512, 1024])
-def test_mixed_rows_alone_and_in_batches_agree(rbc, Nx, Nz=10):
+def test_rows_alone_and_in_batches_agree(rbc, Nx, precision, Nz=10):
     """15 rows (one per block, every pass spread), 345 and 2250 rows (several per block, a ragged last one)."""
-    F = rbc.Propagator(1e5, 1.0, 2.0, Nx, Nz, 1e-4, 1)
+    F = rbc.Propagator(1e5, 1.0, 2.0, Nx, Nz, 1e-4, precision)
     o = RBC(1e5, 1.0, 2.0, Nx, Nz, 1e-4)
     alone = F.new_states(1)
     alone[0].copy_(torch.from_numpy(to_abi(nonlinear_state(o, 5))))
