@@ -139,18 +139,15 @@ class Clocks:
 # sources are those that were captured.
 NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_kernels.cu",
-    "paper_2001_01609_gb300/csrc/rbc_rows_fx.cu",
-    "paper_2001_01609_gb300/csrc/rbc_rows_f32.cu",
-    "paper_2001_01609_gb300/csrc/rbc_zfx.cu",
+    "paper_2001_01609_gb300/csrc/rbc_rows_f64.cu",
     "paper_2001_01609_gb300/csrc/rbc_solve.cu",
-    "paper_2001_01609_gb300/csrc/rbc_fx.cuh",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "8e467adf1e08a0b5c6ab88616c88d6fa8a39b8aa669e8d551f6a48a9848d0efe"
+NCU_TRAFFIC_SHA256 = "03295c7e7e7714a4a67836c25e095dbd06f7ab5271493b549abd87e0f0f682bb"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 143155, "coarse:k_rows": 368896, "coarse:k_zfwd": 123328, "coarse:k_solve": 803200,
-    "fine:k_zinv@32": 9588685, "fine:k_rows@32": 37884621, "fine:k_zfwd@32": 12628736, "fine:k_solve@32": 23855488,
-    "fine:k_zinv@2": 675379, "fine:k_rows@2": 2458624, "fine:k_zfwd@2": 830144, "fine:k_solve@2": 2763648,
+    "coarse:k_zinv": 128666, "coarse:k_rows": 483430, "coarse:k_zfwd": 119552, "coarse:k_solve": 802112,
+    "fine:k_zinv@32": 8569754, "fine:k_rows@32": 56721408, "fine:k_zfwd@32": 12623296, "fine:k_solve@32": 23862400,
+    "fine:k_zinv@2": 661811, "fine:k_rows@2": 3584307, "fine:k_zfwd@2": 821312, "fine:k_solve@2": 2763904,
 }
 
 
@@ -450,7 +447,7 @@ def run_gb300(args, w):
                                        sampled_launches=v["launches"])
     dom = max(kern, key=lambda k: kern[k]["ms"])
     pk = kern[dom]
-    # FP64 work is counted against the FP64 pipe: 152 SMs x 4 FP64 flop/clk/SM x 2070 MHz
+    # FP64 work is bound by the FP64 pipe: 152 SMs x 4 FP64 flop/clk/SM x 2070 MHz
     peak_fp64 = 152 * 4 * 2070e6 / 1e12
     achieved = pk["flops_per"] / (pk["per_ms"] / 1e3) / 1e12
     total_ms = sum(v["ms"] for v in kern.values())
@@ -459,8 +456,6 @@ def run_gb300(args, w):
     traffic = ncu_traffic(dom if dom.startswith("coarse:") else f"{dom}@{kern[dom].get('sampled_batch')}")
     roofline = dict(bound="alu", achieved=achieved, peak=peak_fp64, unit="TFLOP/s", frac=achieved / peak_fp64,
                     traffic=traffic, traffic_source="ncu, one RK443 step, cold cache (profiles/)", kernel=dom, peak_source="derived: 152 SMs x 4 FP64 flop/clk/SM x 2070 MHz",
-                    note="FP64-equivalent flops; the z transforms and the row kernel compute them in 64-bit "
-                         "fixed point on the integer pipe and can exceed the FP64 peak",
                     launch_us=1e3 * pk["per_ms"], flops_per_launch=pk["flops_per"],
                     algorithmic_bytes_per_launch=pk["bytes_per"],
                     kernel_share={k: v["ms"] / total_ms for k, v in kern.items()},
@@ -498,8 +493,7 @@ def run_gb300(args, w):
                         batch=N, kernels=fine_batch, hbm_peak_gbs=hbm,
                         note="one launch per kernel covers all 32 fine slices; FP64 peak derived "
                              "(152 SMs x 4 flop/clk x 2070 MHz), HBM of measured; the batch's working "
-                             "set stays in L2, so the FP64 pipe (k_solve) and the integer pipe (the others, "
-                             "whose FP64-equivalent rate can exceed the FP64 peak), not HBM, bound them"))
+                             "set stays in L2, so the FP64 pipe, not HBM, bounds these kernels"))
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()

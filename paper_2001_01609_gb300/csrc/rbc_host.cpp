@@ -6,7 +6,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
-#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -112,71 +111,6 @@ Mat lobatto_interp(int N, const std::vector<double>& theta) {
       W[(size_t)n * N + j] = 2.0 / (N - 1) * std::cos(n * theta[j]) / (cn * cj);
     }
   return W;
-}
-
-// ---------------------------------------------------------------------------
-// Fixed-point tables (62 fractional bits), in double-double arithmetic: the
-// same integers on every host.
-// ---------------------------------------------------------------------------
-struct DD {
-  double h, l;
-};
-DD dd_fast(double a, double b) {
-  const double s = a + b;
-  return {s, b - (s - a)};
-}
-DD dd_add(DD a, DD b) {
-  const double s = a.h + b.h, t = s - a.h;
-  const double e = (a.h - (s - t)) + (b.h - t);
-  return dd_fast(s, e + (a.l + b.l));
-}
-DD dd_mul(DD a, DD b) {
-  const double p = a.h * b.h, e = std::fma(a.h, b.h, -p);
-  return dd_fast(p, e + (a.h * b.l + a.l * b.h));
-}
-DD dd_div(DD a, double b) {
-  const double q = a.h / b;
-  const double r = std::fma(-q, b, a.h) + a.l;
-  return dd_fast(q, r / b);
-}
-long long q62(DD v) {
-  const double x = std::ldexp(v.h, 62), f = std::floor(x);
-  return (long long)f + std::llround((x - f) + std::ldexp(v.l, 62));
-}
-// cos and sin of (pi / 2) rem / N, 0 <= rem <= N / 2, by the Taylor series
-void q62_octant(int rem, int N, long long* c, long long* s) {
-  const DD x = dd_div(dd_mul({1.5707963267948966, 6.123233995736766e-17}, {(double)rem, 0.0}), (double)N);
-  DD term{1.0, 0.0}, cs{0.0, 0.0}, sn{0.0, 0.0};
-  for (int k = 0; k <= 20; ++k) {   // term = x^k / k!, below 2^-70 at k = 21
-    if (k > 0) term = dd_div(dd_mul(term, x), k);
-    DD& acc = (k & 1) ? sn : cs;
-    acc = dd_add(acc, (k & 2) ? DD{-term.h, -term.l} : term);
-  }
-  *c = q62(cs);
-  *s = q62(sn);
-}
-// cos and sin of 2 pi t / N, 0 <= t < N, interleaved
-std::vector<long long> q62_circle(int N) {
-  std::vector<long long> out((size_t)2 * N), oct((size_t)2 * (N / 2 + 1), -1);   // cos >= 0 once known
-  for (int t = 0; t < N; ++t) {
-    const int quad = (int)((4LL * t) / N);
-    int rem = (int)(4LL * t - (long long)quad * N);   // angle = (pi / 2) (quad + rem / N)
-    const bool swap = 2 * rem > N;
-    if (swap) rem = N - rem;
-    long long* o = &oct[(size_t)2 * rem];
-    if (o[0] < 0) q62_octant(rem, N, o, o + 1);
-    const long long a = o[swap ? 1 : 0], b = o[swap ? 0 : 1];
-    const long long cc[4] = {a, -b, -a, b}, ss[4] = {b, a, -b, -a};
-    out[2 * t] = cc[quad];
-    out[2 * t + 1] = ss[quad];
-  }
-  return out;
-}
-// v = h 2^32 + l with |l| < 2^31, as w[0] = h, w[1] = l
-void q_halves(long long v, int* w) {
-  if ((int)v == INT32_MIN) ++v;
-  w[1] = (int)v;
-  w[0] = (int)((v - w[1]) >> 32);
 }
 
 // ---------------------------------------------------------------------------
@@ -792,6 +726,11 @@ static rbc_status upload_tables(rbc_t h) {
   Mat Wn = lobatto_interp(N, thn);
 
   if (seg) mp.clear();   // (laid out by matrix row in seg_mp)
+  // FP64 transform tables: all of them in FP64 mode, the z inverse for the averages
+  // of Sec. 2.2 in any
+  add(zinv);
+  add(g.mixed ? std::vector<double>() : zfwd);
+  add(g.mixed ? std::vector<double>() : tw);
   add(cc); add(s2); add(s4); add(mp);
   for (UlTables* t : {&uT, &uP, &uU}) {
     add(t->multB); add(t->multD); add(t->Dinv); add(t->Lb); add(t->invd);
@@ -824,31 +763,6 @@ static rbc_status upload_tables(rbc_t h) {
     add(packed);
   };
   add_f32(zinv); add_f32(zfwd); add_f32(tw);
-  {
-    // fixed-point twiddles of the FP64 mode's x FFTs and 2 / k of the x-means
-    std::vector<double> twfx(g.mixed ? 0 : (size_t)2 * g.Mx);
-    const std::vector<long long> cs = q62_circle(g.mixed ? 0 : g.Mx);
-    for (size_t t = 0; t < cs.size() / 2; ++t) {
-      int w[4];
-      q_halves(cs[2 * t], w);
-      q_halves(-cs[2 * t + 1], w + 2);
-      memcpy(&twfx[2 * t], w, sizeof(w));
-    }
-    add(twfx);
-    std::vector<double> rk(nm, 0.0);
-    for (int m = 1; m < nm; ++m) rk[m] = 2.0 / (g.kfac * m);
-    add(rk);
-  }
-  {
-    // fixed-point z transforms
-    std::vector<int> A, Ae, G, W, We;
-    zfx_build(g, zinv.data(), zfwd.data(), A, Ae, G, W, We);
-    for (const std::vector<int>* v : {&A, &Ae, &G, &W, &We}) {
-      std::vector<double> packed((v->size() + 1) / 2, 0.0);
-      memcpy(packed.data(), v->data(), v->size() * sizeof(int));
-      add(packed);
-    }
-  }
   add(Tinv); add(Pinv); add(Uinv);
   // tensor-core z-inverse operator images (mixed precision only)
   const bool tc = g.mixed && tc_zinv_supported(g);
@@ -879,6 +793,9 @@ static rbc_status upload_tables(rbc_t h) {
   const double* b = h->d_tables;
   int i = 0;
   Tables& T = h->t;
+  T.zinv = b + offs[i++];
+  T.zfwd = b + offs[i++];
+  T.tw = reinterpret_cast<const double2*>(b + offs[i++]);
   T.cc = b + offs[i++];
   T.s2 = b + offs[i++];
   T.s4 = b + offs[i++];
@@ -900,13 +817,6 @@ static rbc_status upload_tables(rbc_t h) {
   T.zinv32 = reinterpret_cast<const float*>(b + offs[i++]);
   T.zfwd32 = reinterpret_cast<const float*>(b + offs[i++]);
   T.tw32 = reinterpret_cast<const float2*>(b + offs[i++]);
-  T.twfx = reinterpret_cast<const int4*>(b + offs[i++]);
-  T.rk = b + offs[i++];
-  T.zfxA = reinterpret_cast<const int2*>(b + offs[i++]);
-  T.zfxAe = reinterpret_cast<const int*>(b + offs[i++]);
-  T.zfxG = reinterpret_cast<const int4*>(b + offs[i++]);
-  T.zfxW = reinterpret_cast<const int2*>(b + offs[i++]);
-  T.zfxWe = reinterpret_cast<const int*>(b + offs[i++]);
   T.T_inv = dense ? b + offs[i] : nullptr;
   ++i;
   T.P_inv = dense ? b + offs[i] : nullptr;

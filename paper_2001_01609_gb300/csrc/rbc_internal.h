@@ -67,14 +67,9 @@ struct SegFactors {
 // Parity-split tables are laid out [p][row][j][m] so that threads with
 // consecutive Fourier index m read consecutive addresses.
 struct Tables {
-  // z transforms of the FP64 mode (and of the Sec. 2.2 averages) in fixed point,
-  // see rbc_zfx.cu: entries as halves (h, l), h 2^30 + l; Kp, Kh: nq and
-  // ceil(Mz/2) padded to a multiple of eight, Mh = ceil(Mz/2)
-  const int2* zfxA;     // [Mh][2][Kp][4]  d^q T_n / ds^q 2^-G_q(n) at the padded points, n = 2 k + parity
-  const int* zfxAe;     // [4][Mh]         exponent of each row
-  const int4* zfxG;     // [Nz]            G_q(n), q = 0..3
-  const int2* zfxW;     // [Nz][Kh]        padded Lobatto values -> T coefficients
-  const int* zfxWe;     // [Nz]            exponent of each row
+  const double* zinv;   // [4][Mz][Nz]  d^q T_n / ds^q at the padded Lobatto points, q = 0..3
+  const double* zfwd;   // [Nz][Mz]     padded Lobatto values -> T coefficients n < Nz (FP64 mode)
+  const double2* tw;    // [Mx]         exp(-2 pi i t / Mx) (FP64 mode)
   const double* cc;     // [Mz]         Clenshaw-Curtis weights on the padded points
   const double* s2;     // [2][nq][3]   C^(2) conversion S1 S0, tau row t, columns q = t..t+2
   const double* s4;     // [2][nq][5]   C^(4) conversion S3 S2 S1 S0, columns q = t..t+4
@@ -107,10 +102,6 @@ struct Tables {
   const float* zinv32;  // [4][Mz][Nz]
   const float* zfwd32;  // [Nz][Mz]
   const float2* tw32;   // [Mx]         exp(-2 pi i t / Mx)
-  // x FFTs of the FP64 mode: the same twiddles with 62 fractional bits, each part
-  // as signed 32-bit halves (re hi, re lo, im hi, im lo; part = hi 2^32 + lo)
-  const int4* twfx;     // [Mx]
-  const double* rk;     // [nm]         2 / k_m (0 for m = 0): Parseval sums of the x-means
   // tensor-core z-inverse operands (RBC_MIXED): TF32 hi/lo images of the
   // interleaved operator rows, pre-swizzled per 128-row tile and 32-wide K-chunk
   const float *tcA_psi_hi, *tcA_psi_lo, *tcA_T_hi, *tcA_T_lo;
@@ -153,9 +144,10 @@ struct Shapes {
   int solve_tms = 0;   // Fourier modes per k_solve block (power of two, <= 16)
   int zfwd_tm = 0;     // Fourier modes per k_zfwd block (power of two, <= 32)
   int zfwd_nch = 0;    // chunks of the n range per k_zfwd block (1, 2, 4, 8)
-  int rows_cl = -1;    // 1: one row per row-kernel block, 0: as many as fill it
-  int rows_threads = 0;   // largest row-kernel block (256, 512 or 1024; FP32 uses up to 256, FP64 up to 320)
-  int rows_lean = -1;  // kept for callers that pin shapes; the row kernels have one layout
+  int rows_cl = -1;    // row kernel, FP64: 1 a cluster per row, 0 a block per row; mixed: 1 one row
+                       // per block, 0 as many as fill it
+  int rows_threads = 0;   // threads of a k_rows block (256, 512 or 1024; FP64)
+  int rows_lean = -1;  // 1: k_rows with 5 + 3 shared rows, 0: 5 + 5 (where either fits; FP64)
 };
 
 // Per-call workspace pointers (capacity >= B states).
@@ -163,7 +155,7 @@ struct Work {
   double* Xs;      // stage state, B states
   double* F;       // explicit-term coefficients, B states
   double* R;       // RK accumulators, [B][4] states (tau rows in the coefficient slots)
-  double* Z;       // z-inverse output, [B][6][Mz][nm] complex in FP64, [B][9][Mz][nm] in FP32 (mixed)
+  double* Z;       // z-inverse output, [B][9][Mz][nm] complex (FP64, or FP32 in the first half)
   double* Q;       // row-kernel output, [B][2][Mz][nm] complex (FP64 or FP32)
   double* wT;      // [B][Mz] x-mean of w T
   int* maxs;       // [1] max over nsteps, right before nsteps (copied with it)
@@ -220,9 +212,7 @@ inline cudaError_t launch_pdl(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 blo
 #define RBC_HD
 #endif
 RBC_HD inline size_t state_doubles(const Grid& g) { return (size_t)2 * g.Nz * g.nm * 2; }
-// z-inverse output: six FP64 fields (u, w, d_x omega, d_z omega, d_x T, d_z T); the nine
-// FP32 fields of the mixed mode take less
-RBC_HD inline size_t z_doubles(const Grid& g) { return (size_t)6 * g.Mz * g.nm * 2; }
+RBC_HD inline size_t z_doubles(const Grid& g) { return (size_t)9 * g.Mz * g.nm * 2; }
 RBC_HD inline size_t q_doubles(const Grid& g) { return (size_t)2 * g.Mz * g.nm * 2; }
 
 // ---- launchers (rbc_kernels.cu) ----
@@ -267,9 +257,14 @@ cudaError_t launch_correct_norm(const Grid& gf, const Grid& gc, const Tables& tf
 // row kernel of the mixed mode (rbc_rows_f32.cu)
 cudaError_t configure_rows_f32(const Grid& g);
 cudaError_t launch_rows_f32(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
-// row kernel of the FP64 mode (rbc_rows_fx.cu)
-cudaError_t configure_rows_fx(const Grid& g);
-cudaError_t launch_rows_fx(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
+// row kernel of the FP64 mode (rbc_rows_f64.cu)
+cudaError_t configure_rows_f64(const Grid& g);
+cudaError_t launch_rows_f64(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
+// shared memory of its forms: one block per row, the smaller layout of that (available
+// where the five inverse FFTs run together), a cluster per row
+size_t rows_f64_bytes(const Grid& g, bool lean);
+bool rows_f64_batched(const Grid& g);
+size_t rows_f64_cl_bytes(const Grid& g);
 // whether a launch shape can run on this grid (shared memory, threads)
 bool shapes_valid(const Grid& g, const Shapes& sh, size_t es);
 size_t static_scratch_doubles_needed(const Grid& g);
@@ -293,14 +288,6 @@ inline bool solve_segmented(const Grid& g) { return !g.mixed && g.nq > kDenseSol
 cudaError_t configure_solve_seg(const Grid& g);
 cudaError_t launch_solve_seg(const Grid& g, const Tables& t, const Work& w, double* X, int B, int stage, double* nu,
                              cudaStream_t s);
-// z transforms in fixed point (rbc_zfx.cu); diag: T in place of d_x T
-cudaError_t configure_zfx(const Grid& g);
-cudaError_t launch_zinv_fx(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
-                           bool diag, cudaStream_t s);
-cudaError_t launch_zfwd_fx(const Grid& g, const Tables& t, const Work& w, int B, cudaStream_t s);
-// tables from the FP64 matrices zinv[4][Mz][Nz] and zfwd[Nz][Mz], as ints in the layouts of Tables
-void zfx_build(const Grid& g, const double* zinv, const double* zfwd, std::vector<int>& A, std::vector<int>& Ae,
-               std::vector<int>& G, std::vector<int>& W, std::vector<int>& We);
 // tensor-core z inverse transform (rbc_tcgen05.cu)
 RBC_HD int tc_zinv_mtiles(const Grid& g, int nops);
 RBC_HD int tc_zinv_kchunks(const Grid& g);

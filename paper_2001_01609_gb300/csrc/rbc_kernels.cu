@@ -3,11 +3,11 @@
 // One RK443 stage (Sec. 3.2, Sec. 3.6) of B batched time slices is four
 // launches:
 //   z inverse  Chebyshev coefficients -> fields at the 3/2-padded Lobatto points,
-//              with the Fourier-mode factors ik (FP64: rbc_zfx.cu; mixed:
-//              rbc_tcgen05.cu from Nz = 64, else k_zinv here);
+//              with the Fourier-mode factors ik (k_zinv; mixed from Nz = 64:
+//              rbc_tcgen05.cu);
 //   rows       per padded z-row: packed inverse real FFTs in x, advective products,
 //              one packed forward FFT, truncation to the kept modes, x-means
-//              (FP64: rbc_rows_fx.cu; mixed: rbc_rows_f32.cu);
+//              (FP64: rbc_rows_f64.cu; mixed: rbc_rows_f32.cu);
 //   z forward  the products to T coefficients n < Nz (files as the inverse; k_zfwd);
 //   solve      per (slice, Fourier mode, Chebyshev parity): RK443 right-hand
 //              side in tau rows, solve of the implicit system (temperature first,
@@ -326,11 +326,6 @@ static int zinv_warps(const Grid& g) {
   while (kp < 8 && (g.Nz / 2) / (2 * kp) >= 2) kp *= 2;
   return kp;
 }
-
-// Bounds of the row-kernel shapes that rbc_set_shapes accepts (shared memory of
-// the forms its fourth and sixth values once named; the row kernels take any).
-static bool rows_batched(const Grid& g, size_t es) { return (size_t)g.Mx * 11 * 2 * es <= 200 * 1024; }
-static size_t rows_cl_bytes(const Grid& g, size_t es) { return (size_t)g.Mx * 5 * 2 * es + (size_t)2 * g.Mx * 8; }
 
 // Deterministic block sum: the fixed tree red[t] += red[t + s], s = blockDim/2
 // down to 1 (blockDim a power of two, at least 32).  Levels s >= 32 go through
@@ -1150,10 +1145,10 @@ bool shapes_valid(const Grid& g, const Shapes& sh, size_t es) {
                          (size_t)2 * ((g.Mz + 1) / 2) * sh.zfwd_tm * 2 * es > 200 * 1024))
     return false;
   if (sh.zfwd_nch > 0 && (sh.zfwd_nch > 8 || (sh.zfwd_nch & (sh.zfwd_nch - 1)))) return false;
-  if (sh.rows_cl == 1 && rows_cl_bytes(g, es) > 200 * 1024) return false;
+  if (es == 8 && sh.rows_cl == 1 && rows_f64_cl_bytes(g) > 200 * 1024) return false;
   if (sh.rows_threads != 0 && sh.rows_threads != 256 && sh.rows_threads != 512 && sh.rows_threads != 1024)
     return false;
-  if (sh.rows_lean < -1 || sh.rows_lean > 1 || (sh.rows_lean == 1 && !rows_batched(g, es))) return false;
+  if (sh.rows_lean < -1 || sh.rows_lean > 1 || (es == 8 && sh.rows_lean == 1 && !rows_f64_batched(g))) return false;
   return true;
 }
 
@@ -1226,16 +1221,14 @@ __global__ void k_l2_diff(Grid g, const double* __restrict__ gram, const double*
 
 // Algorithmic work of one launch over B slices (all active).
 static double zinv_flops(const Grid& g, int B) { return 24.0 * B * ((g.Mz + 1) / 2) * g.nm * g.Nz; }
-// (nf z-inverse fields of es-byte reals; nfft x FFTs per row)
-static double z_reals(const Grid& g, int nf) { return 2.0 * nf * g.Mz * g.nm; }
-static double zinv_bytes(const Grid& g, int B, int nf, size_t es) {
-  return 8.0 * B * state_doubles(g) + (double)es * B * z_reals(g, nf);
+static double zinv_bytes(const Grid& g, int B, size_t es) {
+  return 8.0 * B * state_doubles(g) + (double)es * B * z_doubles(g);
 }
-static double rows_flops(const Grid& g, int B, int nfft) {
-  return (double)B * g.Mz * (nfft * 5.0 * g.Mx * std::log2((double)g.Mx) + 10.0 * g.Mx);
+static double rows_flops(const Grid& g, int B) {
+  return (double)B * g.Mz * (6.0 * 5.0 * g.Mx * std::log2((double)g.Mx) + 10.0 * g.Mx);
 }
-static double rows_bytes(const Grid& g, int B, int nf, size_t es) {
-  return (double)es * B * (z_reals(g, nf) + q_doubles(g)) + 8.0 * B * g.Mz;
+static double rows_bytes(const Grid& g, int B, size_t es) {
+  return (double)es * B * (z_doubles(g) + q_doubles(g)) + 8.0 * B * g.Mz;
 }
 static double zfwd_flops(const Grid& g, int B) { return 4.0 * B * g.Nz * g.nm * ((g.Mz + 1) / 2) * 2.0; }
 static double zfwd_bytes(const Grid& g, int B, size_t es = 8) {
@@ -1262,68 +1255,66 @@ cudaError_t configure_kernels(const Grid& g) {
                                         kCorrTile * 512 * (int)sizeof(double2));
   if (l2 == cudaSuccess) l2 = cudaFuncSetAttribute(k_l2_diff, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (l2 != cudaSuccess) return l2;
-  static int a_zfwd_f = 48 * 1024;
-  cudaError_t e = configure_zfx(g);   // also the averages of Sec. 2.2 of a mixed handle
-  if (e == cudaSuccess) e = g.mixed ? configure_rows_f32(g) : configure_rows_fx(g);
+  static int a_zfwd_d = 48 * 1024, a_zfwd_f = 48 * 1024;
+  cudaError_t e = g.mixed ? configure_rows_f32(g) : configure_rows_f64(g);
   if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
   if (e == cudaSuccess && g.mixed && g.nq > kDenseSolveMaxNq)
     for (auto* fn : {k_solve<1, false>, k_solve<2, false>, k_solve<4, false>, k_solve<4, true>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmem);
-  if (e == cudaSuccess && g.mixed)
-    e = allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f);
+  if (e == cudaSuccess)
+    e = g.mixed ? allow_smem(k_zfwd<float>, (int)std::max(zfwd_smem(g, 1, 4), zfwd_smem(g, 1 << 20, 4)), a_zfwd_f)
+                : allow_smem(k_zfwd<double>, (int)std::max(zfwd_smem(g, 1, 8), zfwd_smem(g, 1 << 20, 8)), a_zfwd_d);
   return e;
 }
 
-// FP32 transforms (mixed): z inverse and row kernel.
-static void launch_transforms_f32(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
-                                  Prof* pf, cudaStream_t s) {
+// z inverse on the CUDA cores.
+template <typename T>
+static cudaError_t launch_zinv(bool pdl, const Grid& g, const T* Bz, const Work& w, const double* X, int B, const int* ns,
+                               cudaStream_t s) {
   const int kp = zinv_warps(g);
-  const unsigned zb = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
-  float* Z = reinterpret_cast<float*>(w.Z);
-  const size_t es = sizeof(float);
-  if (pf) pf->begin(RBC_KERNEL_ZINV, s);
-  if (t.tcA_psi_hi != nullptr)
-    launch_zinv_tc(g, t, w, X, B, ns, s);              // tensor cores, TF32 with split compensation
-  else
-    launch_pdl(w.pdl != 0, k_zinv<float>, zb, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * es : 0, s, g, t.zinv32, X,
-               state_doubles(g), Z, B, ns, w.step);
-  if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 9, es));
-  if (pf) pf->begin(RBC_KERNEL_ROWS, s);
-  launch_rows_f32(g, t, w, B, ns, s);
-  if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B, 6), rows_bytes(g, B, 9, es));
+  const unsigned blocks = (unsigned)(B * ((g.Mz + 1) / 2) * ((g.nm + 31) / 32));
+  return launch_pdl(pdl, k_zinv<T>, blocks, 32 * kp, kp > 1 ? (size_t)kp * 12 * 32 * 2 * sizeof(T) : 0, s, g, Bz, X,
+                    state_doubles(g), reinterpret_cast<T*>(w.Z), B, ns, w.step);
 }
 
-// FP64: the transforms and products in fixed point (three inverse FFTs and one forward).
-static void launch_transforms_f64(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
-                                  Prof* pf, cudaStream_t s) {
+// z inverse and row kernel.
+static cudaError_t launch_transforms(const Grid& g, const Tables& t, const Work& w, const double* X, int B, const int* ns,
+                                     Prof* pf, cudaStream_t s) {
+  const size_t es = g.mixed ? sizeof(float) : sizeof(double);
   if (pf) pf->begin(RBC_KERNEL_ZINV, s);
-  launch_zinv_fx(g, t, w, X, B, ns, false, s);
-  if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, 6, sizeof(double)));
+  cudaError_t e;
+  if (t.tcA_psi_hi != nullptr)
+    e = launch_zinv_tc(g, t, w, X, B, ns, s);          // tensor cores, TF32 or BF16 with split compensation
+  else
+    e = g.mixed ? launch_zinv<float>(w.pdl != 0, g, t.zinv32, w, X, B, ns, s)
+                : launch_zinv<double>(w.pdl != 0, g, t.zinv, w, X, B, ns, s);
+  if (e != cudaSuccess) return e;
+  if (pf) pf->end(RBC_KERNEL_ZINV, s, zinv_flops(g, B), zinv_bytes(g, B, es));
   if (pf) pf->begin(RBC_KERNEL_ROWS, s);
-  launch_rows_fx(g, t, w, B, ns, s);
-  if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B, 4), rows_bytes(g, B, 6, sizeof(double)));
+  e = g.mixed ? launch_rows_f32(g, t, w, B, ns, s) : launch_rows_f64(g, t, w, B, ns, s);
+  if (pf) pf->end(RBC_KERNEL_ROWS, s, rows_flops(g, B), rows_bytes(g, B, es));
+  return e;
 }
 
 cudaError_t launch_explicit(const Grid& g, const Tables& t, const Work& w, const double* X, int B, bool all_active,
                             cudaStream_t s) {
   const int* ns = all_active ? nullptr : w.nsteps;
   Prof* pf = (w.prof && w.prof->on && !all_active) ? w.prof : nullptr;
-  if (g.mixed)
-    launch_transforms_f32(g, t, w, X, B, ns, pf, s);
-  else
-    launch_transforms_f64(g, t, w, X, B, ns, pf, s);
+  const cudaError_t e = launch_transforms(g, t, w, X, B, ns, pf, s);
+  if (e != cudaSuccess) return e;
   count(2);
   return cudaGetLastError();
 }
 
-static void launch_zfwd_f32(const Grid& g, const Tables& t, const Work& w, int B, cudaStream_t s) {
-  const size_t S = state_doubles(g), es = sizeof(float);
+template <typename T>
+static cudaError_t launch_zfwd(const Grid& g, const T* W, const Work& w, int B, cudaStream_t s) {
+  const size_t S = state_doubles(g), es = sizeof(T);
   const int tm = zfwd_tm_of(g, w, B, es);
   const int mt = (g.nm + tm - 1) / tm;
   const int nch = zfwd_nch_of(g, w, B, tm);
   const size_t smem = (size_t)2 * ((g.Mz + 1) / 2) * tm * 2 * es;
-  launch_pdl(w.pdl != 0, k_zfwd<float>, (unsigned)(B * 2 * mt * nch), 128, smem, s, g, t.zfwd32,
-             reinterpret_cast<const float*>(w.Q), w.F, S, B, tm, nch, w.nsteps, w.step);
+  return launch_pdl(w.pdl != 0, k_zfwd<T>, (unsigned)(B * 2 * mt * nch), 128, smem, s, g, W,
+                    reinterpret_cast<const T*>(w.Q), w.F, S, B, tm, nch, w.nsteps, w.step);
 }
 
 cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* X, int B, int stage, double* nu,
@@ -1335,11 +1326,10 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   Prof* pf = (w.prof && w.prof->on) ? w.prof : nullptr;
   if (pf) pf->begin(RBC_KERNEL_ZFWD, s);
   if (g.mixed && t.tcW_hi[0] != nullptr)
-    launch_zfwd_tc(g, t, w, B, s);                     // tensor cores, TF32 with split compensation
-  else if (g.mixed)
-    launch_zfwd_f32(g, t, w, B, s);
+    e = launch_zfwd_tc(g, t, w, B, s);                 // tensor cores, TF32 or BF16 with split compensation
   else
-    launch_zfwd_fx(g, t, w, B, s);
+    e = g.mixed ? launch_zfwd<float>(g, t.zfwd32, w, B, s) : launch_zfwd<double>(g, t.zfwd, w, B, s);
+  if (e != cudaSuccess) return e;
   if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, g.mixed ? 4 : 8));
   if (pf) pf->begin(RBC_KERNEL_SOLVE, s);
   if (solve_segmented(g)) {
@@ -1432,7 +1422,7 @@ cudaError_t launch_nusselt(const Grid& g, const Tables& t, const Work& w, const 
 }
 
 // Consistency-check averages of Sec. 2.2, pass 1.  Z holds the FP64 z inverse
-// of every state (fields u, w, d_x omega, d_z omega, T at the padded rows).  Block per (state, padded row j): x-means by Parseval over the kept
+// of every state (fields u, w, d_x omega, d_z omega, ..., T, ... at the padded rows).  Block per (state, padded row j): x-means by Parseval over the kept
 // modes (weight 1 for m = 0, 2 otherwise; Re(a conj b) for a pair of fields):
 //   u^2 + w^2,   u.lap u = -u d_z omega + w d_x omega,   w T,
 //   (T - <T>_x)^2 (modes m >= 1),   <T>_x = Re T_0(s_j).
@@ -1441,13 +1431,13 @@ __global__ void __launch_bounds__(128) k_diag_rows(Grid g, const double* __restr
   __shared__ double red[128];
   const int b = blockIdx.x / g.Mz, j = blockIdx.x - b * g.Mz;
   const size_t fs = (size_t)g.Mz * g.nm * 2;
-  const double* zb = Z + (size_t)b * 6 * fs + (size_t)j * g.nm * 2;
+  const double* zb = Z + (size_t)b * 9 * fs + (size_t)j * g.nm * 2;
   double ke = 0.0, ep = 0.0, wt = 0.0, tv = 0.0;
   for (int m = threadIdx.x; m < g.nm; m += blockDim.x) {
     const double c = m == 0 ? 1.0 : 2.0;
     const double2 u = ld2(zb + 2 * m), w = ld2(zb + fs + 2 * m);
     const double2 dxo = ld2(zb + 2 * fs + 2 * m), dzo = ld2(zb + 3 * fs + 2 * m);
-    const double2 t = ld2(zb + 4 * fs + 2 * m);
+    const double2 t = ld2(zb + 6 * fs + 2 * m);
     ke += c * (u.x * u.x + u.y * u.y + w.x * w.x + w.y * w.y);
     ep += c * (w.x * dxo.x + w.y * dxo.y - u.x * dzo.x - u.y * dzo.y);
     wt += c * (w.x * t.x + w.y * t.y);
@@ -1463,7 +1453,7 @@ __global__ void __launch_bounds__(128) k_diag_rows(Grid g, const double* __restr
     r[g.Mz] = ep;
     r[2 * g.Mz] = wt;
     r[3 * g.Mz] = tv;
-    r[4 * g.Mz] = zb[4 * fs];
+    r[4 * g.Mz] = zb[6 * fs];
   }
 }
 
@@ -1513,7 +1503,7 @@ cudaError_t launch_diagnostics(const Grid& g, const Tables& t, const Work& w, co
                                cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   // FP64 z inverse of all states (no step mask), whatever the handle's precision
-  cudaError_t e = launch_zinv_fx(g, t, w, X, B, nullptr, true, s);
+  cudaError_t e = launch_zinv<double>(false, g, t.zinv, w, X, B, nullptr, s);
   if (e != cudaSuccess) return e;
   k_diag_rows<<<(unsigned)(B * g.Mz), 128, 0, s>>>(g, w.Z, w.Q);
   k_diag_final<<<(unsigned)B, 128, 0, s>>>(g, t.cc, X, w.Q, out);
@@ -1966,10 +1956,8 @@ static std::atomic<double*> g_static_ptr[kMaxDevices] = {};
 
 // Layout: Z, Q, the <wT>_x profile (Mz rounded up to even), then 8 doubles:
 // the three Nusselt numbers and, in the fifth, the int error bits of the call.
-// The admission bound counts nine FP64 z-inverse fields (the header's 132 Nx Nz
-// bytes), so the grids it refuses do not depend on how many the kernels keep.
 size_t static_scratch_doubles_needed(const Grid& g) {
-  return z_doubles(g) / 6 * 9 + q_doubles(g) + (size_t)((g.Mz + 1) & ~1) + 8;
+  return z_doubles(g) + q_doubles(g) + (size_t)((g.Mz + 1) & ~1) + 8;
 }
 
 cudaError_t launch_nusselt_static(const Grid& g, const Tables& t, const double* X, double* host_out3,
