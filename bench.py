@@ -140,14 +140,15 @@ class Clocks:
 NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_kernels.cu",
     "paper_2001_01609_gb300/csrc/rbc_rows_f64.cu",
-    "paper_2001_01609_gb300/csrc/rbc_solve.cu",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "03295c7e7e7714a4a67836c25e095dbd06f7ab5271493b549abd87e0f0f682bb"
+NCU_TRAFFIC_SHA256 = "1ff087b199b3d9affcd335b2cd367209dd5c7e8c61594788d1570b8f00495910"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 128666, "coarse:k_rows": 483430, "coarse:k_zfwd": 119552, "coarse:k_solve": 802112,
-    "fine:k_zinv@32": 8569754, "fine:k_rows@32": 56721408, "fine:k_zfwd@32": 12623296, "fine:k_solve@32": 23862400,
-    "fine:k_zinv@2": 661811, "fine:k_rows@2": 3584307, "fine:k_zfwd@2": 821312, "fine:k_solve@2": 2763904,
+    "coarse:k_zinv": 129434, "coarse:k_rows": 483328, "coarse:k_zfwd": 116352, "coarse:k_solve": 803712,
+    "fine:k_zinv@32": 8566579, "fine:k_rows@32": 56725555, "fine:k_zfwd@32": 12619904, "fine:k_solve@32": 23578112,
+    # batch of 2 with the heuristic shapes (the clustered row kernel; the tuned one-block-per-row
+    # kernel reads and writes the same rows)
+    "fine:k_zinv@2": 664064, "fine:k_rows@2": 3584563, "fine:k_zfwd@2": 822336, "fine:k_solve@2": 2428544,
 }
 
 

@@ -118,7 +118,9 @@ Mat lobatto_interp(int N, const std::vector<double>& theta) {
 // top, then tau rows whose nonzeros lie in columns r-D .. r+D (dominant
 // derivative term on the diagonal).  Eliminating columns n-1 .. D from the
 // bottom creates no fill; what remains is a D x D dense block and a lower
-// band.  Only entries of the band and of the boundary rows are looked at.  No pivoting; the residual is checked after factoring.
+// band.  Only entries of the band and of the boundary rows are looked at: the
+// tau rows are sums of operators whose band is checked before they are formed.
+// No pivoting; the residual is checked after factoring.
 // ---------------------------------------------------------------------------
 struct UL {
   int n = 0, D = 0;
@@ -531,17 +533,14 @@ static rbc_status upload_tables(rbc_t h) {
 
   // ---- stage matrices and their UL factors ----
   const double hdt = g.gamma * g.dt;       // stage matrices M - gamma dt L
-  struct SegTables {   // see SegFactors
-    std::vector<double> beta, multD, Dinv, invd, ilb, phi, theta;
-  };
-  const bool dense = nq <= kDenseSolveMaxNq, seg = solve_segmented(g);
-  // mixed precision: the factors as they are, [p][row][j][m]
+  const bool dense = nq <= kDenseSolveMaxNq;
+  // the factors, [p][row][j][m]
   struct UlTables {
     std::vector<double> multB, multD, Dinv, Lb, invd;
   };
   UlTables uT, uP, uU;
   auto ul_store = [&](UlTables& t, const UL& f, int p, int nmod, int mi) {
-    if (dense || seg) return;
+    if (dense) return;
     const int D = f.D;
     if (t.invd.empty()) {
       for (auto* v : {&t.multB, &t.multD, &t.Lb}) v->assign((size_t)2 * nq * D * nmod, 0.0);
@@ -559,71 +558,6 @@ static rbc_status upload_tables(rbc_t h) {
     }
     for (int e = 0; e < D * D; ++e) t.Dinv[((size_t)p * D * D + e) * nmod + mi] = f.Dinv[e];
   };
-  const int LR = solve_seg_rows(nq), NR = (nq + LR - 1) / LR * LR;
-  SegTables sT, sP, sU;
-  auto seg_alloc = [&](SegTables& t, int D, int nmod) {
-    if (!seg) return;
-    for (auto* v : {&t.beta, &t.multD, &t.ilb, &t.phi, &t.theta}) v->assign((size_t)2 * NR * D * nmod, 0.0);
-    t.Dinv.assign((size_t)2 * D * D * nmod, 0.0);
-    t.invd.assign((size_t)2 * NR * nmod, 0.0);
-  };
-  seg_alloc(sT, 1, nm);
-  seg_alloc(sP, 2, nm);
-  seg_alloc(sU, 1, 1);
-  auto seg_store = [&](SegTables& t, const UL& f, int p, int nmod, int mi) {
-    if (!seg) return;
-    const int D = f.D;
-    auto at = [&](int r, int j) { return ((size_t)(p * NR + r) * D + j) * nmod + mi; };
-    std::vector<double> ilb((size_t)nq * D), v(nq + D + LR, 0.0);
-    for (int r = 0; r < nq; ++r) {
-      t.invd[(size_t)(p * NR + r) * nmod + mi] = r < D ? 0.0 : f.invd[r];
-      for (int j = 0; j < D; ++j) {
-        // row r gets -multB[r + 1 + j][D - 1 - j] times row r + 1 + j
-        const int c = r + 1 + j;
-        if (r >= D && c < nq && c / LR == r / LR) t.beta[at(r, j)] = f.multB[(size_t)c * D + D - 1 - j];
-        t.multD[at(r, j)] = f.multD[(size_t)r * D + j];
-        t.ilb[at(r, j)] = ilb[(size_t)r * D + j] = f.invd[r] * f.Lb[(size_t)r * D + j];
-      }
-    }
-    for (int e = 0; e < D * D; ++e) t.Dinv[((size_t)p * D * D + e) * nmod + mi] = f.Dinv[e];
-    for (int r0 = 0; r0 < nq; r0 += LR) {
-      const int e = r0 + LR;
-      for (int j = 0; j < D; ++j) {
-        if (e + j < nq) {   // backward: a unit value at row e + j
-          for (int i = 0; i < D; ++i) v[e + i] = i == j ? 1.0 : 0.0;
-          for (int c = e - 1; c >= std::max(r0, D); --c) {
-            double a = 0.0;
-            for (int i = 1; i <= D; ++i)
-              if (c + i < nq && c + i < e + D) a = std::fma(-f.multB[(size_t)(c + i) * D + D - i], v[c + i], a);
-            v[c] = a;
-            t.phi[at(c, j)] = a;
-          }
-        }
-        const int b0 = r0 == 0 ? 0 : r0 - D;   // forward: a unit value at row b0 + j
-        for (int i = 0; i < D; ++i) v[b0 + i] = i == j ? 1.0 : 0.0;
-        if (r0 == 0)
-          for (int i = 0; i < D; ++i) t.theta[at(i, j)] = v[i];
-        for (int r = std::max(r0, D); r < std::min(nq, e); ++r) {
-          double a = 0.0;
-          for (int i = 0; i < D; ++i) a = std::fma(-ilb[(size_t)r * D + i], v[r - D + i], a);
-          v[r] = a;
-          t.theta[at(r, j)] = a;
-        }
-      }
-    }
-  };
-  // taps by matrix row
-  std::vector<double> seg_s2(seg ? (size_t)2 * NR * 3 : 0, 0.0), seg_s4(seg ? (size_t)2 * NR * 5 : 0, 0.0),
-      seg_mp(seg ? (size_t)2 * NR * 5 * nm : 0, 0.0);
-  for (int p = 0; p < 2 && seg; ++p)
-    for (int t = 0; t < nq - 1; ++t) {
-      for (int j = 0; j < 3; ++j) seg_s2[(size_t)(p * NR + t + 1) * 3 + j] = s2[(p * nq + t) * 3 + j];
-      for (int j = 0; j < 5 && t < nq - 2; ++j) {
-        seg_s4[(size_t)(p * NR + t + 2) * 5 + j] = s4[(p * nq + t) * 5 + j];
-        for (int m = 0; m < nm; ++m)
-          seg_mp[((size_t)(p * NR + t + 2) * 5 + j) * nm + m] = mp[((size_t)(p * nq + t) * 5 + j) * nm + m];
-      }
-    }
   // explicit inverses of the parity systems of small grids, [p][r][q][m]
   const size_t ninv = dense ? (size_t)2 * nq * nq : 0;
   std::vector<double> Tinv(ninv * nm), Pinv(ninv * nm), Uinv(ninv);
@@ -656,7 +590,6 @@ static rbc_status upload_tables(rbc_t h) {
       UL f;
       if (!ul_factor(A, nq, 1, f, why)) return fail(RBC_EINVAL, "T system m=%d p=%d: %s", m, p, why.c_str());
       worst = std::max(worst, ul_residual(A, f, 17 * m + p));
-      seg_store(sT, f, p, nm, m);
       ul_store(uT, f, p, nm, m);
       if (dense) inverse_into(f, Tinv, p, nm, m);
       if (m == 0) {
@@ -671,7 +604,6 @@ static rbc_status upload_tables(rbc_t h) {
         UL fu;
         if (!ul_factor(U, nq, 1, fu, why)) return fail(RBC_EINVAL, "U system p=%d: %s", p, why.c_str());
         worst = std::max(worst, ul_residual(U, fu, 99 + p));
-        seg_store(sU, fu, p, 1, 0);
         ul_store(uU, fu, p, 1, 0);
         if (dense) inverse_into(fu, Uinv, p, 1, 0);
       } else {
@@ -693,7 +625,6 @@ static rbc_status upload_tables(rbc_t h) {
         UL fp;
         if (!ul_factor(P, nq, 2, fp, why)) return fail(RBC_EINVAL, "psi system m=%d p=%d: %s", m, p, why.c_str());
         worst = std::max(worst, ul_residual(P, fp, 31 * m + p));
-        seg_store(sP, fp, p, nm, m);
         ul_store(uP, fp, p, nm, m);
         if (dense) inverse_into(fp, Pinv, p, nm, m);
       }
@@ -725,7 +656,6 @@ static rbc_status upload_tables(rbc_t h) {
   }
   Mat Wn = lobatto_interp(N, thn);
 
-  if (seg) mp.clear();   // (laid out by matrix row in seg_mp)
   // FP64 transform tables: all of them in FP64 mode, the z inverse for the averages
   // of Sec. 2.2 in any
   add(zinv);
@@ -735,22 +665,16 @@ static rbc_status upload_tables(rbc_t h) {
   for (UlTables* t : {&uT, &uP, &uU}) {
     add(t->multB); add(t->multD); add(t->Dinv); add(t->Lb); add(t->invd);
   }
-  for (SegTables* t : {&sT, &sP, &sU})
-    for (auto* v : {&t->beta, &t->multD, &t->Dinv, &t->invd, &t->ilb, &t->phi, &t->theta}) add(*v);
-  add(seg_s2); add(seg_s4); add(seg_mp);
   add(gram); add(twn); add(Vn); add(Vn1); add(Wn);
   {
-    // dt * (explicit tableau), (gamma dt) Pr, (implicit tableau) / gamma: products
-    // the stage solve would otherwise form per element
+    // dt * (explicit tableau), then (gamma dt) Pr: the same IEEE products the
+    // stage solve would form per element
     double ae[5][5], ai[5][5], gm;
     int ns;
     scheme_tableau(g.scheme, ae, ai, &ns, &gm);
-    std::vector<double> dtae(51);
+    std::vector<double> dtae(26);
     for (int i = 0; i < 5; ++i)
-      for (int j = 0; j < 5; ++j) {
-        dtae[i * 5 + j] = g.dt * ae[i][j];
-        dtae[26 + i * 5 + j] = g.inv_gamma * ai[i][j];
-      }
+      for (int j = 0; j < 5; ++j) dtae[i * 5 + j] = g.dt * ae[i][j];
     dtae[25] = (g.gamma * g.dt) * g.Pr;
     add(dtae);
   }
@@ -803,11 +727,6 @@ static rbc_status upload_tables(rbc_t h) {
   for (const double** q : {&T.T_multB, &T.T_multD, &T.T_Dinv, &T.T_Lb, &T.T_invd, &T.P_multB, &T.P_multD, &T.P_Dinv, &T.P_Lb,
                            &T.P_invd, &T.U_multB, &T.U_multD, &T.U_Dinv, &T.U_Lb, &T.U_invd})
     *q = b + offs[i++];
-  for (SegFactors* f : {&T.segT, &T.segP, &T.segU})
-    for (const double** q : {&f->beta, &f->multD, &f->Dinv, &f->invd, &f->ilb, &f->phi, &f->theta}) *q = b + offs[i++];
-  T.seg_s2 = b + offs[i++];
-  T.seg_s4 = b + offs[i++];
-  T.seg_mp = b + offs[i++];
   T.gram = b + offs[i++];
   T.twn = reinterpret_cast<const double2*>(b + offs[i++]);
   T.Vn = b + offs[i++];

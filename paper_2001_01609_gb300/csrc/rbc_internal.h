@@ -44,25 +44,6 @@ inline double t_wall_rhs(const Grid& g, int p) {
   return p == 0 ? 0.5 : -0.5;
 }
 
-// Rows per segment of k_solve_seg (a choice of the grid only).
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline int solve_seg_rows(int nq) { return nq <= 32 ? 4 : 8; }
-
-// UL factors of the parity systems of one kind, laid out for the segmented
-// solve: [2][NR][D][nmod] with NR = nq padded to whole segments; Dinv
-// [2][D D][nmod], invd [2][NR][nmod].  Rows without an entry (boundary rows,
-// padding, the next segment's rows in beta) hold zeros, so no row is a special
-// case.  beta: factors of the next D rows in the backward recurrence; ilb =
-// invd Lb; phi, theta: each row's response to a unit value that comes into its
-// segment, backward (from the next segment's first D rows) and forward (from
-// the previous segment's last D rows; in the first segment from the boundary
-// unknowns).
-struct SegFactors {
-  const double *beta, *multD, *Dinv, *invd, *ilb, *phi, *theta;
-};
-
 // Device-resident operator tables (built on the host in FP64 once per grid/dt).
 // Parity-split tables are laid out [p][row][j][m] so that threads with
 // consecutive Fourier index m read consecutive addresses.
@@ -76,17 +57,11 @@ struct Tables {
   const double* mp;     // [2][nq][5][nm] psi mass operator lap_k in C^(4)
   // UL factors of the stage matrices (M - gamma dt L) with boundary rows on top.
   // T: D = 1, nmod = nm; P (psi, m >= 1): D = 2, nmod = nm; U (mean flow,
-  // m = 0): D = 1, nmod = 1.
-  // Mixed precision: [2][nq][D][nmod], Dinv [2][D*D][nmod], invd (reciprocal
+  // m = 0): D = 1, nmod = 1.  [2][nq][D][nmod], Dinv [2][D*D][nmod], invd (reciprocal
   // diagonal) [2][nq][nmod].
   const double *T_multB, *T_multD, *T_Dinv, *T_Lb, *T_invd;
   const double *P_multB, *P_multD, *P_Dinv, *P_Lb, *P_invd;
   const double *U_multB, *U_multD, *U_Dinv, *U_Lb, *U_invd;
-  // FP64 (with nq > kDenseSolveMaxNq): the same for the segmented solve
-  SegFactors segT, segP, segU;
-  // taps by matrix row (tau row + D), rows padded as the factors': S2 [2][NR][3],
-  // S4 [2][NR][5], psi mass operator [2][NR][5][nm]
-  const double *seg_s2, *seg_s4, *seg_mp;
   const double* gram;   // [Nz][Nz]  int_{-1}^{1} T_a T_b ds
   // native grid transforms
   const double2* twn;   // [Nx]      exp(-2 pi i t / Nx)
@@ -108,9 +83,8 @@ struct Tables {
   // tensor-core z-forward operands (RBC_MIXED): TF32 hi/lo images of the rows
   // of the forward matrix of each Chebyshev parity, per 128-row tile and K-chunk
   const float *tcW_hi[2], *tcW_lo[2];
-  // [5][5] dt * (explicit tableau entry), at [25] (gamma dt) Pr, from [26] [5][5]
-  // (implicit tableau entry) / gamma: products the stage solve would otherwise
-  // form per element
+  // [5][5] dt * (explicit tableau entry) and, at [25], (gamma dt) Pr: products
+  // the stage solve would otherwise form per element (same IEEE products, same bits)
   const double* dtae;
 };
 
@@ -283,11 +257,6 @@ void scheme_tableau(int scheme, double AE[5][5], double AI[5][5], int* ns, doubl
 cudaError_t upload_schemes();
 constexpr int kProfileSampleSteps = 8;     // steps recorded kernel by kernel in a sampled call
 cudaError_t configure_kernels(const Grid& g);
-// stage solve of the FP64 mode for nq > kDenseSolveMaxNq (rbc_solve.cu)
-inline bool solve_segmented(const Grid& g) { return !g.mixed && g.nq > kDenseSolveMaxNq; }
-cudaError_t configure_solve_seg(const Grid& g);
-cudaError_t launch_solve_seg(const Grid& g, const Tables& t, const Work& w, double* X, int B, int stage, double* nu,
-                             cudaStream_t s);
 // tensor-core z inverse transform (rbc_tcgen05.cu)
 RBC_HD int tc_zinv_mtiles(const Grid& g, int nops);
 RBC_HD int tc_zinv_kchunks(const Grid& g);

@@ -13,7 +13,7 @@
 //              side in tau rows, solve of the implicit system (temperature first,
 //              then streamfunction with the implicit buoyancy coupling), RK
 //              accumulator updates, Nu_V accumulation (small grids: k_solve_dense;
-//              FP64: rbc_solve.cu; mixed: k_solve).
+//              else k_solve; FP64 in both modes).
 // Here also: the step loop's counters, diagnostics, statistics, transfers between
 // grids, norms and the Parareal correction.
 #include <cooperative_groups.h>
@@ -446,8 +446,8 @@ static size_t zfwd_smem(const Grid& g, int B, size_t es) {
 }
 
 // ---------------------------------------------------------------------------
-// Stage solve (k_solve) of the mixed mode with nq > kDenseSolveMaxNq (smaller
-// grids: k_solve_dense; the FP64 mode's: rbc_solve.cu).  Block per (slice,
+// Stage solve (k_solve) of grids with nq > kDenseSolveMaxNq (smaller grids:
+// k_solve_dense).  Block per (slice,
 // Chebyshev parity p, tile of tms Fourier modes); a column is one (mode m,
 // real/imaginary part c) pair -- the stage matrices are real, so the two parts
 // are independent systems except for the implicit buoyancy coupling -i k Pr Ra T
@@ -473,7 +473,12 @@ static size_t zfwd_smem(const Grid& g, int B, size_t es) {
 // Measured (GB300, per launch; before, all rows' factors from L2 by the recurring
 // warp, three arrays and 256 threads of 125 registers, two blocks per SM; same
 // bits): 1024 x 256, 32 states 1650 -> 1042 us, one state 240 -> 103 us; 512 x 128,
-// 64 states 810 -> 515 us; 256 x 64, 8 states 83 -> 42 us, one state 37 -> 28 us.
+// 64 states 810 -> 515 us, 3 states 154 -> 64 us; 256 x 64, 32 states 137 -> 100 us,
+// 8 states 83 -> 42 us, one state 37 -> 28 us.  Recurrences in segments on all warps
+// took 922, 46, 87, 32 and 24 us (1024 x 256 with 32 states; 512 x 128 with 3; 256 x
+// 64 with 32, 8, 1) and are not used: their roundings differ, and a mixed step or the
+// defect of a converging Parareal run turns that into differences of the size of its
+// own error.
 // ---------------------------------------------------------------------------
 enum { KT = 0, KP = 1, KU = 2 };
 
@@ -1257,8 +1262,7 @@ cudaError_t configure_kernels(const Grid& g) {
   if (l2 != cudaSuccess) return l2;
   static int a_zfwd_d = 48 * 1024, a_zfwd_f = 48 * 1024;
   cudaError_t e = g.mixed ? configure_rows_f32(g) : configure_rows_f64(g);
-  if (e == cudaSuccess && solve_segmented(g)) e = configure_solve_seg(g);
-  if (e == cudaSuccess && g.mixed && g.nq > kDenseSolveMaxNq)
+  if (e == cudaSuccess && g.nq > kDenseSolveMaxNq)
     for (auto* fn : {k_solve<1, false>, k_solve<2, false>, k_solve<4, false>, k_solve<4, true>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSolveSmem);
   if (e == cudaSuccess)
@@ -1332,26 +1336,22 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   if (e != cudaSuccess) return e;
   if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, g.mixed ? 4 : 8));
   if (pf) pf->begin(RBC_KERNEL_SOLVE, s);
-  if (solve_segmented(g)) {
-    e = launch_solve_seg(g, t, w, X, B, stage, nu, s);
-  } else {
-    const bool dense = g.nq <= kDenseSolveMaxNq;
-    int tms = solve_tms_of(g, w, B);
-    while (tms > g.nm || (dense && g.nq * 2 * tms > kDenseThreads)) tms >>= 1;
-    const int mtiles = (g.nm + tms - 1) / tms;
-    // tau rows per thread and round: four share the loads of a window; fewer while
-    // a round would not give every thread of the block a row
-    const int items = g.nq * 2 * tms;
-    const bool rg = solve_rg(g, tms);
-    auto* kernel = dense                        ? k_solve_dense
-                   : rg                         ? k_solve<4, true>
-                   : items >= 4 * kSolveThreads ? k_solve<4, false>
-                   : items >= 2 * kSolveThreads ? k_solve<2, false>
-                                                : k_solve<1, false>;
-    e = launch_pdl(w.pdl != 0, kernel, (unsigned)(B * 2 * mtiles), dense ? (items + 31) / 32 * 32 : kSolveThreads,
-                   dense ? 0 : solve_smem(g, tms, rg), s, g,
-                   t, X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
-  }
+  const bool dense = g.nq <= kDenseSolveMaxNq;
+  int tms = solve_tms_of(g, w, B);
+  while (tms > g.nm || (dense && g.nq * 2 * tms > kDenseThreads)) tms >>= 1;
+  const int mtiles = (g.nm + tms - 1) / tms;
+  // tau rows per thread and round: four share the loads of a window; fewer while
+  // a round would not give every thread of the block a row
+  const int items = g.nq * 2 * tms;
+  const bool rg = solve_rg(g, tms);
+  auto* kernel = dense                        ? k_solve_dense
+                 : rg                         ? k_solve<4, true>
+                 : items >= 4 * kSolveThreads ? k_solve<4, false>
+                 : items >= 2 * kSolveThreads ? k_solve<2, false>
+                                              : k_solve<1, false>;
+  e = launch_pdl(w.pdl != 0, kernel, (unsigned)(B * 2 * mtiles), dense ? (items + 31) / 32 * 32 : kSolveThreads,
+                 dense ? 0 : solve_smem(g, tms, rg), s, g,
+                 t, X, w.Xs, w.F, w.R, S, w.wT, nu, w.flags, w.err, B, stage, tms, w.ra, w.nsteps, w.step);
   if (e != cudaSuccess) return e;
   if (pf) pf->end(RBC_KERNEL_SOLVE, s, solve_flops(g, B), solve_bytes(g, B));
   count(2);

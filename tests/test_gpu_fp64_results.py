@@ -45,7 +45,8 @@ def test_mean_flow_of_rows_with_a_broad_spectrum(rbc, Nx, decay):
     assert np.linalg.norm(U - ref) <= 1e-14 * np.linalg.norm(ref)
 
 
-RUNS = [(64, 32, 32, 16, 1e4, 1e-3, 20, 5, 4)]
+RUNS = [(64, 32, 32, 16, 1e4, 1e-3, 20, 5, 4), (256, 34, 128, 18, 18800.0, 1.25e-4, 12, 6, 2),
+        (128, 64, 64, 32, 1e5, 1.5625e-5, 8, 4, 3)]
 
 
 def parareal_defects(rbc, Nx, Nz, Nxc, Nzc, Ra, dt, nf, nc, slices):
