@@ -142,13 +142,13 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_rows_f64.cu",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "1ff087b199b3d9affcd335b2cd367209dd5c7e8c61594788d1570b8f00495910"
+NCU_TRAFFIC_SHA256 = "a6047ac8f84c8b15ebf7620e7b6b7d865fe1b92e7753e93b2b4a12d23d0977e3"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 129434, "coarse:k_rows": 483328, "coarse:k_zfwd": 116352, "coarse:k_solve": 803712,
-    "fine:k_zinv@32": 8566579, "fine:k_rows@32": 56725555, "fine:k_zfwd@32": 12619904, "fine:k_solve@32": 23578112,
+    "coarse:k_zinv": 128768, "coarse:k_rows": 483533, "coarse:k_zfwd": 116224, "coarse:k_solve": 802176,
+    "fine:k_zinv@32": 8628480, "fine:k_rows@32": 56726682, "fine:k_zfwd@32": 12619520, "fine:k_solve@32": 23583232,
     # batch of 2 with the heuristic shapes (the clustered row kernel; the tuned one-block-per-row
     # kernel reads and writes the same rows)
-    "fine:k_zinv@2": 664064, "fine:k_rows@2": 3584563, "fine:k_zfwd@2": 822336, "fine:k_solve@2": 2428544,
+    "fine:k_zinv@2": 662118, "fine:k_rows@2": 3583949, "fine:k_zfwd@2": 821120, "fine:k_solve@2": 2431744,
 }
 
 

@@ -238,6 +238,8 @@ struct DriverApi {
   CUresult (*from_green)(CUcontext*, CUgreenCtx) = nullptr;
   CUresult (*ctx_get)(CUcontext*) = nullptr;
   CUresult (*ctx_set)(CUcontext) = nullptr;
+  CUresult (*stream_green)(CUstream, CUgreenCtx*) = nullptr;
+  CUresult (*ctx_resource)(CUcontext, CUdevResource*, CUdevResourceType) = nullptr;
   bool ok = false;
 };
 
@@ -257,9 +259,27 @@ static const DriverApi& driver_api() {
            get("cuCtxFromGreenCtx", reinterpret_cast<void**>(&a.from_green)) &&
            get("cuCtxGetCurrent", reinterpret_cast<void**>(&a.ctx_get)) &&
            get("cuCtxSetCurrent", reinterpret_cast<void**>(&a.ctx_set));
+    if (!get("cuStreamGetGreenCtx", reinterpret_cast<void**>(&a.stream_green))) a.stream_green = nullptr;
+    if (!get("cuCtxGetDevResource", reinterpret_cast<void**>(&a.ctx_resource))) a.ctx_resource = nullptr;
     return a;
   }();
   return api;
+}
+
+// Whether launches on `stream` may be confined to a part of the SMs: it belongs to a
+// green context, or the current context has fewer SMs than the device (or that cannot
+// be told).
+static bool stream_confined(cudaStream_t stream) {
+  const DriverApi& d = driver_api();
+  if (!d.ok || !d.stream_green || !d.ctx_resource) return true;
+  CUgreenCtx green = nullptr;
+  CUcontext ctx = nullptr;
+  CUdevResource part{}, all{};
+  int dev = 0;
+  return d.stream_green(stream, &green) != CUDA_SUCCESS || green != nullptr || d.ctx_get(&ctx) != CUDA_SUCCESS ||
+         ctx == nullptr || d.ctx_resource(ctx, &part, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS ||
+         cudaGetDevice(&dev) != cudaSuccess || d.get_resource((CUdevice)dev, &all, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS ||
+         part.sm.smCount < all.sm.smCount;
 }
 
 // Makes `ctx` (a partition's context) current for the scope; nullptr keeps
@@ -1219,7 +1239,8 @@ extern "C" rbc_status rbc_parareal_correct(rbc_t fine, rbc_t coarse, const void*
 extern "C" rbc_status rbc_l2_diff(rbc_t h, const void* d_A, const void* d_B, int B, double* d_out,
                                   cudaStream_t stream) {
   if (!h || B < 0 || (B > 0 && (!d_A || !d_out))) return fail(RBC_EINVAL, "null argument or B < 0");
-  CK(launch_l2_diff(h->g, h->t, static_cast<const double*>(d_A), static_cast<const double*>(d_B), B, d_out, stream));
+  CK(launch_l2_diff(h->g, h->t, static_cast<const double*>(d_A), static_cast<const double*>(d_B), B, d_out,
+                    l2_large_clusters(h->g, B) && stream_confined(stream), stream));
   return RBC_OK;
 }
 
@@ -1514,7 +1535,8 @@ extern "C" rbc_status rbc_l2_temperature(rbc_t h, const void* d_state, double* o
   if (!h || !d_state || !out) return fail(RBC_EINVAL, "null argument");
   rbc_status s = rbc_reserve(h, 1);
   if (s != RBC_OK) return s;
-  CK(launch_l2_diff(h->g, h->t, static_cast<const double*>(d_state), nullptr, 1, h->w.small, stream));
+  CK(launch_l2_diff(h->g, h->t, static_cast<const double*>(d_state), nullptr, 1, h->w.small,
+                    l2_large_clusters(h->g, 1) && stream_confined(stream), stream));
   double v = 0.0;
   CK(cudaMemcpyAsync(&v, h->w.small, sizeof(double), cudaMemcpyDeviceToHost, stream));
   CK(cudaStreamSynchronize(stream));

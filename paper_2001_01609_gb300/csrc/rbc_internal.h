@@ -210,8 +210,11 @@ cudaError_t launch_diagnostics(const Grid& g, const Tables& t, const Work& w, co
 cudaError_t launch_stat_sample(const Grid& g, double* d, int B, cudaStream_t s);
 cudaError_t launch_stat_accum(double* acc, double* prev, const double* cur, double h2, long n, cudaStream_t s);
 cudaError_t launch_add(double* a, const double* b, int n, cudaStream_t s);
+// norms of nst states; confined: the stream may not have all SMs (asked where
+// l2_large_clusters, clusters of more than eight blocks, says so)
+bool l2_large_clusters(const Grid& g, int nst);
 cudaError_t launch_l2_diff(const Grid& g, const Tables& t, const double* A, const double* Bm, int nst,
-                           double* out, cudaStream_t s);
+                           double* out, bool confined, cudaStream_t s);
 cudaError_t launch_set_state(const Grid& g, const Tables& t, const double* gT, const double* gu,
                              const double* gw, double* scratch, double* X, cudaStream_t s);
 cudaError_t launch_get_state(const Grid& g, const Tables& t, const double* X, double* scratch, double* gT,

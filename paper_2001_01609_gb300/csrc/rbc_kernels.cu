@@ -1632,25 +1632,36 @@ __global__ void __launch_bounds__(kCorrThreads) k_l2_diff(Grid g, const double* 
   }
 }
 
-// Blocks per state: one per tile up to a cluster of 16, eight (the portable size)
-// from 38 states on, where 38 x 8 already makes two blocks per SM.
+// Blocks per state: one per tile up to a cluster of 16, eight from 38 states on, where
+// 38 x 8 already makes two blocks per SM.  More than eight, the portable size, only
+// where the stream has the whole GPU (not in an SM partition, `confined`); fewer where
+// the device cannot place one such cluster.  (With eight, 256 x 64, one state takes 27
+// us instead of 16.5, 1024 x 256, one state 1170 instead of 591.)
+bool l2_large_clusters(const Grid& g, int nst) { return nst < 38 && g.nm > 8 * kCorrTile; }
+
 cudaError_t launch_l2_diff(const Grid& g, const Tables& t, const double* A, const double* Bm, int nst, double* out,
-                           cudaStream_t s) {
+                           bool confined, cudaStream_t s) {
   if (nst <= 0) return cudaSuccess;
   const int tiles = (g.nm + kCorrTile - 1) / kCorrTile;
-  int ncta = 1;
-  while (2 * ncta <= std::min(tiles, nst >= 38 ? 8 : 16)) ncta *= 2;
+  int ncta = l2_large_clusters(g, nst) && !confined ? 16 : 8;
+  while (ncta > tiles) ncta /= 2;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = (unsigned)(nst * ncta);
   cfg.blockDim = kCorrThreads;
   cfg.dynamicSmemBytes = (size_t)kCorrTile * g.Nz * sizeof(double2);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)ncta;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  for (;; ncta /= 2) {
+    cfg.gridDim = (unsigned)(nst * ncta);
+    at[0].val.clusterDim.x = (unsigned)ncta;
+    int fit = 0;
+    if (ncta == 1) break;
+    if (cudaOccupancyMaxActiveClusters(&fit, k_l2_diff, &cfg) == cudaSuccess && fit > 0) break;
+    cudaGetLastError();   // (a size that the device refuses)
+  }
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_l2_diff, g, t.gram, A, Bm, out, ncta);
   count();
   return e == cudaSuccess ? cudaGetLastError() : e;

@@ -9,6 +9,8 @@ blocks of the C ABI, and the continuous-batching engine.
   slice counts, chunked fine batches, memory-limited admission) reproduces its
   solo result bitwise.
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -133,6 +135,40 @@ def test_l2_norms_of_every_cluster_size(rbc, Nx, Nz):
     bound = 2.0 ** -52 * (2 * Nz + Nx) * terms      # additions in a row, at most, on either side
     assert (abs(out[39].cpu().numpy() - ref) <= bound).all()      # Lx / 2 = 1
     assert torch.equal(out[37], out[39][:37]) and torch.equal(out[1], out[39][:1])
+
+
+@pytest.fixture
+def partition_stream():
+    """A stream confined to eight SMs (a green context), through the driver's C interface."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    torch.zeros(1, device="cuda")                       # the primary context is current
+    dev, n, desc, green, stream = ctypes.c_int(), ctypes.c_uint(1), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+    res = [(ctypes.c_ubyte * 1024)() for _ in range(3)]   # CUdevResource: the device's, the group, the rest
+    call = lambda name, *args: (name, getattr(cu, name)(*args))   # noqa: E731
+    done = [call("cuDeviceGet", ctypes.byref(dev), 0),
+            call("cuDeviceGetDevResource", dev, res[0], 1),        # 1: SMs
+            call("cuDevSmResourceSplitByCount", res[1], ctypes.byref(n), res[0], res[2], 0, 8),
+            call("cuDevResourceGenerateDesc", ctypes.byref(desc), res[1], 1)]
+    done.append(call("cuGreenCtxCreate", ctypes.byref(green), desc, dev, 1))
+    done.append(call("cuGreenCtxStreamCreate", ctypes.byref(stream), green, 1, 0))
+    assert all(status == 0 for _, status in done), done
+    yield torch.cuda.ExternalStream(stream.value)
+    torch.cuda.synchronize()
+    cu.cuStreamDestroy_v2(stream)
+    cu.cuGreenCtxDestroy(green)
+
+
+@pytest.mark.parametrize("Nx,Nz,B", [(256, 12, 1), (256, 12, 40), (1024, 512, 2), (16, 10, 3)])
+def test_l2_norms_on_a_partition_of_the_sms(rbc, partition_stream, Nx, Nz, B):
+    """Up to eight blocks per state there, 16 on the whole GPU: the same bits."""
+    F = rbc.Propagator(1e4, 1.0, 2.0, Nx, Nz, 1e-5, 0)
+    A, Bm = torch.randn((2, B) + F.state_shape, dtype=torch.float64, device="cuda")
+    whole, part = torch.zeros((2, B), dtype=torch.float64, device="cuda")
+    rbc.l2_diff(F, A, Bm, whole)
+    torch.cuda.synchronize()
+    rbc.l2_diff(F, A, Bm, part, stream=partition_stream)
+    partition_stream.synchronize()
+    assert torch.equal(whole, part) and (whole > 0).all()
 
 
 def small_classes(Nx, Nz, precision):
