@@ -142,13 +142,13 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_rows_f64.cu",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "a6047ac8f84c8b15ebf7620e7b6b7d865fe1b92e7753e93b2b4a12d23d0977e3"
+NCU_TRAFFIC_SHA256 = "ff1eeb63723cae373579ebbfe62b9b22d41d13fbcb281a2cb8e2086cb049db81"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 128768, "coarse:k_rows": 483533, "coarse:k_zfwd": 116224, "coarse:k_solve": 802176,
-    "fine:k_zinv@32": 8628480, "fine:k_rows@32": 56726682, "fine:k_zfwd@32": 12619520, "fine:k_solve@32": 23583232,
+    "coarse:k_zinv": 129229, "coarse:k_rows": 483686, "coarse:k_zfwd": 116096, "coarse:k_solve": 802368,
+    "fine:k_zinv@32": 8584294, "fine:k_rows@32": 56754278, "fine:k_zfwd@32": 12619328, "fine:k_solve@32": 23582400,
     # batch of 2 with the heuristic shapes (the clustered row kernel; the tuned one-block-per-row
     # kernel reads and writes the same rows)
-    "fine:k_zinv@2": 662118, "fine:k_rows@2": 3583949, "fine:k_zfwd@2": 821120, "fine:k_solve@2": 2431744,
+    "fine:k_zinv@2": 665344, "fine:k_rows@2": 3586970, "fine:k_zfwd@2": 820928, "fine:k_solve@2": 2428800,
 }
 
 

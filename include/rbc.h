@@ -364,17 +364,21 @@ int parareal_coarse_sms(parareal_t p);
 /* Autotuner (outside the paper's method).  rbc_autotune times, on the device,
  * RK443 steps of a batch of B states with candidate launch shapes that leave
  * every result unchanged bit for bit (modes per stage-solve block, modes and
- * n-chunks per z-forward block, rows per block of the x-FFT kernel and its
- * block size; reduction orders depend on the grid only), by a coordinate search
- * from the built-in heuristics, and keeps the fastest for batches of B states
- * on this handle (and on the library's copies of it that Parareal uses).
+ * n-chunks per z-forward block, the form of the x-FFT kernel, its block size
+ * and shared-memory layout; reduction orders depend on the grid only), by a
+ * coordinate search from the built-in heuristics, and keeps the fastest for
+ * batches of B states on this handle (and on the library's copies of it that
+ * Parareal uses).
  * out_ms (may be NULL): the time per step with the heuristics and with the
  * shapes kept.  Synchronous on `stream`; allocates B scratch states for the
  * duration of the call; RBC_EINVAL for B < 1.  rbc_tuned_shapes writes the
  * shapes kept for B (0 / -1: the heuristic) to host out[6] = (solve modes,
- * z-forward modes, z-forward chunks, rows per row-kernel block: 1 one, 0 as
- * many as fit, row-kernel threads, row-kernel layout: there is one, the value
- * is checked and kept).  rbc_set_shapes keeps the host array
+ * z-forward modes, z-forward chunks, row-kernel form: FP64 1 a cluster per row,
+ * 0 a block per row, mixed 1 one row per block, 0 as many as fit; row-kernel
+ * threads and row-kernel layout (1 lean, 0 full), of FP64 handles' block per
+ * row).  The z-forward fields act on FP64 handles and, below Nz = 64 or where
+ * the tensor-core kernel does not fit, on mixed ones; a shape without effect
+ * on a handle is neither timed nor picked.  rbc_set_shapes keeps the host array
  * in[6] (same order and meaning) for batches of B states without timing
  * anything; RBC_EINVAL if a shape is not valid for the grid (a power of two
  * up to 16 solve modes or 32 z-forward modes, 1-8 chunks, 256/512/1024 row

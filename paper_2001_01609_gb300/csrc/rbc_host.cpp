@@ -1368,9 +1368,10 @@ extern "C" rbc_status rbc_autotune(rbc_t h, int B, double out_ms[2], cudaStream_
   s = time_shapes(h, X, B, best, steps, stream, &t_best);
   if (s != RBC_OK) return s;
   const float t_heur = t_best;
-  // coordinate search: row kernel form, then z-forward tile and chunks, then solve tile
+  // coordinate search: row kernel form, then z-forward tile and chunks, then solve
+  // tile; a candidate whose launches are those of the best so far is not timed
   auto trial = [&](Shapes c) -> rbc_status {
-    if (!shapes_valid(g, c, es)) return RBC_OK;
+    if (!shapes_valid(g, c, es) || resolved_shapes(g, h->t, c, B) == resolved_shapes(g, h->t, best, B)) return RBC_OK;
     float t = 0.f;
     rbc_status r = time_shapes(h, X, B, c, steps, stream, &t);
     if (r != RBC_OK) return r;
@@ -1385,9 +1386,14 @@ extern "C" rbc_status rbc_autotune(rbc_t h, int B, double out_ms[2], cudaStream_
     c.rows_cl = cl;
     if ((s = trial(c)) != RBC_OK) return s;
   }
-  for (int th = 512; th <= 1024; th *= 2) {   // largest block of the row kernel
+  for (int th = 512; th <= 1024; th *= 2) {   // block size of the one-block-per-row kernel (FP64)
     Shapes c = best;
     c.rows_threads = th;
+    if ((s = trial(c)) != RBC_OK) return s;
+  }
+  for (int ln = 0; ln <= 1; ++ln) {             // its shared-memory layout
+    Shapes c = best;
+    c.rows_lean = ln;
     if ((s = trial(c)) != RBC_OK) return s;
   }
   for (int tm = 4; tm <= 32; tm *= 2)

@@ -122,6 +122,10 @@ struct Shapes {
                        // per block, 0 as many as fill it
   int rows_threads = 0;   // threads of a k_rows block (256, 512 or 1024; FP64)
   int rows_lean = -1;  // 1: k_rows with 5 + 3 shared rows, 0: 5 + 5 (where either fits; FP64)
+  bool operator==(const Shapes& o) const {
+    return solve_tms == o.solve_tms && zfwd_tm == o.zfwd_tm && zfwd_nch == o.zfwd_nch && rows_cl == o.rows_cl &&
+           rows_threads == o.rows_threads && rows_lean == o.rows_lean;
+  }
 };
 
 // Per-call workspace pointers (capacity >= B states).
@@ -234,14 +238,20 @@ cudaError_t launch_correct_norm(const Grid& gf, const Grid& gc, const Tables& tf
 // row kernel of the mixed mode (rbc_rows_f32.cu)
 cudaError_t configure_rows_f32(const Grid& g);
 cudaError_t launch_rows_f32(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
+int rows_f32_per_block(const Grid& g, const Shapes& sh, int B);
 // row kernel of the FP64 mode (rbc_rows_f64.cu)
 cudaError_t configure_rows_f64(const Grid& g);
 cudaError_t launch_rows_f64(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s);
+// form of a launch: cluster per row (1) or block per row (0) of so many threads and layout
+void rows_f64_form(const Grid& g, const Shapes& sh, int B, int* cl, int* threads, int* lean);
 // shared memory of its forms: one block per row, the smaller layout of that (available
 // where the five inverse FFTs run together), a cluster per row
 size_t rows_f64_bytes(const Grid& g, bool lean);
 bool rows_f64_batched(const Grid& g);
 size_t rows_f64_cl_bytes(const Grid& g);
+// what a launch of B states uses of `sh` and of the heuristics; fields without effect on
+// this grid and precision at their defaults (rows_cl of the mixed mode: rows per block)
+Shapes resolved_shapes(const Grid& g, const Tables& t, const Shapes& sh, int B);
 // whether a launch shape can run on this grid (shared memory, threads)
 bool shapes_valid(const Grid& g, const Shapes& sh, size_t es);
 size_t static_scratch_doubles_needed(const Grid& g);

@@ -1133,14 +1133,29 @@ static int solve_tile(const Grid& g, int B) {
 }
 
 // The shapes of a launch: the tuned ones where set, else the heuristics.
-static int solve_tms_of(const Grid& g, const Work& w, int B) {
-  return (w.shapes && w.shapes->solve_tms > 0) ? w.shapes->solve_tms : solve_tile(g, B);
+static int solve_tms_of(const Grid& g, const Shapes* sh, int B) {
+  int tms = (sh && sh->solve_tms > 0) ? sh->solve_tms : solve_tile(g, B);
+  while (tms > g.nm || (g.nq <= kDenseSolveMaxNq && g.nq * 2 * tms > kDenseThreads)) tms >>= 1;
+  return tms;
 }
-static int zfwd_tm_of(const Grid& g, const Work& w, int B, size_t es) {
-  return (w.shapes && w.shapes->zfwd_tm > 0) ? w.shapes->zfwd_tm : zfwd_tile(g, B, es);
+static int zfwd_tm_of(const Grid& g, const Shapes* sh, int B, size_t es) {
+  return (sh && sh->zfwd_tm > 0) ? sh->zfwd_tm : zfwd_tile(g, B, es);
 }
-static int zfwd_nch_of(const Grid& g, const Work& w, int B, int tm) {
-  return (w.shapes && w.shapes->zfwd_nch > 0) ? w.shapes->zfwd_nch : zfwd_chunks(g, B, tm);
+static int zfwd_nch_of(const Grid& g, const Shapes* sh, int B, int tm) {
+  return (sh && sh->zfwd_nch > 0) ? sh->zfwd_nch : zfwd_chunks(g, B, tm);
+}
+Shapes resolved_shapes(const Grid& g, const Tables& t, const Shapes& sh, int B) {
+  Shapes r;
+  r.solve_tms = solve_tms_of(g, &sh, B);
+  if (t.tcW_hi[0] == nullptr) {
+    r.zfwd_tm = zfwd_tm_of(g, &sh, B, g.mixed ? 4 : 8);
+    r.zfwd_nch = zfwd_nch_of(g, &sh, B, r.zfwd_tm);
+  }
+  if (g.mixed)
+    r.rows_cl = rows_f32_per_block(g, sh, B);
+  else
+    rows_f64_form(g, sh, B, &r.rows_cl, &r.rows_threads, &r.rows_lean);
+  return r;
 }
 bool shapes_valid(const Grid& g, const Shapes& sh, size_t es) {
   if (sh.solve_tms > 0 && (sh.solve_tms > 16 || (sh.solve_tms & (sh.solve_tms - 1)) ||
@@ -1313,9 +1328,9 @@ cudaError_t launch_explicit(const Grid& g, const Tables& t, const Work& w, const
 template <typename T>
 static cudaError_t launch_zfwd(const Grid& g, const T* W, const Work& w, int B, cudaStream_t s) {
   const size_t S = state_doubles(g), es = sizeof(T);
-  const int tm = zfwd_tm_of(g, w, B, es);
+  const int tm = zfwd_tm_of(g, w.shapes, B, es);
   const int mt = (g.nm + tm - 1) / tm;
-  const int nch = zfwd_nch_of(g, w, B, tm);
+  const int nch = zfwd_nch_of(g, w.shapes, B, tm);
   const size_t smem = (size_t)2 * ((g.Mz + 1) / 2) * tm * 2 * es;
   return launch_pdl(w.pdl != 0, k_zfwd<T>, (unsigned)(B * 2 * mt * nch), 128, smem, s, g, W,
                     reinterpret_cast<const T*>(w.Q), w.F, S, B, tm, nch, w.nsteps, w.step);
@@ -1337,8 +1352,7 @@ cudaError_t launch_stage(const Grid& g, const Tables& t, const Work& w, double* 
   if (pf) pf->end(RBC_KERNEL_ZFWD, s, zfwd_flops(g, B), zfwd_bytes(g, B, g.mixed ? 4 : 8));
   if (pf) pf->begin(RBC_KERNEL_SOLVE, s);
   const bool dense = g.nq <= kDenseSolveMaxNq;
-  int tms = solve_tms_of(g, w, B);
-  while (tms > g.nm || (dense && g.nq * 2 * tms > kDenseThreads)) tms >>= 1;
+  const int tms = solve_tms_of(g, w.shapes, B);
   const int mtiles = (g.nm + tms - 1) / tms;
   // tau rows per thread and round: four share the loads of a window; fewer while
   // a round would not give every thread of the block a row

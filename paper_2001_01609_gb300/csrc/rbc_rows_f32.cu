@@ -283,7 +283,6 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : 512) k_rows_f32(Grid g
   if constexpr (SPLIT) {
     for (int i = tid; i < NR * 5 * NK; i += T) {
       const int r = i / (5 * NK), i1 = i - r * 5 * NK, pr = i1 / NK, k = i1 - pr * NK;
-      if (!SPLIT && !act[r]) continue;
       C* h = H(r) + pr * FS + (k & (RA - 1)) * LD + RC * (k / RA);
       C x[RC];
 #pragma unroll
@@ -410,20 +409,22 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : 512) k_rows_f32(Grid g
 // 26.1 without; beyond, blocks of 640 threads crowd each other out.
 constexpr int kSplitRows = 2 * 152;
 
+// Rows per block: up to 256 C items and 48 KB, fewer while the launch would not
+// give every SM two blocks; a row alone takes threads for the A items too.
+template <int P> int per_block(const Shapes& sh, int nrows) {
+  using PL = Plan32<P>;
+  int nr = 1;
+  while (nr < kMaxRows && 2 * nr * PL::NK <= 256 && 2 * nr * PL::row_bytes <= 48 * 1024) nr *= 2;
+  if (sh.rows_cl == 1) return 1;
+  if (sh.rows_cl < 0)
+    while (nr > 1 && (long)nrows < 2L * 152 * nr) nr /= 2;
+  return nr;
+}
+
 template <int P>
 cudaError_t launch_rows_P(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s) {
   using PL = Plan32<P>;
-  // rows per block: up to 256 C items and 48 KB, fewer while the launch would
-  // not give every SM two blocks; a row alone takes threads for the A items too
-  const int nrows = B * g.Mz;
-  const int cap = (w.shapes && w.shapes->rows_threads > 0) ? std::min(256, w.shapes->rows_threads) : 256;
-  int nr = 1;
-  while (nr < kMaxRows && 2 * nr * PL::NK <= cap && 2 * nr * PL::row_bytes <= 48 * 1024) nr *= 2;
-  const int form = w.shapes ? w.shapes->rows_cl : -1;
-  if (form == 1)
-    nr = 1;
-  else if (form < 0)
-    while (nr > 1 && (long)nrows < 2L * 152 * nr) nr /= 2;
+  const int nrows = B * g.Mz, nr = per_block<P>(w.shapes ? *w.shapes : Shapes{}, nrows);
   const unsigned blocks = (unsigned)((nrows + nr - 1) / nr);
   const float* Z = reinterpret_cast<const float*>(w.Z);
   float* Q = reinterpret_cast<float*>(w.Q);
@@ -457,6 +458,15 @@ cudaError_t configure_rows_f32(const Grid& g) {
 #undef X
   }
   return cudaErrorInvalidValue;
+}
+
+int rows_f32_per_block(const Grid& g, const Shapes& sh, int B) {
+  switch (g.nm) {
+#define X(P) case 1 << P: return per_block<P>(sh, B * g.Mz);
+    RBC_ROWS_CASES(X)
+#undef X
+  }
+  return 0;
 }
 
 cudaError_t launch_rows_f32(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s) {

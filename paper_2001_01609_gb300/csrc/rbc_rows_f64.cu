@@ -423,15 +423,23 @@ cudaError_t configure_rows_f64(const Grid& g) {
   return e;
 }
 
+void rows_f64_form(const Grid& g, const Shapes& sh, int B, int* cl, int* threads, int* lean) {
+  *cl = sh.rows_cl >= 0 ? sh.rows_cl : use_cluster(g, B);
+  *threads = 0;
+  *lean = -1;
+  if (*cl) return;
+  *threads = sh.rows_threads > 0 ? sh.rows_threads : kRowsThreads;
+  if (rows_f64_batched(g)) *lean = sh.rows_lean >= 0 ? sh.rows_lean : lean_default(g);
+}
+
 cudaError_t launch_rows_f64(const Grid& g, const Tables& t, const Work& w, int B, const int* ns, cudaStream_t s) {
-  const Shapes sh = w.shapes ? *w.shapes : Shapes{};
-  if (sh.rows_cl >= 0 ? sh.rows_cl != 0 : use_cluster(g, B))
+  int cl, threads, lean;
+  rows_f64_form(g, w.shapes ? *w.shapes : Shapes{}, B, &cl, &threads, &lean);
+  if (cl)
     return launch_pdl(w.pdl != 0, k_rows_cl, (unsigned)(B * g.Mz * kRowsCluster), kRowsThreads, rows_f64_cl_bytes(g), s,
                       g, t.tw, w.Z, w.Q, w.wT, B, ns, w.step);
-  const bool lean = sh.rows_lean >= 0 ? sh.rows_lean != 0 : lean_default(g);
-  return launch_pdl(w.pdl != 0, k_rows, (unsigned)(B * g.Mz), sh.rows_threads > 0 ? sh.rows_threads : kRowsThreads,
-                    rows_f64_bytes(g, lean), s, g, t.tw, w.Z, w.Q, w.wT, B, rows_f64_batched(g) ? 1 : 0, lean ? 1 : 0,
-                    ns, w.step);
+  return launch_pdl(w.pdl != 0, k_rows, (unsigned)(B * g.Mz), threads, rows_f64_bytes(g, lean == 1), s, g, t.tw, w.Z,
+                    w.Q, w.wT, B, rows_f64_batched(g) ? 1 : 0, lean == 1 ? 1 : 0, ns, w.step);
 }
 
 }  // namespace rbc

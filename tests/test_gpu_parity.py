@@ -423,6 +423,17 @@ def test_autotuned_shapes_give_identical_bits(rbc, precision, Nx, Nz, B):
     assert F.check_diverged() == T.check_diverged() == rbc.RBC_OK
 
 
+@pytest.mark.parametrize("precision", [1, 2])
+def test_autotune_picks_only_shapes_that_have_an_effect(rbc, precision):
+    """A mixed handle from Nz = 64 on has no z-forward tile, row-kernel block size or layout to choose: a trial of one
+    would repeat the launch that it is compared with, and timer noise decide."""
+    F = rbc.Propagator(2e4, 1.0, 2.0, 64, 64, 2e-4, precision)
+    for B in (1, 3, 12):
+        F.autotune(B)
+        _, tm, nch, _, threads, lean = F.tuned_shapes(B)
+        assert (tm, nch, threads, lean) == (0, 0, 0, -1)
+
+
 @pytest.mark.parametrize("precision,Nx,Nz,B", [(0, 32, 16, 6), (1, 64, 64, 3), (2, 128, 64, 2), (1, 256, 64, 4)])
 def test_pinned_launch_shapes_give_identical_bits(rbc, precision, Nx, Nz, B):
     """rbc_set_shapes: every valid combination of the row kernel's form, block
