@@ -142,13 +142,13 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_rows_f64.cu",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "ff1eeb63723cae373579ebbfe62b9b22d41d13fbcb281a2cb8e2086cb049db81"
+NCU_TRAFFIC_SHA256 = "05c4fecffa11faf7877d4e5225e9d9d129a767977d7e7ee2ed71f37daa8ab100"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 129229, "coarse:k_rows": 483686, "coarse:k_zfwd": 116096, "coarse:k_solve": 802368,
-    "fine:k_zinv@32": 8584294, "fine:k_rows@32": 56754278, "fine:k_zfwd@32": 12619328, "fine:k_solve@32": 23582400,
+    "coarse:k_zinv": 128717, "coarse:k_rows": 483379, "coarse:k_zfwd": 116096, "coarse:k_solve": 801856,
+    "fine:k_zinv@32": 8590234, "fine:k_rows@32": 56717875, "fine:k_zfwd@32": 12619776, "fine:k_solve@32": 23579200,
     # batch of 2 with the heuristic shapes (the clustered row kernel; the tuned one-block-per-row
     # kernel reads and writes the same rows)
-    "fine:k_zinv@2": 665344, "fine:k_rows@2": 3586970, "fine:k_zfwd@2": 820928, "fine:k_solve@2": 2428800,
+    "fine:k_zinv@2": 662579, "fine:k_rows@2": 3584563, "fine:k_zfwd@2": 820992, "fine:k_solve@2": 2431680,
 }
 
 

@@ -222,9 +222,11 @@ __device__ __forceinline__ void zinv_item(const Grid& g, const T* __restrict__ B
     asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(t) : "l"(Bz + (size_t)(lane * g.Mz + j) * g.Nz + min(2 * p0, g.Nz - 1)));
   }
   pdl_wait();
-  // small grids look at whether the state is active once its values are on their way
+  // a state or two alone look at whether they are active once their values are on their
+  // way; in a batch the blocks hide each other's latency, and states that have taken
+  // their steps shall cost nothing
   const int now = nsteps ? *step : 0, last = nsteps ? nsteps[b] : 1;   // (the grid is exact: b < B)
-  if (kp == 1 && now >= last) return;
+  if ((kp == 1 || B > kPdlMaxBatch) && now >= last) return;
   V E[6], O[6];
 #pragma unroll
   for (int q = 0; q < 6; ++q) E[q] = O[q] = mk2<T>(0, 0);
@@ -383,6 +385,7 @@ __device__ __forceinline__ void zfwd_item(const Grid& g, const T* __restrict__ W
   }
   pdl_wait();
   const int now = nsteps ? *step : 0, last = nsteps ? nsteps[b] : 1;   // (the grid is exact: b < B)
+  if (B > kPdlMaxBatch && now >= last) return;                         // as in zinv_item
   const size_t qs = (size_t)g.Mz * g.nm * 2;
   const T* q = Q + (size_t)(b * 2 + f) * qs;
   const int ltm = __ffs(tm) - 1;             // tm is a power of two
