@@ -484,7 +484,7 @@ static rbc_status upload_tables(rbc_t h) {
   std::vector<size_t> offs;
   auto add = [&](const std::vector<double>& v) {
     size_t o = buf.size();
-    o = (o + 1) & ~(size_t)1;   // 16-byte alignment for double2 loads
+    o = (o + 31) & ~(size_t)31;   // 256 bytes: whole cache lines, whatever tables a mode leaves out
     buf.resize(o);
     buf.insert(buf.end(), v.begin(), v.end());
     offs.push_back(o);
