@@ -1,11 +1,12 @@
 """The transform kernels at the edges of their sizes, against the FP64 oracle.
 
-One step of every row length (Nx = 4 .. 1024: one, two and three passes per
-FFT) and batch size (several rows per block, a ragged last block), and of the
-column lengths around the groups, chunks and segments of the z sums and stage
-solves, in batches that take each split of a row pair, alone and together.
-Tolerances: FP64 1e-12 relative to the largest coefficient, ten times the
-largest difference of the two implementations' roundings seen on these grids;
+One step of every row length (Nx = 4 .. 1024: odd and even numbers of radix-4
+steps, rows in shared memory together and in turn) and batch size (a cluster or
+a block per row, several rows per block, a ragged last block), and of column
+lengths up to the largest, around the dense solve's limit, the chunks of the
+recurrences and the tensor-core tiles, alone and in batches of other tilings.
+Tolerances: FP64 1e-12 relative to the largest coefficient (the
+implementations' roundings differ by up to 2e-15 in one step of the tall grids);
 FP32 products 1e-5, the bound of the mixed mode's parity tests.
 """
 import numpy as np
@@ -53,7 +54,7 @@ def test_every_row_length_matches_oracle(rbc, Nx, precision, tol):
         assert abs(nu[b].item() - integ) <= tol * max(abs(integ), 1e-30)
 
 
-@pytest.mark.parametrize("Nz", [8, 16, 18, 32, 34, 36, 64, 66, 128, 130, 258])
+@pytest.mark.parametrize("Nz", [8, 16, 18, 32, 34, 36, 64, 66, 128, 130, 258, 384, 510, 512])
 def test_column_lengths_match_oracle_and_batches_agree(rbc, Nz, Nx=8):
     Ra, dt = 1e4, 1e-5
     o = RBC(Ra, 1.0, 2.0, Nx, Nz, dt)
@@ -77,7 +78,8 @@ def test_column_lengths_match_oracle_and_batches_agree(rbc, Nz, Nx=8):
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("Nx", [4, 8, 16, 32, 64, 128, 256, 512, 1024])
 def test_rows_alone_and_in_batches_agree(rbc, Nx, precision, Nz=10):
-    """15 rows (one per block, every pass spread), 345 and 2250 rows (several per block, a ragged last one)."""
+    """15 rows (FP64: a cluster each; mixed: one per block, the last inverse pass spread), 345 and 2250 rows (FP64: a
+    block each; mixed: several per block, a ragged last one)."""
     F = rbc.Propagator(1e5, 1.0, 2.0, Nx, Nz, 1e-4, precision)
     o = RBC(1e5, 1.0, 2.0, Nx, Nz, 1e-4)
     alone = F.new_states(1)
@@ -93,10 +95,11 @@ def test_rows_alone_and_in_batches_agree(rbc, Nx, precision, Nz=10):
 
 
 @pytest.mark.parametrize("precision", [1, 2])
-@pytest.mark.parametrize("Nz", [34, 62, 64, 66, 96, 128, 130, 256, 258])
+@pytest.mark.parametrize("Nz", [34, 62, 64, 66, 96, 128, 130, 256, 258, 384, 510, 512])
 def test_mixed_column_lengths_match_oracle_and_batches_agree(rbc, Nz, precision, Nx=16):
     """K-chunks and row tiles of the tensor-core transforms (one per CTA alone, all of a field's in batches), rows per
-    thread and chunks of the stage solve; above Nz = 256 the FP32 CUDA-core transforms."""
+    thread and chunks of the stage solve; the FP32 CUDA-core transforms where TF32 operands do not fit (Nz = 384: the
+    inverse, 510 and 512: both)."""
     Ra, dt = 1e4, 1e-5
     o = RBC(Ra, 1.0, 2.0, Nx, Nz, dt)
     F = rbc.Propagator(Ra, 1.0, 2.0, Nx, Nz, dt, precision)
