@@ -142,13 +142,13 @@ NCU_TRAFFIC_SOURCES = (
     "paper_2001_01609_gb300/csrc/rbc_rows_f64.cu",
     "paper_2001_01609_gb300/csrc/rbc_internal.h",
 )
-NCU_TRAFFIC_SHA256 = "05c4fecffa11faf7877d4e5225e9d9d129a767977d7e7ee2ed71f37daa8ab100"
+NCU_TRAFFIC_SHA256 = "156344432593751fb1438ff6e4b1e9f117687d863e41746817f4f12dc60aff05"
 NCU_TRAFFIC = {
-    "coarse:k_zinv": 128717, "coarse:k_rows": 483379, "coarse:k_zfwd": 116096, "coarse:k_solve": 801856,
-    "fine:k_zinv@32": 8590234, "fine:k_rows@32": 56717875, "fine:k_zfwd@32": 12619776, "fine:k_solve@32": 23579200,
+    "coarse:k_zinv": 129382, "coarse:k_rows": 483430, "coarse:k_zfwd": 116352, "coarse:k_solve": 801856,
+    "fine:k_zinv@32": 8577485, "fine:k_rows@32": 56725914, "fine:k_zfwd@32": 12640448, "fine:k_solve@32": 23583232,
     # batch of 2 with the heuristic shapes (the clustered row kernel; the tuned one-block-per-row
     # kernel reads and writes the same rows)
-    "fine:k_zinv@2": 662579, "fine:k_rows@2": 3584563, "fine:k_zfwd@2": 820992, "fine:k_solve@2": 2431680,
+    "fine:k_zinv@2": 670515, "fine:k_rows@2": 3586509, "fine:k_zfwd@2": 820736, "fine:k_solve@2": 2429952,
 }
 
 

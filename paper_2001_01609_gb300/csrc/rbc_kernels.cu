@@ -217,14 +217,15 @@ __device__ __forceinline__ void zinv_item(const Grid& g, const T* __restrict__ B
   const int npair = g.Nz / 2;
   const int per = (npair + kp - 1) / kp;
   const int p0 = w * per, p1 = min(npair, p0 + per);
-  if (kp > 1 && lane < 4) {   // the warp's table entries into L1 while the launch before this one finishes
+  if (kp > 1 && B <= kPdlMaxBatch && lane < 4) {   // table entries into L1 while the launch before this one finishes
     float t;
     asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(t) : "l"(Bz + (size_t)(lane * g.Mz + j) * g.Nz + min(2 * p0, g.Nz - 1)));
   }
   pdl_wait();
   // a state or two alone look at whether they are active once their values are on their
   // way; in a batch the blocks hide each other's latency, and states that have taken
-  // their steps shall cost nothing
+  // their steps shall cost nothing (64 x 32, 23 states of 0 to 9 steps, all launches in
+  // FP64: 2904 us, 3121 with the values of all states loaded first; even steps alike)
   const int now = nsteps ? *step : 0, last = nsteps ? nsteps[b] : 1;   // (the grid is exact: b < B)
   if ((kp == 1 || B > kPdlMaxBatch) && now >= last) return;
   V E[6], O[6];
@@ -378,7 +379,7 @@ __device__ __forceinline__ void zfwd_item(const Grid& g, const T* __restrict__ W
   const int mi = threadIdx.x & (tm - 1), n0 = threadIdx.x / tm;
   const int nper = (g.Nz + nch - 1) / nch;
   const int nlo = ch * nper, nhi = min(g.Nz, nlo + nper);
-  {   // the first table row into L1 while the launch before this one finishes
+  if (B <= kPdlMaxBatch) {   // the first table row into L1 while the launch before this one finishes
     float t;
     const T* wr = W + (size_t)min(nlo + n0, g.Nz - 1) * g.Mz;
     for (int jh = mi * 32; jh < Mh; jh += tm * 32) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(t) : "l"(wr + jh));

@@ -398,12 +398,16 @@ size_t rows_f64_cl_bytes(const Grid& g) {
 }
 
 namespace {
-// The lean layout by default where the full one leaves room for a single block
-// per SM and the lean one for two.
+// The lean layout by default where the full one leaves room for a single block per SM
+// and the lean one for two (512 x 128: one state 107 us, 115 in the full layout; 16
+// states 1057 and 1194).
 bool lean_default(const Grid& g) {
   return rows_f64_batched(g) && batched_bytes(g) > 113 * 1024 && lean_bytes(g) <= 113 * 1024;
 }
-// A cluster per row up to two rows per SM, where a block per row would leave SMs idle.
+// A cluster per row up to two rows per SM, where a block per row leaves SMs idle: a
+// first choice, of which the autotuner times the other side (64 x 32, one state 18.2
+// us, 19.5 with a block per row; 512 x 128, one state 105 and 107; but 256 x 64, one
+// state 41.4 and 36.5, three states 72 and 56).
 bool use_cluster(const Grid& g, int B) { return (long)B * g.Mz <= 2L * 152 && rows_f64_cl_bytes(g) <= 200 * 1024; }
 
 // The dynamic shared-memory allowances only ever grow, so that a later handle
